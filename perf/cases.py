@@ -312,7 +312,8 @@ def _scan_points(c, seed):
                              torch.arange(runs, device=DEV), right=True).sub_(1).clamp_(0, ns - 1)
     reach = patches * min(1.0, 100.0 / c["box"])
     pick = t[who, 0] / c["box"] * patches + (2.0 * _uniform(g, runs) - 1.0) * reach
-    pick = pick.long().clamp_(0, patches - 1)
+    pick = pick.long().abs_()  # reflected at both ends
+    pick = torch.where(pick >= patches, 2 * patches - 1 - pick, pick).clamp_(0, patches - 1)
     scan = torch.repeat_interleave(torch.arange(ns, device=DEV), per)
     pts = torch.empty(n, 3, dtype=F64, device=DEV)
     step = 1 << 24
