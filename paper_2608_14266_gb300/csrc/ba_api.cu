@@ -507,7 +507,7 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   }
 
   // iteration buffers
-  h->n_cost = voxel_pass_blocks(n_voxels);
+  h->n_cost = h->mixed ? voxel_pass_blocks(n_voxels) : voxel_pass_f64_blocks(n_voxels);
   h->poses2 = (double*)dev_alloc(h, h->keep, sizeof(double) * 24 * (size_t)n_scans);
   h->planes2 = (double*)dev_alloc(h, h->keep, sizeof(double) * 2 * kPlaneStride * (size_t)n_voxels);
   h->gH = (double*)dev_alloc(h, h->keep, sizeof(double) * kGH * (size_t)n_scans);
@@ -940,7 +940,7 @@ ba_status ba_shard_trial(ba_handle* h, double* trial_cost) {
                          h->mixed ? h->mb.stab2 : nullptr, h->stream),
      "solve");
   CK(h, voxel_pass(h, nullptr, 1, -1), "trial voxel pass");
-  CK(h, launch_shard_cost(h->L, h->cost_part, h->d_shard, h->stream), "trial cost");
+  CK(h, launch_shard_cost(h->cost_part, h->n_cost, h->d_shard, h->stream), "trial cost");
   h->launches += 4;
   CK(h, cudaMemcpyAsync(trial_cost, h->d_shard, sizeof(double), cudaMemcpyDeviceToHost, h->stream), "read cost");
   CK(h, cudaStreamSynchronize(h->stream), "synchronize");
@@ -1210,7 +1210,7 @@ ba_status refresh(ba_batch* b) {
   for (size_t k = 0; k < n; ++k) {
     const ba_handle* h = b->jobs[k];
     views[k] = job_view(h);
-    pre[k + 1] = pre[k] + voxel_pass_blocks(h->L.n_voxels);
+    pre[k + 1] = pre[k] + h->n_cost;
     pre[(n + 1) + k + 1] = pre[(n + 1) + k] + h->L.n_scans;
     pre[2 * (n + 1) + k + 1] = pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans);
   }

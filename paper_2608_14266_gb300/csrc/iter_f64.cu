@@ -8,10 +8,12 @@
 namespace mmba {
 
 // ---------------------------------------------------------------------------
-// Voxel pass: one thread per voxel over the SELL-32 slices.
+// Voxel pass: a block of 128 threads takes kV voxels (a slice or a part of
+// one) of the SELL-32 slices, 128 / kV threads to a voxel, each thread every
+// (128 / kV)-th of the voxel's observations.
 //
 // For voxel i with observations o = (i, j): q_o = R_j m_o + t_j is the posed
-// cluster mean; with an anchor a (the first q_o of the voxel) the thread sums
+// cluster mean; with an anchor a (the first q_o of the voxel) the threads sum
 //   n = sum N_o,  s = sum N_o (q_o - a),  M = sum [R_j S_o R_j^T + N_o (q_o - a)(q_o - a)^T]
 // so that the centroid is c = a + s / n and the world-point covariance of
 // Eq. 1 is A = M / n - (c - a)(c - a)^T.  The anchor keeps the subtraction
@@ -19,33 +21,56 @@ namespace mmba {
 // slot's pivoted LDL^T of S_o (ldlt3_pivoted): 61 FP64 operations per
 // observation instead of 76 with S itself.  Then lambda_min(A) and its
 // eigenvector give the plane (u, d = u^T c); the voxel's cost is lambda_min.
+//
+// Bound: the FP64 pipe, which a warp instruction holds for 64 cycles of its
+// scheduler whatever the number of its active lanes.  A voxel's observations
+// are therefore a chain of ~80 such instructions each, and a problem of a few
+// hundred voxels with one thread per voxel is that chain on a few warps.
+// Splitting a voxel over the block's warps shortens it; the 3x3 eigenproblem
+// (~250 instructions) runs once per voxel, in one warp of the block (warp
+// blk % 4, so that the four schedulers share them).  Against one thread per
+// voxel: 118 -> 32 us at 200 voxels, 258 -> 206 us at 50,000, 2.01 -> 1.97 ms
+// at 500,000 (15M observations).
 // ---------------------------------------------------------------------------
-template <bool kFull>
+template <int kV, bool kFull>
 __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const double* __restrict__ poses2,
                                                     double* __restrict__ planes2, double* __restrict__ full_out,
                                                     double* __restrict__ cost_part,
                                                     const double* __restrict__ pred_part, DevState* __restrict__ st,
                                                     int use_trial, int decide_mode, int64_t blk, double* red,
-                                                    int* is_last) {
+                                                    double (*sums)[10][32], int* is_last) {
+  static_assert(kVoxelThreads == 128 && (kV == 8 || kV == 16 || kV == 32), "four warps per block");
   if (st->honor_stop && st->stop) {
     // a stopped solve takes no step, so no gradient is pending either
     if (decide_mode == 0 && blk == 0 && threadIdx.x == 0) st->scan_pending = 0;
     return;
   }
+  constexpr int kRows = kVoxelThreads / kV;  // threads per voxel
   const int buf = use_trial ? 1 - st->cur : st->cur;
   const double* __restrict__ poses = poses2 + (int64_t)buf * L.n_scans * 12;
   double* __restrict__ planes = planes2 + (int64_t)buf * L.n_voxels * kPlaneStride;
-  const int64_t p = blk * kVoxelThreads + threadIdx.x;
-  double lam0 = 0.0;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t p = blk * kV + (threadIdx.x & (kV - 1));
+  // the sums n, s, M of this thread's observations
+  double acc[10] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  double ax = 0.0, ay = 0.0, az = 0.0;
   if (p < L.n_voxels) {
-    const int64_t s = p >> 5;
-    const int lane = (int)(p & 31);
     const int len = L.vlen[p];
-    const int64_t base = L.slice_off[s] + lane;
+    const int64_t base = L.slice_off[p >> 5] + (p & 31);
     const int64_t ne = L.n_elems;
-    double n = 0.0, ax = 0.0, ay = 0.0, az = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-    double m00 = 0.0, m01 = 0.0, m02 = 0.0, m11 = 0.0, m12 = 0.0, m22 = 0.0;
-    for (int k = 0; k < len; ++k) {
+    const int k0 = threadIdx.x / kV;
+    if (k0 < len || w == (int)(blk & 3)) {
+      // the anchor: the first observation's posed mean, formed by every thread
+      const uint32_t sv = (uint32_t)__ldg(L.ve_scan + base);
+      int p0, p1, p2;
+      perm_decode(sv >> kPermShift, p0, p1, p2);
+      const double* __restrict__ P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
+      const double m0 = __ldg(L.ve + 6 * ne + base), m1 = __ldg(L.ve + 7 * ne + base), m2 = __ldg(L.ve + 8 * ne + base);
+      ax = fma(P[p0], m0, fma(P[p1], m1, fma(P[p2], m2, P[9])));
+      ay = fma(P[3 + p0], m0, fma(P[3 + p1], m1, fma(P[3 + p2], m2, P[10])));
+      az = fma(P[6 + p0], m0, fma(P[6 + p1], m1, fma(P[6 + p2], m2, P[11])));
+    }
+    for (int k = k0; k < len; k += kRows) {
       const int64_t e = base + (int64_t)k * kSlice;
       const uint32_t sv = (uint32_t)__ldg(L.ve_scan + e);
       int p0, p1, p2;
@@ -62,11 +87,6 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
       const double qx = fma(a0, m0, fma(b0, m1, fma(c0, m2, P[9])));
       const double qy = fma(a1, m0, fma(b1, m1, fma(c1, m2, P[10])));
       const double qz = fma(a2, m0, fma(b2, m1, fma(c2, m2, P[11])));
-      if (k == 0) {
-        ax = qx;
-        ay = qy;
-        az = qz;
-      }
       const double dx = qx - ax, dy = qy - ay, dz = qz - az;
       // R S R^T = sum_a D_a W_a W_a^T with W = R P^T L
       const double w00 = fma(l10, b0, fma(l20, c0, a0)), w01 = fma(l10, b1, fma(l20, c1, a1)),
@@ -76,48 +96,89 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
       const double u10 = D1 * w10, u11 = D1 * w11, u12 = D1 * w12;
       const double u20 = D2 * c0, u21 = D2 * c1, u22 = D2 * c2;
       const double Nx = N * dx, Ny = N * dy, Nz = N * dz;
-      m00 = fma(u00, w00, fma(u10, w10, fma(u20, c0, fma(Nx, dx, m00))));
-      m01 = fma(u00, w01, fma(u10, w11, fma(u20, c1, fma(Nx, dy, m01))));
-      m02 = fma(u00, w02, fma(u10, w12, fma(u20, c2, fma(Nx, dz, m02))));
-      m11 = fma(u01, w01, fma(u11, w11, fma(u21, c1, fma(Ny, dy, m11))));
-      m12 = fma(u01, w02, fma(u11, w12, fma(u21, c2, fma(Ny, dz, m12))));
-      m22 = fma(u02, w02, fma(u12, w12, fma(u22, c2, fma(Nz, dz, m22))));
-      sx += Nx;
-      sy += Ny;
-      sz += Nz;
-      n += N;
+      acc[4] = fma(u00, w00, fma(u10, w10, fma(u20, c0, fma(Nx, dx, acc[4]))));
+      acc[5] = fma(u00, w01, fma(u10, w11, fma(u20, c1, fma(Nx, dy, acc[5]))));
+      acc[6] = fma(u00, w02, fma(u10, w12, fma(u20, c2, fma(Nx, dz, acc[6]))));
+      acc[7] = fma(u01, w01, fma(u11, w11, fma(u21, c1, fma(Ny, dy, acc[7]))));
+      acc[8] = fma(u01, w02, fma(u11, w12, fma(u21, c2, fma(Ny, dz, acc[8]))));
+      acc[9] = fma(u02, w02, fma(u12, w12, fma(u22, c2, fma(Nz, dz, acc[9]))));
+      acc[1] += Nx;
+      acc[2] += Ny;
+      acc[3] += Nz;
+      acc[0] += N;
     }
-    const double inv = 1.0 / n;
-    const double cx = sx * inv, cy = sy * inv, cz = sz * inv;  // centroid - anchor
-    double A[6] = {fma(-cx, cx, m00 * inv), fma(-cx, cy, m01 * inv), fma(-cx, cz, m02 * inv),
-                   fma(-cy, cy, m11 * inv), fma(-cy, cz, m12 * inv), fma(-cz, cz, m22 * inv)};
-    double lam[3], V[9];
-    eig3_sym(A, lam, V);
-    const double ux = V[0], uy = V[1], uz = V[2];
-    const double Cx = ax + cx, Cy = ay + cy, Cz = az + cz;
-    double* pl = planes + p * kPlaneStride;
-    pl[0] = ux;
-    pl[1] = uy;
-    pl[2] = uz;
-    pl[3] = fma(ux, Cx, fma(uy, Cy, uz * Cz));
-    if (kFull) {
-      double* f = full_out + 9 * (int64_t)L.vperm[p];
-      f[0] = lam[0];
-      f[1] = lam[1];
-      f[2] = lam[2];
-      f[3] = ux;
-      f[4] = uy;
-      f[5] = uz;
-      f[6] = Cx;
-      f[7] = Cy;
-      f[8] = Cz;
-    }
-    lam0 = lam[0];
   }
-  const double tot = block_sum<kVoxelThreads>(lam0, red);
-  if (threadIdx.x == 0) cost_part[blk] = tot;
-  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_blocks(L.n_voxels), pred_part, solve_blocks(L.n_scans), st,
-                                   decide_mode, red, is_last);
+  // a voxel's threads of one warp (kV < 32), then of the four warps, in a fixed order
+#pragma unroll
+  for (int o = 16; o >= kV; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < 10; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+  if (lane < kV)
+#pragma unroll
+    for (int q = 0; q < 10; ++q) sums[w][q][lane] = acc[q];
+  __syncthreads();
+  if (w == (int)(blk & 3)) {
+    double lam0 = 0.0;
+    if (lane < kV && p < L.n_voxels) {
+#pragma unroll
+      for (int q = 0; q < 10; ++q)
+        acc[q] = (sums[0][q][lane] + sums[1][q][lane]) + (sums[2][q][lane] + sums[3][q][lane]);
+      const double inv = 1.0 / acc[0];
+      const double cx = acc[1] * inv, cy = acc[2] * inv, cz = acc[3] * inv;  // centroid - anchor
+      double A[6] = {fma(-cx, cx, acc[4] * inv), fma(-cx, cy, acc[5] * inv), fma(-cx, cz, acc[6] * inv),
+                     fma(-cy, cy, acc[7] * inv), fma(-cy, cz, acc[8] * inv), fma(-cz, cz, acc[9] * inv)};
+      double lam[3], V[9];
+      eig3_sym(A, lam, V);
+      const double ux = V[0], uy = V[1], uz = V[2];
+      const double Cx = ax + cx, Cy = ay + cy, Cz = az + cz;
+      double* pl = planes + p * kPlaneStride;
+      pl[0] = ux;
+      pl[1] = uy;
+      pl[2] = uz;
+      pl[3] = fma(ux, Cx, fma(uy, Cy, uz * Cz));
+      if (kFull) {
+        double* f = full_out + 9 * (int64_t)L.vperm[p];
+        f[0] = lam[0];
+        f[1] = lam[1];
+        f[2] = lam[2];
+        f[3] = ux;
+        f[4] = uy;
+        f[5] = uz;
+        f[6] = Cx;
+        f[7] = Cy;
+        f[8] = Cz;
+      }
+      lam0 = lam[0];
+    }
+#pragma unroll
+    for (int o = kV / 2; o > 0; o >>= 1) lam0 += __shfl_down_sync(0xffffffffu, lam0, o);
+    if (lane == 0) cost_part[blk] = lam0;
+  }
+  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_f64_blocks(L.n_voxels), pred_part, solve_blocks(L.n_scans),
+                                   st, decide_mode, red, is_last, (int)(blk & 3) * 32);
+}
+
+// the body for a problem of this size (voxel_pass_f64_width)
+template <bool kFull>
+__device__ __forceinline__ void voxel_pass_f64_sized(const DevLayout& L, const double* poses2, double* planes2,
+                                                     double* full_out, double* cost_part, const double* pred_part,
+                                                     DevState* st, int use_trial, int decide_mode, int64_t blk) {
+  __shared__ double red[kVoxelThreads / 32];
+  __shared__ double sums[kVoxelThreads / 32][10][32];
+  __shared__ int is_last;
+  switch (voxel_pass_f64_width(L.n_voxels)) {
+    case 8:
+      voxel_pass_f64_body<8, kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
+                                    blk, red, sums, &is_last);
+      break;
+    case 16:
+      voxel_pass_f64_body<16, kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
+                                     blk, red, sums, &is_last);
+      break;
+    default:
+      voxel_pass_f64_body<32, kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
+                                     blk, red, sums, &is_last);
+  }
 }
 
 template <bool kFull>
@@ -128,20 +189,16 @@ __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_kernel(DevLayout
                                                                       const double* __restrict__ pred_part,
                                                                       DevState* __restrict__ st, int use_trial,
                                                                       int decide_mode) {
-  __shared__ double red[kVoxelThreads / 32];
-  __shared__ int is_last;
-  voxel_pass_f64_body<kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
-                             blockIdx.x, red, &is_last);
+  voxel_pass_f64_sized<kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
+                              blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_batch_kernel(const __grid_constant__ JobGroup G,
                                                                              int use_trial) {
-  __shared__ double red[kVoxelThreads / 32];
-  __shared__ int is_last;
   const int job = find_job(G.vblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  voxel_pass_f64_body<false>(J.L, J.poses2, J.planes2, nullptr, J.cost_part, J.pred_part, J.st, use_trial,
-                             use_trial ? 0 : 1, (int64_t)blockIdx.x - G.vblk[job], red, &is_last);
+  voxel_pass_f64_sized<false>(J.L, J.poses2, J.planes2, nullptr, J.cost_part, J.pred_part, J.st, use_trial,
+                              use_trial ? 0 : 1, (int64_t)blockIdx.x - G.vblk[job]);
 }
 
 // ---------------------------------------------------------------------------
@@ -161,7 +218,7 @@ __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_batch_kernel(con
 __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const double* __restrict__ poses2,
                                                    const double* __restrict__ planes2, double* __restrict__ gH,
                                                    const DevState* __restrict__ st, int force, int j,
-                                                   double (*red)[kGH]) {
+                                                   double (*red)[32]) {
   // a rejected step (or an iteration after the solve stopped) leaves g, H unchanged
   if (!force && !st->scan_pending) return;
   const int buf = st->cur;
@@ -171,10 +228,11 @@ __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const dou
   const double r00 = P[0], r01 = P[1], r02 = P[2], r10 = P[3], r11 = P[4], r12 = P[5], r20 = P[6], r21 = P[7],
                r22 = P[8];
   const double tx = P[9], ty = P[10], tz = P[11];
-  double acc[kGH];
+  // the 27 sums, then those of w_a m'_a (exact Hessian's diagonal), padded to
+  // a warp for the reduce-scatter
+  double acc[32];
 #pragma unroll
-  for (int k = 0; k < kGH; ++k) acc[k] = 0.0;
-  double dg0 = 0.0, dg1 = 0.0, dg2 = 0.0;  // sums of w_a m'_a (exact Hessian's diagonal)
+  for (int k = 0; k < 32; ++k) acc[k] = 0.0;
   const int64_t lo = L.scan_off[j], hi = L.scan_off[j + 1];
   const int64_t no = L.n_obs;
   for (int64_t o = lo + threadIdx.x; o < hi; o += kScanThreads) {
@@ -220,15 +278,15 @@ __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const dou
     acc[17] = fma(wx, b21, fma(-wy, b20, acc[17]));
     if (!gn) {
       // exact term sym(w m'^T) - (w . m') I: the off-diagonal halves go into
-      // the sums here, the diagonal products into dg (the trace is taken off
-      // once per thread after the loop, as the term is linear)
+      // the sums here, the diagonal products into sums of their own (the trace
+      // is taken off once per scan, as the term is linear)
       const double hx = 0.5 * mpx, hy = 0.5 * mpy, hz = 0.5 * mpz;
       acc[7] = fma(wx, hy, fma(hx, wy, acc[7]));
       acc[8] = fma(wx, hz, fma(hx, wz, acc[8]));
       acc[13] = fma(wy, hz, fma(hy, wz, acc[13]));
-      dg0 = fma(wx, mpx, dg0);
-      dg1 = fma(wy, mpy, dg1);
-      dg2 = fma(wz, mpz, dg2);
+      acc[27] = fma(wx, mpx, acc[27]);
+      acc[28] = fma(wy, mpy, acc[28]);
+      acc[29] = fma(wz, mpz, acc[29]);
     }
     // rotation-translation block: N (m x w) w^T
     const double cx = Nmy * wz - Nmz * wy, cy = Nmz * wx - Nmx * wz, cz = Nmx * wy - Nmy * wx;
@@ -250,62 +308,60 @@ __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const dou
     acc[25] += Nwy * wz;
     acc[26] += N * wz * wz;
   }
-  if (!gn) {
-    const double tr = dg0 + dg1 + dg2;
-    acc[6] += dg0 - tr;
-    acc[12] += dg1 - tr;
-    acc[17] += dg2 - tr;
-  }
-  // deterministic block reduction
+  // Deterministic block reduction, then the rotation to the world frame, one
+  // output entry per lane of warp 0.  On the FP64 pipe these cost what their
+  // warp instructions are, however few lanes they hold: 31 + 3 additions and
+  // ~20 operations of the rotation (a butterfly per sum and one thread's
+  // rotation of the whole 6x6, ~1,000 instructions a scan, were 16% of the
+  // pass at 1,500 observations a scan and most of it at 100: 3.43 -> 2.88 ms
+  // at 10,000 scans of 1,500, 31 -> 16 us at 40 scans of 120).
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < kGH; ++k) {
-    double v = acc[k];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (l == 0) red[w][k] = v;
-  }
+  warp_reduce_scatter32(acc);
+  red[w][l] = acc[0];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double a[kGH];
+  if (w != 0) return;
+  double tot = red[0][l];
 #pragma unroll
-    for (int k = 0; k < kGH; ++k) {
-      double v = 0.0;
+  for (int q = 1; q < kScanThreads / 32; ++q) tot += red[q][l];
+  __syncwarp();
+  red[0][l] = tot;
+  if (l < 9) red[1][l] = P[l];
+  __syncwarp();
+  const double* a = red[0];
+  const double* R = red[1];
+  double* out = gH + (int64_t)j * kGH;
+  if (l < 6) {
+    const int b = l / 3, r = l % 3;
+    out[l] = fma(R[3 * r], a[3 * b], fma(R[3 * r + 1], a[3 * b + 1], R[3 * r + 2] * a[3 * b + 2]));
+  } else if (l < kGH) {
+    // entry (r, c) of the upper triangle: its 3x3 block B of the scan frame's 6x6 as R B R^T
+    int r = 0, rem = l - 6;
+    while (rem >= 6 - r) {
+      rem -= 6 - r;
+      ++r;
+    }
+    const int c = r + rem;
+    const int br = r / 3, bc = c / 3, rr = r % 3, cc = c % 3;
+    const double tr = br + bc == 0 ? a[27] + a[28] + a[29] : 0.0;
+    double v = 0.0;
 #pragma unroll
-      for (int q = 0; q < kScanThreads / 32; ++q) v += red[q][k];
-      a[k] = v;
-    }
-    // scan-frame 6x6 (upper triangle layout of acc[6..26], row-major over the 6x6)
-    double Hs[6][6];
-    int idx = 6;
-    for (int r = 0; r < 6; ++r)
-      for (int c = r; c < 6; ++c) {
-        Hs[r][c] = a[idx];
-        Hs[c][r] = a[idx];
-        ++idx;
+    for (int x = 0; x < 3; ++x) {
+      double t = 0.0;
+#pragma unroll
+      for (int y = 0; y < 3; ++y) {
+        int i = 3 * br + x, k = 3 * bc + y;
+        if (i > k) {
+          const int s = i;
+          i = k;
+          k = s;
+        }
+        double h = a[6 + 6 * i - i * (i - 1) / 2 + (k - i)];
+        if (x == y && br + bc == 0) h += a[27 + x] - tr;
+        t = fma(h, R[3 * cc + y], t);
       }
-    const double R[3][3] = {{r00, r01, r02}, {r10, r11, r12}, {r20, r21, r22}};
-    double* out = gH + (int64_t)j * kGH;
-    for (int r = 0; r < 3; ++r) {
-      out[r] = R[r][0] * a[0] + R[r][1] * a[1] + R[r][2] * a[2];
-      out[3 + r] = R[r][0] * a[3] + R[r][1] * a[4] + R[r][2] * a[5];
+      v = fma(R[3 * rr + x], t, v);
     }
-    // world blocks: R B R^T for each 3x3 block of Hs
-    double Hw[6][6];
-    for (int br = 0; br < 2; ++br)
-      for (int bc = 0; bc < 2; ++bc) {
-        double T[3][3];
-        for (int r = 0; r < 3; ++r)
-          for (int c = 0; c < 3; ++c)
-            T[r][c] = R[r][0] * Hs[3 * br + 0][3 * bc + c] + R[r][1] * Hs[3 * br + 1][3 * bc + c] +
-                      R[r][2] * Hs[3 * br + 2][3 * bc + c];
-        for (int r = 0; r < 3; ++r)
-          for (int c = 0; c < 3; ++c)
-            Hw[3 * br + r][3 * bc + c] = T[r][0] * R[c][0] + T[r][1] * R[c][1] + T[r][2] * R[c][2];
-      }
-    idx = 6;
-    for (int r = 0; r < 6; ++r)
-      for (int c = r; c < 6; ++c) out[idx++] = 0.5 * (Hw[r][c] + Hw[c][r]);
+    out[l] = v;
   }
 }
 
@@ -313,12 +369,12 @@ __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_kernel(DevLayout L
                                                                     const double* __restrict__ planes2,
                                                                     double* __restrict__ gH,
                                                                     const DevState* __restrict__ st, int force) {
-  __shared__ double red[kScanThreads / 32][kGH];
+  __shared__ double red[kScanThreads / 32][32];
   scan_pass_f64_body(L, poses2, planes2, gH, st, force, MMBA_IDX(scan_of_block(L, blockIdx.x), L.n_scans, st), red);
 }
 
 __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const __grid_constant__ JobGroup G) {
-  __shared__ double red[kScanThreads / 32][kGH];
+  __shared__ double red[kScanThreads / 32][32];
   const int job = find_job(G.sblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
   scan_pass_f64_body(J.L, J.poses2, J.planes2, J.gH, J.st, 0,
@@ -473,7 +529,7 @@ __global__ void __launch_bounds__(kDecideThreads) shard_decide_kernel(const doub
 cudaError_t launch_voxel_pass_f64(const DevLayout& L, const double* poses2, double* planes2, double* full_out,
                                   double* cost_part, const double* pred_part, DevState* st, int use_trial,
                                   int decide_mode, cudaStream_t stream) {
-  const int64_t nb = voxel_pass_blocks(L.n_voxels);
+  const int64_t nb = voxel_pass_f64_blocks(L.n_voxels);
   if (full_out)
     voxel_pass_f64_kernel<true><<<(unsigned)nb, kVoxelThreads, 0, stream>>>(L, poses2, planes2, full_out, cost_part,
                                                                             pred_part, st, use_trial, decide_mode);
@@ -490,8 +546,8 @@ cudaError_t launch_scan_pass_f64(const DevLayout& L, const double* poses2, const
   return cudaGetLastError();
 }
 
-cudaError_t launch_shard_cost(const DevLayout& L, const double* cost_part, double* out, cudaStream_t stream) {
-  shard_cost_kernel<<<1, kDecideThreads, 0, stream>>>(cost_part, voxel_pass_blocks(L.n_voxels), out);
+cudaError_t launch_shard_cost(const double* cost_part, int64_t n_cost, double* out, cudaStream_t stream) {
+  shard_cost_kernel<<<1, kDecideThreads, 0, stream>>>(cost_part, n_cost, out);
   return cudaGetLastError();
 }
 

@@ -798,15 +798,16 @@ __device__ inline double strided_sum(const double* __restrict__ p, int64_t n) {
 // At the level with offset o, the lanes with bit o set keep the upper half of
 // their remaining values and receive it from the partner lane, the others
 // keep and receive the lower half.
-__device__ __forceinline__ void warp_reduce_scatter32(float (&a)[32]) {
+template <typename T>
+__device__ __forceinline__ void warp_reduce_scatter32(T (&a)[32]) {
   const int l = threadIdx.x & 31;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const bool up = (l & o) != 0;
 #pragma unroll
     for (int k = 0; k < o; ++k) {
-      const float send = up ? a[k] : a[k + o];
-      const float keep = up ? a[k + o] : a[k];
+      const T send = up ? a[k] : a[k + o];
+      const T keep = up ? a[k + o] : a[k];
       a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
     }
   }
@@ -946,14 +947,14 @@ __device__ __forceinline__ void decide_apply(DevState* st, double csum, double p
 // the block that brings the counter to n_cost sums all partials (in the same
 // fixed order as a separate decision launch, so results do not depend on which
 // block finishes last), decides, and re-arms the counter.  mode as for
-// decide_body; with mode < 0 nothing is decided.
+// decide_body; with mode < 0 nothing is decided.  leader is the thread that
+// wrote the block's partial.
 template <int kThreads>
 __device__ __forceinline__ void voxel_pass_decide(const double* cost_part, int64_t n_cost, const double* pred_part,
                                                   int64_t n_pred, DevState* st, int mode, double* red,
-                                                  int* is_last) {
+                                                  int* is_last, int leader = 0) {
   if (mode < 0) return;
-  __syncthreads();  // thread 0 has written this block's partial
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == leader) {
     __threadfence();
     const unsigned prev = atomicAdd(&st->blocks_done, 1u);
     *is_last = prev == (unsigned)(n_cost - 1);

@@ -15,6 +15,22 @@ constexpr int kDecideThreads = 256;  // one block; FP64 sums are 1/64 rate, so f
 constexpr int kSolveThreads = 64;  // FP64-serial per scan: small blocks spread the scans over every SM
 
 __host__ __device__ inline int64_t voxel_pass_blocks(int64_t n_voxels) { return (n_voxels + kVoxelThreads - 1) / kVoxelThreads; }
+// FP64 voxel pass: voxels per block of kVoxelThreads (a part of a 32-voxel
+// slice; the rest of the block's threads share the voxels' observations).
+// Fewer voxels per block spread a small problem over more of the FP64 pipes;
+// the price is the eigenproblem's warp, which then holds fewer voxels.
+// Measured (us per pass, 8-40 observations per voxel, event-timed; 8 / 16 / 32
+// voxels per block, and one thread per voxel before):
+//     200 voxels   32 /  37 /  47   (118)      9,728   85 /  66 /  64   (121)
+//   2,432          37 /  38 /  49   (121)     19,456  149 / 116 /  97   (129)
+//   4,864          47 /  43 /  49   (120)     50,000  344 / 245 / 206   (258)
+__host__ __device__ inline int voxel_pass_f64_width(int64_t n_voxels) {
+  return n_voxels <= 2432 ? 8 : n_voxels <= 6144 ? 16 : 32;
+}
+__host__ __device__ inline int64_t voxel_pass_f64_blocks(int64_t n_voxels) {
+  const int v = voxel_pass_f64_width(n_voxels);
+  return (n_voxels + v - 1) / v;
+}
 __host__ __device__ inline int64_t solve_blocks(int64_t n_scans) { return (n_scans + kSolveThreads - 1) / kSolveThreads; }
 
 // ---- batched launches over a job group (one launch per kind for the group's jobs) ----
@@ -39,7 +55,7 @@ cudaError_t launch_scan_pass_f64(const DevLayout& L, const double* poses2, const
 // sref/stab2 non-null: also write the trial FP32 scan table (mixed precision)
 // voxel-sharded solve: this handle's summed trial cost into *out (device);
 // the LM decision from the total trial cost over all shards
-cudaError_t launch_shard_cost(const DevLayout& L, const double* cost_part, double* out, cudaStream_t stream);
+cudaError_t launch_shard_cost(const double* cost_part, int64_t n_cost, double* out, cudaStream_t stream);
 cudaError_t launch_shard_decide(const DevLayout& L, const double* pred_part, DevState* st, double trial_total,
                                 cudaStream_t stream);
 cudaError_t launch_solve_f64(const DevLayout& L, double* poses2, const double* gH, double* pred_part, DevState* st,
