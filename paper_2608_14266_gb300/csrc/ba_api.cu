@@ -248,17 +248,18 @@ void fill_stats(const DevState& s, double cost_before, int32_t iters_call, ba_st
 
 // Voxel pass with the decision folded into its last block (decide_mode as
 // for launch_voxel_pass_*).
-cudaError_t voxel_pass(ba_handle* h, double* full, int use_trial, int decide_mode) {
+// dependent: an iteration's launch (launch_dependent).
+cudaError_t voxel_pass(ba_handle* h, double* full, int use_trial, int decide_mode, bool dependent = false) {
   if (h->mixed)
     return launch_voxel_pass_mixed(h->L, h->X, full, h->cost_part, h->pred_part, h->d_state, use_trial, decide_mode,
-                                   h->stream);
+                                   h->stream, dependent);
   return launch_voxel_pass_f64(h->L, h->poses2, h->planes2, full, h->cost_part, h->pred_part, h->d_state, use_trial,
-                               decide_mode, h->stream);
+                               decide_mode, h->stream, dependent);
 }
 
-cudaError_t scan_pass(ba_handle* h, int force) {
+cudaError_t scan_pass(ba_handle* h, int force, bool dependent = false) {
   if (h->mixed) return launch_scan_pass_mixed(h->L, h->X, h->poses2, h->gH, h->d_state, force, h->stream);
-  return launch_scan_pass_f64(h->L, h->poses2, h->planes2, h->gH, h->d_state, force, h->stream);
+  return launch_scan_pass_f64(h->L, h->poses2, h->planes2, h->gH, h->d_state, force, h->stream, dependent);
 }
 
 ba_status evaluate_current(ba_handle* h) {
@@ -290,19 +291,29 @@ cudaError_t prof_end(ba_handle* h, size_t idx) {
   return cudaEventRecord(h->ev_pool[idx + 1], h->stream);
 }
 
+// The solve may start under the scan pass's tail (launch_dependent) in FP64,
+// and in the mixed path up to this many observations, whose copies L2 holds:
+// a solve block that starts early keeps its SM from changing between the
+// scan pass's split of shared memory and L1 and the voxel pass's, which at
+// larger sizes costs the voxel pass its L1.  Measured, us an iteration without
+// / with: 58.3 / 56.3 at 0.6M observations, 90.7 / 88.6 at 2.4M, 145.4 / 147.9
+// at 4.8M, 307 / 319 at 15M.
+constexpr int64_t kDependentSolveObs = 2500000;
+
 ba_status launch_iteration(ba_handle* h) {
+  const bool early_solve = !h->mixed || h->L.n_obs <= kDependentSolveObs;
   size_t ev = 0;
   CK(h, prof_begin(h, BA_KERNEL_SOLVE, &ev), "event");
   CK(h, launch_solve_f64(h->L, h->poses2, h->gH, h->pred_part, h->d_state, h->mixed ? h->mb.sref : nullptr,
-                         h->mixed ? h->mb.stab2 : nullptr, h->stream),
+                         h->mixed ? h->mb.stab2 : nullptr, h->stream, early_solve),
      "solve");
   CK(h, prof_end(h, ev), "event");
   CK(h, prof_begin(h, BA_KERNEL_VOXEL_PASS, &ev), "event");
   // the trial cost and the LM decision (in the pass's last block)
-  CK(h, voxel_pass(h, nullptr, 1, 0), "trial voxel pass");
+  CK(h, voxel_pass(h, nullptr, 1, 0, true), "trial voxel pass");
   CK(h, prof_end(h, ev), "event");
   CK(h, prof_begin(h, BA_KERNEL_SCAN_PASS, &ev), "event");
-  CK(h, scan_pass(h, 0), "scan pass");
+  CK(h, scan_pass(h, 0, true), "scan pass");
   CK(h, prof_end(h, ev), "event");
   h->launches += 3;
   return BA_OK;

@@ -33,13 +33,17 @@ namespace mmba {
 // at 500,000 (15M observations).
 // ---------------------------------------------------------------------------
 template <int kV, bool kFull>
-__device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const double* __restrict__ poses2,
-                                                    double* __restrict__ planes2, double* __restrict__ full_out,
-                                                    double* __restrict__ cost_part,
-                                                    const double* __restrict__ pred_part, DevState* __restrict__ st,
-                                                    int use_trial, int decide_mode, int64_t blk, double* red,
+__device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const double* poses2, double* planes2,
+                                                    double* full_out, double* cost_part, const double* pred_part,
+                                                    DevState* st, int use_trial, int decide_mode, int64_t blk, double* red,
                                                     double (*sums)[10][32], int* is_last) {
   static_assert(kVoxelThreads == 128 && (kV == 8 || kV == 16 || kV == 32), "four warps per block");
+  const int64_t p = blk * kV + (threadIdx.x & (kV - 1));
+  const int len = p < L.n_voxels ? L.vlen[p] : 0;
+  const int64_t base = p < L.n_voxels ? L.slice_off[p >> 5] + (p & 31) : 0;
+  grid_wait();
+  grid_launch_next();
+  st = after_wait(st);
   if (st->honor_stop && st->stop) {
     // a stopped solve takes no step, so no gradient is pending either
     if (decide_mode == 0 && blk == 0 && threadIdx.x == 0) st->scan_pending = 0;
@@ -47,16 +51,13 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
   }
   constexpr int kRows = kVoxelThreads / kV;  // threads per voxel
   const int buf = use_trial ? 1 - st->cur : st->cur;
-  const double* __restrict__ poses = poses2 + (int64_t)buf * L.n_scans * 12;
-  double* __restrict__ planes = planes2 + (int64_t)buf * L.n_voxels * kPlaneStride;
+  const double* poses = after_wait(poses2) + (int64_t)buf * L.n_scans * 12;
+  double* planes = planes2 + (int64_t)buf * L.n_voxels * kPlaneStride;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t p = blk * kV + (threadIdx.x & (kV - 1));
   // the sums n, s, M of this thread's observations
   double acc[10] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   double ax = 0.0, ay = 0.0, az = 0.0;
   if (p < L.n_voxels) {
-    const int len = L.vlen[p];
-    const int64_t base = L.slice_off[p >> 5] + (p & 31);
     const int64_t ne = L.n_elems;
     const int k0 = threadIdx.x / kV;
     if (k0 < len || w == (int)(blk & 3)) {
@@ -64,7 +65,7 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
       const uint32_t sv = (uint32_t)__ldg(L.ve_scan + base);
       int p0, p1, p2;
       perm_decode(sv >> kPermShift, p0, p1, p2);
-      const double* __restrict__ P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
+      const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
       const double m0 = __ldg(L.ve + 6 * ne + base), m1 = __ldg(L.ve + 7 * ne + base), m2 = __ldg(L.ve + 8 * ne + base);
       ax = fma(P[p0], m0, fma(P[p1], m1, fma(P[p2], m2, P[9])));
       ay = fma(P[3 + p0], m0, fma(P[3 + p1], m1, fma(P[3 + p2], m2, P[10])));
@@ -75,7 +76,7 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
       const uint32_t sv = (uint32_t)__ldg(L.ve_scan + e);
       int p0, p1, p2;
       perm_decode(sv >> kPermShift, p0, p1, p2);
-      const double* __restrict__ P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
+      const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
       const double l10 = __ldg(L.ve + e), l20 = __ldg(L.ve + ne + e), l21 = __ldg(L.ve + 2 * ne + e);
       const double D0 = __ldg(L.ve + 3 * ne + e), D1 = __ldg(L.ve + 4 * ne + e), D2 = __ldg(L.ve + 5 * ne + e);
       const double m0 = __ldg(L.ve + 6 * ne + e), m1 = __ldg(L.ve + 7 * ne + e), m2 = __ldg(L.ve + 8 * ne + e);
@@ -182,13 +183,10 @@ __device__ __forceinline__ void voxel_pass_f64_sized(const DevLayout& L, const d
 }
 
 template <bool kFull>
-__global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_kernel(DevLayout L, const double* __restrict__ poses2,
-                                                                      double* __restrict__ planes2,
-                                                                      double* __restrict__ full_out,
-                                                                      double* __restrict__ cost_part,
-                                                                      const double* __restrict__ pred_part,
-                                                                      DevState* __restrict__ st, int use_trial,
-                                                                      int decide_mode) {
+__global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_kernel(DevLayout L, const double* poses2,
+                                                                      double* planes2, double* full_out,
+                                                                      double* cost_part, const double* pred_part,
+                                                                      DevState* st, int use_trial, int decide_mode) {
   voxel_pass_f64_sized<kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
                               blockIdx.x);
 }
@@ -215,15 +213,18 @@ __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_batch_kernel(con
 // S and N.  The world-frame blocks are R (.) R^T.  Gauss-Newton mode drops
 // the (w m'^T + m' w^T)/2 - (w^T m') I term.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const double* __restrict__ poses2,
-                                                   const double* __restrict__ planes2, double* __restrict__ gH,
-                                                   const DevState* __restrict__ st, int force, int j,
+__device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const double* poses2, const double* planes2,
+                                                   double* gH, const DevState* st, int force, int j,
                                                    double (*red)[32]) {
+  const int64_t lo = L.scan_off[j], hi = L.scan_off[j + 1];
+  grid_wait();
+  grid_launch_next();
+  st = after_wait(st);
   // a rejected step (or an iteration after the solve stopped) leaves g, H unchanged
   if (!force && !st->scan_pending) return;
   const int buf = st->cur;
-  const double* __restrict__ P = poses2 + ((int64_t)buf * L.n_scans + j) * 12;
-  const double* __restrict__ planes = planes2 + (int64_t)buf * L.n_voxels * kPlaneStride;
+  const double* P = after_wait(poses2) + ((int64_t)buf * L.n_scans + j) * 12;
+  const double* planes = after_wait(planes2) + (int64_t)buf * L.n_voxels * kPlaneStride;
   const bool gn = st->hess_mode != 0;
   const double r00 = P[0], r01 = P[1], r02 = P[2], r10 = P[3], r11 = P[4], r12 = P[5], r20 = P[6], r21 = P[7],
                r22 = P[8];
@@ -233,7 +234,6 @@ __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const dou
   double acc[32];
 #pragma unroll
   for (int k = 0; k < 32; ++k) acc[k] = 0.0;
-  const int64_t lo = L.scan_off[j], hi = L.scan_off[j + 1];
   const int64_t no = L.n_obs;
   for (int64_t o = lo + threadIdx.x; o < hi; o += kScanThreads) {
     const double4_32a pl =
@@ -365,10 +365,9 @@ __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const dou
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_pass_f64_kernel(DevLayout L, const double* __restrict__ poses2,
-                                                                    const double* __restrict__ planes2,
-                                                                    double* __restrict__ gH,
-                                                                    const DevState* __restrict__ st, int force) {
+__global__ void __launch_bounds__(kScanThreads) scan_pass_f64_kernel(DevLayout L, const double* poses2,
+                                                                    const double* planes2, double* gH,
+                                                                    const DevState* st, int force) {
   __shared__ double red[kScanThreads / 32][32];
   scan_pass_f64_body(L, poses2, planes2, gH, st, force, MMBA_IDX(scan_of_block(L, blockIdx.x), L.n_scans, st), red);
 }
@@ -389,8 +388,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const
 // ---------------------------------------------------------------------------
 // *stepped = false: the pose is kept (fixed scan, no observation, failed
 // factorisation); otherwise dlt holds the increment.
-__device__ inline double solve_scan(const DevLayout& L, int j, const double* __restrict__ P, double* __restrict__ Pt,
-                                    const double* __restrict__ gH, DevState* st, double* dlt, bool* stepped) {
+__device__ inline double solve_scan(const DevLayout& L, int j, const double* P, double* Pt, const double* gH,
+                                    DevState* st, double* dlt, bool* stepped) {
   *stepped = false;
   const double* a = gH + (int64_t)j * kGH;
   // a scan nobody observes keeps its pose: no observation in this handle's
@@ -447,10 +446,14 @@ __device__ inline double solve_scan(const DevLayout& L, int j, const double* __r
 // written too, from the trial pose and the scan's reference pose.  Block blk
 // (scans blk * kSolveThreads ..) writes the sum of its scans' predicted
 // reductions to pred_part[blk], in a fixed order.
-__device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* __restrict__ poses2,
-                                               const double* __restrict__ gH, double* __restrict__ pred_part,
-                                               DevState* st, const double* __restrict__ sref,
-                                               float* __restrict__ stab2, int64_t blk, double* red) {
+__device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* poses2, const double* gH,
+                                               double* pred_part, DevState* st, const double* sref, float* stab2,
+                                               int64_t blk, double* red) {
+  grid_wait();
+  grid_launch_next();
+  st = after_wait(st);
+  gH = after_wait(gH);
+  poses2 = after_wait(poses2);
   if (st->honor_stop && st->stop) return;  // uniform over the block
   const int64_t j = blk * kSolveThreads + threadIdx.x;
   double pred = 0.0;
@@ -464,7 +467,7 @@ __device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* __res
     if (stab2) {
       // FP64 quaternion of the trial dR: the step's Exp composed onto the
       // current one (no matrix-to-quaternion conversion per step)
-      double* sq2 = sq2_of(sref, L.n_scans);
+      double* sq2 = after_wait(sq2_of(sref, L.n_scans));
       const double* qc = sq2 + ((int64_t)cur * L.n_scans + j) * 4;
       double* qt = sq2 + ((int64_t)(1 - cur) * L.n_scans + j) * 4;
       double qn[4];
@@ -483,11 +486,9 @@ __device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* __res
   if (threadIdx.x == 0) pred_part[blk] = tot;
 }
 
-__global__ void __launch_bounds__(kSolveThreads) solve_f64_kernel(DevLayout L, double* __restrict__ poses2,
-                                                                 const double* __restrict__ gH,
-                                                                 double* __restrict__ pred_part, DevState* st,
-                                                                 const double* __restrict__ sref,
-                                                                 float* __restrict__ stab2) {
+__global__ void __launch_bounds__(kSolveThreads) solve_f64_kernel(DevLayout L, double* poses2, const double* gH,
+                                                                 double* pred_part, DevState* st, const double* sref,
+                                                                 float* stab2) {
   __shared__ double red[kSolveThreads / 32];
   solve_f64_body(L, poses2, gH, pred_part, st, sref, stab2, blockIdx.x, red);
 }
@@ -528,22 +529,17 @@ __global__ void __launch_bounds__(kDecideThreads) shard_decide_kernel(const doub
 
 cudaError_t launch_voxel_pass_f64(const DevLayout& L, const double* poses2, double* planes2, double* full_out,
                                   double* cost_part, const double* pred_part, DevState* st, int use_trial,
-                                  int decide_mode, cudaStream_t stream) {
-  const int64_t nb = voxel_pass_f64_blocks(L.n_voxels);
-  if (full_out)
-    voxel_pass_f64_kernel<true><<<(unsigned)nb, kVoxelThreads, 0, stream>>>(L, poses2, planes2, full_out, cost_part,
-                                                                            pred_part, st, use_trial, decide_mode);
-  else
-    voxel_pass_f64_kernel<false><<<(unsigned)nb, kVoxelThreads, 0, stream>>>(L, poses2, planes2, nullptr, cost_part,
-                                                                             pred_part, st, use_trial, decide_mode);
-  return cudaGetLastError();
+                                  int decide_mode, cudaStream_t stream, bool dependent) {
+  return launch_dependent(full_out ? voxel_pass_f64_kernel<true> : voxel_pass_f64_kernel<false>,
+                          voxel_pass_f64_blocks(L.n_voxels), kVoxelThreads, stream, dependent, L, poses2, planes2,
+                          full_out, cost_part, pred_part, st, use_trial, decide_mode);
 }
 
 cudaError_t launch_scan_pass_f64(const DevLayout& L, const double* poses2, const double* planes2, double* gH,
-                                 const DevState* st, int force, cudaStream_t stream) {
+                                 const DevState* st, int force, cudaStream_t stream, bool dependent) {
   if (L.n_scans == 0) return cudaSuccess;
-  scan_pass_f64_kernel<<<(unsigned)L.n_scans, kScanThreads, 0, stream>>>(L, poses2, planes2, gH, st, force);
-  return cudaGetLastError();
+  return launch_dependent(scan_pass_f64_kernel, L.n_scans, kScanThreads, stream, dependent, L, poses2, planes2, gH, st,
+                          force);
 }
 
 cudaError_t launch_shard_cost(const double* cost_part, int64_t n_cost, double* out, cudaStream_t stream) {
@@ -558,10 +554,9 @@ cudaError_t launch_shard_decide(const DevLayout& L, const double* pred_part, Dev
 }
 
 cudaError_t launch_solve_f64(const DevLayout& L, double* poses2, const double* gH, double* pred_part, DevState* st,
-                             const double* sref, float* stab2, cudaStream_t stream) {
-  solve_f64_kernel<<<(unsigned)solve_blocks(L.n_scans), kSolveThreads, 0, stream>>>(L, poses2, gH, pred_part, st, sref,
-                                                                                    stab2);
-  return cudaGetLastError();
+                             const double* sref, float* stab2, cudaStream_t stream, bool dependent) {
+  return launch_dependent(solve_f64_kernel, solve_blocks(L.n_scans), kSolveThreads, stream, dependent, L, poses2, gH,
+                          pred_part, st, sref, stab2);
 }
 
 cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double* pred_part, int64_t n_pred,
@@ -571,18 +566,15 @@ cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double*
 }
 
 cudaError_t launch_batch_solve(const JobGroup& T, int64_t n_blocks, cudaStream_t stream) {
-  solve_f64_batch_kernel<<<(unsigned)n_blocks, kSolveThreads, 0, stream>>>(T);
-  return cudaGetLastError();
+  return launch_dependent(solve_f64_batch_kernel, n_blocks, kSolveThreads, stream, false, T);
 }
 
 cudaError_t launch_batch_voxel_pass_f64(const JobGroup& T, int64_t n_blocks, int use_trial, cudaStream_t stream) {
-  voxel_pass_f64_batch_kernel<<<(unsigned)n_blocks, kVoxelThreads, 0, stream>>>(T, use_trial);
-  return cudaGetLastError();
+  return launch_dependent(voxel_pass_f64_batch_kernel, n_blocks, kVoxelThreads, stream, true, T, use_trial);
 }
 
 cudaError_t launch_batch_scan_pass_f64(const JobGroup& T, int64_t n_blocks, cudaStream_t stream) {
-  scan_pass_f64_batch_kernel<<<(unsigned)n_blocks, kScanThreads, 0, stream>>>(T);
-  return cudaGetLastError();
+  return launch_dependent(scan_pass_f64_batch_kernel, n_blocks, kScanThreads, stream, true, T);
 }
 
 }  // namespace mmba

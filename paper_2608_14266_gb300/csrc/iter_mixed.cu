@@ -37,42 +37,54 @@ __device__ __forceinline__ void apply_E(const float* ph, float a, float b, float
 // keeps lambda_min relatively accurate; an FP32 Jacobi in B gives the plane,
 // and B and delta then move to the new eigenvectors and centroid.
 // ---------------------------------------------------------------------------
-template <bool kFull>
+// kDependent: the launch may overlap the tail of the kernel before it
+// (grid_wait).  The batch's launches do not: they are long, and the pointers
+// that a wait pins in registers would spill there.
+template <bool kFull, bool kDependent>
 __device__ __forceinline__ void voxel_pass_mixed_body(const DevLayout& L, const DevMixed& X,
-                                                      double* __restrict__ full_out, double* __restrict__ cost_part,
-                                                      const double* __restrict__ pred_part, DevState* __restrict__ st,
-                                                      int use_trial, int decide_mode, int64_t blk, float* red,
-                                                      double* dred, int* is_last, int pf) {
+                                                      double* full_out, double* cost_part, const double* pred_part,
+                                                      DevState* st, int use_trial, int decide_mode, int64_t blk,
+                                                      float* red, double* dred, int* is_last, int pf) {
+  // what no pass writes, read while the kernel before drains: the voxel's
+  // length and place, its anchor and its first slot
+  const int64_t p = blk * kVoxelThreads + threadIdx.x;
+  const float4* __restrict__ slot = X.ve32;
+  int len = 0;
+  float4 an = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 n0 = an, n1 = an, n2 = an;
+  if (p < L.n_voxels) {
+    len = L.vlen[p];
+    slot += kVe32 * (L.slice_off[p >> 5] + (p & 31));
+    an = X.vanchor[p];
+    if (len > 0) {
+      n0 = __ldg(slot);
+      n1 = __ldg(slot + 1);
+      n2 = __ldg(slot + 2);
+    }
+  }
+  if (kDependent) {
+    grid_wait();
+    grid_launch_next();
+    st = after_wait(st);
+  }
   if (st->honor_stop && st->stop) {
     // a stopped solve takes no step, so no gradient is pending either
     if (decide_mode == 0 && blk == 0 && threadIdx.x == 0) st->scan_pending = 0;
     return;
   }
   const int buf = use_trial ? 1 - st->cur : st->cur;
-  const float* __restrict__ stab = X.stab2 + (int64_t)buf * L.n_scans * kTab;
-  float4* __restrict__ planes = X.planes32_2 + (int64_t)buf * L.n_voxels * 2;
-  const int64_t p = blk * kVoxelThreads + threadIdx.x;
+  const float* stab = (kDependent ? after_wait(X.stab2) : X.stab2) + (int64_t)buf * L.n_scans * kTab;
+  float4* planes = X.planes32_2 + (int64_t)buf * L.n_voxels * 2;
+  float4* vstate = kDependent ? after_wait(X.vstate) : X.vstate;
   float lam0 = 0.f;
   if (p < L.n_voxels) {
-    const int64_t sl = p >> 5;
-    const int lane = (int)(p & 31);
-    const int len = L.vlen[p];
-    const int64_t base = L.slice_off[sl] + lane;
-    const float4 an = X.vanchor[p];
-    const float4 qb = X.vstate[2 * p];
-    const float4 dw = X.vstate[2 * p + 1];
+    const float4 qb = vstate[2 * p];
+    const float4 dw = vstate[2 * p + 1];
     float B[9];
     quat_to_mat_f(qb.x, qb.y, qb.z, qb.w, B);
     float n = 0.f, s0 = 0.f, s1 = 0.f, s2 = 0.f;
     float m00 = 0.f, m01 = 0.f, m02 = 0.f, m11 = 0.f, m12 = 0.f, m22 = 0.f;
     // the slot of observation k + 1 (three 128-bit loads) is fetched while k is processed
-    const float4* __restrict__ slot = X.ve32 + kVe32 * base;
-    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0;
-    if (len > 0) {
-      n0 = __ldg(slot);
-      n1 = __ldg(slot + 1);
-      n2 = __ldg(slot + 2);
-    }
     for (int k = 0; k < len; ++k) {
       const float4 f0 = n0, f1 = n1, f2 = n2;
       // rows further ahead go to L2 without holding registers (the lanes'
@@ -86,7 +98,8 @@ __device__ __forceinline__ void voxel_pass_mixed_body(const DevLayout& L, const 
       }
       const int j = MMBA_IDX(__float_as_int(f1.w), L.n_scans, st);
       const float4* T4 = reinterpret_cast<const float4*>(stab + (int64_t)j * kTab);
-      const float4 qd = __ldg(T4), t1 = __ldg(T4 + 1), t2 = __ldg(T4 + 2);
+      const float4 qd = kDependent ? T4[0] : __ldg(T4), t1 = kDependent ? T4[1] : __ldg(T4 + 1),
+                   t2 = kDependent ? T4[2] : __ldg(T4 + 2);
       const float ph[3] = {qd.y, qd.z, qd.w};
       const float b0 = f0.x, b1 = f0.y, b2 = f0.z, N = f0.w;
       // posed mean about the latest centroid (world axes), then voxel frame:
@@ -151,8 +164,8 @@ __device__ __forceinline__ void voxel_pass_mixed_body(const DevLayout& L, const 
       }
       float qn[4];
       mat_to_quat<float>(U, qn);
-      X.vstate[2 * p] = make_float4(qn[0], qn[1], qn[2], qn[3]);
-      X.vstate[2 * p + 1] = make_float4(cw0, cw1, cw2, 0.f);
+      vstate[2 * p] = make_float4(qn[0], qn[1], qn[2], qn[3]);
+      vstate[2 * p + 1] = make_float4(cw0, cw1, cw2, 0.f);
     } else {
       double* f = full_out + 9 * (int64_t)L.vperm[p];
       f[0] = lam[0];
@@ -177,15 +190,13 @@ __device__ __forceinline__ void voxel_pass_mixed_body(const DevLayout& L, const 
 
 template <bool kFull>
 __global__ void __launch_bounds__(kVoxelThreads, 6) voxel_pass_mixed_kernel(DevLayout L, DevMixed X,
-                                                                        double* __restrict__ full_out,
-                                                                        double* __restrict__ cost_part,
-                                                                        const double* __restrict__ pred_part,
-                                                                        DevState* __restrict__ st, int use_trial,
-                                                                        int decide_mode) {
+                                                                        double* full_out, double* cost_part,
+                                                                        const double* pred_part, DevState* st,
+                                                                        int use_trial, int decide_mode) {
   __shared__ float red[kVoxelThreads / 32];
   __shared__ double dred[kVoxelThreads / 32];
   __shared__ int is_last;
-  voxel_pass_mixed_body<kFull>(L, X, full_out, cost_part, pred_part, st, use_trial, decide_mode, blockIdx.x, red,
+  voxel_pass_mixed_body<kFull, true>(L, X, full_out, cost_part, pred_part, st, use_trial, decide_mode, blockIdx.x, red,
                                dred, &is_last, kVoxPrefetch);
 }
 
@@ -199,7 +210,7 @@ __global__ void __launch_bounds__(kVoxelThreads, kMinBlocks)
   __shared__ int is_last;
   const int job = find_job(G.vblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  voxel_pass_mixed_body<false>(J.L, J.X, nullptr, J.cost_part, J.pred_part, J.st, use_trial, use_trial ? 0 : 1,
+  voxel_pass_mixed_body<false, false>(J.L, J.X, nullptr, J.cost_part, J.pred_part, J.st, use_trial, use_trial ? 0 : 1,
                                (int64_t)blockIdx.x - G.vblk[job], red, dred, &is_last, pf);
 }
 
@@ -314,9 +325,15 @@ __device__ __forceinline__ void issue_scan_chunk(ScanChunk& S, uint32_t bar, con
 }
 
 __device__ __forceinline__ void scan_pass_mixed_body(const DevLayout& L, const DevMixed& X,
-                                                     double* __restrict__ gH, DevState* __restrict__ st,
-                                                     int force, int j, float (*red)[kGH], float* tot, float* dR,
+                                                     double* __restrict__ gH, DevState* __restrict__ st, int force,
+                                                     int j, float (*red)[kGH], float* tot, float* dR,
                                                      ScanChunk* chunks, uint64_t* bars) {
+  // launched after the voxel pass has drained, not dependent on it: its shared
+  // memory and the voxel pass's L1 want different splits of the SM's memory,
+  // which changes only between blocks (as a dependent launch its first blocks
+  // would settle for the voxel pass's split: 61 -> 73 us an iteration at 0.6M
+  // observations, 307 -> 316 at 15M)
+  grid_launch_next();
   if (!force && !st->scan_pending) return;
   const int lane = threadIdx.x & 31;
   const int buf = st->cur;
@@ -458,8 +475,7 @@ __device__ __forceinline__ void scan_pass_mixed_body(const DevLayout& L, const D
 }
 
 __global__ void __launch_bounds__(kScanMixedThreads, 24) scan_pass_mixed_kernel(DevLayout L, DevMixed X,
-                                                                                  double* __restrict__ gH,
-                                                                                  DevState* __restrict__ st, int force) {
+                                                                                  double* gH, DevState* st, int force) {
   __shared__ float red[1][kGH];
   __shared__ float tot[kGH];
   __shared__ float dR[9];
@@ -509,43 +525,29 @@ __global__ void scan_table_kernel(int32_t n_scans, const double* poses2, const d
 
 cudaError_t launch_voxel_pass_mixed(const DevLayout& L, const DevMixed& X, double* full_out, double* cost_part,
                                     const double* pred_part, DevState* st, int use_trial, int decide_mode,
-                                    cudaStream_t stream) {
-  const int64_t nb = voxel_pass_blocks(L.n_voxels);
-  if (full_out)
-    voxel_pass_mixed_kernel<true><<<(unsigned)nb, kVoxelThreads, 0, stream>>>(L, X, full_out, cost_part, pred_part,
-                                                                              st, use_trial, decide_mode);
-  else
-    voxel_pass_mixed_kernel<false><<<(unsigned)nb, kVoxelThreads, 0, stream>>>(L, X, nullptr, cost_part, pred_part,
-                                                                               st, use_trial, decide_mode);
-  return cudaGetLastError();
+                                    cudaStream_t stream, bool dependent) {
+  return launch_dependent(full_out ? voxel_pass_mixed_kernel<true> : voxel_pass_mixed_kernel<false>,
+                          voxel_pass_blocks(L.n_voxels), kVoxelThreads, stream, dependent, L, X, full_out, cost_part,
+                          pred_part, st, use_trial, decide_mode);
 }
 
 cudaError_t launch_scan_pass_mixed(const DevLayout& L, const DevMixed& X, const double* poses2, double* gH,
                                    DevState* st, int force, cudaStream_t stream) {
   if (L.n_scans == 0) return cudaSuccess;
   (void)poses2;
-  scan_pass_mixed_kernel<<<(unsigned)L.n_scans, kScanMixedThreads, 0, stream>>>(L, X, gH, st, force);
-  return cudaGetLastError();
+  return launch_dependent(scan_pass_mixed_kernel, L.n_scans, kScanMixedThreads, stream, false, L, X, gH, st, force);
 }
 
 cudaError_t launch_batch_voxel_pass_mixed(const JobGroup& T, int64_t n_blocks, int use_trial, cudaStream_t stream,
                                           int min_blocks, int pf) {
-  switch (min_blocks) {
-    case 4:
-      voxel_pass_mixed_batch_kernel<4><<<(unsigned)n_blocks, kVoxelThreads, 0, stream>>>(T, use_trial, pf);
-      break;
-    case 8:
-      voxel_pass_mixed_batch_kernel<8><<<(unsigned)n_blocks, kVoxelThreads, 0, stream>>>(T, use_trial, pf);
-      break;
-    default:
-      voxel_pass_mixed_batch_kernel<6><<<(unsigned)n_blocks, kVoxelThreads, 0, stream>>>(T, use_trial, pf);
-  }
-  return cudaGetLastError();
+  return launch_dependent(min_blocks == 4   ? voxel_pass_mixed_batch_kernel<4>
+                          : min_blocks == 8 ? voxel_pass_mixed_batch_kernel<8>
+                                            : voxel_pass_mixed_batch_kernel<6>,
+                          n_blocks, kVoxelThreads, stream, false, T, use_trial, pf);
 }
 
 cudaError_t launch_batch_scan_pass_mixed(const JobGroup& T, int64_t n_blocks, cudaStream_t stream) {
-  scan_pass_mixed_batch_kernel<<<(unsigned)n_blocks, kScanMixedThreads, 0, stream>>>(T);
-  return cudaGetLastError();
+  return launch_dependent(scan_pass_mixed_batch_kernel, n_blocks, kScanMixedThreads, stream, false, T);
 }
 
 cudaError_t launch_wait_probe(int limit, int32_t* out, cudaStream_t stream) {

@@ -813,6 +813,30 @@ __device__ __forceinline__ void warp_reduce_scatter32(T (&a)[32]) {
   }
 }
 
+// ---- programmatic dependent launch ----
+// The kernels of an iteration are launched so that each may start while the
+// one before it in the stream still drains (launch_dependent): its blocks take
+// the SM slots the last wave leaves idle, read what no kernel of the iteration
+// writes (lengths, offsets, clusters), and wait in grid_wait() until every
+// block of the kernel before has finished and its writes are visible.  Every
+// block calls grid_wait() before it returns, so a finished kernel implies that
+// all kernels before it in the stream have finished too.  grid_launch_next()
+// comes after the wait, so at most one kernel runs ahead.  Both do nothing in
+// a launch without the attribute.  An FP64 iteration of 200 voxels takes 53.7
+// us instead of 58.6 with only its voxel pass launched so.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A pointer to data that the kernels before may write, for use after
+// grid_wait(): loads through it can neither move above the wait nor take the
+// read-only path (pass it by plain, not __restrict__, parameters).
+// (through a global address, so that they stay global, not generic, loads)
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+  size_t g = __cvta_generic_to_global(p);
+  asm volatile("" : "+l"(g)::"memory");
+  return (T*)__cvta_global_to_generic(g);
+}
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- bulk asynchronous copies (TMA engine) into shared memory ----
 // A copy needs 16-byte aligned source and destination and a size that is a
 // multiple of 16; it completes on an mbarrier as transaction bytes.

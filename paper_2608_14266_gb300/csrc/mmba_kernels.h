@@ -33,6 +33,23 @@ __host__ __device__ inline int64_t voxel_pass_f64_blocks(int64_t n_voxels) {
 }
 __host__ __device__ inline int64_t solve_blocks(int64_t n_scans) { return (n_scans + kSolveThreads - 1) / kSolveThreads; }
 
+// Launch of an iteration kernel; with dependent = true it may start while the
+// kernel before it in the stream drains (see grid_wait in mmba_internal.cuh).
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), int64_t blocks, int threads, cudaStream_t stream,
+                                    bool dependent, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- batched launches over a job group (one launch per kind for the group's jobs) ----
 cudaError_t launch_batch_solve(const JobGroup& T, int64_t n_blocks, cudaStream_t stream);
 cudaError_t launch_batch_voxel_pass_f64(const JobGroup& T, int64_t n_blocks, int use_trial, cudaStream_t stream);
@@ -44,14 +61,16 @@ cudaError_t launch_batch_voxel_pass_mixed(const JobGroup& T, int64_t n_blocks, i
 cudaError_t launch_batch_scan_pass_mixed(const JobGroup& T, int64_t n_blocks, cudaStream_t stream);
 
 // ---- iteration (FP64) ----
+// dependent = true: an iteration's launch, which may overlap the tail of the
+// kernel before it (launch_dependent).
 // decide_mode: 0 = LM decision in the launch's last block (an iteration's
 // trial pass), 1 = only install the summed cost (evaluation at the current
 // poses), -1 = no decision (planes for output)
 cudaError_t launch_voxel_pass_f64(const DevLayout& L, const double* poses2, double* planes2, double* full_out,
                                   double* cost_part, const double* pred_part, DevState* st, int use_trial,
-                                  int decide_mode, cudaStream_t stream);
+                                  int decide_mode, cudaStream_t stream, bool dependent = false);
 cudaError_t launch_scan_pass_f64(const DevLayout& L, const double* poses2, const double* planes2, double* gH,
-                                 const DevState* st, int force, cudaStream_t stream);
+                                 const DevState* st, int force, cudaStream_t stream, bool dependent = false);
 // sref/stab2 non-null: also write the trial FP32 scan table (mixed precision)
 // voxel-sharded solve: this handle's summed trial cost into *out (device);
 // the LM decision from the total trial cost over all shards
@@ -59,7 +78,7 @@ cudaError_t launch_shard_cost(const double* cost_part, int64_t n_cost, double* o
 cudaError_t launch_shard_decide(const DevLayout& L, const double* pred_part, DevState* st, double trial_total,
                                 cudaStream_t stream);
 cudaError_t launch_solve_f64(const DevLayout& L, double* poses2, const double* gH, double* pred_part, DevState* st,
-                             const double* sref, float* stab2, cudaStream_t stream);
+                             const double* sref, float* stab2, cudaStream_t stream, bool dependent = false);
 cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double* pred_part, int64_t n_pred,
                           DevState* st, int mode, cudaStream_t stream);
 
@@ -163,7 +182,7 @@ cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBoun
 // ---- mixed precision ----
 cudaError_t launch_voxel_pass_mixed(const DevLayout& L, const DevMixed& X, double* full_out, double* cost_part,
                                     const double* pred_part, DevState* st, int use_trial, int decide_mode,
-                                    cudaStream_t stream);
+                                    cudaStream_t stream, bool dependent = false);
 cudaError_t launch_scan_pass_mixed(const DevLayout& L, const DevMixed& X, const double* poses2, double* gH,
                                    DevState* st, int force, cudaStream_t stream);
 cudaError_t launch_scan_table(int32_t n_scans, const double* poses2, const double* sref, float* stab2, int buf,
