@@ -4,6 +4,7 @@
 // Everything here runs once per load; none of it is on the per-iteration path.
 #include <cfloat>
 
+#include "block_order.cuh"
 #include "mmba_internal.cuh"
 #include "mmba_kernels.h"
 
@@ -758,22 +759,35 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
 //
 // The sums are exact integer sums in fixed point.  An observation's scale is
 // 2^-F with F = 1076 - E0, E0 the largest biased binary exponent of p0's
-// coordinates: p0's largest coordinate then has its last bit at 2^-F, every
-// coordinate of that size or larger (up to 2^9 times) is an exact integer
-// multiple of 2^-F, and smaller ones are rounded to it (an error below half
-// the last bit of p0's largest coordinate, the resolution of FP64 arithmetic
-// on these points).  d, sum d and sum d d^T are then 64- and 128-bit integer
-// sums with no rounding at all, on the integer pipe; GB300's FP64 pipe (1/64
-// of FP32) only converts the nine sums and forms m and S once per
-// observation.  An observation whose points do not fit (a coordinate over 2^9
-// times p0's largest, a spread over 2^56 steps, more than 2^14 points, a
-// first point at the origin, or a scale outside 2^-500 .. 2^500) takes the
-// same shifted sums in FP64.
-// ============================================================================
+// coordinates: half the last bit of p0's largest coordinate.  Every coordinate
+// of that size or larger (up to 2^9 times) is an exact integer multiple of
+// 2^-F, and smaller ones are rounded to it (an error below half the last bit
+// of p0's largest coordinate, the resolution of FP64 arithmetic on these
+// points).  d, sum d and sum d d^T are then 64- and 128-bit integer sums with
+// no rounding at all, on the integer pipe; GB300's FP64 pipe (1/64 of FP32)
+// only forms m and S once per observation.  An observation whose points do not
+// fit (a coordinate over 2^9 times p0's largest, a spread over 2^56 steps,
+// more than 2^14 points, a first point at the origin, or a scale outside
+// 2^-400 .. 2^400) takes the same shifted sums in FP64.
+//
+// Points within 2^54 steps of the first (two metres at one metre's range, 128
+// m at 100 m) take d split at 27 bits into two 32-bit halves, each product of
+// halves in a 64-bit sum of its own, one multiply-add each: 21 a point instead
+// of six 128-bit multiply-adds.  The bounds: both halves are below 2^27 in
+// size, a pair of cross products is below 2^55, and 254 of those below 2^63,
+// the lanes' sums added; longer observations are joined 254 points at a time.
+//
+// A block takes 256 observations in order of their lengths, so that the sixteen
+// of a warp are about as long (a warp runs as long as its longest), and each
+// lane has its next two points on their way while it sums one.
+//
+// Bound: instruction issue (0.56 a cycle; ~176 instructions a point, ~1,400 a
+// warp for the sixteen records) and the loads' latency at 16 warps an SM.
+// Measured, before (128-bit sums, observations in input order) and now:
+// 0.6M observations of 1-64 points 576 -> 265 us, 1M of 32 454 -> 386 us, 0.2M of
+// 100 319 -> 222 us, 3M of 1-8 614 -> 586 us, 60,000 of 200-400 645 -> 267 us.
 constexpr int kAggLanes = 2;
-
-// 2^-F as an FP64 value, for F in [-1022, 1022]
-__device__ __forceinline__ double pow2_neg(int F) { return __hiloint2double((1023 - F) << 20, 0); }
+constexpr int kAggShort = 254;  // points whose sums of halves fit 64 bits (whole lane pairs)
 
 // round(p 2^F) to the nearest integer (halves away from zero); ok is cleared
 // when the result would reach 2^62
@@ -795,14 +809,45 @@ __device__ __forceinline__ long long fix_round(double p, int F, bool& ok) {
   return (b >> 63) ? -(long long)v : (long long)v;
 }
 
-// the nearest FP64 values to the magnitude's two 64-bit halves, combined by
-// one FMA (an error of about one unit in the last place); the sign is set in
-// the bits
-__device__ __forceinline__ double i128_to_double(__int128 v) {
+// v 2^e rounded to the nearest FP64 value, ties to even, in integer
+// arithmetic (the conversions of the hardware run on the FP64 pipe); for
+// |v| < 2^127 and results in the normal range
+__device__ __forceinline__ double i128_scaled(__int128 v, int e) {
   const bool neg = v < 0;
   const unsigned __int128 u = neg ? (unsigned __int128)(-v) : (unsigned __int128)v;
-  const double r = fma((double)(unsigned long long)(u >> 64), 0x1p64, (double)(unsigned long long)u);
-  return __longlong_as_double(__double_as_longlong(r) | ((long long)neg << 63));
+  unsigned long long hi = (unsigned long long)(u >> 64), lo = (unsigned long long)u;
+  if ((hi | lo) == 0) return 0.0;
+  int top = 127;  // exponent of the leading bit
+  if (hi == 0) {
+    hi = lo;
+    lo = 0;
+    top = 63;
+  }
+  const int lz = __clzll((long long)hi);
+  if (lz) {
+    hi = (hi << lz) | (lo >> (64 - lz));
+    lo <<= lz;
+  }
+  top -= lz;
+  unsigned long long m = hi >> 11;  // 53 bits, the leading one included
+  const unsigned rest = (unsigned)hi & 2047u;
+  m += (rest > 1024u || (rest == 1024u && (lo != 0 || (m & 1ull)))) ? 1ull : 0ull;
+  // the leading bit adds one to the exponent field (two where rounding carried out of the fraction)
+  const unsigned long long r = ((unsigned long long)(unsigned)(1022 + top + e) << 52) + m;
+  return __longlong_as_double((long long)(r | ((unsigned long long)neg << 63)));
+}
+
+// the same for |v| < 2^63
+__device__ __forceinline__ double i64_scaled(long long v, int e) {
+  if (v == 0) return 0.0;
+  const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)u);
+  const unsigned long long h = u << lz;
+  const unsigned rest = (unsigned)h & 2047u;
+  unsigned long long m = h >> 11;
+  m += (rest > 1024u || (rest == 1024u && (m & 1ull))) ? 1ull : 0ull;
+  const unsigned long long r = ((unsigned long long)(unsigned)(1022 + 63 - lz + e) << 52) + m;
+  return __longlong_as_double((long long)(r | ((unsigned long long)v & 0x8000000000000000ull)));
 }
 
 __device__ __forceinline__ __int128 shfl_xor_i128(unsigned mask, __int128 v, int lane) {
@@ -829,15 +874,11 @@ __device__ void aggregate_f64(int64_t a, int64_t b, int sub, unsigned mask, cons
     c12 = fma(y, z, c12);
     c22 = fma(z, z, c22);
   }
-  sx += __shfl_xor_sync(mask, sx, 1);
-  sy += __shfl_xor_sync(mask, sy, 1);
-  sz += __shfl_xor_sync(mask, sz, 1);
-  c00 += __shfl_xor_sync(mask, c00, 1);
-  c01 += __shfl_xor_sync(mask, c01, 1);
-  c02 += __shfl_xor_sync(mask, c02, 1);
-  c11 += __shfl_xor_sync(mask, c11, 1);
-  c12 += __shfl_xor_sync(mask, c12, 1);
-  c22 += __shfl_xor_sync(mask, c22, 1);
+  double* sums[9] = {&sx, &sy, &sz, &c00, &c01, &c02, &c11, &c12, &c22};
+#pragma unroll
+  for (int o = 1; o < kAggLanes; o <<= 1)
+#pragma unroll
+    for (int q = 0; q < 9; ++q) *sums[q] += __shfl_xor_sync(mask, *sums[q], o);
   const double n = (double)(b - a);
   const double rn = 1.0 / n;
   const double dx = sx * rn, dy = sy * rn, dz = sz * rn;
@@ -847,7 +888,7 @@ __device__ void aggregate_f64(int64_t a, int64_t b, int sub, unsigned mask, cons
     r[2] = fma(-sx, dz, c02);
     r[3] = fma(-sy, dy, c11);
     r[4] = fma(-sy, dz, c12);
-  } else {
+  } else if (sub == 1) {
     r[5] = fma(-sz, dz, c22);
     r[6] = p0x + dx;
     r[7] = p0y + dy;
@@ -856,14 +897,39 @@ __device__ void aggregate_f64(int64_t a, int64_t b, int sub, unsigned mask, cons
   }
 }
 
-__global__ void aggregate_points_kernel(int64_t n_obs, const int64_t* __restrict__ off,
-                                        const double* __restrict__ pts, double* __restrict__ out) {
-  const int64_t o = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kAggLanes;
-  const int sub = threadIdx.x & (kAggLanes - 1);
-  const unsigned mask = 0x3u << (threadIdx.x & 30);  // the two lanes of this observation
-  if (o >= n_obs) return;  // both lanes of a pair leave together
-  const int64_t a = off[o], b = off[o + 1];
-  double* r = out + 10 * o;
+// 1 / n for a whole n <= 2^14: Newton's iteration for the reciprocal from the
+// binary32 quotient, twice (24 -> 48 -> 53 bits)
+__device__ __forceinline__ double recip_count(double n, float nf) {
+  const double r0 = f32_to_f64(__frcp_rn(nf));
+  const double r1 = fma(r0, fma(-n, r0, 1.0), r0);
+  return fma(r1, fma(-n, r1, 1.0), r1);
+}
+
+// A coordinate in steps of 2^-F as fix_round gives it, for the short sums: no
+// test inside; the largest biased exponent met and the bits of the offsets
+// from X0 are kept in emax and wide and tested once per observation.  sh =
+// 1075 - F, so that the value is mantissa 2^(E - sh).
+__device__ __forceinline__ long long fix_offset(double p, int sh, long long X0, int& emax, unsigned& wide) {
+  const unsigned hi = (unsigned)__double2hiint(p), lo = (unsigned)__double2loint(p);
+  const int E = (int)(hi >> 20) & 0x7ff;
+  emax = max(emax, E);
+  // twice the mantissa, shifted down by at most 63 (zero and subnormal values: E - sh < -63)
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  const int s = E - sh;
+  // at or above the unit: exact; below: rounded to nearest, halves away from zero
+  const unsigned long long v = s >= 0 ? m << (s & 15) : ((m >> min(-s - 1, 63)) + 1ull) >> 1;
+  const long long neg = (long long)((int)hi >> 31);
+  const long long d = (((long long)v ^ neg) - neg) - X0;
+  const int dh = (int)(d >> 32);
+  wide |= (unsigned)(dh ^ (dh >> 31));
+  return d;
+}
+
+// one observation by a pair of lanes (sub = 0, 1; mask = the pair's lanes;
+// totals: five values of this thread's, kOrderBlock apart)
+__device__ __forceinline__ void aggregate_one(int64_t a, int64_t b, int sub, unsigned mask,
+                                              const double* __restrict__ pts, double* __restrict__ r,
+                                              __int128* totals) {
   if (b <= a) {
     for (int k = sub; k < 10; k += kAggLanes) r[k] = 0.0;
     return;
@@ -873,68 +939,203 @@ __global__ void aggregate_points_kernel(int64_t n_obs, const int64_t* __restrict
   E0 = max(E0, (__double2hiint(p0y) >> 20) & 0x7ff);
   E0 = max(E0, (__double2hiint(p0z) >> 20) & 0x7ff);
   const int F = 1076 - E0;
-  bool ok = E0 != 0 && F >= -500 && F <= 500 && b - a <= (1 << 14);
-  const long long X0x = fix_round(p0x, F, ok), X0y = fix_round(p0y, F, ok), X0z = fix_round(p0z, F, ok);
-  __int128 s1x = 0, s1y = 0, s1z = 0, s00 = 0, s01 = 0, s02 = 0, s11 = 0, s12 = 0, s22 = 0;
-  constexpr long long kMaxD = 1ll << 56;
-  for (int64_t k = a + sub; k < b && ok; k += kAggLanes) {
-    const long long dx = fix_round(pts[3 * k], F, ok) - X0x;
-    const long long dy = fix_round(pts[3 * k + 1], F, ok) - X0y;
-    const long long dz = fix_round(pts[3 * k + 2], F, ok) - X0z;
-    ok = ok && dx > -kMaxD && dx < kMaxD && dy > -kMaxD && dy < kMaxD && dz > -kMaxD && dz < kMaxD;
-    s1x += dx;
-    s1y += dy;
-    s1z += dz;
-    s00 += (__int128)dx * dx;
-    s01 += (__int128)dx * dy;
-    s02 += (__int128)dx * dz;
-    s11 += (__int128)dy * dy;
-    s12 += (__int128)dy * dz;
-    s22 += (__int128)dz * dz;
-  }
-  // both lanes take the shuffle (a short-circuit would skip it on one of them)
-  const int partner_ok = __shfl_xor_sync(mask, (int)ok, 1);
-  ok = ok && partner_ok != 0;
-  if (!ok) {
-    aggregate_f64(a, b, sub, mask, pts, r);
-    return;
-  }
-  s1x += shfl_xor_i128(mask, s1x, 1);
-  s1y += shfl_xor_i128(mask, s1y, 1);
-  s1z += shfl_xor_i128(mask, s1z, 1);
-  s00 += shfl_xor_i128(mask, s00, 1);
-  s01 += shfl_xor_i128(mask, s01, 1);
-  s02 += shfl_xor_i128(mask, s02, 1);
-  s11 += shfl_xor_i128(mask, s11, 1);
-  s12 += shfl_xor_i128(mask, s12, 1);
-  s22 += shfl_xor_i128(mask, s22, 1);
-  // Both lanes hold the exact sums.  Each converts five of them and writes
-  // half of the record through one instruction sequence whose operands are
-  // chosen per lane (lane 0: S xx, xy, xz, yy, yz = C - s_a d_b; lane 1: S zz,
-  // then m = p0 + d and N), since GB300 issues an FP64 warp instruction at the
-  // same cost whatever the number of lanes on each side of a branch.
-  const double sc = pow2_neg(F);  // F is in [-500, 500]
-  const double sc2 = sc * sc;
-  const double n = (double)(b - a);
-  const double rn = 1.0 / n;
-  const double sx = i128_to_double(s1x) * sc, sy = i128_to_double(s1y) * sc, sz = i128_to_double(s1z) * sc;
-  const double dx = sx * rn, dy = sy * rn, dz = sz * rn;
-  const bool l0 = sub == 0;
-  const __int128 v[5] = {l0 ? s00 : s22, l0 ? s01 : (__int128)X0x, l0 ? s02 : (__int128)X0y,
-                         l0 ? s11 : (__int128)X0z, l0 ? s12 : (__int128)0};
-  const double A[5] = {l0 ? -sx : -sz, l0 ? -sx : 1.0, l0 ? -sx : 1.0, l0 ? -sy : 1.0, l0 ? -sy : n};
-  const double B[5] = {l0 ? dx : dz, l0 ? dy : dx, l0 ? dz : dy, l0 ? dy : dz, l0 ? dz : 1.0};
-  const double S[5] = {sc2, l0 ? sc2 : sc, l0 ? sc2 : sc, l0 ? sc2 : sc, sc2};
-  double* w = r + 5 * sub;
+  bool fits = E0 != 0 && F >= -400 && F <= 400 && b - a <= (1 << 14);
+  const long long X0x = fix_round(p0x, F, fits), X0y = fix_round(p0y, F, fits), X0z = fix_round(p0z, F, fits);
+  // lane 0 ends with S xx, xy, xz, yy in u[0 .. 3], lane 1 with S yz, zz and
+  // sum d in u[0 .. 4], all exact
+  __int128 u[5] = {0, 0, 0, 0, 0};
+  bool ok = fits;
+#pragma unroll 1
+  for (int64_t a1 = a; ok && a1 < b; a1 += kAggShort) {
+    // h, c, l (products of the high halves, cross products, products of the
+    // low halves) of each entry of S, then sum d; the diagonal entries hold
+    // half their cross products
+    long long v[21];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) w[k] = fma(A[k], B[k], i128_to_double(v[k]) * S[k]);
+    for (int k = 0; k < 21; ++k) v[k] = 0;
+    const double* q = pts + 3 * (a1 + sub);
+    const int n1 = (int)(b - a1 < kAggShort ? b - a1 : kAggShort);
+    const int cnt = (n1 - sub + kAggLanes - 1) / kAggLanes;  // points of this lane
+    const int sh = 1075 - F;
+    int emax = 0;
+    unsigned wide = 0;
+    auto add = [&](double x, double y, double z) {
+      const long long dx = fix_offset(x, sh, X0x, emax, wide);
+      const long long dy = fix_offset(y, sh, X0y, emax, wide);
+      const long long dz = fix_offset(z, sh, X0z, emax, wide);
+      const int xh = (int)(dx >> 27), yh = (int)(dy >> 27), zh = (int)(dz >> 27);
+      const int xl = (int)dx & 0x7ffffff, yl = (int)dy & 0x7ffffff, zl = (int)dz & 0x7ffffff;
+      v[0] += (long long)xh * xh;  // xx
+      v[1] += (long long)xh * xl;
+      v[2] += (long long)xl * xl;
+      v[3] += (long long)xh * yh;  // xy
+      v[4] += (long long)xh * yl;
+      v[4] += (long long)xl * yh;
+      v[5] += (long long)xl * yl;
+      v[6] += (long long)xh * zh;  // xz
+      v[7] += (long long)xh * zl;
+      v[7] += (long long)xl * zh;
+      v[8] += (long long)xl * zl;
+      v[9] += (long long)yh * yh;  // yy
+      v[10] += (long long)yh * yl;
+      v[11] += (long long)yl * yl;
+      v[12] += (long long)yh * zh;  // yz
+      v[13] += (long long)yh * zl;
+      v[13] += (long long)yl * zh;
+      v[14] += (long long)yl * zl;
+      v[15] += (long long)zh * zh;  // zz
+      v[16] += (long long)zh * zl;
+      v[17] += (long long)zl * zl;
+      v[18] += dx;
+      v[19] += dy;
+      v[20] += dz;
+    };
+    double ax = p0x, ay = p0y, az = p0z, bx = p0x, by = p0y, bz = p0z;
+    if (cnt > 0) {
+      ax = q[0];
+      ay = q[1];
+      az = q[2];
+    }
+    if (cnt > 1) {
+      bx = q[3 * kAggLanes];
+      by = q[3 * kAggLanes + 1];
+      bz = q[3 * kAggLanes + 2];
+    }
+    for (int k = 0; k < cnt; k += 2) {
+      q += 6 * kAggLanes;
+      {
+        const double x = ax, y = ay, z = az;
+        if (k + 2 < cnt) {
+          ax = q[0];
+          ay = q[1];
+          az = q[2];
+        }
+        add(x, y, z);
+      }
+      if (k + 1 < cnt) {
+        const double x = bx, y = by, z = bz;
+        if (k + 3 < cnt) {
+          bx = q[3 * kAggLanes];
+          by = q[3 * kAggLanes + 1];
+          bz = q[3 * kAggLanes + 2];
+        }
+        add(x, y, z);
+      }
+    }
+    // every coordinate within 2^9 of p0's largest, every offset below 2^54
+    ok = __all_sync(mask, emax - sh <= 9 && (wide >> 22) == 0u);
+    // lane 0 takes the pair's first 12 sums, lane 1 the other 9
+    long long w[12];
+    const bool up = sub != 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const long long hi = k < 9 ? v[k + 12 < 21 ? k + 12 : 20] : 0;
+      w[k] = (up ? hi : v[k]) + __shfl_xor_sync(mask, up ? v[k] : hi, 1);
+    }
+    auto join = [](long long h, long long c, int cs, long long l) {
+      return ((__int128)h << 54) + ((__int128)c << cs) + (__int128)l;
+    };
+    u[0] = join(w[0], w[1], up ? 27 : 28, w[2]);  // yz or xx
+    u[1] = join(w[3], w[4], up ? 28 : 27, w[5]);  // zz or xy
+    u[2] = up ? (__int128)w[6] : join(w[6], w[7], 27, w[8]);
+    u[3] = up ? (__int128)w[7] : join(w[9], w[10], 28, w[11]);
+    u[4] = w[8];  // (lane 1)
+    if (b - a > kAggShort) {  // the sums so far wait in shared memory, not in registers
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        if (a1 > a) u[k] += totals[k * kOrderBlock];
+        totals[k * kOrderBlock] = u[k];
+      }
+    }
+  }
+  if (!ok) {  // wide observations: 128-bit sums, or FP64
+    ok = fits;
+    constexpr long long kMaxD = 1ll << 56;
+    __int128 t[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (int64_t k = a + sub; k < b && ok; k += kAggLanes) {
+      const long long dx = fix_round(pts[3 * k], F, ok) - X0x;
+      const long long dy = fix_round(pts[3 * k + 1], F, ok) - X0y;
+      const long long dz = fix_round(pts[3 * k + 2], F, ok) - X0z;
+      ok = ok && dx > -kMaxD && dx < kMaxD && dy > -kMaxD && dy < kMaxD && dz > -kMaxD && dz < kMaxD;
+      t[0] += (__int128)dx * dx;
+      t[1] += (__int128)dx * dy;
+      t[2] += (__int128)dx * dz;
+      t[3] += (__int128)dy * dy;
+      t[4] += (__int128)dy * dz;
+      t[5] += (__int128)dz * dz;
+      t[6] += dx;
+      t[7] += dy;
+      t[8] += dz;
+    }
+    if (!__all_sync(mask, ok)) {
+      aggregate_f64(a, b, sub, mask, pts, r);
+      return;
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) t[q] += shfl_xor_i128(mask, t[q], 1);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) u[q] = sub == 0 ? t[q] : t[4 + q];
+  }
+  // S = C - s_a d_b and m = p0 + d from the exact sums, one instruction
+  // sequence with operands chosen per lane (an FP64 warp instruction costs the
+  // same whatever the number of lanes on each side of a branch)
+  const bool up = sub != 0;
+  const int e2 = up ? -F : -2 * F;
+  double c[5] = {i128_scaled(u[0], -2 * F), i128_scaled(u[1], -2 * F), i128_scaled(u[2], e2), i128_scaled(u[3], e2), 0.0};
+  // sum d is below 2^56 2^14: slot 4 of lane 1 may need 128 bits
+  const int lane0 = threadIdx.x & 30;
+  if (up) c[4] = i128_scaled(u[4], -F);
+  const double sx = __shfl_sync(mask, c[2], lane0 + 1), sy = __shfl_sync(mask, c[3], lane0 + 1),
+               sz = __shfl_sync(mask, c[4], lane0 + 1);
+  // p0 in whole steps: x by lane 0, y by lane 1, then z
+  const double xy = i64_scaled(up ? X0y : X0x, -F), mx0 = __shfl_sync(mask, xy, lane0), mz0 = i64_scaled(X0z, -F);
+  if (up) {
+    c[2] = mx0;
+    c[3] = xy;
+    c[4] = mz0;
+  }
+  const float nf = (float)(int)(b - a);
+  const double n = f32_to_f64(nf);
+  const double rn = recip_count(n, nf);
+  const double dx = sx * rn, dy = sy * rn, dz = sz * rn;
+  double* w = r + (up ? 4 : 0);
+  w[0] = fma(up ? -sy : -sx, up ? dz : dx, c[0]);  // yz or xx
+  w[1] = fma(up ? -sz : -sx, up ? dz : dy, c[1]);  // zz or xy
+  w[2] = fma(up ? 1.0 : -sx, up ? dx : dz, c[2]);  // m x or xz
+  w[3] = fma(up ? 1.0 : -sy, dy, c[3]);            // m y or yy
+  if (up) {
+    w[4] = c[4] + dz;
+    w[5] = n;
+  }
+}
+
+__global__ void __launch_bounds__(kOrderBlock, 2) aggregate_points_kernel(int64_t n_obs, const int64_t* __restrict__ off,
+                                                                       const double* __restrict__ pts,
+                                                                       double* __restrict__ out) {
+  __shared__ int s_cnt[32], s_order[kOrderBlock];
+  __shared__ __int128 s_totals[5 * kOrderBlock];
+  const int64_t o0 = (int64_t)blockIdx.x * kOrderBlock;
+  {
+    const int64_t o = o0 + threadIdx.x;
+    const int64_t len = o < n_obs ? off[o + 1] - off[o] : 0;
+    block_order_by_key(len < 0 ? 0 : len < 124 ? (int)(len >> 2) : 31, s_cnt, s_order);
+  }
+  constexpr int kGroups = kOrderBlock / kAggLanes;
+  const int sub = threadIdx.x & (kAggLanes - 1), group = threadIdx.x / kAggLanes;
+  const unsigned mask = ((1u << kAggLanes) - 1u) << (threadIdx.x & 31 & ~(kAggLanes - 1));
+#pragma unroll 1
+  for (int round = 0; round < kAggLanes; ++round) {
+    // every second round from the other end, so that every warp takes short and long ones
+    const int64_t o = o0 + s_order[kGroups * round + (round & 1 ? kGroups - 1 - group : group)];
+    if (o < n_obs) aggregate_one(off[o], off[o + 1], sub, mask, pts, out + 10 * o, s_totals + threadIdx.x);
+  }
 }
 
 cudaError_t launch_aggregate_points(int64_t n_obs, const int64_t* point_off, const double* points, double* agg_out,
                                     cudaStream_t stream) {
   if (n_obs <= 0) return cudaSuccess;
-  const int64_t threads = n_obs * kAggLanes;
-  aggregate_points_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(n_obs, point_off, points, agg_out);
+  aggregate_points_kernel<<<(unsigned)((n_obs + kOrderBlock - 1) / kOrderBlock), kOrderBlock, 0, stream>>>(
+      n_obs, point_off, points, agg_out);
   return cudaGetLastError();
 }
 
