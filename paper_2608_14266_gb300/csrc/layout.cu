@@ -5,6 +5,7 @@
 #include <cfloat>
 
 #include "block_order.cuh"
+#include "fixed_sums.cuh"
 #include "mmba_internal.cuh"
 #include "mmba_kernels.h"
 
@@ -787,74 +788,6 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
 // 0.6M observations of 1-64 points 576 -> 265 us, 1M of 32 454 -> 386 us, 0.2M of
 // 100 319 -> 222 us, 3M of 1-8 614 -> 586 us, 60,000 of 200-400 645 -> 267 us.
 constexpr int kAggLanes = 2;
-constexpr int kAggShort = 254;  // points whose sums of halves fit 64 bits (whole lane pairs)
-
-// round(p 2^F) to the nearest integer (halves away from zero); ok is cleared
-// when the result would reach 2^62
-__device__ __forceinline__ long long fix_round(double p, int F, bool& ok) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(p);
-  const int E = (int)((b >> 52) & 0x7ffu);
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = E - 1075 + F;
-  unsigned long long v = 0;
-  if (E != 0) {  // zero and subnormal values are below the resolution
-    if (sh >= 0) {
-      ok = ok && sh <= 9;
-      v = m << (sh & 15);
-    } else if (sh > -63) {
-      const int r = -sh;
-      v = (m + (1ull << (r - 1))) >> r;
-    }
-  }
-  return (b >> 63) ? -(long long)v : (long long)v;
-}
-
-// v 2^e rounded to the nearest FP64 value, ties to even, in integer
-// arithmetic (the conversions of the hardware run on the FP64 pipe); for
-// |v| < 2^127 and results in the normal range
-__device__ __forceinline__ double i128_scaled(__int128 v, int e) {
-  const bool neg = v < 0;
-  const unsigned __int128 u = neg ? (unsigned __int128)(-v) : (unsigned __int128)v;
-  unsigned long long hi = (unsigned long long)(u >> 64), lo = (unsigned long long)u;
-  if ((hi | lo) == 0) return 0.0;
-  int top = 127;  // exponent of the leading bit
-  if (hi == 0) {
-    hi = lo;
-    lo = 0;
-    top = 63;
-  }
-  const int lz = __clzll((long long)hi);
-  if (lz) {
-    hi = (hi << lz) | (lo >> (64 - lz));
-    lo <<= lz;
-  }
-  top -= lz;
-  unsigned long long m = hi >> 11;  // 53 bits, the leading one included
-  const unsigned rest = (unsigned)hi & 2047u;
-  m += (rest > 1024u || (rest == 1024u && (lo != 0 || (m & 1ull)))) ? 1ull : 0ull;
-  // the leading bit adds one to the exponent field (two where rounding carried out of the fraction)
-  const unsigned long long r = ((unsigned long long)(unsigned)(1022 + top + e) << 52) + m;
-  return __longlong_as_double((long long)(r | ((unsigned long long)neg << 63)));
-}
-
-// the same for |v| < 2^63
-__device__ __forceinline__ double i64_scaled(long long v, int e) {
-  if (v == 0) return 0.0;
-  const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-  const int lz = __clzll((long long)u);
-  const unsigned long long h = u << lz;
-  const unsigned rest = (unsigned)h & 2047u;
-  unsigned long long m = h >> 11;
-  m += (rest > 1024u || (rest == 1024u && (m & 1ull))) ? 1ull : 0ull;
-  const unsigned long long r = ((unsigned long long)(unsigned)(1022 + 63 - lz + e) << 52) + m;
-  return __longlong_as_double((long long)(r | ((unsigned long long)v & 0x8000000000000000ull)));
-}
-
-__device__ __forceinline__ __int128 shfl_xor_i128(unsigned mask, __int128 v, int lane) {
-  const unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)((unsigned __int128)v >> 64);
-  const unsigned long long lo2 = __shfl_xor_sync(mask, lo, lane), hi2 = __shfl_xor_sync(mask, hi, lane);
-  return (__int128)(((unsigned __int128)hi2 << 64) | lo2);
-}
 
 // the shifted sums in FP64 (observations the fixed point does not fit)
 __device__ void aggregate_f64(int64_t a, int64_t b, int sub, unsigned mask, const double* __restrict__ pts,
@@ -897,34 +830,6 @@ __device__ void aggregate_f64(int64_t a, int64_t b, int sub, unsigned mask, cons
   }
 }
 
-// 1 / n for a whole n <= 2^14: Newton's iteration for the reciprocal from the
-// binary32 quotient, twice (24 -> 48 -> 53 bits)
-__device__ __forceinline__ double recip_count(double n, float nf) {
-  const double r0 = f32_to_f64(__frcp_rn(nf));
-  const double r1 = fma(r0, fma(-n, r0, 1.0), r0);
-  return fma(r1, fma(-n, r1, 1.0), r1);
-}
-
-// A coordinate in steps of 2^-F as fix_round gives it, for the short sums: no
-// test inside; the largest biased exponent met and the bits of the offsets
-// from X0 are kept in emax and wide and tested once per observation.  sh =
-// 1075 - F, so that the value is mantissa 2^(E - sh).
-__device__ __forceinline__ long long fix_offset(double p, int sh, long long X0, int& emax, unsigned& wide) {
-  const unsigned hi = (unsigned)__double2hiint(p), lo = (unsigned)__double2loint(p);
-  const int E = (int)(hi >> 20) & 0x7ff;
-  emax = max(emax, E);
-  // twice the mantissa, shifted down by at most 63 (zero and subnormal values: E - sh < -63)
-  const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  const int s = E - sh;
-  // at or above the unit: exact; below: rounded to nearest, halves away from zero
-  const unsigned long long v = s >= 0 ? m << (s & 15) : ((m >> min(-s - 1, 63)) + 1ull) >> 1;
-  const long long neg = (long long)((int)hi >> 31);
-  const long long d = (((long long)v ^ neg) - neg) - X0;
-  const int dh = (int)(d >> 32);
-  wide |= (unsigned)(dh ^ (dh >> 31));
-  return d;
-}
-
 // one observation by a pair of lanes (sub = 0, 1; mask = the pair's lanes;
 // totals: five values of this thread's, kOrderBlock apart)
 __device__ __forceinline__ void aggregate_one(int64_t a, int64_t b, int sub, unsigned mask,
@@ -946,49 +851,20 @@ __device__ __forceinline__ void aggregate_one(int64_t a, int64_t b, int sub, uns
   __int128 u[5] = {0, 0, 0, 0, 0};
   bool ok = fits;
 #pragma unroll 1
-  for (int64_t a1 = a; ok && a1 < b; a1 += kAggShort) {
-    // h, c, l (products of the high halves, cross products, products of the
-    // low halves) of each entry of S, then sum d; the diagonal entries hold
-    // half their cross products
-    long long v[21];
-#pragma unroll
-    for (int k = 0; k < 21; ++k) v[k] = 0;
+  for (int64_t a1 = a; ok && a1 < b; a1 += kHalfPoints) {
+    HalfSums h;
+    h.clear();
     const double* q = pts + 3 * (a1 + sub);
-    const int n1 = (int)(b - a1 < kAggShort ? b - a1 : kAggShort);
+    const int n1 = (int)(b - a1 < kHalfPoints ? b - a1 : kHalfPoints);
     const int cnt = (n1 - sub + kAggLanes - 1) / kAggLanes;  // points of this lane
     const int sh = 1075 - F;
-    int emax = 0;
+    int emax = -2048;
     unsigned wide = 0;
     auto add = [&](double x, double y, double z) {
       const long long dx = fix_offset(x, sh, X0x, emax, wide);
       const long long dy = fix_offset(y, sh, X0y, emax, wide);
       const long long dz = fix_offset(z, sh, X0z, emax, wide);
-      const int xh = (int)(dx >> 27), yh = (int)(dy >> 27), zh = (int)(dz >> 27);
-      const int xl = (int)dx & 0x7ffffff, yl = (int)dy & 0x7ffffff, zl = (int)dz & 0x7ffffff;
-      v[0] += (long long)xh * xh;  // xx
-      v[1] += (long long)xh * xl;
-      v[2] += (long long)xl * xl;
-      v[3] += (long long)xh * yh;  // xy
-      v[4] += (long long)xh * yl;
-      v[4] += (long long)xl * yh;
-      v[5] += (long long)xl * yl;
-      v[6] += (long long)xh * zh;  // xz
-      v[7] += (long long)xh * zl;
-      v[7] += (long long)xl * zh;
-      v[8] += (long long)xl * zl;
-      v[9] += (long long)yh * yh;  // yy
-      v[10] += (long long)yh * yl;
-      v[11] += (long long)yl * yl;
-      v[12] += (long long)yh * zh;  // yz
-      v[13] += (long long)yh * zl;
-      v[13] += (long long)yl * zh;
-      v[14] += (long long)yl * zl;
-      v[15] += (long long)zh * zh;  // zz
-      v[16] += (long long)zh * zl;
-      v[17] += (long long)zl * zl;
-      v[18] += dx;
-      v[19] += dy;
-      v[20] += dz;
+      h.add(dx, dy, dz);
     };
     double ax = p0x, ay = p0y, az = p0z, bx = p0x, by = p0y, bz = p0z;
     if (cnt > 0) {
@@ -1023,24 +899,21 @@ __device__ __forceinline__ void aggregate_one(int64_t a, int64_t b, int sub, uns
       }
     }
     // every coordinate within 2^9 of p0's largest, every offset below 2^54
-    ok = __all_sync(mask, emax - sh <= 9 && (wide >> 22) == 0u);
+    ok = __all_sync(mask, emax <= 9 && (wide >> 22) == 0u);
     // lane 0 takes the pair's first 12 sums, lane 1 the other 9
     long long w[12];
     const bool up = sub != 0;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      const long long hi = k < 9 ? v[k + 12 < 21 ? k + 12 : 20] : 0;
-      w[k] = (up ? hi : v[k]) + __shfl_xor_sync(mask, up ? v[k] : hi, 1);
+      const long long hi = k < 9 ? h.v[k + 12 < 21 ? k + 12 : 20] : 0;
+      w[k] = (up ? hi : h.v[k]) + __shfl_xor_sync(mask, up ? h.v[k] : hi, 1);
     }
-    auto join = [](long long h, long long c, int cs, long long l) {
-      return ((__int128)h << 54) + ((__int128)c << cs) + (__int128)l;
-    };
-    u[0] = join(w[0], w[1], up ? 27 : 28, w[2]);  // yz or xx
-    u[1] = join(w[3], w[4], up ? 28 : 27, w[5]);  // zz or xy
-    u[2] = up ? (__int128)w[6] : join(w[6], w[7], 27, w[8]);
-    u[3] = up ? (__int128)w[7] : join(w[9], w[10], 28, w[11]);
+    u[0] = join_halves(w[0], w[1], up ? 27 : 28, w[2]);  // yz or xx
+    u[1] = join_halves(w[3], w[4], up ? 28 : 27, w[5]);  // zz or xy
+    u[2] = up ? (__int128)w[6] : join_halves(w[6], w[7], 27, w[8]);
+    u[3] = up ? (__int128)w[7] : join_halves(w[9], w[10], 28, w[11]);
     u[4] = w[8];  // (lane 1)
-    if (b - a > kAggShort) {  // the sums so far wait in shared memory, not in registers
+    if (b - a > kHalfPoints) {  // the sums so far wait in shared memory, not in registers
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         if (a1 > a) u[k] += totals[k * kOrderBlock];

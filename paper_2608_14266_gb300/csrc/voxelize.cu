@@ -18,6 +18,7 @@
 #include <condition_variable>
 #include <mutex>
 #include <thread>
+#include <type_traits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -26,6 +27,7 @@
 
 #include "../../include/ba.h"
 #include "block_order.cuh"
+#include "fixed_sums.cuh"
 #include "mmba_internal.cuh"
 #include "mmba_kernels.h"
 
@@ -249,87 +251,14 @@ __global__ void mask_starts_kernel(int64_t n_words, const uint32_t* mask, const 
   if (w == 0) start[n_groups] = n;
 }
 
-// ---- clusters (Eq. 2, centred) from shifted sums ----------------------------
-// A piece of a cluster: n points, shift s (its first point), a = sum (p - s),
-// b = sum (p - s)(p - s)^T (xx, xy, xz, yy, yz, zz).  Pieces merge exactly in
-// real arithmetic (shift to the first piece's s); the centred cluster is
+// ---- clusters (Eq. 2, centred) ----------------------------------------------
+// Shifted sums of a merged cluster: n points, shift s, a = sum (p - s),
+// b = sum (p - s)(p - s)^T (xx, xy, xz, yy, yz, zz); the centred cluster is
 // m = s + a/n, S = b - a a^T / n.  The shift keeps every term small (a voxel's
 // extent), so no large cancellation occurs.
 struct Piece {
   double n, s[3], a[3], b[6];
 };
-constexpr int kPieceDoubles = 13;
-
-// one more point of a piece holding cnt points (cnt = 0: p becomes the shift)
-__device__ __forceinline__ void piece_add(Piece& P, int cnt, double p0, double p1, double p2) {
-  if (cnt == 0) {
-    P.s[0] = p0;
-    P.s[1] = p1;
-    P.s[2] = p2;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) P.a[q] = 0.0;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) P.b[q] = 0.0;
-    return;
-  }
-  const double d[3] = {p0 - P.s[0], p1 - P.s[1], p2 - P.s[2]};
-  int k = 0;
-#pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    P.a[x] += d[x];
-#pragma unroll
-    for (int y = x; y < 3; ++y) {
-      P.b[k] = fma(d[x], d[y], P.b[k]);
-      ++k;
-    }
-  }
-}
-
-__device__ __forceinline__ void piece_merge(Piece& A, const Piece& B) {
-  if (B.n == 0.0) return;
-  if (A.n == 0.0) {
-    A = B;
-    return;
-  }
-  const double dl[3] = {B.s[0] - A.s[0], B.s[1] - A.s[1], B.s[2] - A.s[2]};
-  int k = 0;
-#pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    const double nd = B.n * dl[x];
-#pragma unroll
-    for (int y = x; y < 3; ++y) {
-      double t = fma(B.a[x], dl[y], B.b[k]);
-      t = fma(dl[x], B.a[y], t);
-      A.b[k] += fma(nd, dl[y], t);
-      ++k;
-    }
-  }
-#pragma unroll
-  for (int x = 0; x < 3; ++x) A.a[x] += fma(B.n, dl[x], B.a[x]);
-  A.n += B.n;
-}
-
-__device__ __forceinline__ void piece_store(double* o, const Piece& P) {
-  o[0] = P.n;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) o[1 + q] = P.s[q];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) o[4 + q] = P.a[q];
-#pragma unroll
-  for (int q = 0; q < 6; ++q) o[7 + q] = P.b[q];
-}
-
-__device__ __forceinline__ Piece piece_load(const double* o) {
-  Piece P;
-  P.n = o[0];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) P.s[q] = o[1 + q];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) P.a[q] = o[4 + q];
-#pragma unroll
-  for (int q = 0; q < 6; ++q) P.b[q] = o[7 + q];
-  return P;
-}
 
 // centred cluster record (S xx..zz, m, N)
 __device__ __forceinline__ void piece_finish(const Piece& P, double* c) {
@@ -348,108 +277,263 @@ __device__ __forceinline__ void piece_finish(const Piece& P, double* c) {
   c[9] = P.n;
 }
 
-constexpr int kChunk = 32;  // sorted points per thread
+// L1 clusters: the points of each (key, scan) run of the sorted order, as sums
+// of their offsets from the run's first point p0, m = p0 + (sum d) / N and
+// S = sum d d^T - (sum d)(sum d)^T / N.  The sums are exact integer sums in
+// fixed point (RunFrame, fixed_sums.cuh); a run whose points do not fit (the
+// poses stretch it over 2^54 steps, or coordinates outside 2^-400 .. 2^400)
+// takes the same sums in FP64.
+//
+// One thread per run of fewer than kLongRun points, a block's runs in order of
+// their lengths so that a warp's lanes are about as long, each lane with its
+// next point on the way; longer runs by a whole warp each.  The block's two
+// warps take the groups of 32 runs longest first, as they get free (one warp
+// per group leaves the warps of short runs idle until the longest is done).
+//
+// Bound: latency of the gathers (a run's points lie together, its neighbours'
+// elsewhere) against four warps a scheduler, instruction issue 45% active.
+// Measured on 120M points in 12.3M runs, before (FP64 sums over fixed chunks
+// of 32 sorted points, pieces of 104 bytes written and merged per run; the
+// FP64 pipe 69% active): 3.12 + 0.91 ms, now 2.88 ms.  Runs ordered in pools of
+// 256, 512 and 1,024 cost their neighbours' lines in L1 and L2: 2.97, 3.6, 3.7
+// ms.  65,000 points in 7,400 runs: 54 -> 30 us.
+constexpr int kLongRun = 192;  // below kHalfPoints
+static_assert(kLongRun <= kHalfPoints, "a thread's sums must fit");
 
-// L1 clusters, pass 1: each thread sums a chunk of kChunk = 32 sorted points,
-// one piece per (key, scan) run (its key: the packed key, or raw[point] if
-// raw is given); hmask[chunk] flags the run heads of the
-// chunk and base[chunk] counts the heads before it.  The piece where a run starts
-// goes to head_piece[run], the piece of a run continuing from the previous
-// chunk to carry[chunk]; counts are stored as integers (no FP64 work in the
-// divergent stores).  The points reach each thread through shared memory, 8
-// at a time, gathered by its whole warp.
-template <typename K>
-__global__ void __launch_bounds__(128, 5) l1_pieces_kernel(int64_t n, const K* keys, const uint32_t* vals,
-                                                        const int32_t* pscan, const double* pts, const int64_t* base,
-                                                        const uint32_t* hmask, const uint64_t* raw,
-                                                        double* head_piece, double* carry, uint64_t* ckey,
-                                                        int32_t* cscan) {
-  static_assert(kChunk == 32, "one head-mask word per chunk");
-  // per warp, one round of 8 points of each lane's chunk, staged by the whole
-  // warp: lanes 8q..8q+7 load 8 consecutive sorted points of one chunk, so a
-  // load instruction touches 4 runs of consecutive points instead of 32
-  // scattered ones (a chunk's points mostly lie together in the input)
-  __shared__ double sx[4][32][9], sy[4][32][9], sz[4][32][9];
-  __shared__ uint32_t sv[4][32][9];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t wch = ((int64_t)blockIdx.x * blockDim.x) + 32 * w;  // the warp's first chunk
-  const int64_t ch = wch + lane;
-  const int64_t e0 = ch * kChunk;
-  const bool active = e0 < n;
-  const int64_t e1 = e0 + kChunk < n ? e0 + kChunk : n;
-  const uint32_t hm = active ? hmask[ch] : 0u;
-  const bool open = !(hm & 1u);  // the first run continues from the previous chunk
-  const int64_t g0 = active ? base[ch] - 1 : 0;  // the run holding e0 - 1 (a head at e0 starts run g0 + 1)
-  int64_t g = g0;
-  Piece P;
-  int cnt = 0;
-  bool first = true;
-#pragma unroll 1
-  for (int r = 0; r < kChunk / 8; ++r) {
+// bin of a run's length for the block's ordering; 31 = long
+__device__ __forceinline__ int run_bin(int64_t len) {
+  return len <= 8 ? (int)len : len <= 24 ? 4 + (int)(len >> 1) : len < 96 ? 13 + (int)(len >> 3) : len < kLongRun ? 25 + (int)((len - 96) >> 5) : 31;
+}
+
+// Fixed-point frame of a run: per axis the scale (steps of 2^-F) and the first
+// point in steps.  A step is half the last bit of the first point's coordinate,
+// so that a run's coordinates are whole steps, but no finer than 2^-f_cap, about
+// 2^-53 of the voxel's diagonal: where the coordinate itself is smaller than the
+// voxel, rounding to it is what FP64 loses of an offset of the voxel's size.
+struct RunFrame {
+  int F[3];
+  long long X[3];
+  bool fits;
+};
+__device__ __forceinline__ RunFrame run_frame(double x, double y, double z, int f_cap) {
+  const double p[3] = {x, y, z};
+  RunFrame f;
+  f.fits = true;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int t = 4 * i + (lane >> 3), k = lane & 7;
-      const int64_t e = (wch + t) * kChunk + 8 * r + k;
-      if (e < n) {
-        const uint32_t v = vals[e];
-        const double* p = pts + 3 * (int64_t)v;
-        sx[w][t][k] = p[0];
-        sy[w][t][k] = p[1];
-        sz[w][t][k] = p[2];
-        sv[w][t][k] = v;
-      }
-    }
-    __syncwarp();
-    if (active) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int64_t e = e0 + 8 * r + k;
-        if (e >= e1) break;
-        const uint32_t v = sv[w][lane][k];
-        if ((hm >> (int)(e - e0)) & 1u) {
-          if (!first) {  // close the previous run's piece
-            P.n = __longlong_as_double((long long)cnt);
-            piece_store((g == g0 && open) ? carry + kPieceDoubles * ch : head_piece + kPieceDoubles * g, P);
-          }
-          ++g;
-          cnt = 0;
-          ckey[g] = raw ? raw[v] : (uint64_t)keys[e];
-          cscan[g] = pscan[v];
-        }
-        first = false;
-        piece_add(P, cnt, sx[w][lane][k], sy[w][lane][k], sz[w][lane][k]);
-        ++cnt;
-      }
-    }
-    __syncwarp();
+  for (int a = 0; a < 3; ++a) {
+    f.F[a] = min(1076 - ((__double2hiint(p[a]) >> 20) & 0x7ff), f_cap);
+    f.fits = f.fits && f.F[a] >= -400 && f.F[a] <= 400;
+    f.X[a] = fix_round(p[a], f.F[a], f.fits);
   }
-  if (!active) return;
-  P.n = __longlong_as_double((long long)cnt);
-  piece_store((g == g0 && open) ? carry + kPieceDoubles * ch : head_piece + kPieceDoubles * g, P);
+  return f;
 }
 
-__device__ __forceinline__ Piece piece_load_counted(const double* o) {
-  Piece P = piece_load(o);
-  P.n = (double)__double_as_longlong(P.n);
-  return P;
+// record from the exact sums: t = sum d d^T, s = sum d as FP64, n points, rn = 1 / n
+__device__ __forceinline__ void run_record(const RunFrame& f, const __int128* t, const double (&s)[3], double n,
+                                           double rn, double* c) {
+  int k = 0;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    const double d = s[x] * rn;
+#pragma unroll
+    for (int y = x; y < 3; ++y) {
+      c[k] = fma(-s[y], d, i128_scaled(t[k], -(f.F[x] + f.F[y])));
+      ++k;
+    }
+    c[6 + x] = i64_scaled(f.X[x], -f.F[x]) + d;
+  }
+  c[9] = n;
 }
 
-// L1 clusters, pass 2 (per run): the head piece merged in order with the
-// carries of the chunks the run covers, then the centred cluster; a block's
-// 256 runs are taken in order of their carry counts (as in merge_kernel)
-__global__ void __launch_bounds__(kOrderBlock, 3) l1_finish_kernel(int64_t n1, const int64_t* start,
-                                                                const double* head_piece, const double* carry,
-                                                                double* c) {
-  __shared__ int s_cnt[32], s_order[kOrderBlock];
-  const int64_t g0 = (int64_t)blockIdx.x * kOrderBlock + threadIdx.x;
-  const int64_t extra0 = g0 < n1 ? (start[g0 + 1] - 1) / kChunk - start[g0] / kChunk : 0;
-  const int64_t g =
-      (int64_t)blockIdx.x * kOrderBlock + block_order_by_key((int)(extra0 < 31 ? extra0 : 31), s_cnt, s_order);
-  if (g >= n1) return;
-  Piece acc = piece_load_counted(head_piece + kPieceDoubles * g);
-  const int64_t cs = start[g] / kChunk, ce = (start[g + 1] - 1) / kChunk;
-  for (int64_t c2 = cs + 1; c2 <= ce; ++c2) piece_merge(acc, piece_load_counted(carry + kPieceDoubles * c2));
-  piece_finish(acc, c + 10 * g);
+// the sums of every stride-th point from sorted position e on, in FP64 (a = sum d, b = sum d d^T)
+__device__ __noinline__ void run_sums_f64(int64_t e, int64_t end, int stride, const uint32_t* vals, const double* pts,
+                                          double p0x, double p0y, double p0z, double* t) {
+  for (int q = 0; q < 9; ++q) t[q] = 0.0;
+  for (; e < end; e += stride) {
+    const double* p = pts + 3 * (int64_t)vals[e];
+    const double x = p[0] - p0x, y = p[1] - p0y, z = p[2] - p0z;
+    t[0] = fma(x, x, t[0]);
+    t[1] = fma(x, y, t[1]);
+    t[2] = fma(x, z, t[2]);
+    t[3] = fma(y, y, t[3]);
+    t[4] = fma(y, z, t[4]);
+    t[5] = fma(z, z, t[5]);
+    t[6] += x;
+    t[7] += y;
+    t[8] += z;
+  }
+}
+
+__device__ __noinline__ void run_record_f64(const double* t, double n, double p0x, double p0y, double p0z, double* c) {
+  Piece P{n, {p0x, p0y, p0z}, {t[6], t[7], t[8]}, {t[0], t[1], t[2], t[3], t[4], t[5]}};
+  piece_finish(P, c);
+}
+
+constexpr int kClusterThreads = 64;
+
+// adds cnt points, every stride-th from sorted position e on, to h, the next
+// point and the index of the one after it on their way; false if one does not fit
+__device__ __forceinline__ bool run_sums(HalfSums& h, const RunFrame& f, int64_t e, int cnt, int stride,
+                                         const uint32_t* __restrict__ vals, const double* __restrict__ pts) {
+  int emax = -2048;
+  unsigned wide = 0;
+  double x = 0.0, y = 0.0, z = 0.0;
+  uint32_t next = 0;
+  const uint32_t* v = vals + e;
+  if (cnt > 0) {
+    const double* p = pts + 3 * (int64_t)*v;
+    x = p[0];
+    y = p[1];
+    z = p[2];
+  }
+  if (cnt > 1) next = *(v += stride);
+  for (int k = 0; k < cnt; ++k) {
+    const double cx = x, cy = y, cz = z;
+    if (k + 1 < cnt) {
+      const double* p = pts + 3 * (int64_t)next;
+      x = p[0];
+      y = p[1];
+      z = p[2];
+    }
+    if (k + 2 < cnt) next = *(v += stride);
+    const long long dx = fix_offset(cx, 1075 - f.F[0], f.X[0], emax, wide);
+    const long long dy = fix_offset(cy, 1075 - f.F[1], f.X[1], emax, wide);
+    const long long dz = fix_offset(cz, 1075 - f.F[2], f.X[2], emax, wide);
+    h.add(dx, dy, dz);
+  }
+  return emax <= 9 && (wide >> 22) == 0u;
+}
+
+__device__ __forceinline__ void run_totals(const HalfSums& h, __int128* t) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    t[k] = join_halves(h.v[3 * k], h.v[3 * k + 1], k == 0 || k == 3 || k == 5 ? 28 : 27, h.v[3 * k + 2]);
+}
+
+// a run of kLongRun points and more, by a warp
+__device__ __noinline__ void cluster_long(int64_t g, int lane, const int64_t* start, const uint32_t* vals,
+                                          const double* pts, double* c, int f_cap) {
+  const int64_t a = start[g], b = start[g + 1];
+  const uint32_t v0 = vals[a];
+  const double p0x = pts[3 * (int64_t)v0], p0y = pts[3 * (int64_t)v0 + 1], p0z = pts[3 * (int64_t)v0 + 2];
+  const RunFrame f = run_frame(p0x, p0y, p0z, f_cap);
+  bool ok = f.fits;
+  __int128 t[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  for (int64_t e = a; ok && e < b; e += 32 * kHalfPoints) {
+    const int64_t left = (b - e - lane + 31) / 32;  // points of this lane from here on: every 32nd
+    const int cnt = left <= 0 ? 0 : (int)(left < kHalfPoints ? left : kHalfPoints);
+    HalfSums h;
+    h.clear();
+    const bool mine = run_sums(h, f, e + lane, cnt, 32, vals, pts);
+    ok = __all_sync(0xffffffffu, mine);
+    __int128 u[6];
+    run_totals(h, u);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) t[q] += u[q];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) t[6 + q] += h.v[18 + q];
+  }
+  const double n = (double)(b - a);
+  if (ok) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t[q] += shfl_xor_i128(0xffffffffu, t[q], o);
+    const double s[3] = {i128_scaled(t[6], -f.F[0]), i128_scaled(t[7], -f.F[1]), i128_scaled(t[8], -f.F[2])};
+    if (lane == 0) run_record(f, t, s, n, 1.0 / n, c + 10 * g);
+  } else {
+    double t64[9];
+    run_sums_f64(a + lane, b, 32, vals, pts, p0x, p0y, p0z, t64);
+    for (int q = 0; q < 9; ++q)
+      for (int o = 16; o > 0; o >>= 1) t64[q] += __shfl_xor_sync(0xffffffffu, t64[q], o);
+    if (lane == 0) run_record_f64(t64, n, p0x, p0y, p0z, c + 10 * g);
+  }
+}
+
+constexpr int64_t kPoolRuns = 400000;  // runs from which a block orders 128 of them; below, 64 (more blocks)
+
+// (the clusters' keys: the packed key, or raw[point] if raw is given)
+template <typename K, int kPool>
+__global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t n1, const int64_t* __restrict__ start,
+                                                                     const K* __restrict__ keys,
+                                                                     const uint32_t* __restrict__ vals,
+                                                                     const int32_t* __restrict__ pscan,
+                                                                     const double* __restrict__ pts,
+                                                                     const uint64_t* __restrict__ raw, int f_cap,
+                                                                     double* c, uint64_t* ckey, int32_t* cscan) {
+  __shared__ int s_cnt[32], s_next;
+  __shared__ uint16_t s_order[kPool];
+  __shared__ int64_t s_start[kPool];
+  __shared__ int s_len[kPool];
+  __shared__ uint32_t s_first[kPool];
+  const int64_t r0 = (int64_t)blockIdx.x * kPool;
+  const int lane = threadIdx.x & 31;
+  {
+    // the runs' places, first points, keys and scans in input order (coalesced,
+    // independent loads)
+    constexpr int kPer = kPool / kClusterThreads;
+    int bin[kPer];
+    int64_t a[kPer], e[kPer];
+    uint32_t v0[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int64_t g = r0 + k * kClusterThreads + threadIdx.x;
+      a[k] = g < n1 ? start[g] : 0;
+      e[k] = g < n1 ? start[g + 1] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) v0[k] = e[k] > a[k] ? vals[a[k]] : 0u;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int i = k * kClusterThreads + threadIdx.x;
+      bin[k] = run_bin(e[k] - a[k]);
+      s_start[i] = a[k];
+      s_len[i] = (int)(e[k] - a[k] < kLongRun ? e[k] - a[k] : kLongRun);
+      s_first[i] = v0[k];
+      if (e[k] > a[k]) {
+        ckey[r0 + i] = raw ? raw[v0[k]] : (uint64_t)keys[a[k]];
+        cscan[r0 + i] = pscan[v0[k]];
+      }
+    }
+    if (threadIdx.x == 0) s_next = 0;
+    block_order_items<kPer, kClusterThreads>(bin, s_cnt, s_order);
+  }
+  const int n_long = kPool - s_cnt[31];
+  for (;;) {
+    // the next item: the long runs, then the groups of 32, longest first
+    int item = lane == 0 ? atomicAdd(&s_next, 1) : 0;
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item < n_long) {
+      cluster_long(r0 + s_order[kPool - 1 - item], lane, start, vals, pts, c, f_cap);
+      continue;
+    }
+    const int group = kPool / 32 - 1 - (item - n_long);
+    if (group < 0) break;
+    const int i = s_order[group * 32 + lane];
+    const int64_t g = r0 + i, a = s_start[i];
+    const int len = s_len[i];
+    if (len > 0 && len < kLongRun) {
+      const uint32_t v0 = s_first[i];
+      const double p0x = pts[3 * (int64_t)v0], p0y = pts[3 * (int64_t)v0 + 1], p0z = pts[3 * (int64_t)v0 + 2];
+      const RunFrame f = run_frame(p0x, p0y, p0z, f_cap);
+      HalfSums h;
+      h.clear();
+      double* rec = c + 10 * g;
+      if (f.fits && run_sums(h, f, a + 1, len - 1, 1, vals, pts)) {  // p0's own offset is zero
+        __int128 t[6];
+        run_totals(h, t);
+        const double s[3] = {i64_scaled(h.v[18], -f.F[0]), i64_scaled(h.v[19], -f.F[1]),
+                             i64_scaled(h.v[20], -f.F[2])};
+        const float nf = (float)len;
+        const double n = f32_to_f64(nf);
+        run_record(f, t, s, n, recip_count(n, nf), rec);
+      } else {
+        double t[9];
+        run_sums_f64(a + 1, a + len, 1, vals, pts, p0x, p0y, p0z, t);
+        run_record_f64(t, (double)len, p0x, p0y, p0z, rec);
+      }
+    }
+  }
 }
 
 // Eq. 5: parent key of every cluster (level packing pc -> pp); sort keys
@@ -849,13 +933,10 @@ ba_status vfail(ba_status s, const char* fmt, ...) {
                                              : vfail(BA_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e_)); \
   } while (0)
 
-// groups of a sorted (key, scan) sequence: mask (one word per 32 elements),
-// base = exclusive head count before each word (n_words + 1 entries), start
-// (n_groups + 1 entries)
+// groups of a sorted (key, scan) sequence: start (n_groups + 1 entries)
 template <typename K>
 ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int32_t* scan, Buf& tmp,
-                       uint32_t** mask_out, int64_t** base_out, int64_t** start_out, int64_t* n_groups,
-                       cudaStream_t st, int64_t* launches) {
+                       int64_t** start_out, int64_t* n_groups, cudaStream_t st, int64_t* launches) {
   const int64_t nw = (n + 31) / 32;
   uint32_t* mask = tmp.get<uint32_t>(nw);
   int64_t* base = tmp.get<int64_t>(nw + 1);
@@ -874,8 +955,6 @@ ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int
   mask_starts_kernel<<<blocks_for(nw), 256, 0, st>>>(nw, mask, base, n, start, ng);
   VCK(cudaGetLastError(), "voxelize");
   *launches += 2;
-  *mask_out = mask;
-  *base_out = base;
   *start_out = start;
   *n_groups = ng;
   return BA_OK;
@@ -907,7 +986,7 @@ struct Level {
 // (the clusters go to out, the rest to tmp; raw_keys: clusters keep raw keys)
 template <typename K>
 ba_status level1(int64_t n, const uint64_t* raw, uint32_t* vals, const int32_t* pscan, const double* pts, Level& L,
-                 bool raw_keys, Buf& out, Buf& tmp, StageTimer& tm, cudaStream_t st, int64_t* launches) {
+                 bool raw_keys, int f_cap, Buf& out, Buf& tmp, StageTimer& tm, cudaStream_t st, int64_t* launches) {
   K* keys = tmp.get<K>(n);
   K* tkeys = tmp.get<K>(n);
   uint32_t* tvals = tmp.get<uint32_t>(n);
@@ -925,29 +1004,28 @@ ba_status level1(int64_t n, const uint64_t* raw, uint32_t* vals, const int32_t* 
     VCK(radix_sort_pairs64((uint64_t*)keys, vals, (uint64_t*)tkeys, tvals, n, pack_bits(L.pk), scr, st, launches),
         "voxelize sort");
   tm.end();
-  int64_t *base = nullptr, *start = nullptr;
-  uint32_t* hmask = nullptr;
+  int64_t* start = nullptr;
   int64_t n1 = 0;
-  const int64_t n_chunks = (n + kChunk - 1) / kChunk;
   tm.begin(BA_VOX_RUNS);
-  ba_status s = group_starts<K>(n, keys, vals, pscan, tmp, &hmask, &base, &start, &n1, st, launches);
+  ba_status s = group_starts<K>(n, keys, vals, pscan, tmp, &start, &n1, st, launches);
   tm.end();
   if (s != BA_OK) return s;
   L.nc = n1;
   L.c = out.get<double>(10 * n1);
   L.key = out.get<uint64_t>(n1);
   L.scan = out.get<int32_t>(n1);
-  double* hp = tmp.get<double>(kPieceDoubles * n1);
-  double* cr = tmp.get<double>(kPieceDoubles * n_chunks);
-  if (!L.c || !L.key || !L.scan || !hp || !cr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
+  if (!L.c || !L.key || !L.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   tm.begin(BA_VOX_CLUSTER_PASS);
-  l1_pieces_kernel<K><<<blocks_for(n_chunks, 128), 128, 0, st>>>(n, keys, vals, pscan, pts, base, hmask,
-                                                              raw_keys ? raw : nullptr, hp, cr, L.key, L.scan);
+  auto clusters = [&](auto pool) {
+    l1_clusters_kernel<K, decltype(pool)::value><<<blocks_for(n1, decltype(pool)::value), kClusterThreads, 0, st>>>(
+        n1, start, keys, vals, pscan, pts, raw_keys ? raw : nullptr, f_cap, L.c, L.key, L.scan);
+  };
+  if (n1 > kPoolRuns)
+    clusters(std::integral_constant<int, 128>());
+  else
+    clusters(std::integral_constant<int, 64>());
   tm.end();
-  tm.begin(BA_VOX_CLUSTER_FINISH);
-  l1_finish_kernel<<<blocks_for(n1, kOrderBlock), kOrderBlock, 0, st>>>(n1, start, hp, cr, L.c);
-  tm.end();
-  *launches += 2;
+  ++*launches;
   VCK(cudaGetLastError(), "voxelize clusters");
   return BA_OK;
 }
@@ -980,10 +1058,9 @@ ba_status level_up(const Level& ch, Level& P, int32_t n_scans, Buf& tmp, cudaStr
   else
     VCK(radix_sort_pairs64((uint64_t*)k2, cv, (uint64_t*)t2, tcv, nc, pack_bits(P.pk), scr, st, launches),
         "voxelize sort");
-  int64_t *base = nullptr, *pst = nullptr;
-  uint32_t* hmask = nullptr;
+  int64_t* pst = nullptr;
   int64_t np = 0;
-  ba_status s = group_starts<K>(nc, k2, cv, ch.scan, tmp, &hmask, &base, &pst, &np, st, launches);
+  ba_status s = group_starts<K>(nc, k2, cv, ch.scan, tmp, &pst, &np, st, launches);
   if (s != BA_OK) return s;
   P.nc = np;
   P.c = tmp.get<double>(10 * np);
@@ -1040,9 +1117,12 @@ ba_status l1_range(const L1Ctx& c, int64_t p0, int64_t m, const double* pts, boo
     return vfail(BA_ERR_CAPACITY, "point %lld lies outside the voxel index range [-2^20, 2^20) at this voxel size",
                  b2);
   L.pk = make_pack(bb, bb + 3);
-  return pack_bits(L.pk) <= 32 ? level1<uint32_t>(m, raw, vals, pscan, pts, L, raw_keys, out, tmp, *c.tm, c.st,
+  // finest fixed-point step of the cluster sums: the diagonal, 2^e (e from ilogb,
+  // so diagonal < 2^(e + 1)), in fewer than 2^54 steps
+  const int f_cap = 52 - std::ilogb(1.7320508075688772 * c.d);
+  return pack_bits(L.pk) <= 32 ? level1<uint32_t>(m, raw, vals, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
                                                   c.launches)
-                               : level1<uint64_t>(m, raw, vals, pscan, pts, L, raw_keys, out, tmp, *c.tm, c.st,
+                               : level1<uint64_t>(m, raw, vals, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
                                                   c.launches);
 }
 
@@ -1125,10 +1205,9 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
     VCK(cudaGetLastError(), "voxelize merge");
     return BA_OK;
   }
-  uint32_t* hmask = nullptr;
-  int64_t *base = nullptr, *start = nullptr;
+  int64_t* start = nullptr;
   int64_t ng = 0;
-  ba_status s = group_starts<K>(m, keys, vals, scan_all, tmp, &hmask, &base, &start, &ng, c.st, c.launches);
+  ba_status s = group_starts<K>(m, keys, vals, scan_all, tmp, &start, &ng, c.st, c.launches);
   if (s != BA_OK) return s;
   L.nc = ng;
   L.c = out.get<double>(10 * ng);
