@@ -1,6 +1,6 @@
 """The level-1 clusters of ba_voxelize where their kernel branches: runs
 around the length a warp takes over and around the 32 x 254 points of its sums,
-coordinates near zero (where the fixed-point step is set by the voxel, not by
+the integer and the FP64 path of the voxel indices, coordinates near zero (where the fixed-point step is set by the voxel, not by
 the coordinate), few runs (pools of 64) and many (pools of 128)."""
 import numpy as np
 import pytest
@@ -80,3 +80,57 @@ def test_many_short_runs(mm, n):
     tol = 2 * (cnt + 1) * EPS * 3 * cnt * 0.3**2
     assert np.all(np.abs(got["agg"][:, :6] - ref["agg"][:, :6]) <= tol[:, None])
     assert np.all(np.abs(got["agg"][:, 6:9] - ref["agg"][:, 6:9]) <= 4 * EPS * (60.0 + cnt[:, None]))
+
+
+def _rotation(rng):
+    q, _ = np.linalg.qr(rng.normal(size=(3, 3)))
+    return q if np.linalg.det(q) > 0 else -q
+
+
+@pytest.mark.parametrize("d", [0.5, 0.3, 1.0, 0.7, 1e-3, 40.0, 1e-5])
+@pytest.mark.parametrize("form", ["rotation", "identity", "scaled", "far", "long", "limit", "empty"])
+def test_index_paths(mm, d, form):
+    """Indices bit for bit (the oracle forms floor(RN(w / d)) in FP64): points
+    on, just below and just above voxel faces among random ones; poses with a
+    rotation, the identity (faces hit exactly), a matrix larger than the fixed
+    point takes, offsets near 2^20 voxels; points past the integer path's range;
+    coordinates at zero; scans without points between those with some."""
+    rng = np.random.default_rng(5)
+    m = 4000
+    cells = rng.integers(-300, 300, (m, 3)).astype(np.float64)
+    p = np.concatenate([cells * d, np.nextafter(cells * d, np.inf), np.nextafter(cells * d, -np.inf),
+                        (cells + 2.0**-16 * rng.normal(size=(m, 3))) * d, rng.uniform(-400, 400, (m, 3)) * d,
+                        np.zeros((3, 3)), rng.normal(size=(50, 3)) * 1e-300])
+    R, t = np.eye(3), np.zeros(3)
+    if form == "rotation":
+        R, t = _rotation(rng), rng.uniform(-50, 50, 3) * d
+    elif form == "scaled":
+        R = 37.0 * _rotation(rng)
+    elif form == "far":
+        R, t = _rotation(rng), np.array([2.0**20 - 2000, -(2.0**20) + 2000, 12345.678]) * d
+    elif form == "long":
+        R = _rotation(rng)
+        p = np.concatenate([p, rng.uniform(-60000, 60000, (m, 3)) * d])
+    elif form == "limit":
+        t = np.array([2.0**20 - 402.0, 0.0, -(2.0**20) + 402.0]) * d
+    n = len(p)
+    poses = np.stack([np.concatenate([R.ravel(), t]), np.concatenate([np.eye(3).ravel(), np.zeros(3)]),
+                      np.concatenate([R.ravel(), t + d])])
+    spo = np.array([0, n // 2, n // 2 if form == "empty" else n // 2 + 5, n], dtype=np.int64)
+    if form == "empty":
+        poses = np.repeat(poses, [1, 700, 1], axis=0)
+        spo = np.concatenate([[0], np.full(701, n // 2), [n]]).astype(np.int64)
+    ref = oracle.voxelize(spo, p, poses, d)
+    got = mm.voxelize(spo, p, poses, d)
+    for k in ("voxel_off", "obs_scan", "level", "index"):
+        np.testing.assert_array_equal(got[k], ref[k])
+    np.testing.assert_array_equal(got["agg"][:, 9], ref["agg"][:, 9])
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, 1e300, 2.0**20])
+def test_point_outside_the_index_range_is_refused(mm, value):
+    p = np.random.default_rng(1).uniform(-5, 5, (5000, 3))
+    p[3210, 1] = value
+    poses = np.stack([np.concatenate([np.eye(3).ravel(), np.zeros(3)])])
+    with pytest.raises(mm.BAError, match="point 3210"):
+        mm.voxelize(np.array([0, 5000], dtype=np.int64), p, poses, 1.0)
