@@ -552,14 +552,14 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
       // filled while the chunks arrive, the slots placed in their slices
       // (spatial windows draw voxels from every chunk) at the end
       float4* staging = (float4*)dev_alloc(h, h->temp, sizeof(float4) * 3 * (size_t)n_obs);
-      uint32_t* chunk_q = (uint32_t*)dev_alloc(h, h->temp, sizeof(uint32_t) * (size_t)n_obs);
-      if (!staging || !chunk_q) return fail(h, BA_ERR_OOM, "slot staging: out of device memory");
+      const uint32_t* chunk_q = nullptr;
+      if (!staging) return fail(h, BA_ERR_OOM, "slot staging: out of device memory");
       {
         // each chunk's scan-major positions, listed while the first chunk is copied
         ChunkBounds cb{};
         cb.n = n_chunks;
         for (int k = 0; k <= n_chunks; ++k) cb.o[k] = voxel_off[chunk_v[k]];
-        CK(h, group_by_chunk(lb.scan_order, n_obs, cb, chunk_q, temp, h->stream, &h->launches), "chunk order");
+        CK(h, group_by_chunk(lb.scan_order, n_obs, cb, &chunk_q, temp, h->stream, &h->launches), "chunk order");
       }
       for (int k = 0; k < n_chunks; ++k) {
         const int64_t v0 = chunk_v[k], v1 = chunk_v[k + 1];

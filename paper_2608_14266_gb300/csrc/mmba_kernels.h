@@ -84,14 +84,18 @@ cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double*
 
 // ---- layout build / primitives ----
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the
-// keys.  keys/vals are sorted in place; tmp buffers of n entries each and a
-// histogram scratch of radix_scratch_count(n) int64 are supplied by the caller.
+// keys (n < 2^32).  Buffers of n entries each and scratch of
+// radix_scratch_count(n) int64 are supplied by the caller; the sorted pairs end
+// in *keys and *vals, which are exchanged with *tmp_keys and *tmp_vals after an
+// odd number of digits (radix_passes(bits)).  With positions = true the values
+// are the positions 0 .. n - 1 and *vals need not be filled.
 int64_t radix_scratch_count(int64_t n);
-cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* tmp_keys, uint32_t* tmp_vals, int64_t n,
-                             int bits, int64_t* scratch, cudaStream_t stream, int64_t* launches);
+inline int radix_passes(int bits) { return bits <= 0 ? 0 : (bits + 7) / 8; }
+cudaError_t radix_sort_pairs(uint32_t** keys, uint32_t** vals, uint32_t** tmp_keys, uint32_t** tmp_vals, int64_t n,
+                             int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches);
 // The same for 64-bit keys (bits up to 64).
-cudaError_t radix_sort_pairs64(uint64_t* keys, uint32_t* vals, uint64_t* tmp_keys, uint32_t* tmp_vals, int64_t n,
-                               int bits, int64_t* scratch, cudaStream_t stream, int64_t* launches);
+cudaError_t radix_sort_pairs64(uint64_t** keys, uint32_t** vals, uint64_t** tmp_keys, uint32_t** tmp_vals, int64_t n,
+                               int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches);
 // The library's stream-ordered memory pool of a device (freed memory stays
 // mapped for reuse); NULL if it cannot be created.
 cudaMemPool_t library_pool(int device);
@@ -168,15 +172,15 @@ cudaError_t launch_vscale(const LoadInput& in, int64_t v0, int64_t v1, double* v
                           int64_t* launches);
 // A load that copies its clusters in chunks of observations [o[k], o[k + 1])
 // (o[0] = 0, o[n] = n_obs, at most kMaxCopyChunks chunks) groups the
-// scan-major positions by chunk: out_q[o[k] .. o[k + 1]) holds, ascending,
+// scan-major positions by chunk: (*out_q)[o[k] .. o[k + 1]) holds, ascending,
 // the positions q whose observation order[q] lies in chunk k (order is a
-// permutation of 0 .. n_obs - 1).  Temporaries come from temp.
+// permutation of 0 .. n_obs - 1).  *out_q and temporaries come from temp.
 constexpr int kMaxCopyChunks = 20;  // chunks halving in size: up to 2^20 - 1 windows, more than 2^31 voxels
 struct ChunkBounds {
   int64_t o[kMaxCopyChunks + 1];
   int n;
 };
-cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBounds& cb, uint32_t* out_q,
+cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBounds& cb, const uint32_t** out_q,
                            Allocator temp, cudaStream_t stream, int64_t* launches);
 
 // ---- mixed precision ----

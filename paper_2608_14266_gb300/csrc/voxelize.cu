@@ -189,10 +189,10 @@ constexpr int kKeyRounds = 4;  // at most so many times kKeyThreads kKeyPoints c
 // L1 (Eq. 4): world point w = R p + t, index floor(w / d), raw key; the
 // index bounding box (one atomic per block) and the first point whose index
 // leaves the key range.  Blocks take tiles of consecutive points of a batch
-// starting at global point p0 (pts, keys, vals and pscan are indexed within the
+// starting at global point p0 (pts, keys and pscan are indexed within the
 // batch); a thread keeps its scan until a point passes the scan's end.
 //
-// Bound: HBM, 24 bytes read and 16 written a point.  120M points: 0.93 ms (5.2
+// Bound: HBM, 24 bytes read and 12 written a point.  120M points: 0.93 ms (5.2
 // TB/s); 2.63 ms with the index in FP64 (9 multiply-adds and 3 additions a
 // point, 88% of the FP64 pipe).
 __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, const int64_t* __restrict__ spo,
@@ -201,8 +201,7 @@ __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, c
                                                               const double* __restrict__ sposes,
                                                               const ScanFix* __restrict__ fix, int kp, double d,
                                                               int rounds, int64_t p0, int64_t n, uint64_t* __restrict__ keys,
-                                                              uint32_t* __restrict__ vals, int32_t* __restrict__ pscan,
-                                                              long long* bad, int* bbox) {
+                                                              int32_t* __restrict__ pscan, long long* bad, int* bbox) {
   int mn[3] = {INT_MAX, INT_MAX, INT_MAX}, mx[3] = {INT_MIN, INT_MIN, INT_MIN};
   const int64_t tile = (int64_t)kKeyThreads * kKeyPoints * rounds;
   for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < n; t0 += (int64_t)gridDim.x * tile) {
@@ -275,7 +274,6 @@ __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, c
           }
         }
         keys[i] = ok ? raw_key(ix[0], ix[1], ix[2]) : 0;
-        vals[i] = (uint32_t)i;
         pscan[i] = j;
       }
     }
@@ -663,14 +661,13 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
 // Eq. 5: parent key of every cluster (level packing pc -> pp); sort keys
 // (scan first, then parent)
 __global__ void parent_keys_kernel(int64_t nc, const uint64_t* ckey, const int32_t* cscan, KeyPack pc, KeyPack pp,
-                                   uint64_t* pkey, uint32_t* skey, uint32_t* vals) {
+                                   uint64_t* pkey, uint32_t* skey) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nc) return;
   int ix[3];
   unpack_key(pc, ckey[i], ix);
   pkey[i] = pack_key(pp, half_floor(ix[0]), half_floor(ix[1]), half_floor(ix[2]));
   skey[i] = (uint32_t)cscan[i];
-  vals[i] = (uint32_t)i;
 }
 
 template <typename K>
@@ -741,11 +738,6 @@ __global__ void gather_clusters_kernel(int64_t m, const uint32_t* vals, const K*
   for (int q = 0; q < 10; ++q) c[10 * i + q] = c_in[10 * src + q];
   ckey[i] = (uint64_t)keys[i];
   cscan[i] = scan_in[src];
-}
-
-__global__ void iota_kernel(int64_t n, uint32_t* v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] = (uint32_t)i;
 }
 
 // voxels of a level: runs of equal key among its clusters (sorted by key, scan)
@@ -1057,6 +1049,15 @@ ba_status vfail(ba_status s, const char* fmt, ...) {
                                              : vfail(BA_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e_)); \
   } while (0)
 
+cudaError_t sort_keys(uint32_t** k, uint32_t** v, uint32_t** tk, uint32_t** tv, int64_t n, int bits, bool positions,
+                      int64_t* scr, cudaStream_t st, int64_t* launches) {
+  return radix_sort_pairs(k, v, tk, tv, n, bits, positions, scr, st, launches);
+}
+cudaError_t sort_keys(uint64_t** k, uint32_t** v, uint64_t** tk, uint32_t** tv, int64_t n, int bits, bool positions,
+                      int64_t* scr, cudaStream_t st, int64_t* launches) {
+  return radix_sort_pairs64(k, v, tk, tv, n, bits, positions, scr, st, launches);
+}
+
 // groups of a sorted (key, scan) sequence: start (n_groups + 1 entries)
 template <typename K>
 ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int32_t* scan, Buf& tmp,
@@ -1109,24 +1110,20 @@ struct Level {
 // level 1: raw keys -> packed keys, sort, (key, scan) runs, clusters
 // (the clusters go to out, the rest to tmp; raw_keys: clusters keep raw keys)
 template <typename K>
-ba_status level1(int64_t n, const uint64_t* raw, uint32_t* vals, const int32_t* pscan, const double* pts, Level& L,
+ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const double* pts, Level& L,
                  bool raw_keys, int f_cap, Buf& out, Buf& tmp, StageTimer& tm, cudaStream_t st, int64_t* launches) {
   K* keys = tmp.get<K>(n);
   K* tkeys = tmp.get<K>(n);
+  uint32_t* vals = tmp.get<uint32_t>(n);
   uint32_t* tvals = tmp.get<uint32_t>(n);
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(n));
-  if (!keys || !tkeys || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
+  if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   tm.begin(BA_VOX_SORT);
   repack_kernel<K><<<blocks_for(n), 256, 0, st>>>(n, raw, L.pk, keys);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize keys");
   // stable by key over points in scan order: groups ordered by (key, scan, point)
-  if (sizeof(K) == 4)
-    VCK(radix_sort_pairs((uint32_t*)keys, vals, (uint32_t*)tkeys, tvals, n, pack_bits(L.pk), scr, st, launches),
-        "voxelize sort");
-  else
-    VCK(radix_sort_pairs64((uint64_t*)keys, vals, (uint64_t*)tkeys, tvals, n, pack_bits(L.pk), scr, st, launches),
-        "voxelize sort");
+  VCK(sort_keys(&keys, &vals, &tkeys, &tvals, n, pack_bits(L.pk), true, scr, st, launches), "voxelize sort");
   tm.end();
   int64_t* start = nullptr;
   int64_t n1 = 0;
@@ -1168,20 +1165,15 @@ ba_status level_up(const Level& ch, Level& P, int32_t n_scans, Buf& tmp, cudaStr
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(nc));
   if (!pkey || !k2 || !t2 || !skey || !tsk || !cv || !tcv || !scr)
     return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  parent_keys_kernel<<<blocks_for(nc), 256, 0, st>>>(nc, ch.key, ch.scan, ch.pk, P.pk, pkey, skey, cv);
+  parent_keys_kernel<<<blocks_for(nc), 256, 0, st>>>(nc, ch.key, ch.scan, ch.pk, P.pk, pkey, skey);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize levels");
-  VCK(radix_sort_pairs(skey, cv, tsk, tcv, nc, bit_width_u((uint64_t)(n_scans - 1)), scr, st, launches),
+  VCK(radix_sort_pairs(&skey, &cv, &tsk, &tcv, nc, bit_width_u((uint64_t)(n_scans - 1)), true, scr, st, launches),
       "voxelize sort");
   gather_keys_kernel<K><<<blocks_for(nc), 256, 0, st>>>(nc, pkey, cv, k2);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize levels");
-  if (sizeof(K) == 4)
-    VCK(radix_sort_pairs((uint32_t*)k2, cv, (uint32_t*)t2, tcv, nc, pack_bits(P.pk), scr, st, launches),
-        "voxelize sort");
-  else
-    VCK(radix_sort_pairs64((uint64_t*)k2, cv, (uint64_t*)t2, tcv, nc, pack_bits(P.pk), scr, st, launches),
-        "voxelize sort");
+  VCK(sort_keys(&k2, &cv, &t2, &tcv, nc, pack_bits(P.pk), false, scr, st, launches), "voxelize sort");
   int64_t* pst = nullptr;
   int64_t np = 0;
   ba_status s = group_starts<K>(nc, k2, cv, ch.scan, tmp, &pst, &np, st, launches);
@@ -1221,9 +1213,8 @@ struct L1Ctx {
 ba_status l1_range(const L1Ctx& c, int64_t p0, int64_t m, const double* pts, bool raw_keys, Level& L, int* bb,
                    Buf& out, Buf& tmp) {
   uint64_t* raw = tmp.get<uint64_t>(m);
-  uint32_t* vals = tmp.get<uint32_t>(m);
   int32_t* pscan = tmp.get<int32_t>(m);
-  if (!raw || !vals || !pscan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
+  if (!raw || !pscan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   const int bb_init[6] = {INT_MAX, INT_MAX, INT_MAX, INT_MIN, INT_MIN, INT_MIN};
   const long long none = LLONG_MAX;
   VCK(cudaMemcpyAsync(c.bbox, bb_init, sizeof bb_init, cudaMemcpyHostToDevice, c.st), "voxelize");
@@ -1232,8 +1223,7 @@ ba_status l1_range(const L1Ctx& c, int64_t p0, int64_t m, const double* pts, boo
   const int rounds = (int)std::min<int64_t>(std::max<int64_t>(m / (key_blocks * kKeyThreads * kKeyPoints), 1), kKeyRounds);
   c.tm->begin(BA_VOX_KEYS);
   l1_keys_kernel<<<(unsigned)key_blocks, kKeyThreads, 0, c.st>>>(c.n_scans, c.spo, pts, c.T, c.sposes, c.fix, c.kp,
-                                                                 c.d, rounds, p0, m, raw, vals, pscan, c.bad + 2,
-                                                                 c.bbox);
+                                                                 c.d, rounds, p0, m, raw, pscan, c.bad + 2, c.bbox);
   c.tm->end();
   ++*c.launches;
   VCK(cudaGetLastError(), "voxelize keys");
@@ -1248,9 +1238,9 @@ ba_status l1_range(const L1Ctx& c, int64_t p0, int64_t m, const double* pts, boo
   // finest fixed-point step of the cluster sums: the diagonal, 2^e (e from ilogb,
   // so diagonal < 2^(e + 1)), in fewer than 2^54 steps
   const int f_cap = 52 - std::ilogb(1.7320508075688772 * c.d);
-  return pack_bits(L.pk) <= 32 ? level1<uint32_t>(m, raw, vals, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
+  return pack_bits(L.pk) <= 32 ? level1<uint32_t>(m, raw, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
                                                   c.launches)
-                               : level1<uint64_t>(m, raw, vals, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
+                               : level1<uint64_t>(m, raw, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
                                                   c.launches);
 }
 
@@ -1312,16 +1302,9 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(m));
   if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   repack_kernel<K><<<blocks_for(m), 256, 0, c.st>>>(m, raw_all, L.pk, keys);
-  iota_kernel<<<blocks_for(m), 256, 0, c.st>>>(m, vals);
-  *c.launches += 2;
+  ++*c.launches;
   VCK(cudaGetLastError(), "voxelize merge");
-  if (sizeof(K) == 4)
-    VCK(radix_sort_pairs((uint32_t*)keys, vals, (uint32_t*)tkeys, tvals, m, pack_bits(L.pk), scr, c.st, c.launches),
-        "voxelize sort");
-  else
-    VCK(radix_sort_pairs64((uint64_t*)keys, vals, (uint64_t*)tkeys, tvals, m, pack_bits(L.pk), scr, c.st,
-                           c.launches),
-        "voxelize sort");
+  VCK(sort_keys(&keys, &vals, &tkeys, &tvals, m, pack_bits(L.pk), true, scr, c.st, c.launches), "voxelize sort");
   if (!any_split) {
     L.nc = m;
     L.c = out.get<double>(10 * m);
