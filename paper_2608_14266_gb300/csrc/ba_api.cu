@@ -397,7 +397,11 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   if (e != cudaSuccess) return cuda_fail(h, e, "stage voxel offsets");
   in.obs_scan = stage(h, obs_scan, (size_t)n_obs, mem_kind, own, &e);
   if (e != cudaSuccess) return cuda_fail(h, e, "stage obs_scan");
-  if (pipelined) {
+  // clusters in device memory are copied while they are validated, where a
+  // kernel can read them as doubles
+  const bool copy_agg =
+      own && agg_mem_kind == BA_MEM_DEVICE && reinterpret_cast<uintptr_t>(agg) % alignof(double) == 0;
+  if (pipelined || copy_agg) {
     double* d = (double*)dev_alloc(h, h->keep, sizeof(double) * 10 * (size_t)n_obs);
     if (!d) return fail(h, BA_ERR_OOM, "clusters: out of device memory");
     in.agg = d;
@@ -465,9 +469,14 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   init.n_obs_seen = 0;
   init.max_len = 0;
   ValidateResult* d_val = (ValidateResult*)dev_alloc(h, h->temp, sizeof(ValidateResult));
-  if (!d_val) return fail(h, BA_ERR_OOM, "validation buffer: out of device memory");
+  float4* t32 = (float4*)dev_alloc(h, h->temp, sizeof(float4) * (size_t)n_scans);
+  if (!d_val || !t32) return fail(h, BA_ERR_OOM, "validation buffer: out of device memory");
   CK(h, cudaMemcpyAsync(d_val, &init, sizeof init, cudaMemcpyHostToDevice, h->stream), "validation init");
-  CK(h, launch_validate(in, d_val, !pipelined, h->stream, &h->launches), "validate");
+  CK(h, launch_validate(in, d_val, t32, h->stream, &h->launches), "validate");
+  if (!pipelined)
+    CK(h, launch_validate_agg(copy_agg ? agg : in.agg, 0, n_obs, copy_agg ? const_cast<double*>(in.agg) : nullptr,
+                              d_val, h->stream, &h->launches),
+       "validate");
   ValidateResult res;
   CK(h, cudaMemcpyAsync(&res, d_val, sizeof res, cudaMemcpyDeviceToHost, h->stream), "validation result");
   CK(h, cudaStreamSynchronize(h->stream), "validation sync");
@@ -481,7 +490,7 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   Allocator keep{keep_fn, h}, temp{temp_fn, h};
   {
     cudaError_t be =
-        build_layout(in, (int)res.max_len, !h->mixed, pipelined, keep, temp, &lb, h->stream, &h->launches);
+        build_layout(in, t32, (int)res.max_len, !h->mixed, pipelined, keep, temp, &lb, h->stream, &h->launches);
     if (be != cudaSuccess) return cuda_fail(h, be, "layout build");
   }
   DevLayout& L = h->L;
@@ -544,6 +553,7 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
     mb.planes32_2 = (float4*)dev_alloc(h, h->keep, sizeof(float4) * 2 * 2 * (size_t)n_voxels);
     if (!mb.ve32 || !mb.vstate || !mb.se32 || !mb.vanchor || !mb.sref || !mb.stab2 || !mb.planes32_2)
       return fail(h, BA_ERR_OOM, "mixed-precision copies: out of device memory");
+    mb.se_vox = lb.se_vox;
     h->in_keep = in;
     h->in_keep.poses = nullptr;
     if (pipelined) {
@@ -564,7 +574,8 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
       for (int k = 0; k < n_chunks; ++k) {
         const int64_t v0 = chunk_v[k], v1 = chunk_v[k + 1];
         CK(h, cudaStreamWaitEvent(h->stream, h->copy_events[k], 0), "wait for clusters");
-        CK(h, launch_validate_agg(in, voxel_off[v0], voxel_off[v1], d_val, h->stream, &h->launches), "validate");
+        CK(h, launch_validate_agg(in.agg, voxel_off[v0], voxel_off[v1], nullptr, d_val, h->stream, &h->launches),
+           "validate");
         CK(h, launch_vscale(in, v0, v1, lb.vscale, h->stream, &h->launches), "voxel scales");
         CK(h, build_mixed_voxels(in, lb, h->poses2, mb, v0, v1, voxel_off[v0], voxel_off[v1], staging, chunk_q,
                                  h->stream, &h->launches),
@@ -1016,7 +1027,7 @@ int64_t ba_estimate_bytes(int32_t precision, int32_t n_scans, int64_t n_voxels, 
   const int64_t slots = n_obs + n_obs / 8 + 64;
   int64_t per_obs, per_slot;
   if (precision == BA_MIXED) {
-    per_obs = 80 + 4 + 40 + 4 + 4 + 4;  // kept FP64 input, obs_scan, scan-major FP32, se_vox, order, obs_vox
+    per_obs = 80 + 4 + 40 + 4 + 4 + 8;  // kept FP64 input, obs_scan, scan-major FP32, se_vox, order, place
     per_slot = 16 * kVe32;
   } else {
     per_obs = 80 + 4;  // scan-major FP64 copy + se_vox
@@ -1033,7 +1044,7 @@ int64_t ba_estimate_bytes(int32_t precision, int32_t n_scans, int64_t n_voxels, 
   // that grouping's sort keys, buffers and scratch
   const int64_t nsort = n_obs > n_voxels ? n_obs : n_voxels;
   if (peak_extra)
-    *peak_extra = (80 + 4 + 8 + (precision == BA_MIXED ? 16 * kVe32 + 4 + 12 + 2 : 0)) * n_obs + 16 * nsort +
+    *peak_extra = (80 + 4 + 8 + 4 + (precision == BA_MIXED ? 16 * kVe32 + 4 + 12 + 2 : 0)) * n_obs + 16 * nsort +
                   24 * nsort / 16 + (8 + 16 + 8 + 8) * (int64_t)n_voxels;
   return keep;
 }

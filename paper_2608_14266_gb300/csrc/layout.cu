@@ -390,51 +390,47 @@ cudaError_t radix_sort_pairs64(uint64_t** keys, uint32_t** vals, uint64_t** tmp_
 // ============================================================================
 __device__ inline void amin(long long* p, long long v) { atomicMin(p, v); }
 
-// every thread of a block reaches the warp reduction (whole warps: the block
-// size is a multiple of 32)
-__global__ void validate_voxels_kernel(LoadInput in, ValidateResult* r) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  int len = 0;  // the voxel's observation count (capped at 2^31 - 1), 0 if none or invalid
-  if (i <= in.n_voxels) {
-    const int64_t a = in.voxel_off[i];
-    if (i == 0 && a != 0) amin(&r->first_bad_offset, 0);
-    if (i == in.n_voxels) {
-      if (a != in.n_obs) amin(&r->first_bad_offset, i);
-    } else {
-      const int64_t b = in.voxel_off[i + 1];
-      if (b < a || a < 0 || b > in.n_obs) amin(&r->first_bad_offset, i);
-      else if (b == a) amin(&r->first_empty_voxel, i);
-      else len = (int)(b - a > 0x7fffffff ? 0x7fffffff : b - a);
+constexpr int kValidateThreads = 256;
+
+// offsets and voxel lengths, scan ids, and poses (their translations also into
+// t32 in FP32, for the spatial order), a range of blocks each.  Every thread of
+// a voxel block reaches the warp reduction.
+__global__ void __launch_bounds__(kValidateThreads) validate_kernel(LoadInput in, int64_t voxel_blocks,
+                                                                    int64_t scan_blocks, float4* t32,
+                                                                    ValidateResult* r) {
+  int64_t blk = blockIdx.x;
+  if (blk < voxel_blocks) {
+    const int64_t i = blk * kValidateThreads + threadIdx.x;
+    int len = 0;  // the voxel's observation count (capped at 2^31 - 1), 0 if none or invalid
+    if (i <= in.n_voxels) {
+      const int64_t a = in.voxel_off[i];
+      if (i == 0 && a != 0) amin(&r->first_bad_offset, 0);
+      if (i == in.n_voxels) {
+        if (a != in.n_obs) amin(&r->first_bad_offset, i);
+      } else {
+        const int64_t b = in.voxel_off[i + 1];
+        if (b < a || a < 0 || b > in.n_obs) amin(&r->first_bad_offset, i);
+        else if (b == a) amin(&r->first_empty_voxel, i);
+        else len = (int)(b - a > 0x7fffffff ? 0x7fffffff : b - a);
+      }
     }
+    // one atomic per warp (one per voxel serialises on the single word)
+    const int wmax = __reduce_max_sync(0xffffffffu, len);
+    if ((threadIdx.x & 31) == 0 && wmax > 0) atomicMax(&r->max_len, (long long)wmax);
+    return;
   }
-  // one atomic per warp (one per voxel serialises on the single word)
-  const int wmax = __reduce_max_sync(0xffffffffu, len);
-  if ((threadIdx.x & 31) == 0 && wmax > 0) atomicMax(&r->max_len, (long long)wmax);
-}
-
-__global__ void validate_scan_ids_kernel(LoadInput in, ValidateResult* r) {
-  const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= in.n_obs) return;
-  const int32_t j = in.obs_scan[o];
-  if (j < 0 || j >= in.n_scans) amin(&r->first_bad_scan, o);
-}
-
-// clusters of observations [o0, o1): finite, and at least one point
-__global__ void validate_agg_kernel(LoadInput in, int64_t o0, int64_t o1, ValidateResult* r) {
-  const int64_t o = o0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= o1) return;
-  const double* a = in.agg + 10 * o;
-  bool fin = true;
-#pragma unroll
-  for (int k = 0; k < 10; ++k) fin = fin && isfinite(a[k]);
-  if (!fin) amin(&r->first_nonfinite_agg, o);
-  if (!(a[9] >= 1.0)) amin(&r->first_bad_count, o);
-}
-
-__global__ void validate_poses_kernel(LoadInput in, ValidateResult* r) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  blk -= voxel_blocks;
+  if (blk < scan_blocks) {
+    const int64_t o = blk * kValidateThreads + threadIdx.x;
+    if (o < in.n_obs) {
+      const int32_t j = in.obs_scan[o];
+      if (j < 0 || j >= in.n_scans) amin(&r->first_bad_scan, o);
+    }
+    return;
+  }
+  const int64_t j = (blk - scan_blocks) * kValidateThreads + threadIdx.x;
   if (j >= in.n_scans) return;
-  const double* P = in.poses + 12 * (int64_t)j;
+  const double* P = in.poses + 12 * j;
   bool ok = true;
   for (int k = 0; k < 12; ++k) ok = ok && isfinite(P[k]);
   for (int a = 0; a < 3 && ok; ++a)
@@ -448,28 +444,71 @@ __global__ void validate_poses_kernel(LoadInput in, ValidateResult* r) {
     if (det < 0.0) ok = false;
   }
   if (!ok) amin(&r->first_bad_pose, j);
+  t32[j] = make_float4(f64_to_f32(P[9]), f64_to_f32(P[10]), f64_to_f32(P[11]), 0.f);
 }
 
-cudaError_t launch_validate(const LoadInput& in, ValidateResult* d_res, bool with_agg, cudaStream_t stream,
-                            int64_t* launches) {
-  validate_voxels_kernel<<<(unsigned)((in.n_voxels + 1 + 255) / 256), 256, 0, stream>>>(in, d_res);
-  ++*launches;
-  RETURN_IF(cudaGetLastError());
-  if (in.n_obs > 0) {
-    validate_scan_ids_kernel<<<(unsigned)((in.n_obs + 255) / 256), 256, 0, stream>>>(in, d_res);
-    ++*launches;
-    RETURN_IF(cudaGetLastError());
-    if (with_agg) RETURN_IF(launch_validate_agg(in, 0, in.n_obs, d_res, stream, launches));
+// Clusters [o0, o1): finite, and at least one point; with dst given also copied
+// there (the handle's own clusters).  Threads take consecutive pairs of values
+// (kPair: where both arrays are 16-byte aligned) or single values, so that the
+// rows of 80 bytes are read as one stream.  Bound by DRAM: 15M clusters copied
+// and validated in 435 us; a row per thread was 318 us behind a copy of 360 us.
+template <bool kPair>
+__global__ void __launch_bounds__(kValidateThreads) validate_agg_kernel(const double* __restrict__ agg, int64_t o0,
+                                                                        int64_t o1, double* __restrict__ dst,
+                                                                        ValidateResult* r) {
+  constexpr int kUnits = 4;  // loads in flight
+  constexpr int64_t kRow = kPair ? 5 : 10;
+  const int64_t e1 = kRow * o1;
+  const int64_t first = kRow * o0 + (int64_t)blockIdx.x * (kValidateThreads * kUnits) + threadIdx.x;
+  double2 v[kUnits];
+#pragma unroll
+  for (int k = 0; k < kUnits; ++k) {
+    const int64_t e = first + k * kValidateThreads;
+    v[k] = make_double2(1.0, 1.0);
+    if (e < e1) {
+      if (kPair)
+        v[k] = reinterpret_cast<const double2*>(agg)[e];
+      else
+        v[k].x = v[k].y = agg[e];
+    }
   }
-  validate_poses_kernel<<<(unsigned)((in.n_scans + 127) / 128), 128, 0, stream>>>(in, d_res);
+#pragma unroll
+  for (int k = 0; k < kUnits; ++k) {
+    const int64_t e = first + k * kValidateThreads;
+    if (e >= e1) break;
+    if (dst) {
+      if (kPair)
+        reinterpret_cast<double2*>(dst)[e] = v[k];
+      else
+        dst[e] = v[k].x;
+    }
+    const bool fin = isfinite(v[k].x) && isfinite(v[k].y);
+    const bool count = e % kRow == kRow - 1;  // holds N
+    if (!fin) amin(&r->first_nonfinite_agg, e / kRow);
+    if (count && !(v[k].y >= 1.0)) amin(&r->first_bad_count, e / kRow);
+  }
+}
+
+cudaError_t launch_validate(const LoadInput& in, ValidateResult* d_res, float4* t32, cudaStream_t stream,
+                            int64_t* launches) {
+  auto blocks = [](int64_t n) { return (n + kValidateThreads - 1) / kValidateThreads; };
+  const int64_t nv = blocks(in.n_voxels + 1), no = blocks(in.n_obs), ns = blocks(in.n_scans);
+  validate_kernel<<<(unsigned)(nv + no + ns), kValidateThreads, 0, stream>>>(in, nv, no, t32, d_res);
   ++*launches;
   return cudaGetLastError();
 }
 
-cudaError_t launch_validate_agg(const LoadInput& in, int64_t o0, int64_t o1, ValidateResult* d_res,
+cudaError_t launch_validate_agg(const double* agg, int64_t o0, int64_t o1, double* dst, ValidateResult* d_res,
                                 cudaStream_t stream, int64_t* launches) {
   if (o1 <= o0) return cudaSuccess;
-  validate_agg_kernel<<<(unsigned)((o1 - o0 + 255) / 256), 256, 0, stream>>>(in, o0, o1, d_res);
+  // pairs where every row starts on 16 bytes
+  const bool pair = (reinterpret_cast<uintptr_t>(agg) | reinterpret_cast<uintptr_t>(dst)) % 16 == 0;
+  const int64_t units = (pair ? 5 : 10) * (o1 - o0), per = 4 * kValidateThreads;
+  const unsigned nb = (unsigned)((units + per - 1) / per);
+  if (pair)
+    validate_agg_kernel<true><<<nb, kValidateThreads, 0, stream>>>(agg, o0, o1, dst, d_res);
+  else
+    validate_agg_kernel<false><<<nb, kValidateThreads, 0, stream>>>(agg, o0, o1, dst, d_res);
   ++*launches;
   return cudaGetLastError();
 }
@@ -501,8 +540,8 @@ __device__ inline void to_centred(const double* a, int form, double out[10]) {
 }
 
 // ---- spatial order of the voxels ----
-// Mean translation of the scans observing each voxel (FP32, summed in the
-// voxel's observation order), and the bounding box of those means as
+// Mean translation of the scans observing each voxel (FP32, from the table of
+// the validation, summed in the voxel's observation order), and the bounding box of those means as
 // order-preserving unsigned encodings of the floats (min and max are exact,
 // so the box does not depend on the order of the atomics).
 __device__ __forceinline__ uint32_t float_order_key(float f) {
@@ -514,7 +553,7 @@ __device__ __forceinline__ float float_from_order_key(uint32_t k) {
 }
 
 __global__ void observer_mean_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ obs_scan,
-                                     const double* __restrict__ poses, int64_t n_voxels, float4* __restrict__ mean,
+                                     const float4* __restrict__ t32, int64_t n_voxels, float4* __restrict__ mean,
                                      uint32_t* __restrict__ box) {
   __shared__ uint32_t sbox[6];
   if (threadIdx.x < 6) sbox[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
@@ -524,10 +563,10 @@ __global__ void observer_mean_kernel(const int64_t* __restrict__ off, const int3
     const int64_t a0 = off[v], a1 = off[v + 1];
     float x = 0.f, y = 0.f, z = 0.f;
     for (int64_t o = a0; o < a1; ++o) {
-      const double* t = poses + 12 * (int64_t)obs_scan[o] + 9;
-      x += f64_to_f32(t[0]);
-      y += f64_to_f32(t[1]);
-      z += f64_to_f32(t[2]);
+      const float4 t = t32[obs_scan[o]];
+      x += t.x;
+      y += t.y;
+      z += t.z;
     }
     const float inv = 1.0f / (float)(a1 - a0);
     const float m[3] = {x * inv, y * inv, z * inv};
@@ -632,39 +671,46 @@ __global__ void fill_sell_kernel(LoadInput in, const int32_t* vperm, const int32
   }
 }
 
-// voxel of every observation, and (unless vscale is null) each voxel's 2 / N_i
-__global__ void obs_voxel_kernel(LoadInput in, int32_t* obs_vox, double* vscale) {
-  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= in.n_voxels) return;
+// The voxel of every observation of voxels [v0, v1) (unless obs_vox is null), and
+// each voxel's 2 / N_i (unless vscale is null), kVoxelLanes threads to a voxel:
+// a voxel's rows are then read together (15M clusters 268 us as a thread per
+// voxel, 184 us).
+constexpr int kVoxelLanes = 8;
+__global__ void __launch_bounds__(256) obs_voxel_kernel(LoadInput in, int64_t v0, int64_t v1, int32_t* obs_vox,
+                                                        double* vscale) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t v = v0 + t / kVoxelLanes;
+  const int sub = (int)(t % kVoxelLanes);
+  if (v >= v1) return;  // whole groups leave together
+  const unsigned mask = ((1u << kVoxelLanes) - 1u) << (threadIdx.x & 31 & ~(kVoxelLanes - 1));
   double n = 0.0;
-  for (int64_t o = in.voxel_off[v]; o < in.voxel_off[v + 1]; ++o) {
-    obs_vox[o] = (int32_t)v;
+  const int64_t b = in.voxel_off[v + 1];
+  for (int64_t o = in.voxel_off[v] + sub; o < b; o += kVoxelLanes) {
+    if (obs_vox) obs_vox[o] = (int32_t)v;
     if (vscale) n += in.agg[10 * o + 9];
   }
-  if (vscale) vscale[v] = 2.0 / n;
-}
-
-// 2 / N_i of voxels [v0, v1)
-__global__ void vscale_kernel(LoadInput in, int64_t v0, int64_t v1, double* vscale) {
-  const int64_t v = v0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= v1) return;
-  double n = 0.0;
-  for (int64_t o = in.voxel_off[v]; o < in.voxel_off[v + 1]; ++o) n += in.agg[10 * o + 9];
-  vscale[v] = 2.0 / n;
+  if (!vscale) return;
+#pragma unroll
+  for (int o = 1; o < kVoxelLanes; o <<= 1) n += __shfl_xor_sync(mask, n, o);
+  if (sub == 0) vscale[v] = 2.0 / n;
 }
 
 // observations listed by sorted voxel position (pbase[p] = observations of
 // the voxels before position p), keyed by scan for the stable sort that makes
 // the scan-major copy: inside a scan, observations follow the voxel order, so
 // the scan pass gathers the plane records of nearby voxels
+// (and, unless place is null, each observation's sorted voxel position and row)
 __global__ void scan_keys_kernel(LoadInput in, const int32_t* obs_vox, const int32_t* vrank, const int64_t* pbase,
-                                 uint32_t* keys, uint32_t* vals) {
+                                 uint32_t* keys, uint32_t* vals, int2* place) {
   const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= in.n_obs) return;
   const int32_t v = obs_vox[o];
-  const int64_t q = pbase[vrank[v]] + (o - in.voxel_off[v]);
+  const int32_t p = vrank[v];
+  const int32_t row = (int32_t)(o - in.voxel_off[v]);
+  const int64_t q = pbase[p] + row;
   keys[q] = (uint32_t)in.obs_scan[o];
   vals[q] = (uint32_t)o;
+  if (place) place[o] = make_int2(p, row);
 }
 
 // scan_off[j] = the first scan-major position of scan j (n at the end), from
@@ -692,7 +738,6 @@ __global__ void fill_scan_major_kernel(LoadInput in, const uint32_t* order, cons
   const int64_t o = order[q];
   const int32_t v = obs_vox[o];
   se_vox[q] = vrank[v];
-  if (!se) return;
   double c[10];
   to_centred(in.agg + 10 * o, in.agg_form, c);
   const double k = vscale[v];
@@ -724,12 +769,17 @@ static int bit_width(uint64_t x) {
   return b;
 }
 
-cudaError_t launch_vscale(const LoadInput& in, int64_t v0, int64_t v1, double* vscale, cudaStream_t stream,
-                          int64_t* launches) {
+static cudaError_t launch_obs_voxel(const LoadInput& in, int64_t v0, int64_t v1, int32_t* obs_vox, double* vscale,
+                                    cudaStream_t stream, int64_t* launches) {
   if (v1 <= v0) return cudaSuccess;
-  vscale_kernel<<<(unsigned)((v1 - v0 + 255) / 256), 256, 0, stream>>>(in, v0, v1, vscale);
+  obs_voxel_kernel<<<(unsigned)(((v1 - v0) * kVoxelLanes + 255) / 256), 256, 0, stream>>>(in, v0, v1, obs_vox, vscale);
   ++*launches;
   return cudaGetLastError();
+}
+
+cudaError_t launch_vscale(const LoadInput& in, int64_t v0, int64_t v1, double* vscale, cudaStream_t stream,
+                          int64_t* launches) {
+  return launch_obs_voxel(in, v0, v1, nullptr, vscale, stream, launches);
 }
 
 cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBounds& cb, const uint32_t** out_q,
@@ -751,7 +801,7 @@ cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBoun
   return cudaSuccess;
 }
 
-cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool defer_scale, Allocator keep,
+cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bool fill_f64, bool defer_scale, Allocator keep,
                          Allocator temp, LayoutBuffers* out, cudaStream_t stream, int64_t* launches) {
   const int64_t nv = in.n_voxels, no = in.n_obs;
   const int64_t n_slices = (nv + kSlice - 1) / kSlice;
@@ -766,7 +816,8 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
   int64_t* scratch = (int64_t*)temp.fn(temp.self, sizeof(int64_t) * (radix_scratch_count(nsort) +
                                                                       scan_scratch_count(n_slices + no + 2)));
   int32_t* vrank = (int32_t*)maps.fn(maps.self, sizeof(int32_t) * nv);
-  int32_t* obs_vox = (int32_t*)maps.fn(maps.self, sizeof(int32_t) * no);
+  int32_t* obs_vox = (int32_t*)temp.fn(temp.self, sizeof(int32_t) * no);
+  int2* place = fill_f64 ? nullptr : (int2*)keep.fn(keep.self, sizeof(int2) * no);
   double* vscale = (double*)maps.fn(maps.self, sizeof(double) * nv);
   uint32_t* order = fill_f64 ? nullptr : (uint32_t*)keep.fn(keep.self, sizeof(uint32_t) * no);
   // persistent
@@ -778,10 +829,11 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
   // + 4 entries: the staged mixed scan pass copies whole 16-byte groups
   out->se_vox = (int32_t*)keep.fn(keep.self, sizeof(int32_t) * (no + 4));
   if (!keys || !vals || !tk || !tv || !scratch || !vrank || !obs_vox || !vscale || !out->slice_off || !out->vlen ||
-      !out->vperm || !out->scan_off || (fill_f64 && !out->se) || (!fill_f64 && !order) || !out->se_vox)
+      !out->vperm || !out->scan_off || (fill_f64 && !out->se) || (!fill_f64 && (!order || !place)) ||
+      !out->se_vox)
     return cudaErrorMemoryAllocation;
   out->vrank = vrank;
-  out->obs_vox = obs_vox;
+  out->place = place;
   out->vscale = vscale;
   out->scan_order = order;
 
@@ -796,7 +848,7 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
     RETURN_IF(cudaMemsetAsync(box, 0xff, sizeof(uint32_t) * 3, stream));  // minima
     RETURN_IF(cudaMemsetAsync(box + 3, 0, sizeof(uint32_t) * 3, stream));  // maxima
     const unsigned nb = (unsigned)((nv + 255) / 256);
-    observer_mean_kernel<<<nb, 256, 0, stream>>>(in.voxel_off, in.obs_scan, in.poses, nv, mean, box);
+    observer_mean_kernel<<<nb, 256, 0, stream>>>(in.voxel_off, in.obs_scan, t32, nv, mean, box);
     morton_keys_kernel<<<nb, 256, 0, stream>>>(mean, nv, box, keys);
     *launches += 2;
     RETURN_IF(cudaGetLastError());
@@ -829,9 +881,7 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
   }
 
   // ---- scan-major copy ----
-  obs_voxel_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, stream>>>(in, obs_vox, defer_scale ? nullptr : vscale);
-  ++*launches;
-  RETURN_IF(cudaGetLastError());
+  RETURN_IF(launch_obs_voxel(in, 0, nv, obs_vox, defer_scale ? nullptr : vscale, stream, launches));
   {
     // kept by a load that stages its slots (they are staged in this order)
     Allocator pb_alloc = defer_scale ? keep : temp;
@@ -846,7 +896,7 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
     // the order, where it is kept, lands in its own buffer: the sort ends in the
     // buffer it starts from after an even number of digits, else in the other
     if (order) (radix_passes(scan_bits) % 2 == 0 ? vals : tv) = order;
-    scan_keys_kernel<<<(unsigned)((no + 255) / 256), 256, 0, stream>>>(in, obs_vox, vrank, pbase, keys, vals);
+    scan_keys_kernel<<<(unsigned)((no + 255) / 256), 256, 0, stream>>>(in, obs_vox, vrank, pbase, keys, vals, place);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
@@ -854,6 +904,7 @@ cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool d
   scan_off_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, stream>>>(keys, no, in.n_scans, out->scan_off);
   ++*launches;
   RETURN_IF(cudaGetLastError());
+  if (!fill_f64) return cudaSuccess;  // the mixed path fills its own copy, se_vox included
   fill_scan_major_kernel<<<(unsigned)((no + 255) / 256), 256, 0, stream>>>(in, vals, obs_vox, vscale, vrank, out->se,
                                                                            out->se_vox);
   ++*launches;

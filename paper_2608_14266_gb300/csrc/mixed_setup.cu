@@ -17,7 +17,16 @@ namespace {
 
 constexpr int kFillRows = 4;  // slice rows per thread of the slot fill
 
-__device__ inline void centred_cluster(const double* a, int form, double out[10]) {
+// the row at in (80 bytes of the handle's own copy, so 16-byte aligned: five
+// 128-bit loads; a row per thread is bound by the load/store unit)
+__device__ inline void centred_cluster(const double* in, int form, double out[10]) {
+  double a[10];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(in) + k);
+    a[2 * k] = v.x;
+    a[2 * k + 1] = v.y;
+  }
   if (form == 1) {
 #pragma unroll
     for (int k = 0; k < 10; ++k) out[k] = a[k];
@@ -109,6 +118,24 @@ __device__ __forceinline__ DF df_fma(DF acc, float x, DF y) {
   return DF{s.hi, __fadd_rn(s.lo, __fadd_rn(acc.lo, fmaf(x, y.lo, e)))};
 }
 
+// x as binary32 plus the binary32 rounding of the exact remainder: hi is
+// f64_to_f32(x), and the remainder is a signed whole number (at most 2^28) of
+// the last place of x, taken from its bits (an FP64 subtraction and two
+// conversions less).  Small and large x, where an exponent leaves binary32's
+// normal range, take the subtraction.
+__device__ __forceinline__ DF split_f64(double x) {
+  const float hi = f64_to_f32(x);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ef = (int)((b >> 52) & 0x7ffu) - 1023 + 127;  // biased exponent in binary32
+  if (ef <= 60 || ef >= 254) return DF{hi, f64_to_f32(x - f32_to_f64(hi))};
+  const unsigned rest = (unsigned)b & 0x1fffffffu;
+  // hi's last bit against the bits kept of x: rounded up or not
+  const bool up = ((__float_as_uint(hi) ^ (unsigned)(b >> 29)) & 1u) != 0u;
+  const int r = (int)rest - (up ? 0x20000000 : 0);
+  const float lo = __int2float_rn(r) * __uint_as_float((unsigned)(ef - 52) << 23);
+  return DF{hi, (long long)b < 0 ? -lo : lo};
+}
+
 // FP32 copies of a cluster's scatter, mean and count (integer-arithmetic
 // conversions: GB300 converts on its narrow FP64 pipe)
 __device__ __forceinline__ void cluster_f32(const double* c, float* Sf, float* mf, float& N) {
@@ -149,8 +176,8 @@ __device__ __forceinline__ float group_sum(unsigned mask, float x) {
 }
 
 __global__ void __launch_bounds__(128) voxel_frames_kernel(LoadInput in, int64_t v0, int64_t v1, const double* sref,
-                                                           const int32_t* vrank, float4* vstate, float4* vanchor,
-                                                           float4* planes2) {
+                                                           const int32_t* vrank, const double* vscale, float4* vstate,
+                                                           float4* vanchor, float4* planes2) {
   static_assert(32 % kFrameLanes == 0 && 128 % kFrameLanes == 0, "groups must not straddle warps");
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t v = v0 + t / kFrameLanes;
@@ -212,7 +239,8 @@ __global__ void __launch_bounds__(128) voxel_frames_kernel(LoadInput in, int64_t
   // remainder (FP32 arithmetic, exact for the rounding step of a sum)
   const float ax = p0[0] + cx, ay = p0[1] + cy, az = p0[2] + cz;
   const int64_t p = vrank[v];
-  vanchor[p] = make_float4(ax, ay, az, 0.0f);
+  // with the factor 2 / N_i of the scan-major copy
+  vanchor[p] = make_float4(ax, ay, az, f64_to_f32(vscale[v]));
   // the anchor also sits beside the plane in both buffers of plane records
   planes2[2 * p + 1] = make_float4(ax, ay, az, 0.0f);
   planes2[2 * (in.n_voxels + p) + 1] = make_float4(ax, ay, az, 0.0f);
@@ -223,9 +251,9 @@ __global__ void __launch_bounds__(128) voxel_frames_kernel(LoadInput in, int64_t
 // b = R_ref m + t_ref - a (world axes), for an observation of a voxel whose
 // anchor is an
 __device__ inline void offset_b(const double* c, const double* ref, float4 an, double b[3]) {
-  b[0] = ref[0] * c[6] + ref[1] * c[7] + ref[2] * c[8] + (ref[9] - f32_to_f64(an.x));
-  b[1] = ref[3] * c[6] + ref[4] * c[7] + ref[5] * c[8] + (ref[10] - f32_to_f64(an.y));
-  b[2] = ref[6] * c[6] + ref[7] * c[7] + ref[8] * c[8] + (ref[11] - f32_to_f64(an.z));
+  b[0] = fma(ref[0], c[6], fma(ref[1], c[7], fma(ref[2], c[8], ref[9] - f32_to_f64(an.x))));
+  b[1] = fma(ref[3], c[6], fma(ref[4], c[7], fma(ref[5], c[8], ref[10] - f32_to_f64(an.y))));
+  b[2] = fma(ref[6], c[6], fma(ref[7], c[7], fma(ref[8], c[8], ref[11] - f32_to_f64(an.z))));
 }
 
 // the slot of observation o of a voxel with anchor an: offset to the anchor
@@ -241,57 +269,64 @@ __device__ void mixed_slot(const LoadInput& in, int64_t o, const double* sref, f
   // Jacobi gives the variances to FP32 relative precision (the normal one
   // included); V = V0 W_vec.  A direction error d of the stored vectors
   // changes a variance only by (spread) d^2.
+  DF Sd[6];  // S as double-floats
   float sf[6];
 #pragma unroll
-  for (int q = 0; q < 6; ++q) sf[q] = f64_to_f32(c[q]);
-  float lam0[3], v0[9];
-  eig3_sym_f(sf, lam0, v0);  // eigenvectors as rows of v0 (vector c at v0[3c..3c+2])
-  // W = V0^T S V0.  The entries of the two smallest directions (W_00,
-  // W_01, W_11) are small next to S's largest entries and lose digits to
-  // cancellation in FP32, so they are formed in double-float arithmetic (~46
-  // bits, from S's FP64 entries; the FP32 eigenvectors are exact): W_00 is the normal
-  // variance of a planar cluster, and for a rod-like cluster (two small,
-  // nearly equal variances) the voxel normal can be any direction of that
-  // pair.  The entries with the largest direction only need absolute
-  // precision (off-diagonals of order 1e-7 of the spread turn V0 by ~1e-7
-  // rad, a second-order change of the variances).
-  float wf[6];
-  {
-    // S as double-floats: hi the binary32 rounding of each entry, lo the
-    // exact remainder rounded once (one FP64 subtraction per entry)
-    DF Sd[6];
+  for (int q = 0; q < 6; ++q) {
+    Sd[q] = split_f64(c[q]);
+    sf[q] = Sd[q].hi;
+  }
+  // eigenvectors as rows of v0 (vector c at v0[3c..3c+2]), then those of W in
+  // wv; one copy of the Jacobi code for both (with two, the kernel waited for
+  // instructions: 15M slots 1285 us, now 1230 us)
+  float v0[9], wf[6], sg[3], wv[9];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) Sd[q] = DF{sf[q], f64_to_f32(c[q] - f32_to_f64(sf[q]))};
-    const DF S[3][3] = {{Sd[0], Sd[1], Sd[2]}, {Sd[1], Sd[3], Sd[4]}, {Sd[2], Sd[4], Sd[5]}};
-    DF Sv[2][3];  // S v_k, k = 0, 1 (v_k binary32, exact)
+  for (int q = 0; q < 6; ++q) wf[q] = sf[q];
+#pragma unroll 1
+  for (int round = 0; round < 2; ++round) {
+    eig3_sym_f(wf, sg, wv);
+    if (round == 1) break;
 #pragma unroll
-    for (int k = 0; k < 2; ++k)
+    for (int q = 0; q < 9; ++q) v0[q] = wv[q];
+    // W = V0^T S V0.  The entries of the two smallest directions (W_00,
+    // W_01, W_11) are small next to S's largest entries and lose digits to
+    // cancellation in FP32, so they are formed in double-float arithmetic (~46
+    // bits, from S's FP64 entries; the FP32 eigenvectors are exact): W_00 is the normal
+    // variance of a planar cluster, and for a rod-like cluster (two small,
+    // nearly equal variances) the voxel normal can be any direction of that
+    // pair.  The entries with the largest direction only need absolute
+    // precision (off-diagonals of order 1e-7 of the spread turn V0 by ~1e-7
+    // rad, a second-order change of the variances).
+    {
+      const DF S[3][3] = {{Sd[0], Sd[1], Sd[2]}, {Sd[1], Sd[3], Sd[4]}, {Sd[2], Sd[4], Sd[5]}};
+      DF Sv[2][3];  // S v_k, k = 0, 1 (v_k binary32, exact)
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          DF acc{0.f, 0.f};
+#pragma unroll
+          for (int q = 0; q < 3; ++q) acc = df_fma(acc, v0[3 * k + q], S[r][q]);
+          Sv[k][r] = acc;
+        }
+      auto dot = [&](int i, int k) {
         DF acc{0.f, 0.f};
 #pragma unroll
-        for (int q = 0; q < 3; ++q) acc = df_fma(acc, v0[3 * k + q], S[r][q]);
-        Sv[k][r] = acc;
-      }
-    auto dot = [&](int i, int k) {
-      DF acc{0.f, 0.f};
-#pragma unroll
-      for (int r = 0; r < 3; ++r) acc = df_fma(acc, v0[3 * i + r], Sv[k][r]);
-      return __fadd_rn(acc.hi, acc.lo);
-    };
-    wf[0] = dot(0, 0);
-    wf[1] = dot(0, 1);
-    wf[3] = dot(1, 1);
-    const float M[3][3] = {{sf[0], sf[1], sf[2]}, {sf[1], sf[3], sf[4]}, {sf[2], sf[4], sf[5]}};
-    float T[3];  // S v_2 (FP32)
-    for (int r = 0; r < 3; ++r) T[r] = fmaf(M[r][0], v0[6], fmaf(M[r][1], v0[7], M[r][2] * v0[8]));
-    // packed (00, 01, 02, 11, 12, 22)
-    wf[2] = fmaf(v0[0], T[0], fmaf(v0[1], T[1], v0[2] * T[2]));
-    wf[4] = fmaf(v0[3], T[0], fmaf(v0[4], T[1], v0[5] * T[2]));
-    wf[5] = fmaf(v0[6], T[0], fmaf(v0[7], T[1], v0[8] * T[2]));
+        for (int r = 0; r < 3; ++r) acc = df_fma(acc, v0[3 * i + r], Sv[k][r]);
+        return __fadd_rn(acc.hi, acc.lo);
+      };
+      wf[0] = dot(0, 0);
+      wf[1] = dot(0, 1);
+      wf[3] = dot(1, 1);
+      const float M[3][3] = {{sf[0], sf[1], sf[2]}, {sf[1], sf[3], sf[4]}, {sf[2], sf[4], sf[5]}};
+      float T[3];  // S v_2 (FP32)
+      for (int r = 0; r < 3; ++r) T[r] = fmaf(M[r][0], v0[6], fmaf(M[r][1], v0[7], M[r][2] * v0[8]));
+      // packed (00, 01, 02, 11, 12, 22)
+      wf[2] = fmaf(v0[0], T[0], fmaf(v0[1], T[1], v0[2] * T[2]));
+      wf[4] = fmaf(v0[3], T[0], fmaf(v0[4], T[1], v0[5] * T[2]));
+      wf[5] = fmaf(v0[6], T[0], fmaf(v0[7], T[1], v0[8] * T[2]));
+    }
   }
-  float sg[3], wv[9];
-  eig3_sym_f(wf, sg, wv);
   // world-axis eigenvectors as columns: V = R_ref V0^T-rows ... = R_ref [v0 rows]^T W
   const float* Rf = sref32_of(sref, in.n_scans, in.obs_scan[o]);
   float V[9];
@@ -351,16 +386,14 @@ __global__ void __launch_bounds__(128, 8)
 // pipelined load computes each arriving chunk's slots there (each voxel's
 // rows one contiguous run), then places them all in their slices once every
 // chunk is done, each slice reading one contiguous stretch.
-__global__ void fill_staging_kernel(LoadInput in, int64_t o0, int64_t o1, const int32_t* obs_vox,
-                                    const int32_t* vrank, const int64_t* vstart, const double* sref,
-                                    const float4* vanchor, float4* staging) {
+__global__ void fill_staging_kernel(LoadInput in, int64_t o0, int64_t o1, const int2* place, const int64_t* vstart,
+                                    const double* sref, const float4* vanchor, float4* staging) {
   const int64_t o = o0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= o1) return;
-  const int32_t v = obs_vox[o];
-  const int64_t p = vrank[v];
+  const int2 at = place[o];
   float4 s0, s1, s2;
-  mixed_slot(in, o, sref, vanchor[p], s0, s1, s2);
-  float4* dst = staging + 3 * (vstart[p] + (o - in.voxel_off[v]));
+  mixed_slot(in, o, sref, vanchor[at.x], s0, s1, s2);
+  float4* dst = staging + 3 * (vstart[at.x] + at.y);
   dst[0] = s0;
   dst[1] = s1;
   dst[2] = s2;
@@ -398,19 +431,35 @@ __global__ void place_slots_kernel(const int64_t* vstart, const int32_t* vlen, c
 // Scan-major FP32 copy from the slots: the offset and count as they are, the
 // scatter in reference axes rebuilt from its eigenvalues and eigenvector
 // quaternion (R_ref S R_ref^T = V diag(sigma) V^T), each scaled by 2 / N_i.
-// Observation o's slot is at sorted voxel position p, row k:
+// Observation o's slot is at sorted voxel position p, row k (place[o]):
 // slice_off[p / 32] + 32 k + p % 32, or, with staging non-null, at
-// staging[3 (vstart[p] + k)].
-__device__ __forceinline__ void fill_scan_one(int64_t q, int64_t o, int64_t n_obs, const int32_t* obs_vox,
-                                              const double* vscale, const int32_t* vrank, const int64_t* voxel_off,
-                                              const int64_t* slice_off, const float4* ve32, const int64_t* vstart,
-                                              const float4* staging, float* se32) {
-  const int32_t v = obs_vox[o];
-  const int64_t p = vrank[v];
-  const int64_t k = o - voxel_off[v];
-  const float4* src =
-      staging ? staging + 3 * (vstart[p] + k) : ve32 + kVe32 * (slice_off[p >> 5] + k * kSlice + (p & 31));
-  const float4 s0 = src[0], s1 = src[1], s2 = src[2];
+// staging[3 (vstart[p] + k)].  se_vox gets its sorted voxel position.
+// A warp fetches its 32 slots together, three lanes to a slot's 48 bytes (a
+// slot per lane asks L1 for a line per lane three times over, 88% of its
+// throughput), and hands them out through shared memory (w: 96 float4 of the
+// warp's).  Every lane of the warp calls it; q < 0: nothing to do.
+__device__ __forceinline__ void fill_scan_one(int64_t q, int64_t o, int64_t n_obs, const int2* __restrict__ place,
+                                              const float4* __restrict__ vanchor,
+                                              const int64_t* __restrict__ slice_off, const float4* ve32,
+                                              const int64_t* vstart, const float4* staging, float* se32,
+                                              int32_t* se_vox, float4* w) {
+  const int lane = threadIdx.x & 31;
+  const int2 at = q >= 0 ? place[o] : make_int2(0, 0);
+  const int64_t p = at.x, k = at.y;
+  const float4* from = staging ? staging : ve32;
+  // the slot's place, in slots
+  const int64_t slot = q < 0 ? 0 : staging ? vstart[p] + k : slice_off[p >> 5] + k * kSlice + (p & 31);
+  const float ks = vanchor[p].w;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int part = 32 * i + lane;
+    const int64_t sl = __shfl_sync(0xffffffffu, slot, part / 3);
+    w[part] = from[3 * sl + part % 3];
+  }
+  __syncwarp();
+  const float4 s0 = w[3 * lane], s1 = w[3 * lane + 1], s2 = w[3 * lane + 2];
+  if (q < 0) return;
+  se_vox[q] = at.x;
   float V[9];
   quat_to_mat_f(s2.x, s2.y, s2.z, s2.w, V);
   const float sg[3] = {s1.x, s1.y, s1.z};
@@ -421,7 +470,6 @@ __device__ __forceinline__ void fill_scan_one(int64_t q, int64_t o, int64_t n_ob
 #pragma unroll
     for (int c = r; c < 3; ++c)
       sw[idx++] = fmaf(V[3 * r] * sg[0], V[3 * c], fmaf(V[3 * r + 1] * sg[1], V[3 * c + 1], V[3 * r + 2] * sg[2] * V[3 * c + 2]));
-  const float ks = f64_to_f32(vscale[v]);
   float4* bN = reinterpret_cast<float4*>(se32);
   float4* S4 = bN + n_obs;
   float2* S2 = reinterpret_cast<float2*>(S4 + n_obs);
@@ -433,15 +481,16 @@ __device__ __forceinline__ void fill_scan_one(int64_t q, int64_t o, int64_t n_ob
 // thread per scan-major position q = qlist[i] (q = i without a list), i in
 // [i0, i1); order[q] = its observation (a pipelined load fills each chunk's
 // entries as the chunk is set up)
-__global__ void fill_scan_mixed_kernel(int64_t n_obs, const uint32_t* qlist, int64_t i0, int64_t i1,
-                                       const uint32_t* order, const int32_t* obs_vox, const double* vscale,
-                                       const int32_t* vrank, const int64_t* voxel_off, const int64_t* slice_off,
-                                       const float4* ve32, const int64_t* vstart, const float4* staging,
-                                       float* se32) {
+constexpr int kFillScanThreads = 256;
+__global__ void __launch_bounds__(kFillScanThreads) fill_scan_mixed_kernel(int64_t n_obs, const uint32_t* qlist, int64_t i0, int64_t i1,
+                                       const uint32_t* order, const int2* place, const float4* vanchor,
+                                       const int64_t* slice_off, const float4* ve32, const int64_t* vstart, const float4* staging,
+                                       float* se32, int32_t* se_vox) {
+  __shared__ float4 slots[kFillScanThreads / 32][96];
   const int64_t i = i0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= i1) return;
-  const int64_t q = qlist ? (int64_t)qlist[i] : i;
-  fill_scan_one(q, order[q], n_obs, obs_vox, vscale, vrank, voxel_off, slice_off, ve32, vstart, staging, se32);
+  const int64_t q = i >= i1 ? -1 : qlist ? (int64_t)qlist[i] : i;
+  fill_scan_one(q, q >= 0 ? order[q] : 0, n_obs, place, vanchor, slice_off, ve32, vstart, staging, se32, se_vox,
+                slots[threadIdx.x >> 5]);
 }
 
 // blocks of 128 threads for kFrameLanes threads per voxel of n voxels
@@ -462,13 +511,13 @@ cudaError_t build_mixed_voxels(const LoadInput& in, const LayoutBuffers& lb, con
   if (v1 <= v0) return cudaSuccess;
   LoadInput cur = in;
   cur.poses = poses2;  // buffer 0
-  voxel_frames_kernel<<<frame_blocks(v1 - v0), 128, 0, stream>>>(cur, v0, v1, mb.sref, lb.vrank, mb.vstate,
-                                                                 mb.vanchor, mb.planes32_2);
+  voxel_frames_kernel<<<frame_blocks(v1 - v0), 128, 0, stream>>>(cur, v0, v1, mb.sref, lb.vrank, lb.vscale,
+                                                                 mb.vstate, mb.vanchor, mb.planes32_2);
   ++*launches;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || o1 <= o0) return e;
-  fill_staging_kernel<<<(unsigned)((o1 - o0 + 127) / 128), 128, 0, stream>>>(cur, o0, o1, lb.obs_vox, lb.vrank,
-                                                                            lb.vstart, mb.sref, mb.vanchor, staging);
+  fill_staging_kernel<<<(unsigned)((o1 - o0 + 127) / 128), 128, 0, stream>>>(cur, o0, o1, lb.place, lb.vstart, mb.sref,
+                                                                            mb.vanchor, staging);
   ++*launches;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // the chunk's scan-major entries (scattered over the whole copy)
@@ -491,9 +540,10 @@ cudaError_t build_mixed_scan_major(const LoadInput& in, const LayoutBuffers& lb,
                                    const float4* staging, const uint32_t* qlist, int64_t i0, int64_t i1,
                                    cudaStream_t stream, int64_t* launches) {
   if (i1 <= i0) return cudaSuccess;
-  fill_scan_mixed_kernel<<<(unsigned)((i1 - i0 + 255) / 256), 256, 0, stream>>>(
-      in.n_obs, qlist, i0, i1, lb.scan_order, lb.obs_vox, lb.vscale, lb.vrank, in.voxel_off, lb.slice_off, mb.ve32,
-      lb.vstart, staging, mb.se32);
+  fill_scan_mixed_kernel<<<(unsigned)((i1 - i0 + kFillScanThreads - 1) / kFillScanThreads), kFillScanThreads, 0,
+                           stream>>>(
+      in.n_obs, qlist, i0, i1, lb.scan_order, lb.place, mb.vanchor, lb.slice_off, mb.ve32, lb.vstart, staging, mb.se32,
+      mb.se_vox);
   ++*launches;
   return cudaGetLastError();
 }
@@ -516,8 +566,8 @@ cudaError_t build_mixed(const LoadInput& in, const LayoutBuffers& lb, const doub
   cur.poses = poses2;  // buffer 0
   const int64_t nv = in.n_voxels;
   if (nv > 0) {
-    voxel_frames_kernel<<<frame_blocks(nv), 128, 0, stream>>>(cur, 0, nv, mb.sref, lb.vrank, mb.vstate, mb.vanchor,
-                                                               mb.planes32_2);
+    voxel_frames_kernel<<<frame_blocks(nv), 128, 0, stream>>>(cur, 0, nv, mb.sref, lb.vrank, lb.vscale, mb.vstate,
+                                                               mb.vanchor, mb.planes32_2);
     ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // every slot, padding included, by sorted position (coalesced writes)

@@ -126,11 +126,11 @@ struct ValidateResult {
   long long n_obs_seen;
   long long max_len;
 };
-// with_agg = false leaves the clusters unchecked (launch_validate_agg checks a
-// range of them once they are on the device)
-cudaError_t launch_validate(const LoadInput& in, ValidateResult* d_res, bool with_agg, cudaStream_t stream,
+// offsets, scan ids and poses; t32 (n_scans) receives the poses' translations in FP32
+cudaError_t launch_validate(const LoadInput& in, ValidateResult* d_res, float4* t32, cudaStream_t stream,
                             int64_t* launches);
-cudaError_t launch_validate_agg(const LoadInput& in, int64_t o0, int64_t o1, ValidateResult* d_res,
+// clusters [o0, o1) of agg; dst non-null: also copied there, at the same places
+cudaError_t launch_validate_agg(const double* agg, int64_t o0, int64_t o1, double* dst, ValidateResult* d_res,
                                 cudaStream_t stream, int64_t* launches);
 
 // Build the device layout; buffers are allocated through the given allocators
@@ -153,7 +153,7 @@ struct LayoutBuffers {
   int64_t max_len;  // observations of the longest voxel (rows of the longest slice)
   // kept only when the FP64 copies are not built (mixed precision)
   int32_t* vrank;        // input voxel -> sorted position
-  int32_t* obs_vox;      // observation -> input voxel
+  int2* place;           // observation -> (sorted voxel position, row)
   double* vscale;        // input voxel -> 2 / N_i
   uint32_t* scan_order;  // scan-major position -> observation
   // kept only by a load with defer_scale: vstart[p] = observations of the
@@ -163,10 +163,12 @@ struct LayoutBuffers {
 // `keep` allocates the buffers of *out, `temp` the build's temporaries (the
 // caller frees those after the stream has drained).
 // With fill_f64 the FP64 cluster copies are filled; without, only the index
-// structures are built and the maps above are kept for the FP32 copies.
+// structures are built and the maps above are kept for the FP32 copies (se_vox
+// is left for the mixed path's scan-major copy to fill).  t32: the poses'
+// translations in FP32 (launch_validate).
 // With defer_scale the clusters are not read (vscale is left for
 // launch_vscale, voxel range by voxel range, as the clusters arrive).
-cudaError_t build_layout(const LoadInput& in, int max_len, bool fill_f64, bool defer_scale, Allocator keep,
+cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bool fill_f64, bool defer_scale, Allocator keep,
                          Allocator temp, LayoutBuffers* out, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_vscale(const LoadInput& in, int64_t v0, int64_t v1, double* vscale, cudaStream_t stream,
                           int64_t* launches);
@@ -201,6 +203,7 @@ struct MixedBuffers {
   double* sref;
   float* stab2;
   float4* planes32_2;
+  int32_t* se_vox;  // the layout's, filled with the scan-major copy
 };
 cudaError_t build_mixed(const LoadInput& in, const LayoutBuffers& lb, const double* poses2, MixedBuffers& mb,
                         cudaStream_t stream, int64_t* launches);
