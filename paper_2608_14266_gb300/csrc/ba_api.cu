@@ -379,7 +379,6 @@ struct CopyDrain {
 ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_obs, const int64_t* voxel_off,
                     const int32_t* obs_scan, const double* agg, int32_t agg_form, const double* poses, int32_t mem_kind,
                     int32_t agg_mem_kind) {
-  cudaError_t e;
   LoadInput in{};
   in.n_scans = n_scans;
   in.n_voxels = n_voxels;
@@ -393,24 +392,68 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   // anchors, slots staged voxel by voxel in the sorted voxel order) while the
   // next chunk is on its way.
   const bool pipelined = h->mixed && mem_kind == BA_MEM_HOST && agg_mem_kind == BA_MEM_HOST && n_voxels > kWindow;
-  in.voxel_off = stage(h, voxel_off, (size_t)n_voxels + 1, mem_kind, own, &e);
-  if (e != cudaSuccess) return cuda_fail(h, e, "stage voxel offsets");
-  in.obs_scan = stage(h, obs_scan, (size_t)n_obs, mem_kind, own, &e);
-  if (e != cudaSuccess) return cuda_fail(h, e, "stage obs_scan");
-  // clusters in device memory are copied while they are validated, where a
-  // kernel can read them as doubles
-  const bool copy_agg =
-      own && agg_mem_kind == BA_MEM_DEVICE && reinterpret_cast<uintptr_t>(agg) % alignof(double) == 0;
-  if (pipelined || copy_agg) {
-    double* d = (double*)dev_alloc(h, h->keep, sizeof(double) * 10 * (size_t)n_obs);
-    if (!d) return fail(h, BA_ERR_OOM, "clusters: out of device memory");
-    in.agg = d;
-  } else {
-    in.agg = stage(h, agg, (size_t)n_obs * 10, agg_mem_kind, own, &e);
-    if (e != cudaSuccess) return cuda_fail(h, e, "stage clusters");
+  // Device inputs that a kernel can read are read in place, and copied (the
+  // mixed path's own copies, the poses) by the kernels that validate them; all
+  // others are copied first.
+  auto readable = [](const void* p, int kind, size_t align) {
+    return kind == BA_MEM_DEVICE && reinterpret_cast<uintptr_t>(p) % align == 0;
+  };
+  const bool off_read = readable(voxel_off, mem_kind, alignof(int64_t));
+  const bool scan_read = readable(obs_scan, mem_kind, alignof(int32_t));
+  const bool pose_read = readable(poses, mem_kind, alignof(double));
+  const bool agg_read = readable(agg, agg_mem_kind, alignof(double));
+  int64_t* off_own = nullptr;
+  int32_t* scan_own = nullptr;
+  double* agg_own = nullptr;
+  ValidateResult* d_val;
+  float4* t32;
+  uint32_t* box;
+  MixedBuffers& mb = h->mb;
+  h->n_cost = h->mixed ? voxel_pass_blocks(n_voxels) : voxel_pass_f64_blocks(n_voxels);
+  {
+    ArrayGroup inputs, keep, temp;
+    temp.add(&d_val, 1);
+    temp.add(&t32, n_scans);
+    temp.add(&box, 8);
+    if (own || !off_read) inputs.add(&off_own, n_voxels + 1);
+    if (own || !scan_read) inputs.add(&scan_own, n_obs);
+    if (own || !agg_read) inputs.add(&agg_own, 10 * n_obs);
+    // iteration buffers
+    keep.add(&h->poses2, 24 * (size_t)n_scans);
+    keep.add(&h->planes2, 2 * kPlaneStride * (size_t)n_voxels);
+    keep.add(&h->gH, kGH * (size_t)n_scans);
+    keep.add(&h->pred_part, n_scans);
+    keep.add(&h->cost_part, h->n_cost);
+    keep.add(&h->d_state, 1);
+    if (h->mixed) {
+      keep.add(&mb.vstate, 2 * (size_t)n_voxels);
+      // + 4 floats: the staged scan pass copies the float2 array from even indices to even ends
+      keep.add(&mb.se32, 10 * (size_t)n_obs + 4);
+      keep.add(&mb.vanchor, n_voxels);
+      // FP64 reference poses, their FP32 copy (see scan_ref_kernel), then the FP64
+      // quaternions of dR of both pose buffers (sq2_of)
+      keep.add(&mb.sref, (18 + 8) * (size_t)n_scans);
+      keep.add(&mb.stab2, 2 * kTab * (size_t)n_scans);
+      keep.add(&mb.planes32_2, 2 * 2 * (size_t)n_voxels);
+    }
+    if ((!inputs.empty() && !inputs.allocate({own ? keep_fn : temp_fn, h})) || !keep.allocate({keep_fn, h}) ||
+        !temp.allocate({temp_fn, h}))
+      return fail(h, BA_ERR_OOM, "load buffers: out of device memory");
   }
-  in.poses = stage(h, poses, (size_t)n_scans * 12, mem_kind, false, &e);
-  if (e != cudaSuccess) return cuda_fail(h, e, "stage poses");
+  auto copy_in = [&](void* dst, const void* src, size_t bytes, int kind) {
+    return cudaMemcpyAsync(dst, src, bytes, kind == BA_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                           h->stream);
+  };
+  if (!off_read)
+    CK(h, copy_in(off_own, voxel_off, sizeof(int64_t) * ((size_t)n_voxels + 1), mem_kind), "stage voxel offsets");
+  if (!scan_read) CK(h, copy_in(scan_own, obs_scan, sizeof(int32_t) * (size_t)n_obs, mem_kind), "stage obs_scan");
+  if (!pose_read) CK(h, copy_in(h->poses2, poses, sizeof(double) * 12 * (size_t)n_scans, mem_kind), "stage poses");
+  if (!agg_read && !pipelined)
+    CK(h, copy_in(agg_own, agg, sizeof(double) * 10 * (size_t)n_obs, agg_mem_kind), "stage clusters");
+  in.voxel_off = off_own ? off_own : voxel_off;
+  in.obs_scan = scan_own ? scan_own : obs_scan;
+  in.agg = agg_own ? agg_own : agg;
+  in.poses = h->poses2;
 
   // The clusters' copy, chunk by chunk, behind the allocation on the handle's
   // stream, started before validation (the copy of a load that fails is
@@ -463,19 +506,19 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   }
 
   // validation (the clusters of a pipelined load are checked chunk by chunk)
-  ValidateResult init;
-  init.first_bad_offset = init.first_empty_voxel = init.first_bad_scan = init.first_bad_count =
-      init.first_nonfinite_agg = init.first_bad_pose = LLONG_MAX;
-  init.n_obs_seen = 0;
-  init.max_len = 0;
-  ValidateResult* d_val = (ValidateResult*)dev_alloc(h, h->temp, sizeof(ValidateResult));
-  float4* t32 = (float4*)dev_alloc(h, h->temp, sizeof(float4) * (size_t)n_scans);
-  if (!d_val || !t32) return fail(h, BA_ERR_OOM, "validation buffer: out of device memory");
-  CK(h, cudaMemcpyAsync(d_val, &init, sizeof init, cudaMemcpyHostToDevice, h->stream), "validation init");
-  CK(h, launch_validate(in, d_val, t32, h->stream, &h->launches), "validate");
+  CK(h, launch_load_init(d_val, box, h->stream, &h->launches), "validation init");
+  {
+    LoadInput src = in;
+    src.voxel_off = off_read ? voxel_off : off_own;
+    src.obs_scan = scan_read ? obs_scan : scan_own;
+    src.poses = pose_read ? poses : h->poses2;
+    const InputCopies to{off_read ? off_own : nullptr, scan_read ? scan_own : nullptr,
+                         pose_read ? h->poses2 : nullptr, t32};
+    CK(h, launch_validate(src, to, d_val, h->stream, &h->launches), "validate");
+  }
   if (!pipelined)
-    CK(h, launch_validate_agg(copy_agg ? agg : in.agg, 0, n_obs, copy_agg ? const_cast<double*>(in.agg) : nullptr,
-                              d_val, h->stream, &h->launches),
+    CK(h, launch_validate_agg(agg_read ? agg : agg_own, 0, n_obs, agg_read ? agg_own : nullptr, d_val, h->stream,
+                              &h->launches),
        "validate");
   ValidateResult res;
   CK(h, cudaMemcpyAsync(&res, d_val, sizeof res, cudaMemcpyDeviceToHost, h->stream), "validation result");
@@ -490,7 +533,7 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   Allocator keep{keep_fn, h}, temp{temp_fn, h};
   {
     cudaError_t be =
-        build_layout(in, t32, (int)res.max_len, !h->mixed, pipelined, keep, temp, &lb, h->stream, &h->launches);
+        build_layout(in, t32, box, (int)res.max_len, !h->mixed, pipelined, keep, temp, &lb, h->stream, &h->launches);
     if (be != cudaSuccess) return cuda_fail(h, be, "layout build");
   }
   DevLayout& L = h->L;
@@ -508,51 +551,10 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   L.scan_off = lb.scan_off;
   L.se = lb.se;
   L.se_vox = lb.se_vox;
-  {
-    // scan-pass block order: scans by decreasing observation count (ties by
-    // index), so the longest start first
-    std::vector<int64_t> so((size_t)n_scans + 1);
-    CK(h, cudaMemcpyAsync(so.data(), lb.scan_off, sizeof(int64_t) * so.size(), cudaMemcpyDeviceToHost, h->stream),
-       "scan order");
-    CK(h, cudaStreamSynchronize(h->stream), "scan order");
-    std::vector<int32_t> ord((size_t)n_scans);
-    for (int32_t j = 0; j < n_scans; ++j) ord[j] = j;
-    std::stable_sort(ord.begin(), ord.end(),
-                     [&](int32_t a, int32_t b) { return so[a + 1] - so[a] > so[b + 1] - so[b]; });
-    int32_t* d_ord = (int32_t*)dev_alloc(h, h->keep, sizeof(int32_t) * (size_t)n_scans);
-    if (!d_ord) return fail(h, BA_ERR_OOM, "scan order: out of device memory");
-    CK(h, cudaMemcpyAsync(d_ord, ord.data(), sizeof(int32_t) * ord.size(), cudaMemcpyHostToDevice, h->stream),
-       "scan order");
-    L.scan_order = d_ord;
-  }
-
-  // iteration buffers
-  h->n_cost = h->mixed ? voxel_pass_blocks(n_voxels) : voxel_pass_f64_blocks(n_voxels);
-  h->poses2 = (double*)dev_alloc(h, h->keep, sizeof(double) * 24 * (size_t)n_scans);
-  h->planes2 = (double*)dev_alloc(h, h->keep, sizeof(double) * 2 * kPlaneStride * (size_t)n_voxels);
-  h->gH = (double*)dev_alloc(h, h->keep, sizeof(double) * kGH * (size_t)n_scans);
-  h->pred_part = (double*)dev_alloc(h, h->keep, sizeof(double) * (size_t)n_scans);
-  h->cost_part = (double*)dev_alloc(h, h->keep, sizeof(double) * (size_t)h->n_cost);
-  h->d_state = (DevState*)dev_alloc(h, h->keep, sizeof(DevState));
-  if (!h->poses2 || !h->planes2 || !h->gH || !h->pred_part || !h->cost_part || !h->d_state)
-    return fail(h, BA_ERR_OOM, "iteration buffers: out of device memory");
-  CK(h, cudaMemcpyAsync(h->poses2, in.poses, sizeof(double) * 12 * (size_t)n_scans, cudaMemcpyDeviceToDevice,
-                        h->stream),
-     "initial poses");
+  L.scan_order = lb.scans_by_len;
   if (h->mixed) {
-    MixedBuffers& mb = h->mb;
     mb.ve32 = (float4*)dev_alloc(h, h->keep, sizeof(float4) * kVe32 * (size_t)lb.n_elems);
-    mb.vstate = (float4*)dev_alloc(h, h->keep, sizeof(float4) * 2 * (size_t)n_voxels);
-    // + 16 bytes: the staged scan pass copies the float2 array from even indices to even ends
-    mb.se32 = (float*)dev_alloc(h, h->keep, sizeof(float) * 10 * (size_t)n_obs + 16);
-    mb.vanchor = (float4*)dev_alloc(h, h->keep, sizeof(float4) * (size_t)n_voxels);
-    // FP64 reference poses, their FP32 copy (see scan_ref_kernel), then the FP64
-    // quaternions of dR of both pose buffers (sq2_of)
-    mb.sref = (double*)dev_alloc(h, h->keep, (18 + 8) * sizeof(double) * (size_t)n_scans);
-    mb.stab2 = (float*)dev_alloc(h, h->keep, sizeof(float) * 2 * kTab * (size_t)n_scans);
-    mb.planes32_2 = (float4*)dev_alloc(h, h->keep, sizeof(float4) * 2 * 2 * (size_t)n_voxels);
-    if (!mb.ve32 || !mb.vstate || !mb.se32 || !mb.vanchor || !mb.sref || !mb.stab2 || !mb.planes32_2)
-      return fail(h, BA_ERR_OOM, "mixed-precision copies: out of device memory");
+    if (!mb.ve32) return fail(h, BA_ERR_OOM, "mixed-precision copies: out of device memory");
     mb.se_vox = lb.se_vox;
     h->in_keep = in;
     h->in_keep.poses = nullptr;
@@ -1035,17 +1037,17 @@ int64_t ba_estimate_bytes(int32_t precision, int32_t n_scans, int64_t n_voxels, 
   }
   // (+ 8: the mixed layout's spatial-order observation offsets)
   const int64_t per_voxel = 8 + 4 + 4 + 4 + 8 + 2 * 32 + 16 + 32 + 8 + 2 * 32 + 16 + (precision == BA_MIXED ? 8 : 0);
-  const int64_t per_scan = 8 + 24 * 8 + 27 * 8 + 8 + 26 * 8 + 2 * kTab * 4;
+  const int64_t per_scan = 8 + 4 + 24 * 8 + 27 * 8 + 8 + 26 * 8 + 2 * kTab * 4;
   const int64_t keep = per_obs * n_obs + per_slot * slots + per_voxel * n_voxels + per_scan * (int64_t)n_scans +
                        (1 << 16);
   // load: staged inputs (host inputs), sort keys/values and scratch, the
   // spatial order's per-voxel means and prefixes, and (mixed loads of host
   // inputs) the staged slots, the scan-major positions grouped by chunk and
   // that grouping's sort keys, buffers and scratch
-  const int64_t nsort = n_obs > n_voxels ? n_obs : n_voxels;
+  const int64_t nsort = std::max(std::max(n_obs, n_voxels), (int64_t)n_scans);
   if (peak_extra)
     *peak_extra = (80 + 4 + 8 + 4 + (precision == BA_MIXED ? 16 * kVe32 + 4 + 12 + 2 : 0)) * n_obs + 16 * nsort +
-                  24 * nsort / 16 + (8 + 16 + 8 + 8) * (int64_t)n_voxels;
+                  24 * nsort / 16 + (8 + 16 + 8 + 8) * (int64_t)n_voxels + 16 * (int64_t)n_scans;
   return keep;
 }
 

@@ -2,7 +2,9 @@
 // primitives it uses: a stable LSD radix sort of (key, value) pairs, an
 // exclusive scan, input validation and point-cluster formation (Eq. 2).
 // Everything here runs once per load; none of it is on the per-iteration path.
+#include <algorithm>
 #include <cfloat>
+#include <climits>
 #include <utility>
 
 #include "block_order.cuh"
@@ -392,11 +394,28 @@ __device__ inline void amin(long long* p, long long v) { atomicMin(p, v); }
 
 constexpr int kValidateThreads = 256;
 
+__global__ void load_init_kernel(ValidateResult* r, uint32_t* box) {
+  const int k = threadIdx.x;
+  if (k < 6) box[k] = k < 3 ? 0xffffffffu : 0u;  // minima, maxima
+  if (k == 0) {
+    r->first_bad_offset = r->first_empty_voxel = r->first_bad_scan = r->first_bad_count = r->first_nonfinite_agg =
+        r->first_bad_pose = LLONG_MAX;
+    r->n_obs_seen = 0;
+    r->max_len = 0;
+  }
+}
+
+cudaError_t launch_load_init(ValidateResult* d_res, uint32_t* box, cudaStream_t stream, int64_t* launches) {
+  load_init_kernel<<<1, 32, 0, stream>>>(d_res, box);
+  ++*launches;
+  return cudaGetLastError();
+}
+
 // offsets and voxel lengths, scan ids, and poses (their translations also into
-// t32 in FP32, for the spatial order), a range of blocks each.  Every thread of
-// a voxel block reaches the warp reduction.
+// t32 in FP32, for the spatial order), a range of blocks each, and their copies
+// where asked for.  Every thread of a voxel block reaches the warp reduction.
 __global__ void __launch_bounds__(kValidateThreads) validate_kernel(LoadInput in, int64_t voxel_blocks,
-                                                                    int64_t scan_blocks, float4* t32,
+                                                                    int64_t scan_blocks, InputCopies to,
                                                                     ValidateResult* r) {
   int64_t blk = blockIdx.x;
   if (blk < voxel_blocks) {
@@ -404,6 +423,7 @@ __global__ void __launch_bounds__(kValidateThreads) validate_kernel(LoadInput in
     int len = 0;  // the voxel's observation count (capped at 2^31 - 1), 0 if none or invalid
     if (i <= in.n_voxels) {
       const int64_t a = in.voxel_off[i];
+      if (to.voxel_off) to.voxel_off[i] = a;
       if (i == 0 && a != 0) amin(&r->first_bad_offset, 0);
       if (i == in.n_voxels) {
         if (a != in.n_obs) amin(&r->first_bad_offset, i);
@@ -424,16 +444,24 @@ __global__ void __launch_bounds__(kValidateThreads) validate_kernel(LoadInput in
     const int64_t o = blk * kValidateThreads + threadIdx.x;
     if (o < in.n_obs) {
       const int32_t j = in.obs_scan[o];
+      if (to.obs_scan) to.obs_scan[o] = j;
       if (j < 0 || j >= in.n_scans) amin(&r->first_bad_scan, o);
     }
     return;
   }
   const int64_t j = (blk - scan_blocks) * kValidateThreads + threadIdx.x;
   if (j >= in.n_scans) return;
-  const double* P = in.poses + 12 * j;
+  double P[12];
   bool ok = true;
-  for (int k = 0; k < 12; ++k) ok = ok && isfinite(P[k]);
-  for (int a = 0; a < 3 && ok; ++a)
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    P[k] = in.poses[12 * j + k];
+    if (to.poses) to.poses[12 * j + k] = P[k];
+    ok = ok && isfinite(P[k]);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
     for (int b = 0; b < 3; ++b) {
       const double d = P[3 * a] * P[3 * b] + P[3 * a + 1] * P[3 * b + 1] + P[3 * a + 2] * P[3 * b + 2];
       if (fabs(d - (a == b ? 1.0 : 0.0)) > 1e-6) ok = false;
@@ -444,7 +472,7 @@ __global__ void __launch_bounds__(kValidateThreads) validate_kernel(LoadInput in
     if (det < 0.0) ok = false;
   }
   if (!ok) amin(&r->first_bad_pose, j);
-  t32[j] = make_float4(f64_to_f32(P[9]), f64_to_f32(P[10]), f64_to_f32(P[11]), 0.f);
+  to.t32[j] = make_float4(f64_to_f32(P[9]), f64_to_f32(P[10]), f64_to_f32(P[11]), 0.f);
 }
 
 // Clusters [o0, o1): finite, and at least one point; with dst given also copied
@@ -489,11 +517,11 @@ __global__ void __launch_bounds__(kValidateThreads) validate_agg_kernel(const do
   }
 }
 
-cudaError_t launch_validate(const LoadInput& in, ValidateResult* d_res, float4* t32, cudaStream_t stream,
+cudaError_t launch_validate(const LoadInput& in, const InputCopies& to, ValidateResult* d_res, cudaStream_t stream,
                             int64_t* launches) {
   auto blocks = [](int64_t n) { return (n + kValidateThreads - 1) / kValidateThreads; };
   const int64_t nv = blocks(in.n_voxels + 1), no = blocks(in.n_obs), ns = blocks(in.n_scans);
-  validate_kernel<<<(unsigned)(nv + no + ns), kValidateThreads, 0, stream>>>(in, nv, no, t32, d_res);
+  validate_kernel<<<(unsigned)(nv + no + ns), kValidateThreads, 0, stream>>>(in, nv, no, to, d_res);
   ++*launches;
   return cudaGetLastError();
 }
@@ -801,37 +829,84 @@ cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBoun
   return cudaSuccess;
 }
 
-cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bool fill_f64, bool defer_scale, Allocator keep,
-                         Allocator temp, LayoutBuffers* out, cudaStream_t stream, int64_t* launches) {
+// Scans by decreasing observation count, ties by index.  Up to kRankScans in
+// one block, each thread counting the scans before its own (1000 scans: 5 us,
+// where the sort's launches take 12); beyond, the general sort of n_obs - count.
+constexpr int kRankScans = 1024;
+__global__ void __launch_bounds__(kRankScans) scan_rank_kernel(const int64_t* __restrict__ scan_off, int n,
+                                                               int32_t* __restrict__ order) {
+  __shared__ __align__(16) uint32_t len[kRankScans];
+  const int j = threadIdx.x;
+  const uint32_t mine = j < n ? (uint32_t)(scan_off[j + 1] - scan_off[j]) : 0u;
+  len[j] = mine;
+  __syncthreads();
+  if (j >= n) return;
+  int rank = 0;
+#pragma unroll 8
+  for (int i = 0; i < n; ++i) rank += len[i] > mine || (len[i] == mine && i < j);
+  order[rank] = j;
+}
+
+__global__ void scan_len_keys_kernel(const int64_t* scan_off, int32_t n_scans, int64_t n_obs, uint32_t* keys) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < n_scans) keys[j] = (uint32_t)(n_obs - (scan_off[j + 1] - scan_off[j]));
+}
+
+cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, int max_len, bool fill_f64,
+                         bool defer_scale, Allocator keep, Allocator temp, LayoutBuffers* out, cudaStream_t stream,
+                         int64_t* launches) {
   const int64_t nv = in.n_voxels, no = in.n_obs;
-  const int64_t n_slices = (nv + kSlice - 1) / kSlice;
-  const int64_t nsort = nv > no ? nv : no;
+  const int64_t n_slices = (nv + kSlice - 1) / kSlice, n_windows = (nv + kWindow - 1) / kWindow;
+  const int64_t nsort = std::max(std::max(nv, no), (int64_t)in.n_scans);
   const int scan_bits = bit_width((uint64_t)(in.n_scans - 1));
-  // temporaries (the maps are kept when the FP32 copies will be rebuilt later)
-  Allocator maps = fill_f64 ? temp : keep;
-  uint32_t* keys = (uint32_t*)temp.fn(temp.self, sizeof(uint32_t) * nsort);
-  uint32_t* vals = (uint32_t*)temp.fn(temp.self, sizeof(uint32_t) * nsort);
-  uint32_t* tk = (uint32_t*)temp.fn(temp.self, sizeof(uint32_t) * nsort);
-  uint32_t* tv = (uint32_t*)temp.fn(temp.self, sizeof(uint32_t) * nsort);
-  int64_t* scratch = (int64_t*)temp.fn(temp.self, sizeof(int64_t) * (radix_scratch_count(nsort) +
-                                                                      scan_scratch_count(n_slices + no + 2)));
-  int32_t* vrank = (int32_t*)maps.fn(maps.self, sizeof(int32_t) * nv);
-  int32_t* obs_vox = (int32_t*)temp.fn(temp.self, sizeof(int32_t) * no);
-  int2* place = fill_f64 ? nullptr : (int2*)keep.fn(keep.self, sizeof(int2) * no);
-  double* vscale = (double*)maps.fn(maps.self, sizeof(double) * nv);
-  uint32_t* order = fill_f64 ? nullptr : (uint32_t*)keep.fn(keep.self, sizeof(uint32_t) * no);
-  // persistent
-  out->slice_off = (int64_t*)keep.fn(keep.self, sizeof(int64_t) * (n_slices + 1));
-  out->vlen = (int32_t*)keep.fn(keep.self, sizeof(int32_t) * nv);
-  out->vperm = (int32_t*)keep.fn(keep.self, sizeof(int32_t) * nv);
-  out->scan_off = (int64_t*)keep.fn(keep.self, sizeof(int64_t) * (in.n_scans + 1));
-  out->se = fill_f64 ? (double*)keep.fn(keep.self, sizeof(double) * 10 * no) : nullptr;
-  // + 4 entries: the staged mixed scan pass copies whole 16-byte groups
-  out->se_vox = (int32_t*)keep.fn(keep.self, sizeof(int32_t) * (no + 4));
-  if (!keys || !vals || !tk || !tv || !scratch || !vrank || !obs_vox || !vscale || !out->slice_off || !out->vlen ||
-      !out->vperm || !out->scan_off || (fill_f64 && !out->se) || (!fill_f64 && (!order || !place)) ||
-      !out->se_vox)
-    return cudaErrorMemoryAllocation;
+  // Slots of all slices.  Within a window the lengths decrease, so each slice's
+  // padding is at most 32 x (its longest - the next slice's longest) and a
+  // window's at most 32 x max_len: where that bound keeps the slots within the
+  // estimate's share (an eighth more than the observations) it stands for their
+  // number, and the host need not wait for the prefix sum; else the sum is read.
+  const int64_t elem_bound = (no + n_windows * kSlice * (int64_t)max_len + kSlice - 1) / kSlice * kSlice;
+  const bool bounded = elem_bound <= no + no / 8 + 64;
+  uint32_t *keys, *vals, *tk, *tv;
+  int64_t *scratch, *pscratch, *pbase;
+  int32_t *vrank, *obs_vox;
+  int2* place = nullptr;
+  double* vscale;
+  uint32_t* order = nullptr;
+  float4* mean;
+  {
+    ArrayGroup t, k;
+    // the maps are kept when the FP32 copies will be rebuilt later, the
+    // prefixes by a load that stages its slots (they are staged in this order)
+    ArrayGroup& maps = fill_f64 ? t : k;
+    t.add(&keys, nsort);
+    t.add(&vals, nsort);
+    t.add(&tk, nsort);
+    t.add(&tv, nsort);
+    t.add(&scratch, radix_scratch_count(nsort) + scan_scratch_count(n_slices + no + 2));
+    t.add(&pscratch, scan_scratch_count(nv + 1));
+    t.add(&obs_vox, no);
+    t.add(&mean, nv);
+    maps.add(&vrank, nv);
+    maps.add(&vscale, nv);
+    (defer_scale ? k : t).add(&pbase, nv + 1);
+    if (!fill_f64) {
+      k.add(&place, no);
+      k.add(&order, no);
+    }
+    k.add(&out->slice_off, n_slices + 1);
+    k.add(&out->vlen, nv);
+    k.add(&out->vperm, nv);
+    k.add(&out->scan_off, in.n_scans + 1);
+    k.add(&out->scans_by_len, in.n_scans);
+    if (fill_f64) k.add(&out->se, 10 * no);
+    // + 4 entries: the staged mixed scan pass copies whole 16-byte groups
+    k.add(&out->se_vox, no + 4);
+    if (fill_f64 && bounded) {
+      k.add(&out->ve, 10 * elem_bound);
+      k.add(&out->ve_scan, elem_bound);
+    }
+    if (!t.allocate(temp) || !k.allocate(keep)) return cudaErrorMemoryAllocation;
+  }
   out->vrank = vrank;
   out->place = place;
   out->vscale = vscale;
@@ -842,11 +917,6 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bo
   const int win_bits = bit_width((uint64_t)((nv - 1) / kWindow));
   if (len_bits + win_bits > 32) return cudaErrorInvalidValue;
   {
-    float4* mean = (float4*)temp.fn(temp.self, sizeof(float4) * nv);
-    uint32_t* box = (uint32_t*)temp.fn(temp.self, sizeof(uint32_t) * 8);
-    if (!mean || !box) return cudaErrorMemoryAllocation;
-    RETURN_IF(cudaMemsetAsync(box, 0xff, sizeof(uint32_t) * 3, stream));  // minima
-    RETURN_IF(cudaMemsetAsync(box + 3, 0, sizeof(uint32_t) * 3, stream));  // maxima
     const unsigned nb = (unsigned)((nv + 255) / 256);
     observer_mean_kernel<<<nb, 256, 0, stream>>>(in.voxel_off, in.obs_scan, t32, nv, mean, box);
     morton_keys_kernel<<<nb, 256, 0, stream>>>(mean, nv, box, keys);
@@ -863,17 +933,22 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bo
   ++*launches;
   RETURN_IF(cudaGetLastError());
   RETURN_IF(exclusive_scan_i64(out->slice_off, n_slices + 1, scratch, stream, launches));
-  int64_t n_elems = 0;
-  RETURN_IF(cudaMemcpyAsync(&n_elems, out->slice_off + n_slices, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-  RETURN_IF(cudaStreamSynchronize(stream));
+  int64_t n_elems = elem_bound;
+  if (!bounded) {
+    RETURN_IF(cudaMemcpyAsync(&n_elems, out->slice_off + n_slices, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
+    RETURN_IF(cudaStreamSynchronize(stream));
+  }
   out->n_elems = n_elems;
   out->n_slices = n_slices;
   out->max_len = max_len;
   // the FP64 slice copy (the mixed path builds its own FP32 slots)
   if (fill_f64) {
-    out->ve = (double*)keep.fn(keep.self, sizeof(double) * 10 * n_elems);
-    out->ve_scan = (int32_t*)keep.fn(keep.self, sizeof(int32_t) * n_elems);
-    if (!out->ve || !out->ve_scan) return cudaErrorMemoryAllocation;
+    if (!bounded) {
+      ArrayGroup k;
+      k.add(&out->ve, 10 * n_elems);
+      k.add(&out->ve_scan, n_elems);
+      if (!k.allocate(keep)) return cudaErrorMemoryAllocation;
+    }
     fill_sell_kernel<<<(unsigned)((n_slices * kSlice + 255) / 256), 256, 0, stream>>>(
         in, out->vperm, out->vlen, out->slice_off, nv, out->ve, out->ve_scan, n_elems);
     ++*launches;
@@ -883,11 +958,6 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bo
   // ---- scan-major copy ----
   RETURN_IF(launch_obs_voxel(in, 0, nv, obs_vox, defer_scale ? nullptr : vscale, stream, launches));
   {
-    // kept by a load that stages its slots (they are staged in this order)
-    Allocator pb_alloc = defer_scale ? keep : temp;
-    int64_t* pbase = (int64_t*)pb_alloc.fn(pb_alloc.self, sizeof(int64_t) * (nv + 1));
-    int64_t* pscratch = (int64_t*)temp.fn(temp.self, sizeof(int64_t) * scan_scratch_count(nv + 1));
-    if (!pbase || !pscratch) return cudaErrorMemoryAllocation;
     vlen_i64_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, stream>>>(out->vlen, nv, pbase);
     ++*launches;
     RETURN_IF(cudaGetLastError());
@@ -904,11 +974,26 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bo
   scan_off_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, stream>>>(keys, no, in.n_scans, out->scan_off);
   ++*launches;
   RETURN_IF(cudaGetLastError());
-  if (!fill_f64) return cudaSuccess;  // the mixed path fills its own copy, se_vox included
-  fill_scan_major_kernel<<<(unsigned)((no + 255) / 256), 256, 0, stream>>>(in, vals, obs_vox, vscale, vrank, out->se,
-                                                                           out->se_vox);
+  if (fill_f64) {  // the mixed path fills its own copy, se_vox included
+    fill_scan_major_kernel<<<(unsigned)((no + 255) / 256), 256, 0, stream>>>(in, vals, obs_vox, vscale, vrank, out->se,
+                                                                             out->se_vox);
+    ++*launches;
+    RETURN_IF(cudaGetLastError());
+  }
+  // ---- scan-pass block order, so the longest scans start first ----
+  if (in.n_scans <= kRankScans) {
+    scan_rank_kernel<<<1, kRankScans, 0, stream>>>(out->scan_off, in.n_scans, out->scans_by_len);
+    ++*launches;
+    return cudaGetLastError();
+  }
+  const int len_digits = bit_width((uint64_t)no);
+  uint32_t* by_len = (uint32_t*)out->scans_by_len;
+  uint32_t* other = tv;  // free: the scan-major order is in vals
+  scan_len_keys_kernel<<<(unsigned)((in.n_scans + 255) / 256), 256, 0, stream>>>(out->scan_off, in.n_scans, no, keys);
   ++*launches;
   RETURN_IF(cudaGetLastError());
+  if (radix_passes(len_digits) % 2 != 0) std::swap(by_len, other);
+  RETURN_IF(radix_sort_pairs(&keys, &by_len, &tk, &other, in.n_scans, len_digits, true, scratch, stream, launches));
   return cudaSuccess;
 }
 

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "mmba_internal.cuh"
 
@@ -126,8 +127,18 @@ struct ValidateResult {
   long long n_obs_seen;
   long long max_len;
 };
-// offsets, scan ids and poses; t32 (n_scans) receives the poses' translations in FP32
-cudaError_t launch_validate(const LoadInput& in, ValidateResult* d_res, float4* t32, cudaStream_t stream,
+// What the validation of a load's inputs writes besides its result: the inputs'
+// copies in the handle (each may be null), and the poses' translations in FP32.
+struct InputCopies {
+  int64_t* voxel_off;
+  int32_t* obs_scan;
+  double* poses;
+  float4* t32;
+};
+// the result's start values, and those of the spatial order's bounding box (8 words)
+cudaError_t launch_load_init(ValidateResult* d_res, uint32_t* box, cudaStream_t stream, int64_t* launches);
+// offsets, scan ids and poses
+cudaError_t launch_validate(const LoadInput& in, const InputCopies& to, ValidateResult* d_res, cudaStream_t stream,
                             int64_t* launches);
 // clusters [o0, o1) of agg; dst non-null: also copied there, at the same places
 cudaError_t launch_validate_agg(const double* agg, int64_t o0, int64_t o1, double* dst, ValidateResult* d_res,
@@ -139,6 +150,30 @@ struct Allocator {
   void* (*fn)(void* self, size_t bytes);
   void* self;
 };
+// Device arrays of one allocation, each on a 256-byte boundary: a load needs
+// some forty arrays, and an allocation is a call into the driver.
+class ArrayGroup {
+ public:
+  template <typename T>
+  void add(T** p, size_t count) {
+    items_.push_back({(void**)(void*)p, total_});
+    total_ += (sizeof(T) * (count ? count : 1) + 255) & ~(size_t)255;
+  }
+  bool empty() const { return items_.empty(); }
+  bool allocate(Allocator a) {
+    char* base = (char*)a.fn(a.self, total_);
+    for (auto& it : items_) *it.p = base ? base + it.at : nullptr;
+    return base != nullptr;
+  }
+
+ private:
+  struct Item {
+    void** p;
+    size_t at;
+  };
+  std::vector<Item> items_;
+  size_t total_ = 0;
+};
 struct LayoutBuffers {
   int64_t* slice_off;
   int32_t* vlen;
@@ -146,9 +181,10 @@ struct LayoutBuffers {
   double* ve;
   int32_t* ve_scan;
   int64_t* scan_off;
+  int32_t* scans_by_len;  // scans by decreasing observation count, ties by index
   double* se;
   int32_t* se_vox;
-  int64_t n_elems;
+  int64_t n_elems;  // at least the slots of all slices
   int64_t n_slices;
   int64_t max_len;  // observations of the longest voxel (rows of the longest slice)
   // kept only when the FP64 copies are not built (mixed precision)
@@ -165,11 +201,11 @@ struct LayoutBuffers {
 // With fill_f64 the FP64 cluster copies are filled; without, only the index
 // structures are built and the maps above are kept for the FP32 copies (se_vox
 // is left for the mixed path's scan-major copy to fill).  t32: the poses'
-// translations in FP32 (launch_validate).
+// translations in FP32 (launch_validate); box: launch_load_init.
 // With defer_scale the clusters are not read (vscale is left for
 // launch_vscale, voxel range by voxel range, as the clusters arrive).
-cudaError_t build_layout(const LoadInput& in, const float4* t32, int max_len, bool fill_f64, bool defer_scale, Allocator keep,
-                         Allocator temp, LayoutBuffers* out, cudaStream_t stream, int64_t* launches);
+cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, int max_len, bool fill_f64,
+                         bool defer_scale, Allocator keep, Allocator temp, LayoutBuffers* out, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_vscale(const LoadInput& in, int64_t v0, int64_t v1, double* vscale, cudaStream_t stream,
                           int64_t* launches);
 // A load that copies its clusters in chunks of observations [o[k], o[k + 1])

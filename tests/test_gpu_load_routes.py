@@ -86,3 +86,38 @@ def test_bad_cluster_is_named(mm, shift, row, col):
         with mm.BundleAdjuster(precision=prec) as ba:
             with pytest.raises(Exception, match=rf"\b{row}\b"):
                 ba.load_observations(s.n_scans, *args)
+
+
+@pytest.mark.parametrize("n_scans", [1, 1024, 1025, 70001])
+@pytest.mark.parametrize("long_voxel", [0, 6000])
+def test_scan_order_and_slot_bound(mm, n_scans, long_voxel):
+    """The block order of the scans (ranked in one block up to 1024 scans, else
+    sorted) names every scan once, those without an observation included; the
+    number of slots is taken from its bound, or, with one voxel far longer than
+    the others, read back.  Compared with the oracle at the FP64 path's
+    tolerances (1e-10 of the largest entry of g, 1e-11 of H's; with one scan g
+    is zero, a sum that cancels, and is compared at H's)."""
+    rng = np.random.default_rng(n_scans)
+    lens = rng.integers(1, 12, 900)
+    if long_voxel:
+        lens[450] = long_voxel
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    n_obs = int(off[-1])
+    # half of the observations on few scans, so that lengths differ and tie
+    scan = np.where(rng.random(n_obs) < 0.5, rng.integers(0, max(n_scans // 50, 1), n_obs),
+                    rng.integers(0, n_scans, n_obs)).astype(np.int32)
+    pts = rng.normal(size=(n_obs, 8, 3)) * [1.0, 0.7, 0.02] + rng.normal(size=(n_obs, 1, 3))
+    cen = oracle.points_to_centred(np.arange(n_obs + 1, dtype=np.int64) * 8, pts.reshape(-1, 3))
+    pose = np.zeros((n_scans, 12))
+    pose[:, [0, 4, 8]] = 1.0
+    pose[:, 9:] = rng.normal(size=(n_scans, 3))
+    prob = oracle.ObsProblem(n_scans, off, scan, cen)
+    c_ref, planes = oracle.voxel_pass(prob, pose)
+    g_ref, H_ref = oracle.grad_hess(prob, pose, planes, gauss_newton=False)
+    with mm.BundleAdjuster() as ba:
+        ba.load_observations(n_scans, off, scan, cen, pose)
+        assert ba.cost() == pytest.approx(c_ref, rel=1e-10)
+        g, H = ba.gradient()
+        g_tol = 1e-10 * np.abs(g_ref).max() if n_scans > 1 else 1e-11 * np.abs(H_ref).max()
+        np.testing.assert_allclose(g, g_ref, rtol=0, atol=g_tol)
+        np.testing.assert_allclose(H, H_ref, rtol=0, atol=1e-11 * np.abs(H_ref).max())
