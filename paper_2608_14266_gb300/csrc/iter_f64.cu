@@ -381,10 +381,16 @@ __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const
 }
 
 // ---------------------------------------------------------------------------
-// Solver: one thread per scan.  A = H + mu diag(H), A delta = -g by LDL^T,
-// trial pose R' = Exp(dphi) R, t' = t + dt, and the scan's share of the
-// predicted reduction -(g^T delta + delta^T H delta / 2).  The fixed scan and
-// scans without observations keep their pose.
+// Solver: A = H + mu diag(H), A delta = -g by LDL^T, trial pose
+// R' = Exp(dphi) R, t' = t + dt, and the scan's share of the predicted
+// reduction -(g^T delta + delta^T H delta / 2).  The fixed scan and scans
+// without observations keep their pose.
+//
+// Bound by the number of FP64 instructions of a warp (64 cycles of its SM
+// sub-partition each, whatever the lanes): one thread per scan takes 310 for
+// 32 scans, eight lanes per scan 120 for 4.  With fewer warps than
+// sub-partitions the shorter one wins, with several to each the one with less
+// work in all: solve_lanes.
 // ---------------------------------------------------------------------------
 // *stepped = false: the pose is kept (fixed scan, no observation, failed
 // factorisation); otherwise dlt holds the increment.
@@ -442,19 +448,174 @@ __device__ inline double solve_scan(const DevLayout& L, int j, const double* P, 
   return pred;
 }
 
+// Coefficients in th^2, th = |dphi| < 0.1, of sin(th)/th, (1 - cos th)/th^2,
+// cos(th/2) and sin(th/2)/th: the Taylor series to th^8 (the first dropped
+// term is below 1e-17).
+__device__ const double kExpSeries[4][5] = {
+    {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880},
+    {0.5, -1.0 / 24, 1.0 / 720, -1.0 / 40320, 1.0 / 3628800},
+    {1.0, -1.0 / 8, 1.0 / 384, -1.0 / 46080, 1.0 / 10321920},
+    {0.5, -1.0 / 48, 1.0 / 3840, -1.0 / 645120, 1.0 / 185794560},
+};
+
+// Eight lanes per scan.  Lane r < 6 holds row r of [A | -g] and eliminates it
+// by the pivot rows' broadcasts; the substitution runs up the rows' kept
+// factors.  The rotation's columns go to lanes 0..2 (p + a (phi x p) +
+// b phi x (phi x p), the Exp map on a column), the translation to 3..5, the
+// four series and the quaternion's components to 0..3.  Returns this lane's
+// term of the predicted reduction.
+__device__ __forceinline__ double solve_scan_lanes(const DevLayout& L, int64_t j, double* poses2, const double* gH,
+                                                   DevState* st, const double* sref, float* stab2,
+                                                   const double (&series)[5]) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int r = threadIdx.x & 7, row = r < 6 ? r : 5;
+  const unsigned group = 0xffu << (threadIdx.x & 24);
+  const bool live = j < L.n_scans;
+  if (!live) j = L.n_scans - 1;  // computed and not written
+  const int cur = st->cur;
+  const double mu = st->mu;
+  const double* P = poses2 + ((int64_t)cur * L.n_scans + j) * 12;
+  double* Pt = poses2 + ((int64_t)(1 - cur) * L.n_scans + j) * 12;
+  const double* h27 = gH + j * kGH;
+  double h[6], a[7], p[3], q = 0.0, ref = 0.0;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int i = row < c ? row : c, k = row < c ? c : row;
+    h[c] = h27[6 + 6 * i - i * (i - 1) / 2 + (k - i)];
+  }
+  const double g = h27[row];
+  const int pc = r < 3 ? r : 9 + (row - 3);  // a column of R, or an entry of t
+#pragma unroll
+  for (int k = 0; k < 3; ++k) p[k] = P[r < 3 ? pc + 3 * k : pc];
+  double* sq2 = stab2 ? after_wait(sq2_of(sref, L.n_scans)) : nullptr;
+  if (stab2) {
+    q = sq2[((int64_t)cur * L.n_scans + j) * 4 + (r & 3)];
+    ref = sref[12 * j + 9 + (r < 3 ? r : row - 3)];
+  }
+  // a scan nobody observes keeps its pose (see solve_scan)
+  double hd = 0.0;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) hd = row == c ? h[c] : hd;
+  const bool none = (__ballot_sync(kAll, hd != 0.0) & group) == 0;
+  const bool unseen = st->shard ? none : L.scan_off[j + 1] == L.scan_off[j];
+  const bool held = j == L.fixed_scan || unseen;
+
+#pragma unroll
+  for (int c = 0; c < 6; ++c) a[c] = row == c ? fma(mu, h[c], h[c]) : h[c];
+  a[6] = -g;
+  bool ok = true;
+  double inv_row = 0.0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const double d = __shfl_sync(kAll, a[k], k, 8);
+    ok = ok && d > 0.0 && isfinite(d);
+    const double inv = recip_pivot(d);
+    if (row == k) inv_row = inv;
+    if (k == 5) break;
+    const double l = row > k ? a[k] * inv : 0.0;
+#pragma unroll
+    for (int c = k + 1; c < 7; ++c) a[c] = fma(-l, __shfl_sync(kAll, a[c], k, 8), a[c]);
+  }
+  double x = a[6] * inv_row;
+#pragma unroll
+  for (int k = 5; k >= 1; --k) {
+    const double f = row < k ? a[k] * inv_row : 0.0;
+    x = fma(-f, __shfl_sync(kAll, x, k, 8), x);
+  }
+  const unsigned lost = __ballot_sync(kAll, !isfinite(x));  // by every lane, ok or not
+  ok = ok && (lost & group) == 0;
+  const bool stepped = ok && !held;
+  if (live && !held && !ok && r == 0) atomicOr(&st->solve_fail_flag, 1);
+
+  double dlt[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) dlt[c] = __shfl_sync(kAll, x, c, 8);
+  // -(g x + x (H x) / 2) of this row
+  double hx = h[0] * dlt[0];
+#pragma unroll
+  for (int c = 1; c < 6; ++c) hx = fma(h[c], dlt[c], hx);
+  const double pred = live && stepped && r < 6 ? -x * fma(0.5, hx, g) : 0.0;
+
+  const double th2 = fma(dlt[0], dlt[0], fma(dlt[1], dlt[1], dlt[2] * dlt[2]));
+  double v = fma(th2, series[4], series[3]);
+#pragma unroll
+  for (int k = 2; k >= 0; --k) v = fma(th2, v, series[k]);
+  if (!(th2 < 0.01)) {  // uniform over the scan's lanes
+    const double th = sqrt(th2);
+    double sh, ch;
+    sincos(0.5 * th, &sh, &ch);
+    const int w = r & 3;
+    v = w == 0 ? sin(th) / th : w == 1 ? 2.0 * sh * sh / th2 : w == 2 ? ch : sh / th;
+  }
+  __syncwarp();
+  const double ca = __shfl_sync(kAll, v, 0, 8), cb = __shfl_sync(kAll, v, 1, 8);
+  if (live) {
+    if (r < 3) {
+      const double u0 = fma(dlt[1], p[2], -(dlt[2] * p[1])), u1 = fma(dlt[2], p[0], -(dlt[0] * p[2])),
+                   u2 = fma(dlt[0], p[1], -(dlt[1] * p[0]));
+      const double w0 = fma(dlt[1], u2, -(dlt[2] * u1)), w1 = fma(dlt[2], u0, -(dlt[0] * u2)),
+                   w2 = fma(dlt[0], u1, -(dlt[1] * u0));
+      // the increment first: one rounding at the size of p
+      const double n0 = p[0] + fma(ca, u0, cb * w0), n1 = p[1] + fma(ca, u1, cb * w1),
+                   n2 = p[2] + fma(ca, u2, cb * w2);
+      Pt[r] = stepped ? n0 : p[0];
+      Pt[3 + r] = stepped ? n1 : p[1];
+      Pt[6 + r] = stepped ? n2 : p[2];
+    } else if (r < 6) {
+      p[0] = stepped ? p[0] + x : p[0];
+      Pt[6 + r] = p[0];
+    }
+  }
+  if (stab2) {
+    // the step's quaternion times the current one: component i of the product
+    // takes the components i ^ k of the current one, with the signs of the
+    // Hamilton product
+    const double cc = __shfl_sync(kAll, v, 2, 8), cs = __shfl_sync(kAll, v, 3, 8);
+    const int i = r & 3;
+    const double q1 = __shfl_xor_sync(kAll, q, 1), q2 = __shfl_xor_sync(kAll, q, 2), q3 = __shfl_xor_sync(kAll, q, 3);
+    const double s1 = (i & 1) ? q1 : -q1, s2 = i == 1 || i == 2 ? q2 : -q2, s3 = (i & 2) ? q3 : -q3;
+    double qn = fma(cc, q, cs * fma(dlt[0], s1, fma(dlt[1], s2, dlt[2] * s3)));
+    qn = stepped ? qn : q;
+    const double w = __shfl_sync(kAll, qn, 0, 8);
+    const double t = r < 3 ? 0.0 : p[0] - ref;
+    if (live) {
+      if (r < 4) sq2[((int64_t)(1 - cur) * L.n_scans + j) * 4 + r] = qn;
+      // the FP32 table entry (scan_table_from_quat)
+      float* out = stab2 + ((int64_t)(1 - cur) * L.n_scans + j) * kTab;
+      if (r < 4) out[r] = f64_to_f32(w < 0.0 ? -qn : qn);
+      if (r >= 3 && r < 6) out[1 + r] = f64_to_f32(t);
+      if (r < 3) out[7 + r] = f64_to_f32(ref);
+      if (r >= 6) out[4 + r] = 0.0f;
+    }
+  }
+  return pred;
+}
+
 // With stab2 given (mixed precision) the trial scan's FP32 table entry is
 // written too, from the trial pose and the scan's reference pose.  Block blk
-// (scans blk * kSolveThreads ..) writes the sum of its scans' predicted
-// reductions to pred_part[blk], in a fixed order.
+// (kSolveThreads / solve_lanes consecutive scans) writes the sum of its scans'
+// predicted reductions to pred_part[blk], in a fixed order.
 __device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* poses2, const double* gH,
                                                double* pred_part, DevState* st, const double* sref, float* stab2,
                                                int64_t blk, double* red) {
+  const int lanes = solve_lanes(L.n_scans);
+  double series[5];
+  if (lanes == 8) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) series[k] = kExpSeries[threadIdx.x & 3][k];
+  }
   grid_wait();
   grid_launch_next();
   st = after_wait(st);
   gH = after_wait(gH);
   poses2 = after_wait(poses2);
   if (st->honor_stop && st->stop) return;  // uniform over the block
+  if (lanes == 8) {
+    const double tot = block_sum<kSolveThreads>(
+        solve_scan_lanes(L, blk * (kSolveThreads / 8) + threadIdx.x / 8, poses2, gH, st, sref, stab2, series), red);
+    if (threadIdx.x == 0) pred_part[blk] = tot;
+    return;
+  }
   const int64_t j = blk * kSolveThreads + threadIdx.x;
   double pred = 0.0;
   if (j < L.n_scans) {

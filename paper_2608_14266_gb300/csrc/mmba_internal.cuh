@@ -695,13 +695,28 @@ __device__ __forceinline__ float4 quat_mul_f(float4 p, float4 q) {
                      fmaf(p.x, q.w, fmaf(p.y, q.z, fmaf(-p.z, q.y, p.w * q.x))));
 }
 
+// 1 / d for a pivot d: the mantissa's binary32 reciprocal r (|1 - m r| < 2^-22)
+// and one step r + r (e + e^2), e = 1 - m r, of the cubic iteration, which
+// leaves e^3 < 2^-66; the exponent is put back in the bits.  Pivots so small or
+// large that the result is near the ends of the range, and those that are not
+// positive and finite (whose result is not used), divide.
+__device__ __forceinline__ double recip_pivot(double d) {
+  const int hi = __double2hiint(d);
+  const int ex = (hi >> 20) - 1023;  // of a positive d
+  if (ex < -1000 || ex > 1000) return 1.0 / d;
+  const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(d));
+  const double r = f32_to_f64(__frcp_rn(f64_to_f32(m)));
+  const double e = fma(-m, r, 1.0);
+  const double y = fma(r, fma(e, e, e), r);
+  return __hiloint2double(__double2hiint(y) - (ex << 20), __double2loint(y));
+}
+
 // LDL^T of the symmetric 6x6 A (full, row-major) without pivoting, then
 // solve A x = b.  Returns false if a pivot is not positive and finite.
 __device__ inline bool ldlt6_solve(const double* A, const double* b, double* x) {
   // LD[i][k] = L[i][k] D[k], kept as the numerator it is (before the scaling
   // by 1 / D[k]), so every update is one FMA; the pivots' reciprocals serve
-  // the factorisation and the diagonal solve alike (an FP64 division is a
-  // long instruction sequence on this part)
+  // the factorisation and the diagonal solve alike
   double L[6][6], LD[6][6], Di[6];
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
@@ -709,7 +724,7 @@ __device__ inline bool ldlt6_solve(const double* A, const double* b, double* x) 
 #pragma unroll
     for (int k = 0; k < j; ++k) dj = fma(-L[j][k], LD[j][k], dj);
     if (!(dj > 0.0) || !isfinite(dj)) return false;
-    const double inv = 1.0 / dj;
+    const double inv = recip_pivot(dj);
     Di[j] = inv;
 #pragma unroll
     for (int i = j + 1; i < 6; ++i) {

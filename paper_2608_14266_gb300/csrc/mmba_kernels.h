@@ -13,7 +13,7 @@ constexpr int kVoxelThreads = 128;
 constexpr int kScanThreads = 128;      // FP64 scan pass: threads per scan
 constexpr int kScanMixedThreads = 32;  // mixed scan pass: one warp per scan (long pipelined loops, no block barrier)
 constexpr int kDecideThreads = 256;  // one block; FP64 sums are 1/64 rate, so few warps and few adds
-constexpr int kSolveThreads = 64;  // FP64-serial per scan: small blocks spread the scans over every SM
+constexpr int kSolveThreads = 64;  // small blocks spread the scans over every SM
 
 __host__ __device__ inline int64_t voxel_pass_blocks(int64_t n_voxels) { return (n_voxels + kVoxelThreads - 1) / kVoxelThreads; }
 // FP64 voxel pass: voxels per block of kVoxelThreads (a part of a 32-voxel
@@ -32,7 +32,16 @@ __host__ __device__ inline int64_t voxel_pass_f64_blocks(int64_t n_voxels) {
   const int v = voxel_pass_f64_width(n_voxels);
   return (n_voxels + v - 1) / v;
 }
-__host__ __device__ inline int64_t solve_blocks(int64_t n_scans) { return (n_scans + kSolveThreads - 1) / kSolveThreads; }
+// Lanes per scan in the solve kernel: 8 while the GPU has few warps to each of
+// its 608 SM sub-partitions, else 1.  Both sides, launch included: 500 scans
+// 18.5 us with one lane and 12.4 with eight, 4000 scans 19.6 and 16.3, 6000
+// scans 20.5 and 18.4, 10,000 scans 21.7 and 31.6.
+constexpr int64_t kLaneSolveScans = 6144;
+__host__ __device__ inline int solve_lanes(int64_t n_scans) { return n_scans <= kLaneSolveScans ? 8 : 1; }
+__host__ __device__ inline int64_t solve_blocks(int64_t n_scans) {
+  const int per = kSolveThreads / solve_lanes(n_scans);
+  return (n_scans + per - 1) / per;
+}
 
 // Launch of an iteration kernel; with dependent = true it may start while the
 // kernel before it in the stream drains (see grid_wait in mmba_internal.cuh).

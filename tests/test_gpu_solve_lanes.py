@@ -1,0 +1,112 @@
+"""The solve kernel gives eight lanes to a scan up to 6144 scans and one
+beyond: one LM step on both sides of the line, with ragged last blocks, scans
+without observations, a fixed scan, steps below and above the small-angle
+series' 0.1 rad, and a factorisation that fails."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mm():
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2608_14266_gb300 as mm
+    assert torch.cuda.is_available()
+    return mm
+
+
+def _problem(n_scans, tilt, seed):
+    """Planes seen by every scan but each seventh, from poses `tilt` rad off."""
+    rng = np.random.default_rng(seed)
+    seen = np.array([j for j in range(n_scans) if j % 7 != 5 or n_scans < 8])
+    n_vox = 6 * len(seen)
+    lens = rng.integers(2, 5, n_vox)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    n_obs = int(off[-1])
+    scan = seen[(np.repeat(np.arange(n_vox), lens) + rng.integers(0, 4, n_obs)) % len(seen)].astype(np.int32)
+    axes = np.linalg.qr(rng.normal(size=(n_vox, 3, 3)))[0]
+    centre = rng.normal(size=(n_vox, 3)) * 4.0
+    flat = rng.normal(size=(n_obs, 10, 3)) * [1.0, 0.8, 0.01]
+    vox = np.repeat(np.arange(n_vox), lens)
+    world = np.einsum("oij,opj->opi", axes[vox], flat) + centre[vox][:, None, :]
+    # the true poses are identities: the scan frames hold the world points
+    cen = oracle.points_to_centred(np.arange(n_obs + 1, dtype=np.int64) * 10, world.reshape(-1, 3))
+    pose = np.zeros((n_scans, 12))
+    for j in range(n_scans):
+        w = rng.normal(size=3)
+        w *= tilt / np.linalg.norm(w)
+        K = np.array([[0, -w[2], w[1]], [w[2], 0, -w[0]], [-w[1], w[0], 0]])
+        pose[j, :9] = (np.eye(3) + np.sin(tilt) / tilt * K + (1 - np.cos(tilt)) / tilt**2 * K @ K).reshape(-1)
+        pose[j, 9:] = 0.02 * rng.normal(size=3)
+    return n_scans, off, scan, cen, pose
+
+
+@pytest.mark.parametrize("n_scans", [1, 3, 8, 9, 500, 6144, 6145])
+@pytest.mark.parametrize("tilt", [1e-3, 0.3])
+def test_step_matches_oracle(mm, n_scans, tilt):
+    """Tolerances: the pose of a step is the solution of a 6x6 system; its
+    relative error is the condition number (measured here per scan) times the
+    1e-11 the path's H and g are held to, plus rounding."""
+    ns, off, scan, cen, pose = _problem(n_scans, tilt, n_scans)
+    prob = oracle.ObsProblem(ns, off, scan, cen)
+    _, planes = oracle.voxel_pass(prob, pose)
+    g, H = oracle.grad_hess(prob, pose, planes, gauss_newton=True)
+    mu = 1e-2
+    want = pose.copy()
+    tol = np.full(ns, 1e-12)
+    for j in range(ns):
+        if j == 2 or not np.any(np.diag(H[j])):
+            continue
+        A = H[j] + mu * np.diag(np.diag(H[j]))
+        d = np.linalg.solve(A, -g[j])
+        th = np.linalg.norm(d[:3])
+        K = np.array([[0, -d[2], d[1]], [d[2], 0, -d[0]], [-d[1], d[0], 0]])
+        E = np.eye(3) + np.sinc(th / np.pi) * K + 0.5 * np.sinc(th / 2 / np.pi) ** 2 * K @ K
+        want[j, :9] = (E @ pose[j, :9].reshape(3, 3)).reshape(-1)
+        want[j, 9:] += d[3:]
+        s = 1 / np.sqrt(np.diag(A))
+        tol[j] += 1e-11 * np.linalg.cond(A * s[:, None] * s) * (1 + np.abs(d).max())
+    with mm.BundleAdjuster(hessian_mode=1, mu0=mu, fixed_scan=2 if ns > 2 else -1) as ba:
+        ba.load_observations(ns, off, scan, cen, pose)
+        c0 = ba.cost()
+        st = ba.iterate(1)
+        got = ba.poses()
+        if not st["last_accepted"]:
+            assert st["cost"] == c0
+            np.testing.assert_array_equal(got, pose)
+            want = None
+        elif ns > 2:
+            np.testing.assert_array_equal(got[2], pose[2])
+    assert want is not None or n_scans == 1
+    if want is not None:
+        assert (np.abs(got - want).max(axis=1) <= tol).all(), (np.abs(got - want).max(axis=1) / tol).max()
+
+
+@pytest.mark.parametrize("n_scans", [9, 6145])
+def test_failed_factorisation_keeps_the_pose(mm, n_scans):
+    """Boxes of eight corners stacked along z, seen from identity poses: every
+    normal is e_z exactly, so the Gauss-Newton Hessian's entries for x and y
+    are zero, every factorisation fails, and the step is refused."""
+    n_vox = n_scans
+    off = np.arange(n_vox + 1, dtype=np.int64) * 2
+    scan = np.stack([np.arange(n_vox), (np.arange(n_vox) + 1) % n_scans], 1).reshape(-1).astype(np.int32)
+    corner = np.array([[x, y, z] for x in (-2, 2) for y in (-1, 1) for z in (-0.25, 0.25)])
+    pts = np.tile(corner, (2 * n_vox, 1, 1))
+    pts[1::2, :, 2] += 0.125
+    pts += np.repeat(np.arange(n_vox) % 5 - 2.0, 2)[:, None, None] * [1.0, 0.5, 0.0]
+    cen = oracle.points_to_centred(np.arange(2 * n_vox + 1, dtype=np.int64) * 8, pts.reshape(-1, 3))
+    pose = np.zeros((n_scans, 12))
+    pose[:, [0, 4, 8]] = 1.0
+    with mm.BundleAdjuster(hessian_mode=1, fixed_scan=-1) as ba:
+        ba.load_observations(n_scans, off, scan, cen, pose)
+        _, H = ba.gradient()
+        assert (H[:, 3, 3] == 0).all() and (H[:, 5, 5] > 0).all()
+        cost = ba.cost()
+        st = ba.iterate(1)
+        assert not st["last_accepted"] and st["cost"] == cost
+        np.testing.assert_array_equal(ba.poses(), pose)
