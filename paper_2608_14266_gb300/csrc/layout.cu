@@ -29,6 +29,8 @@ constexpr int kScanItems = 8;
 constexpr int64_t kScanTile = (int64_t)kScanBlock * kScanItems;
 
 __global__ void __launch_bounds__(kScanBlock) scan_tiles_kernel(int64_t* data, int64_t n, int64_t* tile_sums) {
+  grid_wait();
+  grid_launch_next();
   __shared__ int64_t warp_tot[kScanBlock / 32];
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   int64_t v[kScanItems];
@@ -68,6 +70,8 @@ __global__ void __launch_bounds__(kScanBlock) scan_tiles_kernel(int64_t* data, i
 }
 
 __global__ void scan_add_kernel(int64_t* data, int64_t n, const int64_t* tile_pre) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) data[i] += tile_pre[i / kScanTile];
 }
@@ -85,16 +89,16 @@ cudaError_t exclusive_scan_i64(int64_t* data, int64_t n, int64_t* scratch, cudaS
   if (n <= 0) return cudaSuccess;
   const int64_t tiles = (n + kScanTile - 1) / kScanTile;
   if (tiles == 1) {
-    scan_tiles_kernel<<<1, kScanBlock, 0, stream>>>(data, n, nullptr);
+    launch_chained(scan_tiles_kernel, 1, kScanBlock, 0, stream, data, n, nullptr);
     ++*launches;
     return cudaGetLastError();
   }
   int64_t* sums = scratch;
-  scan_tiles_kernel<<<(unsigned)tiles, kScanBlock, 0, stream>>>(data, n, sums);
+  launch_chained(scan_tiles_kernel, (unsigned)tiles, kScanBlock, 0, stream, data, n, sums);
   ++*launches;
   RETURN_IF(cudaGetLastError());
   RETURN_IF(exclusive_scan_i64(sums, tiles, scratch + tiles + 1, stream, launches));
-  scan_add_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(data, n, sums);
+  launch_chained(scan_add_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, data, n, sums);
   ++*launches;
   return cudaGetLastError();
 }
@@ -153,8 +157,10 @@ __device__ __forceinline__ void look_store(uint64_t* p, uint64_t v) {
 
 // histograms of the first `passes` digits: hist[256 pass + digit]
 template <typename K>
-__global__ void __launch_bounds__(kRadixBlock) radix_count_kernel(const K* __restrict__ keys, int64_t n, int passes,
+__global__ void __launch_bounds__(kRadixBlock) radix_count_kernel(const K* keys, int64_t n, int passes,
                                                                   uint32_t* hist) {
+  grid_wait();
+  grid_launch_next();
   __shared__ uint32_t cnt[kRadixPasses * 256];
   for (int k = threadIdx.x; k < passes * 256; k += kRadixBlock) cnt[k] = 0;
   __syncthreads();
@@ -310,9 +316,11 @@ __device__ __forceinline__ void radix_tile(const K* __restrict__ keys_in, const 
 // kBlocks: resident blocks per SM that the registers are held to
 template <typename K, int kBlocks>
 __global__ void __launch_bounds__(kRadixBlock, kBlocks)
-    radix_scatter_kernel(const K* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
-                         K* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int64_t n, int pass,
-                         const uint32_t* __restrict__ hist, uint32_t* ticket, uint64_t* look) {
+    radix_scatter_kernel(const K* keys_in, const uint32_t* vals_in,
+                         K* keys_out, uint32_t* vals_out, int64_t n, int pass,
+                         const uint32_t* hist, uint32_t* ticket, uint64_t* look) {
+  grid_wait();
+  grid_launch_next();
   extern __shared__ __align__(16) unsigned char radix_smem[];
   K* skey = reinterpret_cast<K*>(radix_smem);
   uint32_t* sval = reinterpret_cast<uint32_t*>(radix_smem + sizeof(K) * kRadixTile);
@@ -332,6 +340,8 @@ __global__ void __launch_bounds__(kRadixBlock, kBlocks)
 }
 
 __global__ void positions_kernel(int64_t n, uint32_t* v) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) v[i] = (uint32_t)i;
 }
@@ -348,7 +358,7 @@ static cudaError_t radix_sort_pairs_t(K** keys, uint32_t** vals, K** tmp_keys, u
   const int passes = radix_passes(bits);
   if (n <= 1 || passes == 0) {
     if (!positions || n <= 0) return cudaSuccess;
-    positions_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(n, *vals);
+    launch_chained(positions_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, n, *vals);
     ++*launches;
     return cudaGetLastError();
   }
@@ -361,13 +371,11 @@ static cudaError_t radix_sort_pairs_t(K** keys, uint32_t** vals, K** tmp_keys, u
   const auto scatter = tiles <= 2 * 152 ? radix_scatter_kernel<K, 2> : radix_scatter_kernel<K, sizeof(K) == 4 ? 4 : 3>;
   RETURN_IF(cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)radix_scatter_smem<K>()));
   RETURN_IF(cudaMemsetAsync(scratch, 0, sizeof(int64_t) * (size_t)radix_scratch_count(n), stream));
-  radix_count_kernel<K><<<(unsigned)(tiles < kCountBlocks ? tiles : kCountBlocks), kRadixBlock, 0, stream>>>(
-      *keys, n, passes, hist);
+  launch_chained(radix_count_kernel<K>, (unsigned)(tiles < kCountBlocks ? tiles : kCountBlocks), kRadixBlock, 0, stream, *keys, n, passes, hist);
   ++*launches;
   RETURN_IF(cudaGetLastError());
   for (int p = 0; p < passes; ++p) {
-    scatter<<<(unsigned)tiles, kRadixBlock, radix_scatter_smem<K>(), stream>>>(
-        *keys, p == 0 && positions ? nullptr : *vals, *tmp_keys, *tmp_vals, n, p, hist, ticket, look);
+    launch_chained(scatter, (unsigned)tiles, kRadixBlock, radix_scatter_smem<K>(), stream, *keys, p == 0 && positions ? nullptr : *vals, *tmp_keys, *tmp_vals, n, p, hist, ticket, look);
     ++*launches;
     RETURN_IF(cudaGetLastError());
     std::swap(*keys, *tmp_keys);
@@ -395,6 +403,7 @@ __device__ inline void amin(long long* p, long long v) { atomicMin(p, v); }
 constexpr int kValidateThreads = 256;
 
 __global__ void load_init_kernel(ValidateResult* r, uint32_t* box) {
+  grid_launch_next();
   const int k = threadIdx.x;
   if (k < 6) box[k] = k < 3 ? 0xffffffffu : 0u;  // minima, maxima
   if (k == 0) {
@@ -417,6 +426,8 @@ cudaError_t launch_load_init(ValidateResult* d_res, uint32_t* box, cudaStream_t 
 __global__ void __launch_bounds__(kValidateThreads) validate_kernel(LoadInput in, int64_t voxel_blocks,
                                                                     int64_t scan_blocks, InputCopies to,
                                                                     ValidateResult* r) {
+  grid_wait();
+  grid_launch_next();
   int64_t blk = blockIdx.x;
   if (blk < voxel_blocks) {
     const int64_t i = blk * kValidateThreads + threadIdx.x;
@@ -481,9 +492,11 @@ __global__ void __launch_bounds__(kValidateThreads) validate_kernel(LoadInput in
 // rows of 80 bytes are read as one stream.  Bound by DRAM: 15M clusters copied
 // and validated in 435 us; a row per thread was 318 us behind a copy of 360 us.
 template <bool kPair>
-__global__ void __launch_bounds__(kValidateThreads) validate_agg_kernel(const double* __restrict__ agg, int64_t o0,
-                                                                        int64_t o1, double* __restrict__ dst,
+__global__ void __launch_bounds__(kValidateThreads) validate_agg_kernel(const double* agg, int64_t o0,
+                                                                        int64_t o1, double* dst,
                                                                         ValidateResult* r) {
+  grid_wait();
+  grid_launch_next();
   constexpr int kUnits = 4;  // loads in flight
   constexpr int64_t kRow = kPair ? 5 : 10;
   const int64_t e1 = kRow * o1;
@@ -521,7 +534,7 @@ cudaError_t launch_validate(const LoadInput& in, const InputCopies& to, Validate
                             int64_t* launches) {
   auto blocks = [](int64_t n) { return (n + kValidateThreads - 1) / kValidateThreads; };
   const int64_t nv = blocks(in.n_voxels + 1), no = blocks(in.n_obs), ns = blocks(in.n_scans);
-  validate_kernel<<<(unsigned)(nv + no + ns), kValidateThreads, 0, stream>>>(in, nv, no, to, d_res);
+  launch_chained(validate_kernel, (unsigned)(nv + no + ns), kValidateThreads, 0, stream, in, nv, no, to, d_res);
   ++*launches;
   return cudaGetLastError();
 }
@@ -534,9 +547,9 @@ cudaError_t launch_validate_agg(const double* agg, int64_t o0, int64_t o1, doubl
   const int64_t units = (pair ? 5 : 10) * (o1 - o0), per = 4 * kValidateThreads;
   const unsigned nb = (unsigned)((units + per - 1) / per);
   if (pair)
-    validate_agg_kernel<true><<<nb, kValidateThreads, 0, stream>>>(agg, o0, o1, dst, d_res);
+    launch_chained(validate_agg_kernel<true>, nb, kValidateThreads, 0, stream, agg, o0, o1, dst, d_res);
   else
-    validate_agg_kernel<false><<<nb, kValidateThreads, 0, stream>>>(agg, o0, o1, dst, d_res);
+    launch_chained(validate_agg_kernel<false>, nb, kValidateThreads, 0, stream, agg, o0, o1, dst, d_res);
   ++*launches;
   return cudaGetLastError();
 }
@@ -580,9 +593,11 @@ __device__ __forceinline__ float float_from_order_key(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-__global__ void observer_mean_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ obs_scan,
-                                     const float4* __restrict__ t32, int64_t n_voxels, float4* __restrict__ mean,
-                                     uint32_t* __restrict__ box) {
+__global__ void observer_mean_kernel(const int64_t* off, const int32_t* obs_scan,
+                                     const float4* t32, int64_t n_voxels, float4* mean,
+                                     uint32_t* box) {
+  grid_wait();
+  grid_launch_next();
   __shared__ uint32_t sbox[6];
   if (threadIdx.x < 6) sbox[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
   __syncthreads();
@@ -619,8 +634,10 @@ __device__ __forceinline__ uint32_t spread3(uint32_t v) {
   return v;
 }
 
-__global__ void morton_keys_kernel(const float4* __restrict__ mean, int64_t n_voxels, const uint32_t* __restrict__ box,
-                                   uint32_t* __restrict__ keys) {
+__global__ void morton_keys_kernel(const float4* mean, int64_t n_voxels, const uint32_t* box,
+                                   uint32_t* keys) {
+  grid_wait();
+  grid_launch_next();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= n_voxels) return;
   const float4 m = mean[v];
@@ -640,8 +657,10 @@ __global__ void morton_keys_kernel(const float4* __restrict__ mean, int64_t n_vo
 
 // after the spatial sort (vals[r] = voxel of spatial rank r): window of the
 // rank, then length descending
-__global__ void window_keys_kernel(const int64_t* __restrict__ off, const uint32_t* __restrict__ vals,
-                                   int64_t n_voxels, int max_len, int len_bits, uint32_t* __restrict__ keys) {
+__global__ void window_keys_kernel(const int64_t* off, const uint32_t* vals,
+                                   int64_t n_voxels, int max_len, int len_bits, uint32_t* keys) {
+  grid_wait();
+  grid_launch_next();
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n_voxels) return;
   const uint32_t v = vals[r];
@@ -651,6 +670,8 @@ __global__ void window_keys_kernel(const int64_t* __restrict__ off, const uint32
 
 __global__ void slice_len_kernel(const int64_t* off, const uint32_t* vperm, int64_t n_voxels, int64_t n_slices,
                                  int64_t* slice_off, int32_t* vlen, int32_t* vperm_out, int32_t* vrank) {
+  grid_wait();
+  grid_launch_next();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n_voxels) {
     const uint32_t v = vperm[p];
@@ -665,6 +686,8 @@ __global__ void slice_len_kernel(const int64_t* off, const uint32_t* vperm, int6
 
 __global__ void fill_sell_kernel(LoadInput in, const int32_t* vperm, const int32_t* vlen, const int64_t* slice_off,
                                  int64_t n_voxels, double* ve, int32_t* ve_scan, int64_t n_elems) {
+  grid_wait();
+  grid_launch_next();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t s = p >> 5;
   if (s * kSlice >= n_voxels) return;
@@ -706,6 +729,8 @@ __global__ void fill_sell_kernel(LoadInput in, const int32_t* vperm, const int32
 constexpr int kVoxelLanes = 8;
 __global__ void __launch_bounds__(256) obs_voxel_kernel(LoadInput in, int64_t v0, int64_t v1, int32_t* obs_vox,
                                                         double* vscale) {
+  grid_wait();
+  grid_launch_next();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t v = v0 + t / kVoxelLanes;
   const int sub = (int)(t % kVoxelLanes);
@@ -730,6 +755,8 @@ __global__ void __launch_bounds__(256) obs_voxel_kernel(LoadInput in, int64_t v0
 // (and, unless place is null, each observation's sorted voxel position and row)
 __global__ void scan_keys_kernel(LoadInput in, const int32_t* obs_vox, const int32_t* vrank, const int64_t* pbase,
                                  uint32_t* keys, uint32_t* vals, int2* place) {
+  grid_wait();
+  grid_launch_next();
   const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= in.n_obs) return;
   const int32_t v = obs_vox[o];
@@ -746,6 +773,8 @@ __global__ void scan_keys_kernel(LoadInput in, const int32_t* obs_vox, const int
 // predecessor's id up to its own (scans with no observation included), so
 // each entry is written once
 __global__ void scan_off_kernel(const uint32_t* keys, int64_t n, int32_t n_scans, int64_t* scan_off) {
+  grid_wait();
+  grid_launch_next();
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q > n) return;
   const int64_t lo = q == 0 ? 0 : (int64_t)keys[q - 1] + 1;
@@ -754,6 +783,8 @@ __global__ void scan_off_kernel(const uint32_t* keys, int64_t n, int32_t n_scans
 }
 
 __global__ void vlen_i64_kernel(const int32_t* vlen, int64_t n_voxels, int64_t* out) {
+  grid_wait();
+  grid_launch_next();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n_voxels) out[p] = vlen[p];
   if (p == 0) out[n_voxels] = 0;
@@ -761,6 +792,8 @@ __global__ void vlen_i64_kernel(const int32_t* vlen, int64_t n_voxels, int64_t* 
 
 __global__ void fill_scan_major_kernel(LoadInput in, const uint32_t* order, const int32_t* obs_vox,
                                        const double* vscale, const int32_t* vrank, double* se, int32_t* se_vox) {
+  grid_wait();
+  grid_launch_next();
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= in.n_obs) return;
   const int64_t o = order[q];
@@ -800,7 +833,7 @@ static int bit_width(uint64_t x) {
 static cudaError_t launch_obs_voxel(const LoadInput& in, int64_t v0, int64_t v1, int32_t* obs_vox, double* vscale,
                                     cudaStream_t stream, int64_t* launches) {
   if (v1 <= v0) return cudaSuccess;
-  obs_voxel_kernel<<<(unsigned)(((v1 - v0) * kVoxelLanes + 255) / 256), 256, 0, stream>>>(in, v0, v1, obs_vox, vscale);
+  launch_chained(obs_voxel_kernel, (unsigned)(((v1 - v0) * kVoxelLanes + 255) / 256), 256, 0, stream, in, v0, v1, obs_vox, vscale);
   ++*launches;
   return cudaGetLastError();
 }
@@ -833,8 +866,10 @@ cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBoun
 // one block, each thread counting the scans before its own (1000 scans: 5 us,
 // where the sort's launches take 12); beyond, the general sort of n_obs - count.
 constexpr int kRankScans = 1024;
-__global__ void __launch_bounds__(kRankScans) scan_rank_kernel(const int64_t* __restrict__ scan_off, int n,
-                                                               int32_t* __restrict__ order) {
+__global__ void __launch_bounds__(kRankScans) scan_rank_kernel(const int64_t* scan_off, int n,
+                                                               int32_t* order) {
+  grid_wait();
+  grid_launch_next();
   __shared__ __align__(16) uint32_t len[kRankScans];
   const int j = threadIdx.x;
   const uint32_t mine = j < n ? (uint32_t)(scan_off[j + 1] - scan_off[j]) : 0u;
@@ -848,6 +883,8 @@ __global__ void __launch_bounds__(kRankScans) scan_rank_kernel(const int64_t* __
 }
 
 __global__ void scan_len_keys_kernel(const int64_t* scan_off, int32_t n_scans, int64_t n_obs, uint32_t* keys) {
+  grid_wait();
+  grid_launch_next();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < n_scans) keys[j] = (uint32_t)(n_obs - (scan_off[j + 1] - scan_off[j]));
 }
@@ -918,17 +955,17 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
   if (len_bits + win_bits > 32) return cudaErrorInvalidValue;
   {
     const unsigned nb = (unsigned)((nv + 255) / 256);
-    observer_mean_kernel<<<nb, 256, 0, stream>>>(in.voxel_off, in.obs_scan, t32, nv, mean, box);
-    morton_keys_kernel<<<nb, 256, 0, stream>>>(mean, nv, box, keys);
+    launch_chained(observer_mean_kernel, nb, 256, 0, stream, in.voxel_off, in.obs_scan, t32, nv, mean, box);
+    launch_chained(morton_keys_kernel, nb, 256, 0, stream, mean, nv, box, keys);
     *launches += 2;
     RETURN_IF(cudaGetLastError());
     RETURN_IF(radix_sort_pairs(&keys, &vals, &tk, &tv, nv, 30, true, scratch, stream, launches));
-    window_keys_kernel<<<nb, 256, 0, stream>>>(in.voxel_off, vals, nv, max_len, len_bits, keys);
+    launch_chained(window_keys_kernel, nb, 256, 0, stream, in.voxel_off, vals, nv, max_len, len_bits, keys);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
   RETURN_IF(radix_sort_pairs(&keys, &vals, &tk, &tv, nv, len_bits + win_bits, false, scratch, stream, launches));
-  slice_len_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, stream>>>(in.voxel_off, vals, nv, n_slices,
+  launch_chained(slice_len_kernel, (unsigned)((nv + 255) / 256), 256, 0, stream, in.voxel_off, vals, nv, n_slices,
                                                                      out->slice_off, out->vlen, out->vperm, vrank);
   ++*launches;
   RETURN_IF(cudaGetLastError());
@@ -949,8 +986,7 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
       k.add(&out->ve_scan, n_elems);
       if (!k.allocate(keep)) return cudaErrorMemoryAllocation;
     }
-    fill_sell_kernel<<<(unsigned)((n_slices * kSlice + 255) / 256), 256, 0, stream>>>(
-        in, out->vperm, out->vlen, out->slice_off, nv, out->ve, out->ve_scan, n_elems);
+    launch_chained(fill_sell_kernel, (unsigned)((n_slices * kSlice + 255) / 256), 256, 0, stream, in, out->vperm, out->vlen, out->slice_off, nv, out->ve, out->ve_scan, n_elems);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
@@ -958,7 +994,7 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
   // ---- scan-major copy ----
   RETURN_IF(launch_obs_voxel(in, 0, nv, obs_vox, defer_scale ? nullptr : vscale, stream, launches));
   {
-    vlen_i64_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, stream>>>(out->vlen, nv, pbase);
+    launch_chained(vlen_i64_kernel, (unsigned)((nv + 255) / 256), 256, 0, stream, out->vlen, nv, pbase);
     ++*launches;
     RETURN_IF(cudaGetLastError());
     RETURN_IF(exclusive_scan_i64(pbase, nv + 1, pscratch, stream, launches));
@@ -966,30 +1002,30 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
     // the order, where it is kept, lands in its own buffer: the sort ends in the
     // buffer it starts from after an even number of digits, else in the other
     if (order) (radix_passes(scan_bits) % 2 == 0 ? vals : tv) = order;
-    scan_keys_kernel<<<(unsigned)((no + 255) / 256), 256, 0, stream>>>(in, obs_vox, vrank, pbase, keys, vals, place);
+    launch_chained(scan_keys_kernel, (unsigned)((no + 255) / 256), 256, 0, stream, in, obs_vox, vrank, pbase, keys, vals, place);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
   RETURN_IF(radix_sort_pairs(&keys, &vals, &tk, &tv, no, scan_bits, false, scratch, stream, launches));
-  scan_off_kernel<<<(unsigned)((no + 1 + 255) / 256), 256, 0, stream>>>(keys, no, in.n_scans, out->scan_off);
+  launch_chained(scan_off_kernel, (unsigned)((no + 1 + 255) / 256), 256, 0, stream, keys, no, in.n_scans, out->scan_off);
   ++*launches;
   RETURN_IF(cudaGetLastError());
   if (fill_f64) {  // the mixed path fills its own copy, se_vox included
-    fill_scan_major_kernel<<<(unsigned)((no + 255) / 256), 256, 0, stream>>>(in, vals, obs_vox, vscale, vrank, out->se,
+    launch_chained(fill_scan_major_kernel, (unsigned)((no + 255) / 256), 256, 0, stream, in, vals, obs_vox, vscale, vrank, out->se,
                                                                              out->se_vox);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
   // ---- scan-pass block order, so the longest scans start first ----
   if (in.n_scans <= kRankScans) {
-    scan_rank_kernel<<<1, kRankScans, 0, stream>>>(out->scan_off, in.n_scans, out->scans_by_len);
+    launch_chained(scan_rank_kernel, 1, kRankScans, 0, stream, out->scan_off, in.n_scans, out->scans_by_len);
     ++*launches;
     return cudaGetLastError();
   }
   const int len_digits = bit_width((uint64_t)no);
   uint32_t* by_len = (uint32_t*)out->scans_by_len;
   uint32_t* other = tv;  // free: the scan-major order is in vals
-  scan_len_keys_kernel<<<(unsigned)((in.n_scans + 255) / 256), 256, 0, stream>>>(out->scan_off, in.n_scans, no, keys);
+  launch_chained(scan_len_keys_kernel, (unsigned)((in.n_scans + 255) / 256), 256, 0, stream, out->scan_off, in.n_scans, no, keys);
   ++*launches;
   RETURN_IF(cudaGetLastError());
   if (radix_passes(len_digits) % 2 != 0) std::swap(by_len, other);

@@ -51,6 +51,8 @@ __device__ inline void centred_cluster(const double* in, int form, double out[10
 // every scan in FP32 (sref32), so per-observation set-up needs no FP64 -> FP32
 // conversions of the rotation
 __global__ void scan_ref_kernel(int32_t n_scans, const double* poses, double* sref) {
+  grid_wait();
+  grid_launch_next();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_scans) return;
   const double* P = poses + 12 * (int64_t)j;
@@ -178,6 +180,8 @@ __device__ __forceinline__ float group_sum(unsigned mask, float x) {
 __global__ void __launch_bounds__(128) voxel_frames_kernel(LoadInput in, int64_t v0, int64_t v1, const double* sref,
                                                            const int32_t* vrank, const double* vscale, float4* vstate,
                                                            float4* vanchor, float4* planes2) {
+  grid_wait();
+  grid_launch_next();
   static_assert(32 % kFrameLanes == 0 && 128 % kFrameLanes == 0, "groups must not straddle warps");
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t v = v0 + t / kFrameLanes;
@@ -359,6 +363,8 @@ __global__ void __launch_bounds__(128, 8)
     fill_sell_mixed_kernel(LoadInput in, const int32_t* vperm, const int32_t* vlen, const int64_t* slice_off,
                            int64_t n_voxels, int64_t p0, int64_t p1, const double* sref, const float4* vanchor,
                            float4* ve32) {
+  grid_wait();
+  grid_launch_next();
   const int64_t p = p0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t s = p >> 5;
   if (s * kSlice >= n_voxels || s * kSlice >= p1) return;
@@ -486,6 +492,8 @@ __global__ void __launch_bounds__(kFillScanThreads) fill_scan_mixed_kernel(int64
                                        const uint32_t* order, const int2* place, const float4* vanchor,
                                        const int64_t* slice_off, const float4* ve32, const int64_t* vstart, const float4* staging,
                                        float* se32, int32_t* se_vox) {
+  grid_wait();
+  grid_launch_next();
   __shared__ float4 slots[kFillScanThreads / 32][96];
   const int64_t i = i0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t q = i >= i1 ? -1 : qlist ? (int64_t)qlist[i] : i;
@@ -500,7 +508,7 @@ unsigned frame_blocks(int64_t n) { return (unsigned)((n * kFrameLanes + 127) / 1
 
 cudaError_t build_mixed_begin(const LoadInput& in, const double* poses2, MixedBuffers& mb, cudaStream_t stream,
                               int64_t* launches) {
-  scan_ref_kernel<<<(in.n_scans + 127) / 128, 128, 0, stream>>>(in.n_scans, poses2, mb.sref);
+  launch_chained(scan_ref_kernel, (in.n_scans + 127) / 128, 128, 0, stream, in.n_scans, poses2, mb.sref);
   ++*launches;
   return cudaGetLastError();
 }
@@ -511,7 +519,7 @@ cudaError_t build_mixed_voxels(const LoadInput& in, const LayoutBuffers& lb, con
   if (v1 <= v0) return cudaSuccess;
   LoadInput cur = in;
   cur.poses = poses2;  // buffer 0
-  voxel_frames_kernel<<<frame_blocks(v1 - v0), 128, 0, stream>>>(cur, v0, v1, mb.sref, lb.vrank, lb.vscale,
+  launch_chained(voxel_frames_kernel, frame_blocks(v1 - v0), 128, 0, stream, cur, v0, v1, mb.sref, lb.vrank, lb.vscale,
                                                                  mb.vstate, mb.vanchor, mb.planes32_2);
   ++*launches;
   cudaError_t e = cudaGetLastError();
@@ -540,9 +548,7 @@ cudaError_t build_mixed_scan_major(const LoadInput& in, const LayoutBuffers& lb,
                                    const float4* staging, const uint32_t* qlist, int64_t i0, int64_t i1,
                                    cudaStream_t stream, int64_t* launches) {
   if (i1 <= i0) return cudaSuccess;
-  fill_scan_mixed_kernel<<<(unsigned)((i1 - i0 + kFillScanThreads - 1) / kFillScanThreads), kFillScanThreads, 0,
-                           stream>>>(
-      in.n_obs, qlist, i0, i1, lb.scan_order, lb.place, mb.vanchor, lb.slice_off, mb.ve32, lb.vstart, staging, mb.se32,
+  launch_chained(fill_scan_mixed_kernel, (unsigned)((i1 - i0 + kFillScanThreads - 1) / kFillScanThreads), kFillScanThreads, 0, stream, in.n_obs, qlist, i0, i1, lb.scan_order, lb.place, mb.vanchor, lb.slice_off, mb.ve32, lb.vstart, staging, mb.se32,
       mb.se_vox);
   ++*launches;
   return cudaGetLastError();
@@ -566,7 +572,7 @@ cudaError_t build_mixed(const LoadInput& in, const LayoutBuffers& lb, const doub
   cur.poses = poses2;  // buffer 0
   const int64_t nv = in.n_voxels;
   if (nv > 0) {
-    voxel_frames_kernel<<<frame_blocks(nv), 128, 0, stream>>>(cur, 0, nv, mb.sref, lb.vrank, lb.vscale, mb.vstate,
+    launch_chained(voxel_frames_kernel, frame_blocks(nv), 128, 0, stream, cur, 0, nv, mb.sref, lb.vrank, lb.vscale, mb.vstate,
                                                                mb.vanchor, mb.planes32_2);
     ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -574,8 +580,7 @@ cudaError_t build_mixed(const LoadInput& in, const LayoutBuffers& lb, const doub
     const int64_t p1 = ((nv + kSlice - 1) / kSlice) * kSlice;
     const unsigned row_blocks =
         (unsigned)std::min<int64_t>(std::max<int64_t>((lb.max_len + kFillRows - 1) / kFillRows, 1), 65535);
-    fill_sell_mixed_kernel<<<dim3((unsigned)((p1 + 127) / 128), row_blocks), 128, 0, stream>>>(
-        cur, lb.vperm, lb.vlen, lb.slice_off, nv, 0, p1, mb.sref, mb.vanchor, mb.ve32);
+    launch_chained(fill_sell_mixed_kernel, dim3((unsigned)((p1 + 127) / 128), row_blocks), 128, 0, stream, cur, lb.vperm, lb.vlen, lb.slice_off, nv, 0, p1, mb.sref, mb.vanchor, mb.ve32);
     ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -68,6 +68,7 @@ __host__ __device__ __forceinline__ int half_floor(int i) { return i >= 0 ? i / 
 // LLONG_MAX); poses finite
 __global__ void check_inputs_kernel(int32_t n_scans, const int64_t* spo, int64_t n, const double* poses,
                                     long long* bad_off, long long* bad_pose) {
+  grid_launch_next();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j > n_scans) return;
   if (j == 0 && spo[0] != 0) atomicMin(bad_off, 0ll);
@@ -126,6 +127,8 @@ static_assert(sizeof(ScanFix) == 64, "four 16-byte loads");
 // poses divided by the voxel size (rd = 1 / d): in FP64, and in fixed point
 __global__ void scaled_poses_kernel(int32_t n_scans, const double* poses, double rd, int kS, int kp, double* out,
                                     ScanFix* fix) {
+  grid_wait();
+  grid_launch_next();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_scans) return;
   ScanFix f;
@@ -202,6 +205,7 @@ __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, c
                                                               const ScanFix* __restrict__ fix, int kp, double d,
                                                               int rounds, int64_t p0, int64_t n, uint64_t* __restrict__ keys,
                                                               int32_t* __restrict__ pscan, long long* bad, int* bbox) {
+  grid_launch_next();
   int mn[3] = {INT_MAX, INT_MAX, INT_MAX}, mx[3] = {INT_MIN, INT_MIN, INT_MIN};
   const int64_t tile = (int64_t)kKeyThreads * kKeyPoints * rounds;
   for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < n; t0 += (int64_t)gridDim.x * tile) {
@@ -302,6 +306,8 @@ __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, c
 // raw keys -> level-1 keys packed to the index range
 template <typename K>
 __global__ void repack_kernel(int64_t n, const uint64_t* raw, KeyPack p, K* keys) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint64_t r = raw[i];
@@ -319,6 +325,8 @@ constexpr int kHeadWords = 4;
 template <typename K>
 __global__ void head_mask_kernel(int64_t n, const K* keys, const uint32_t* vals, const int32_t* scan, uint32_t* mask,
                                  int64_t* wcount) {
+  grid_wait();
+  grid_launch_next();
   const int lane = threadIdx.x & 31;
   const int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kHeadWords;
   K key[kHeadWords], key0[kHeadWords];
@@ -362,6 +370,8 @@ __global__ void head_mask_kernel(int64_t n, const K* keys, const uint32_t* vals,
 // end sentinel
 __global__ void mask_starts_kernel(int64_t n_words, const uint32_t* mask, const int64_t* base, int64_t n,
                                    int64_t* start, int64_t n_groups) {
+  grid_wait();
+  grid_launch_next();
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= n_words) return;
   uint32_t m = mask[w];
@@ -583,6 +593,7 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
                                                                      const double* __restrict__ pts,
                                                                      const uint64_t* __restrict__ raw, int f_cap,
                                                                      double* c, uint64_t* ckey, int32_t* cscan) {
+  grid_launch_next();
   __shared__ int s_cnt[32], s_next;
   __shared__ uint16_t s_order[kPool];
   __shared__ int64_t s_start[kPool];
@@ -662,6 +673,8 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
 // (scan first, then parent)
 __global__ void parent_keys_kernel(int64_t nc, const uint64_t* ckey, const int32_t* cscan, KeyPack pc, KeyPack pp,
                                    uint64_t* pkey, uint32_t* skey) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nc) return;
   int ix[3];
@@ -672,6 +685,8 @@ __global__ void parent_keys_kernel(int64_t nc, const uint64_t* ckey, const int32
 
 template <typename K>
 __global__ void gather_keys_kernel(int64_t n, const uint64_t* src, const uint32_t* vals, K* dst) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = (K)src[vals[i]];
 }
@@ -686,6 +701,8 @@ __global__ void __launch_bounds__(kOrderBlock) merge_kernel(int64_t np, const in
                                                             const double* child, const K* pkeys_sorted,
                                                             const int32_t* cscan, double* c, uint64_t* ckey,
                                                             int32_t* oscan) {
+  grid_wait();
+  grid_launch_next();
   __shared__ int s_cnt[32], s_order[kOrderBlock];
   const int64_t g0 = (int64_t)blockIdx.x * kOrderBlock + threadIdx.x;
   const int64_t len0 = g0 < np ? start[g0 + 1] - start[g0] : 0;
@@ -731,6 +748,8 @@ __global__ void __launch_bounds__(kOrderBlock) merge_kernel(int64_t np, const in
 template <typename K>
 __global__ void gather_clusters_kernel(int64_t m, const uint32_t* vals, const K* keys, const double* c_in,
                                        const int32_t* scan_in, double* c, uint64_t* ckey, int32_t* cscan) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
   const int64_t src = vals[i];
@@ -742,12 +761,16 @@ __global__ void gather_clusters_kernel(int64_t m, const uint32_t* vals, const K*
 
 // voxels of a level: runs of equal key among its clusters (sorted by key, scan)
 __global__ void voxel_heads_kernel(int64_t nc, const uint64_t* ckey, int64_t* pos) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nc) pos[i] = (i == 0 || ckey[i] != ckey[i - 1]) ? 1 : 0;
 }
 
 __global__ void voxel_starts_kernel(int64_t nc, const uint64_t* ckey, const int64_t* pos, int64_t* vstart,
                                     int64_t nv) {
+  grid_wait();
+  grid_launch_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nc && (i == 0 || ckey[i] != ckey[i - 1])) vstart[pos[i]] = i;
   if (i == 0) vstart[nv] = nc;
@@ -760,6 +783,8 @@ __global__ void voxel_starts_kernel(int64_t nc, const uint64_t* ckey, const int6
 // answer is checked against its error bound.  vpos[t + 1] - 1 is t's voxel.
 __global__ void world_terms_kernel(int64_t nc, const double* c, const int32_t* cscan, const double* poses,
                                    const int64_t* vpos, const int64_t* vstart, float4* rel, float4* rsr) {
+  grid_wait();
+  grid_launch_next();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nc) return;
   const int64_t a = vstart[vpos[t + 1] - 1];
@@ -860,6 +885,8 @@ __device__ __noinline__ bool planar_f64(const double* A, double tau) {
 __global__ void select_kernel(int64_t nv, const int64_t* vstart, const float4* rel, const float4* rsr, float tau,
                               int32_t min_obs, int64_t* keep_obs, int64_t* keep_vox, uint32_t* close,
                               unsigned long long* n_close) {
+  grid_wait();
+  grid_launch_next();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= nv) return;
   const int64_t a = vstart[v], b = vstart[v + 1];
@@ -914,6 +941,8 @@ __global__ void select_kernel(int64_t nv, const int64_t* vstart, const float4* r
 __global__ void select_close_kernel(const uint32_t* close, const unsigned long long* n_close, const int64_t* vstart,
                                     const double* c, const int32_t* cscan, const double* poses, double tau,
                                     int64_t* keep_obs, int64_t* keep_vox) {
+  grid_wait();
+  grid_launch_next();
   const int64_t m = (int64_t)*n_close;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t v = close[i];
@@ -931,6 +960,8 @@ __global__ void emit_kernel(int64_t nv, const int64_t* vstart, const uint64_t* c
                             const double* c, const int64_t* obs_pos, const int64_t* vox_pos, const int64_t* keep_vox,
                             int32_t level, int64_t v_base, int64_t o_base, int64_t* voxel_off, int32_t* obs_scan,
                             double* agg, int32_t* lev, int32_t* index) {
+  grid_wait();
+  grid_launch_next();
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= nv || !keep_vox[v]) return;
   const int64_t a = vstart[v], b = vstart[v + 1];
@@ -1067,7 +1098,7 @@ ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int
   int64_t* base = tmp.get<int64_t>(nw + 1);
   int64_t* scr = tmp.get<int64_t>(scan_scratch_count(nw + 1));
   if (!mask || !base || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  head_mask_kernel<K><<<blocks_for((nw + kHeadWords - 1) / kHeadWords, 8), 256, 0, st>>>(n, keys, vals, scan, mask,
+  launch_chained(head_mask_kernel<K>, blocks_for((nw + kHeadWords - 1) / kHeadWords, 8), 256, 0, st, n, keys, vals, scan, mask,
                                                                                          base);
   VCK(cudaGetLastError(), "voxelize");
   VCK(cudaMemsetAsync(base + nw, 0, sizeof(int64_t), st), "voxelize");
@@ -1077,7 +1108,7 @@ ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int
   VCK(cudaStreamSynchronize(st), "voxelize");
   int64_t* start = tmp.get<int64_t>(ng + 1);
   if (!start) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  mask_starts_kernel<<<blocks_for(nw), 256, 0, st>>>(nw, mask, base, n, start, ng);
+  launch_chained(mask_starts_kernel, blocks_for(nw), 256, 0, st, nw, mask, base, n, start, ng);
   VCK(cudaGetLastError(), "voxelize");
   *launches += 2;
   *start_out = start;
@@ -1119,7 +1150,7 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(n));
   if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   tm.begin(BA_VOX_SORT);
-  repack_kernel<K><<<blocks_for(n), 256, 0, st>>>(n, raw, L.pk, keys);
+  launch_chained(repack_kernel<K>, blocks_for(n), 256, 0, st, n, raw, L.pk, keys);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize keys");
   // stable by key over points in scan order: groups ordered by (key, scan, point)
@@ -1165,12 +1196,12 @@ ba_status level_up(const Level& ch, Level& P, int32_t n_scans, Buf& tmp, cudaStr
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(nc));
   if (!pkey || !k2 || !t2 || !skey || !tsk || !cv || !tcv || !scr)
     return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  parent_keys_kernel<<<blocks_for(nc), 256, 0, st>>>(nc, ch.key, ch.scan, ch.pk, P.pk, pkey, skey);
+  launch_chained(parent_keys_kernel, blocks_for(nc), 256, 0, st, nc, ch.key, ch.scan, ch.pk, P.pk, pkey, skey);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize levels");
   VCK(radix_sort_pairs(&skey, &cv, &tsk, &tcv, nc, bit_width_u((uint64_t)(n_scans - 1)), true, scr, st, launches),
       "voxelize sort");
-  gather_keys_kernel<K><<<blocks_for(nc), 256, 0, st>>>(nc, pkey, cv, k2);
+  launch_chained(gather_keys_kernel<K>, blocks_for(nc), 256, 0, st, nc, pkey, cv, k2);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize levels");
   VCK(sort_keys(&k2, &cv, &t2, &tcv, nc, pack_bits(P.pk), false, scr, st, launches), "voxelize sort");
@@ -1183,7 +1214,7 @@ ba_status level_up(const Level& ch, Level& P, int32_t n_scans, Buf& tmp, cudaStr
   P.key = tmp.get<uint64_t>(np);
   P.scan = tmp.get<int32_t>(np);
   if (!P.c || !P.key || !P.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  merge_kernel<K><<<blocks_for(np, kOrderBlock), kOrderBlock, 0, st>>>(np, pst, cv, ch.c, k2, ch.scan, P.c, P.key,
+  launch_chained(merge_kernel<K>, blocks_for(np, kOrderBlock), kOrderBlock, 0, st, np, pst, cv, ch.c, k2, ch.scan, P.c, P.key,
                                                                        P.scan);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize merge");
@@ -1301,7 +1332,7 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
   uint32_t* tvals = tmp.get<uint32_t>(m);
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(m));
   if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  repack_kernel<K><<<blocks_for(m), 256, 0, c.st>>>(m, raw_all, L.pk, keys);
+  launch_chained(repack_kernel<K>, blocks_for(m), 256, 0, c.st, m, raw_all, L.pk, keys);
   ++*c.launches;
   VCK(cudaGetLastError(), "voxelize merge");
   VCK(sort_keys(&keys, &vals, &tkeys, &tvals, m, pack_bits(L.pk), true, scr, c.st, c.launches), "voxelize sort");
@@ -1311,7 +1342,7 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
     L.key = out.get<uint64_t>(m);
     L.scan = out.get<int32_t>(m);
     if (!L.c || !L.key || !L.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-    gather_clusters_kernel<K><<<blocks_for(m), 256, 0, c.st>>>(m, vals, keys, c_all, scan_all, L.c, L.key, L.scan);
+    launch_chained(gather_clusters_kernel<K>, blocks_for(m), 256, 0, c.st, m, vals, keys, c_all, scan_all, L.c, L.key, L.scan);
     ++*c.launches;
     VCK(cudaGetLastError(), "voxelize merge");
     return BA_OK;
@@ -1325,7 +1356,7 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
   L.key = out.get<uint64_t>(ng);
   L.scan = out.get<int32_t>(ng);
   if (!L.c || !L.key || !L.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  merge_kernel<K><<<blocks_for(ng, kOrderBlock), kOrderBlock, 0, c.st>>>(ng, start, vals, c_all, keys, scan_all,
+  launch_chained(merge_kernel<K>, blocks_for(ng, kOrderBlock), kOrderBlock, 0, c.st, ng, start, vals, c_all, keys, scan_all,
                                                                           L.c, L.key, L.scan);
   ++*c.launches;
   VCK(cudaGetLastError(), "voxelize merge");
@@ -1583,7 +1614,7 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
     // fixed point of the indices: 1 / d < 2^e
     // (far out of that range no pose fits and every point takes the FP64 path)
     const int e = std::min(std::max(std::ilogb(1.0 / cfg->voxel_size), -200), 200) + 1, kS = 30 - e, kp = 18 + e;
-    scaled_poses_kernel<<<blocks_for(n_scans, 128), 128, 0, st>>>(n_scans, T, 1.0 / cfg->voxel_size, kS, kp, sposes,
+    launch_chained(scaled_poses_kernel, blocks_for(n_scans, 128), 128, 0, st, n_scans, T, 1.0 / cfg->voxel_size, kS, kp, sposes,
                                                                   fix);
     ++launches;
     int n_sm = 0;
@@ -1650,7 +1681,7 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
     int64_t* pos = tmp.get<int64_t>(L.nc + 1);
     int64_t* scr = tmp.get<int64_t>(scan_scratch_count(L.nc + 1));
     if (!pos || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-    voxel_heads_kernel<<<blocks_for(L.nc), 256, 0, st>>>(L.nc, L.key, pos);
+    launch_chained(voxel_heads_kernel, blocks_for(L.nc), 256, 0, st, L.nc, L.key, pos);
     VCK(cudaGetLastError(), "voxelize");
     VCK(cudaMemsetAsync(pos + L.nc, 0, sizeof(int64_t), st), "voxelize");
     VCK(exclusive_scan_i64(pos, L.nc + 1, scr, st, &launches), "voxelize");
@@ -1664,7 +1695,7 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
     int64_t* scr3 = tmp.get<int64_t>(scan_scratch_count(L.nv + 1));
     if (!L.vstart || !keep_obs[k] || !keep_vox[k] || !obs_pos[k] || !vox_pos[k] || !scr3)
       return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-    voxel_starts_kernel<<<blocks_for(L.nc), 256, 0, st>>>(L.nc, L.key, pos, L.vstart, L.nv);
+    launch_chained(voxel_starts_kernel, blocks_for(L.nc), 256, 0, st, L.nc, L.key, pos, L.vstart, L.nv);
     launches += 2;
     tm.begin(BA_VOX_SELECT);
     float4 *rel = nullptr, *rsr = nullptr;
@@ -1677,18 +1708,18 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
       n_close = tmp.get<unsigned long long>(1);
       if (!rel || !rsr || !close || !n_close) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
       VCK(cudaMemsetAsync(n_close, 0, sizeof(unsigned long long), st), "voxelize");
-      world_terms_kernel<<<blocks_for(L.nc), 256, 0, st>>>(L.nc, L.c, L.scan, T, pos, L.vstart, rel, rsr);
+      launch_chained(world_terms_kernel, blocks_for(L.nc), 256, 0, st, L.nc, L.c, L.scan, T, pos, L.vstart, rel, rsr);
       ++launches;
     }
     // tau rounded to FP32 moves the test by 2^-24 tau lambda1, inside the error band
-    select_kernel<<<blocks_for(L.nv), 256, 0, st>>>(L.nv, L.vstart, rel, rsr, cfg->tau > 0.0 ? (float)cfg->tau : 0.0f,
+    launch_chained(select_kernel, blocks_for(L.nv), 256, 0, st, L.nv, L.vstart, rel, rsr, cfg->tau > 0.0 ? (float)cfg->tau : 0.0f,
                                                    cfg->min_obs, keep_obs[k], keep_vox[k], close, n_close);
     ++launches;
     if (cfg->tau > 0.0) {
       int n_sm = 0;
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
       const int64_t cb = std::min<int64_t>(blocks_for(L.nv, 128), (int64_t)(n_sm > 0 ? n_sm : 1) * 4);
-      select_close_kernel<<<(unsigned)cb, 128, 0, st>>>(close, n_close, L.vstart, L.c, L.scan, T, cfg->tau,
+      launch_chained(select_close_kernel, (unsigned)cb, 128, 0, st, close, n_close, L.vstart, L.c, L.scan, T, cfg->tau,
                                                         keep_obs[k], keep_vox[k]);
       ++launches;
     }
@@ -1730,7 +1761,7 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
     const Level& L = lv[k];
     if (L.nv == 0) continue;
     tm.begin(BA_VOX_EMIT);
-    emit_kernel<<<blocks_for(L.nv), 256, 0, st>>>(L.nv, L.vstart, L.key, L.pk, L.scan, L.c, obs_pos[k], vox_pos[k],
+    launch_chained(emit_kernel, blocks_for(L.nv), 256, 0, st, L.nv, L.vstart, L.key, L.pk, L.scan, L.c, obs_pos[k], vox_pos[k],
                                                  keep_vox[k], k + 1, vb, ob, v->voxel_off, v->obs_scan, v->agg,
                                                  v->level, v->index);
     tm.end();
