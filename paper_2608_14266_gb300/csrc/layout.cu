@@ -560,7 +560,21 @@ cudaError_t launch_validate_agg(const double* agg, int64_t o0, int64_t o1, doubl
 
 // Input cluster -> centred (S, m, N).  Raw sums: m = v / N and
 // S_ab = fma(-v_a, m_b, P_ab).
-__device__ inline void to_centred(const double* a, int form, double out[10]) {
+// (the row in 128-bit loads where its address allows: a thread with a row of its
+// own is bound by the requests to L1)
+__device__ inline void to_centred(const double* in, int form, double out[10]) {
+  double a[10];
+  if (reinterpret_cast<uintptr_t>(in) % 16 == 0) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const double2 v = reinterpret_cast<const double2*>(in)[k];
+      a[2 * k] = v.x;
+      a[2 * k + 1] = v.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 10; ++k) a[k] = in[k];
+  }
   if (form == 1) {
 #pragma unroll
     for (int k = 0; k < 10; ++k) out[k] = a[k];
@@ -684,6 +698,10 @@ __global__ void slice_len_kernel(const int64_t* off, const uint32_t* vperm, int6
   if (p == 0) slice_off[n_slices] = 0;
 }
 
+// FP64 slots: thread (p, blockIdx.y) fills rows blockIdx.y, blockIdx.y + gridDim.y
+// .. of the voxel at sorted position p.  Bound by the factorisation's FP64
+// divisions; a thread for all rows of a voxel left most of the chip idle (50,000
+// voxels, 1.2M clusters 380 us; a thread per row 165 us).
 __global__ void fill_sell_kernel(LoadInput in, const int32_t* vperm, const int32_t* vlen, const int64_t* slice_off,
                                  int64_t n_voxels, double* ve, int32_t* ve_scan, int64_t n_elems) {
   grid_wait();
@@ -697,7 +715,7 @@ __global__ void fill_sell_kernel(LoadInput in, const int32_t* vperm, const int32
   const bool real = p < n_voxels;
   const int32_t len = real ? vlen[p] : 0;
   const int64_t o0 = real ? in.voxel_off[vperm[p]] : 0;
-  for (int64_t k = 0; k < rows; ++k) {
+  for (int64_t k = blockIdx.y; k < rows; k += gridDim.y) {
     const int64_t e = base + k * kSlice;
     double c[10], f[10];
     uint32_t scan = 0;
@@ -862,24 +880,28 @@ cudaError_t group_by_chunk(const uint32_t* order, int64_t n_obs, const ChunkBoun
   return cudaSuccess;
 }
 
-// Scans by decreasing observation count, ties by index.  Up to kRankScans in
-// one block, each thread counting the scans before its own (1000 scans: 5 us,
-// where the sort's launches take 12); beyond, the general sort of n_obs - count.
-constexpr int kRankScans = 1024;
-__global__ void __launch_bounds__(kRankScans) scan_rank_kernel(const int64_t* scan_off, int n,
-                                                               int32_t* order) {
+// Scans by decreasing observation count, ties by index.  Up to kRankScans, eight
+// lanes count the scans before one (1000 scans: 5 us, a thread per scan in one
+// block 30 us); beyond, the general sort of n_obs - count.
+constexpr int kRankScans = 1024, kRankThreads = 256, kRankLanes = 8;
+__global__ void __launch_bounds__(kRankThreads) scan_rank_kernel(const int64_t* scan_off, int n, int32_t* order) {
   grid_wait();
   grid_launch_next();
   __shared__ __align__(16) uint32_t len[kRankScans];
-  const int j = threadIdx.x;
-  const uint32_t mine = j < n ? (uint32_t)(scan_off[j + 1] - scan_off[j]) : 0u;
-  len[j] = mine;
+  for (int i = threadIdx.x; i < (n + 3) / 4 * 4; i += kRankThreads)
+    len[i] = i < n ? (uint32_t)(scan_off[i + 1] - scan_off[i]) : 0u;
   __syncthreads();
-  if (j >= n) return;
-  int rank = 0;
-#pragma unroll 8
-  for (int i = 0; i < n; ++i) rank += len[i] > mine || (len[i] == mine && i < j);
-  order[rank] = j;
+  const int t = blockIdx.x * kRankThreads + threadIdx.x, j = t / kRankLanes;
+  const uint32_t mine = len[j < n ? j : 0];
+  int rank = 0;  // the padding's 0 is longer than none, and after all
+  for (int i = 4 * (t % kRankLanes); i < n; i += 4 * kRankLanes) {
+    const uint4 v = *reinterpret_cast<const uint4*>(len + i);
+    rank += (v.x > mine || (v.x == mine && i < j)) + (v.y > mine || (v.y == mine && i + 1 < j)) +
+            (v.z > mine || (v.z == mine && i + 2 < j)) + (v.w > mine || (v.w == mine && i + 3 < j));
+  }
+#pragma unroll
+  for (int o = kRankLanes / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+  if (j < n && t % kRankLanes == 0) order[rank] = j;
 }
 
 __global__ void scan_len_keys_kernel(const int64_t* scan_off, int32_t n_scans, int64_t n_obs, uint32_t* keys) {
@@ -986,7 +1008,11 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
       k.add(&out->ve_scan, n_elems);
       if (!k.allocate(keep)) return cudaErrorMemoryAllocation;
     }
-    launch_chained(fill_sell_kernel, (unsigned)((n_slices * kSlice + 255) / 256), 256, 0, stream, in, out->vperm, out->vlen, out->slice_off, nv, out->ve, out->ve_scan, n_elems);
+    // rows over blockIdx.y: enough for voxels of four times the mean length, the
+    // rest of a longer one in further turns
+    const unsigned row_blocks = (unsigned)std::min<int64_t>(std::min<int64_t>(max_len, 4 * (no / nv) + 4), 65535);
+    launch_chained(fill_sell_kernel, dim3((unsigned)((n_slices * kSlice + 255) / 256), row_blocks), 256, 0, stream, in,
+                   out->vperm, out->vlen, out->slice_off, nv, out->ve, out->ve_scan, n_elems);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
@@ -1018,7 +1044,8 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
   }
   // ---- scan-pass block order, so the longest scans start first ----
   if (in.n_scans <= kRankScans) {
-    launch_chained(scan_rank_kernel, 1, kRankScans, 0, stream, out->scan_off, in.n_scans, out->scans_by_len);
+    launch_chained(scan_rank_kernel, (unsigned)(((int64_t)in.n_scans * kRankLanes + kRankThreads - 1) / kRankThreads),
+                   kRankThreads, 0, stream, out->scan_off, in.n_scans, out->scans_by_len);
     ++*launches;
     return cudaGetLastError();
   }
