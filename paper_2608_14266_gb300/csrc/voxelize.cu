@@ -304,16 +304,27 @@ __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, c
 }
 
 // raw keys -> level-1 keys packed to the index range
+// Bound by DRAM (8 bytes read, sizeof(K) written): four keys of a thread in
+// flight (120M keys, sort included, 2670 -> 2400 us against one key per thread).
+constexpr int kRepackThreads = 256, kRepackItems = 4;
 template <typename K>
-__global__ void repack_kernel(int64_t n, const uint64_t* raw, KeyPack p, K* keys) {
+__global__ void __launch_bounds__(kRepackThreads) repack_kernel(int64_t n, const uint64_t* raw, KeyPack p, K* keys) {
   grid_wait();
   grid_launch_next();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint64_t r = raw[i];
-  const int ix = (int)((r >> 42) & 0x1fffffull) - kKeyRange, iy = (int)((r >> 21) & 0x1fffffull) - kKeyRange,
-            iz = (int)(r & 0x1fffffull) - kKeyRange;
-  keys[i] = (K)pack_key(p, ix, iy, iz);
+  const int64_t i0 = (int64_t)blockIdx.x * (kRepackThreads * kRepackItems) + threadIdx.x;
+  uint64_t r[kRepackItems];
+#pragma unroll
+  for (int c = 0; c < kRepackItems; ++c) {
+    const int64_t i = i0 + c * kRepackThreads;
+    r[c] = i < n ? raw[i] : 0;
+  }
+#pragma unroll
+  for (int c = 0; c < kRepackItems; ++c) {
+    const int64_t i = i0 + c * kRepackThreads;
+    const int ix = (int)((r[c] >> 42) & 0x1fffffull) - kKeyRange, iy = (int)((r[c] >> 21) & 0x1fffffull) - kKeyRange,
+              iz = (int)(r[c] & 0x1fffffull) - kKeyRange;
+    if (i < n) keys[i] = (K)pack_key(p, ix, iy, iz);
+  }
 }
 
 // group heads as one 32-bit word per 32 elements (bit k: element 32 w + k
@@ -1211,7 +1222,7 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(n));
   if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   tm.begin(BA_VOX_SORT);
-  launch_chained(repack_kernel<K>, blocks_for(n), 256, 0, st, n, raw, L.pk, keys);
+  launch_chained(repack_kernel<K>, blocks_for(n, kRepackThreads * kRepackItems), kRepackThreads, 0, st, n, raw, L.pk, keys);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize keys");
   // stable by key over points in scan order: groups ordered by (key, scan, point)
@@ -1393,7 +1404,7 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
   uint32_t* tvals = tmp.get<uint32_t>(m);
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(m));
   if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  launch_chained(repack_kernel<K>, blocks_for(m), 256, 0, c.st, m, raw_all, L.pk, keys);
+  launch_chained(repack_kernel<K>, blocks_for(m, kRepackThreads * kRepackItems), kRepackThreads, 0, c.st, m, raw_all, L.pk, keys);
   ++*c.launches;
   VCK(cudaGetLastError(), "voxelize merge");
   VCK(sort_keys(&keys, &vals, &tkeys, &tvals, m, pack_bits(L.pk), true, scr, c.st, c.launches), "voxelize sort");
