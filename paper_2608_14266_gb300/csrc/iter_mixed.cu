@@ -515,6 +515,7 @@ __global__ void wait_probe_kernel(int limit, int32_t* out) {
 
 // Per-scan FP32 table of buffer `buf` from the FP64 poses of that buffer.
 __global__ void scan_table_kernel(int32_t n_scans, const double* poses2, const double* sref, float* stab2, int buf) {
+  grid_wait();  // (and no early start after it: the voxel pass reads the slots before its own wait)
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_scans) return;
   scan_table_entry(poses2 + ((int64_t)buf * n_scans + j) * 12, sref + 12 * (int64_t)j,
@@ -557,8 +558,8 @@ cudaError_t launch_wait_probe(int limit, int32_t* out, cudaStream_t stream) {
 
 cudaError_t launch_scan_table(int32_t n_scans, const double* poses2, const double* sref, float* stab2, int buf,
                               cudaStream_t stream) {
-  scan_table_kernel<<<(n_scans + 127) / 128, 128, 0, stream>>>(n_scans, poses2, sref, stab2, buf);
-  return cudaGetLastError();
+  return launch_chained(scan_table_kernel, (unsigned)((n_scans + 127) / 128), 128, 0, stream, n_scans, poses2, sref, stab2,
+                        buf);
 }
 
 }  // namespace mmba

@@ -15,7 +15,12 @@ namespace mmba {
 
 namespace {
 
-constexpr int kFillRows = 4;  // slice rows per thread of the slot fill
+// Slice rows per thread of the slot fill: four where the grid is large enough
+// (15M clusters 4200 us a load, with two 4233; 1.7M clusters alike), two below (0.44M
+// clusters 386 us a load with four, 373 with two; 87,000 clusters 286 and 274).
+constexpr int kFillRows = 4;
+constexpr int64_t kFewSlots = 2000000;
+int fill_rows(int64_t n_obs) { return n_obs < kFewSlots ? 2 : kFillRows; }
 
 // the row at in (80 bytes of the handle's own copy, so 16-byte aligned: five
 // 128-bit loads; a row per thread is bound by the load/store unit)
@@ -355,14 +360,14 @@ __device__ void mixed_slot(const LoadInput& in, int64_t o, const double* sref, f
 }
 
 // slots of the slices that start at sorted positions [p0, p1) (p0 a multiple
-// of kSlice): thread (p, blockIdx.y) fills rows kFillRows * blockIdx.y ..
-// + kFillRows - 1 of voxel p, then the same rows gridDim.y * kFillRows on
+// of kSlice): thread (p, blockIdx.y) fills rows fill_rows * blockIdx.y ..
+// + fill_rows - 1 of voxel p, then the same rows gridDim.y * fill_rows on
 // (eight resident blocks of 128 per SM: 64 registers, measured faster than
 // five blocks at the registers the compiler takes unbounded)
 __global__ void __launch_bounds__(128, 8)
     fill_sell_mixed_kernel(LoadInput in, const int32_t* vperm, const int32_t* vlen, const int64_t* slice_off,
                            int64_t n_voxels, int64_t p0, int64_t p1, const double* sref, const float4* vanchor,
-                           float4* ve32) {
+                           float4* ve32, int fill_rows) {
   grid_wait();
   grid_launch_next();
   const int64_t p = p0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -375,8 +380,8 @@ __global__ void __launch_bounds__(128, 8)
   const int32_t len = real ? vlen[p] : 0;
   const int64_t o0 = real ? in.voxel_off[vperm[p]] : 0;
   const float4 an = real ? vanchor[p] : make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int64_t k0 = (int64_t)blockIdx.y * kFillRows; k0 < rows; k0 += (int64_t)gridDim.y * kFillRows) {
-    for (int64_t k = k0; k < k0 + kFillRows && k < rows; ++k) {
+  for (int64_t k0 = (int64_t)blockIdx.y * fill_rows; k0 < rows; k0 += (int64_t)gridDim.y * fill_rows) {
+    for (int64_t k = k0; k < k0 + fill_rows && k < rows; ++k) {
       const int64_t e = base + k * kSlice;
       float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0, s2 = s0;
       if (k < len) mixed_slot(in, o0 + k, sref, an, s0, s1, s2);
@@ -578,9 +583,10 @@ cudaError_t build_mixed(const LoadInput& in, const LayoutBuffers& lb, const doub
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // every slot, padding included, by sorted position (coalesced writes)
     const int64_t p1 = ((nv + kSlice - 1) / kSlice) * kSlice;
+    const int per = fill_rows(in.n_obs);
     const unsigned row_blocks =
-        (unsigned)std::min<int64_t>(std::max<int64_t>((lb.max_len + kFillRows - 1) / kFillRows, 1), 65535);
-    launch_chained(fill_sell_mixed_kernel, dim3((unsigned)((p1 + 127) / 128), row_blocks), 128, 0, stream, cur, lb.vperm, lb.vlen, lb.slice_off, nv, 0, p1, mb.sref, mb.vanchor, mb.ve32);
+        (unsigned)std::min<int64_t>(std::max<int64_t>((lb.max_len + per - 1) / per, 1), 65535);
+    launch_chained(fill_sell_mixed_kernel, dim3((unsigned)((p1 + 127) / 128), row_blocks), 128, 0, stream, cur, lb.vperm, lb.vlen, lb.slice_off, nv, 0, p1, mb.sref, mb.vanchor, mb.ve32, per);
     ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
