@@ -1231,23 +1231,26 @@ ba_status refresh(ba_batch* b) {
   }
   std::vector<JobView> views(n);
   std::vector<int64_t> pre(3 * (n + 1), 0);
+  const size_t ng = (n + kGroupJobs - 1) / kGroupJobs;
+  std::vector<int64_t> group_scans(ng, 0);
+  for (size_t k = 0; k < n; ++k) group_scans[k / kGroupJobs] += b->jobs[k]->L.n_scans;
   for (size_t k = 0; k < n; ++k) {
     const ba_handle* h = b->jobs[k];
     views[k] = job_view(h);
     pre[k + 1] = pre[k] + h->n_cost;
     pre[(n + 1) + k + 1] = pre[(n + 1) + k] + h->L.n_scans;
-    pre[2 * (n + 1) + k + 1] = pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans);
+    pre[2 * (n + 1) + k + 1] = pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans, solve_lanes(group_scans[k / kGroupJobs]));
   }
   b->n_vblk = pre[n];
   b->n_sblk = pre[(n + 1) + n];
   b->n_oblk = pre[2 * (n + 1) + n];
-  const size_t ng = (n + kGroupJobs - 1) / kGroupJobs;
   b->groups.assign(ng, JobGroup{});
   b->group_blocks.assign(3 * ng, 0);
   for (size_t g = 0; g < ng; ++g) {
     JobGroup& G = b->groups[g];
     const size_t k0 = g * kGroupJobs, k1 = std::min(n, k0 + kGroupJobs);
     G.n_jobs = (int32_t)(k1 - k0);
+    G.solve_lanes = solve_lanes(group_scans[g]);
     int64_t v = 0, sc = 0, o = 0;
     for (size_t k = k0; k < k1; ++k) {
       const int i = (int)(k - k0);

@@ -155,7 +155,7 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
     for (int o = kV / 2; o > 0; o >>= 1) lam0 += __shfl_down_sync(0xffffffffu, lam0, o);
     if (lane == 0) cost_part[blk] = lam0;
   }
-  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_f64_blocks(L.n_voxels), pred_part, solve_blocks(L.n_scans),
+  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_f64_blocks(L.n_voxels), pred_part, pred_parts(L.n_scans),
                                    st, decide_mode, red, is_last, (int)(blk & 3) * 32);
 }
 
@@ -392,8 +392,57 @@ __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const
 // sub-partitions the shorter one wins, with several to each the one with less
 // work in all: solve_lanes.
 // ---------------------------------------------------------------------------
-// *stepped = false: the pose is kept (fixed scan, no observation, failed
-// factorisation); otherwise dlt holds the increment.
+// Coefficients in th^2, th = |dphi| < 0.1, of sin(th)/th, (1 - cos th)/th^2,
+// cos(th/2) and sin(th/2)/th: the Taylor series to th^8 (the first dropped
+// term is below 1e-17).
+__device__ const double kExpSeries[4][5] = {
+    {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880},
+    {0.5, -1.0 / 24, 1.0 / 720, -1.0 / 40320, 1.0 / 3628800},
+    {1.0, -1.0 / 8, 1.0 / 384, -1.0 / 46080, 1.0 / 10321920},
+    {0.5, -1.0 / 48, 1.0 / 3840, -1.0 / 645120, 1.0 / 185794560},
+};
+
+// The two forms do the same arithmetic in the same order (products and sums that
+// the compiler could contract differently are written out), so a scan's step
+// and a block's sums have the same bits in both.
+//
+// c0 + th^2 (c1 + ..) of one of the series, or its function beyond 0.1 rad
+__device__ __forceinline__ double exp_coef(int which, const double* series, double th2) {
+  if (!(th2 < 0.01)) {
+    const double th = sqrt(th2);
+    double sh, ch;
+    sincos(0.5 * th, &sh, &ch);
+    return which == 0 ? sin(th) / th : which == 1 ? 2.0 * sh * sh / th2 : which == 2 ? ch : sh / th;
+  }
+  double v = fma(th2, series[4], series[3]);
+#pragma unroll
+  for (int k = 2; k >= 0; --k) v = fma(th2, v, series[k]);
+  return v;
+}
+// |dphi|^2
+__device__ __forceinline__ double phi_sq(const double* d) { return fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2])); }
+// a column p of R moved by Exp(dphi): p + a (phi x p) + b phi x (phi x p), the
+// increment first (one rounding at the size of p)
+__device__ __forceinline__ void exp_column(const double* d, double ca, double cb, const double* p, double* n) {
+  const double u0 = fma(d[1], p[2], -(d[2] * p[1])), u1 = fma(d[2], p[0], -(d[0] * p[2])),
+               u2 = fma(d[0], p[1], -(d[1] * p[0]));
+  const double w0 = fma(d[1], u2, -(d[2] * u1)), w1 = fma(d[2], u0, -(d[0] * u2)), w2 = fma(d[0], u1, -(d[1] * u0));
+  n[0] = __dadd_rn(p[0], fma(ca, u0, __dmul_rn(cb, w0)));
+  n[1] = __dadd_rn(p[1], fma(ca, u1, __dmul_rn(cb, w1)));
+  n[2] = __dadd_rn(p[2], fma(ca, u2, __dmul_rn(cb, w2)));
+}
+// component i of (cc, cs dphi) times the quaternion whose components i, i ^ 1,
+// i ^ 2, i ^ 3 are q, q1, q2, q3 (the signs of the Hamilton product)
+__device__ __forceinline__ double exp_quat(int i, const double* d, double cc, double cs, double q, double q1, double q2,
+                                           double q3) {
+  const double s1 = (i & 1) ? q1 : -q1, s2 = i == 1 || i == 2 ? q2 : -q2, s3 = (i & 2) ? q3 : -q3;
+  return fma(cc, q, __dmul_rn(cs, fma(d[0], s1, fma(d[1], s2, __dmul_rn(d[2], s3)))));
+}
+// a row's term of -(g^T x + x^T H x / 2), with half the row's share of H x
+__device__ __forceinline__ double pred_term(double x, double g, double hx) { return __dmul_rn(-x, __dadd_rn(g, hx)); }
+
+// One thread per scan.  *stepped = false: the pose is kept (fixed scan, no
+// observation, failed factorisation); otherwise dlt holds the increment.
 __device__ inline double solve_scan(const DevLayout& L, int j, const double* P, double* Pt, const double* gH,
                                     DevState* st, double* dlt, bool* stepped) {
   *stepped = false;
@@ -428,35 +477,32 @@ __device__ inline double solve_scan(const DevLayout& L, int j, const double* P, 
     for (int k = 0; k < 12; ++k) Pt[k] = P[k];
     return 0.0;
   }
-  // L = -(g^T D + D^T H D / 2); the quadratic form from H's upper triangle
-  double gd = 0.0, half = 0.0;
+  // the quadratic form from H's upper triangle, the rows' terms summed as the
+  // lanes' shuffles do
+  double t[6];
+#pragma unroll
   for (int r = 0; r < 6; ++r) {
-    gd = fma(g[r], dlt[r], gd);
-    double hr = 0.5 * H[7 * r] * dlt[r];
-    for (int c = r + 1; c < 6; ++c) hr = fma(H[6 * r + c], dlt[c], hr);
-    half = fma(dlt[r], hr, half);
+    double hx = __dmul_rn(0.5 * H[7 * r], dlt[r]);
+#pragma unroll
+    for (int c = r + 1; c < 6; ++c) hx = fma(H[6 * r + c], dlt[c], hx);
+    t[r] = pred_term(dlt[r], g[r], hx);
   }
-  const double pred = -(gd + half);
-  double E[9];
-  so3_exp(dlt, E);
-  for (int r = 0; r < 3; ++r)
-    for (int c = 0; c < 3; ++c) Pt[3 * r + c] = E[3 * r] * P[c] + E[3 * r + 1] * P[3 + c] + E[3 * r + 2] * P[6 + c];
-  Pt[9] = P[9] + dlt[3];
-  Pt[10] = P[10] + dlt[4];
-  Pt[11] = P[11] + dlt[5];
+  const double th2 = phi_sq(dlt);
+  const double ca = exp_coef(0, kExpSeries[0], th2), cb = exp_coef(1, kExpSeries[1], th2);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double p[3] = {P[c], P[3 + c], P[6 + c]};
+    double n[3];
+    exp_column(dlt, ca, cb, p, n);
+    Pt[c] = n[0];
+    Pt[3 + c] = n[1];
+    Pt[6 + c] = n[2];
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) Pt[9 + k] = __dadd_rn(P[9 + k], dlt[3 + k]);
   *stepped = true;
-  return pred;
+  return ((t[0] + t[1]) + (t[2] + t[3])) + (t[4] + t[5]);
 }
-
-// Coefficients in th^2, th = |dphi| < 0.1, of sin(th)/th, (1 - cos th)/th^2,
-// cos(th/2) and sin(th/2)/th: the Taylor series to th^8 (the first dropped
-// term is below 1e-17).
-__device__ const double kExpSeries[4][5] = {
-    {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880},
-    {0.5, -1.0 / 24, 1.0 / 720, -1.0 / 40320, 1.0 / 3628800},
-    {1.0, -1.0 / 8, 1.0 / 384, -1.0 / 46080, 1.0 / 10321920},
-    {0.5, -1.0 / 48, 1.0 / 3840, -1.0 / 645120, 1.0 / 185794560},
-};
 
 // Eight lanes per scan.  Lane r < 6 holds row r of [A | -g] and eliminates it
 // by the pivot rows' broadcasts; the substitution runs up the rows' kept
@@ -504,7 +550,7 @@ __device__ __forceinline__ double solve_scan_lanes(const DevLayout& L, int64_t j
   for (int c = 0; c < 6; ++c) a[c] = row == c ? fma(mu, h[c], h[c]) : h[c];
   a[6] = -g;
   bool ok = true;
-  double inv_row = 0.0;
+  double inv_row = 0.0, f[6];  // f: the row of L
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const double d = __shfl_sync(kAll, a[k], k, 8);
@@ -512,15 +558,26 @@ __device__ __forceinline__ double solve_scan_lanes(const DevLayout& L, int64_t j
     const double inv = recip_pivot(d);
     if (row == k) inv_row = inv;
     if (k == 5) break;
-    const double l = row > k ? a[k] * inv : 0.0;
+    // the lower triangle: entry (row, c) takes column k's entry of row c, the
+    // right-hand side the pivot row's
+    const double l = row > k ? __dmul_rn(a[k], inv) : 0.0;
+    f[k] = l;
+    const double y = __shfl_sync(kAll, a[6], k, 8);
 #pragma unroll
-    for (int c = k + 1; c < 7; ++c) a[c] = fma(-l, __shfl_sync(kAll, a[c], k, 8), a[c]);
+    for (int c = k + 1; c < 6; ++c) a[c] = fma(-l, __shfl_sync(kAll, a[k], c, 8), a[c]);
+    a[6] = fma(-l, y, a[6]);
   }
-  double x = a[6] * inv_row;
+  double x = __dmul_rn(a[6], inv_row);
 #pragma unroll
   for (int k = 5; k >= 1; --k) {
-    const double f = row < k ? a[k] * inv_row : 0.0;
-    x = fma(-f, __shfl_sync(kAll, x, k, 8), x);
+    // row k of L to the lanes below: lane i takes its entry i
+    double lk = 0.0;
+#pragma unroll
+    for (int i = 0; i < k; ++i) {
+      const double v = __shfl_sync(kAll, f[i], k, 8);
+      lk = row == i ? v : lk;
+    }
+    x = fma(-lk, __shfl_sync(kAll, x, k, 8), x);
   }
   const unsigned lost = __ballot_sync(kAll, !isfinite(x));  // by every lane, ok or not
   ok = ok && (lost & group) == 0;
@@ -530,51 +587,32 @@ __device__ __forceinline__ double solve_scan_lanes(const DevLayout& L, int64_t j
   double dlt[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) dlt[c] = __shfl_sync(kAll, x, c, 8);
-  // -(g x + x (H x) / 2) of this row
-  double hx = h[0] * dlt[0];
+  // this row's term of the predicted reduction, H's upper triangle only
+  double hx = __dmul_rn(0.5 * hd, x);
 #pragma unroll
-  for (int c = 1; c < 6; ++c) hx = fma(h[c], dlt[c], hx);
-  const double pred = live && stepped && r < 6 ? -x * fma(0.5, hx, g) : 0.0;
-
-  const double th2 = fma(dlt[0], dlt[0], fma(dlt[1], dlt[1], dlt[2] * dlt[2]));
-  double v = fma(th2, series[4], series[3]);
-#pragma unroll
-  for (int k = 2; k >= 0; --k) v = fma(th2, v, series[k]);
-  if (!(th2 < 0.01)) {  // uniform over the scan's lanes
-    const double th = sqrt(th2);
-    double sh, ch;
-    sincos(0.5 * th, &sh, &ch);
-    const int w = r & 3;
-    v = w == 0 ? sin(th) / th : w == 1 ? 2.0 * sh * sh / th2 : w == 2 ? ch : sh / th;
-  }
+  for (int c = 1; c < 6; ++c) hx = fma(c > row ? h[c] : 0.0, dlt[c], hx);
+  const double pred = live && stepped && r < 6 ? pred_term(x, g, hx) : 0.0;
+  const double th2 = phi_sq(dlt);
+  const double v = exp_coef(r & 3, series, th2);  // uniform branch over the scan's lanes
   __syncwarp();
   const double ca = __shfl_sync(kAll, v, 0, 8), cb = __shfl_sync(kAll, v, 1, 8);
   if (live) {
     if (r < 3) {
-      const double u0 = fma(dlt[1], p[2], -(dlt[2] * p[1])), u1 = fma(dlt[2], p[0], -(dlt[0] * p[2])),
-                   u2 = fma(dlt[0], p[1], -(dlt[1] * p[0]));
-      const double w0 = fma(dlt[1], u2, -(dlt[2] * u1)), w1 = fma(dlt[2], u0, -(dlt[0] * u2)),
-                   w2 = fma(dlt[0], u1, -(dlt[1] * u0));
-      // the increment first: one rounding at the size of p
-      const double n0 = p[0] + fma(ca, u0, cb * w0), n1 = p[1] + fma(ca, u1, cb * w1),
-                   n2 = p[2] + fma(ca, u2, cb * w2);
-      Pt[r] = stepped ? n0 : p[0];
-      Pt[3 + r] = stepped ? n1 : p[1];
-      Pt[6 + r] = stepped ? n2 : p[2];
+      double n[3];
+      exp_column(dlt, ca, cb, p, n);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) Pt[3 * k + r] = stepped ? n[k] : p[k];
     } else if (r < 6) {
-      p[0] = stepped ? p[0] + x : p[0];
+      p[0] = stepped ? __dadd_rn(p[0], x) : p[0];
       Pt[6 + r] = p[0];
     }
   }
   if (stab2) {
-    // the step's quaternion times the current one: component i of the product
-    // takes the components i ^ k of the current one, with the signs of the
-    // Hamilton product
+    // the step's quaternion times the current one
     const double cc = __shfl_sync(kAll, v, 2, 8), cs = __shfl_sync(kAll, v, 3, 8);
     const int i = r & 3;
     const double q1 = __shfl_xor_sync(kAll, q, 1), q2 = __shfl_xor_sync(kAll, q, 2), q3 = __shfl_xor_sync(kAll, q, 3);
-    const double s1 = (i & 1) ? q1 : -q1, s2 = i == 1 || i == 2 ? q2 : -q2, s3 = (i & 2) ? q3 : -q3;
-    double qn = fma(cc, q, cs * fma(dlt[0], s1, fma(dlt[1], s2, dlt[2] * s3)));
+    double qn = exp_quat(i, dlt, cc, cs, q, q1, q2, q3);
     qn = stepped ? qn : q;
     const double w = __shfl_sync(kAll, qn, 0, 8);
     const double t = r < 3 ? 0.0 : p[0] - ref;
@@ -593,14 +631,15 @@ __device__ __forceinline__ double solve_scan_lanes(const DevLayout& L, int64_t j
 
 // With stab2 given (mixed precision) the trial scan's FP32 table entry is
 // written too, from the trial pose and the scan's reference pose.  Block blk
-// (kSolveThreads / solve_lanes consecutive scans) writes the sum of its scans'
-// predicted reductions to pred_part[blk], in a fixed order.
+// takes kSolveThreads / kLanes consecutive scans; the sum of the predicted
+// reductions of every kPredScans scans goes to pred_part, in a fixed order.
+template <int kLanes>
 __device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* poses2, const double* gH,
                                                double* pred_part, DevState* st, const double* sref, float* stab2,
                                                int64_t blk, double* red) {
-  const int lanes = solve_lanes(L.n_scans);
+  static_assert(kLanes == 1 || (kLanes == 8 && kSolveThreads == 8 * kPredScans && kPredScans == 8), "shuffle widths");
   double series[5];
-  if (lanes == 8) {
+  if (kLanes == 8) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) series[k] = kExpSeries[threadIdx.x & 3][k];
   }
@@ -610,10 +649,14 @@ __device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* poses
   gH = after_wait(gH);
   poses2 = after_wait(poses2);
   if (st->honor_stop && st->stop) return;  // uniform over the block
-  if (lanes == 8) {
-    const double tot = block_sum<kSolveThreads>(
-        solve_scan_lanes(L, blk * (kSolveThreads / 8) + threadIdx.x / 8, poses2, gH, st, sref, stab2, series), red);
-    if (threadIdx.x == 0) pred_part[blk] = tot;
+  if (kLanes == 8) {
+    // rows, then scans, in pairs, fours and eights
+    double v = solve_scan_lanes(L, blk * kPredScans + threadIdx.x / 8, poses2, gH, st, sref, stab2, series);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) pred_part[blk] = __dadd_rn(red[0], red[1]);
     return;
   }
   const int64_t j = blk * kSolveThreads + threadIdx.x;
@@ -631,34 +674,41 @@ __device__ __forceinline__ void solve_f64_body(const DevLayout& L, double* poses
       double* sq2 = after_wait(sq2_of(sref, L.n_scans));
       const double* qc = sq2 + ((int64_t)cur * L.n_scans + j) * 4;
       double* qt = sq2 + ((int64_t)(1 - cur) * L.n_scans + j) * 4;
+      const double q[4] = {qc[0], qc[1], qc[2], qc[3]};
       double qn[4];
       if (stepped) {
-        double qe[4];
-        so3_exp_quat(dlt, qe);
-        quat_mul_d(qe, qc, qn);
+        const double th2 = phi_sq(dlt);
+        const double cc = exp_coef(2, kExpSeries[2], th2), cs = exp_coef(3, kExpSeries[3], th2);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) qn[i] = exp_quat(i, dlt, cc, cs, q[i], q[i ^ 1], q[i ^ 2], q[i ^ 3]);
       } else {
-        for (int k = 0; k < 4; ++k) qn[k] = qc[k];
+        for (int k = 0; k < 4; ++k) qn[k] = q[k];
       }
       for (int k = 0; k < 4; ++k) qt[k] = qn[k];
       scan_table_from_quat(qn, Pt, sref + 12 * (int64_t)j, stab2 + ((int64_t)(1 - cur) * L.n_scans + j) * kTab);
     }
   }
-  const double tot = block_sum<kSolveThreads>(pred, red);
-  if (threadIdx.x == 0) pred_part[blk] = tot;
+#pragma unroll
+  for (int o = 1; o < kPredScans; o <<= 1) pred = __dadd_rn(pred, __shfl_xor_sync(0xffffffffu, pred, o));
+  const int64_t part = (blk * kSolveThreads + threadIdx.x) / kPredScans;
+  if (threadIdx.x % kPredScans == 0 && part < pred_parts(L.n_scans)) pred_part[part] = pred;
 }
 
+template <int kLanes>
 __global__ void __launch_bounds__(kSolveThreads) solve_f64_kernel(DevLayout L, double* poses2, const double* gH,
                                                                  double* pred_part, DevState* st, const double* sref,
                                                                  float* stab2) {
   __shared__ double red[kSolveThreads / 32];
-  solve_f64_body(L, poses2, gH, pred_part, st, sref, stab2, blockIdx.x, red);
+  solve_f64_body<kLanes>(L, poses2, gH, pred_part, st, sref, stab2, blockIdx.x, red);
 }
 
+template <int kLanes>
 __global__ void __launch_bounds__(kSolveThreads) solve_f64_batch_kernel(const __grid_constant__ JobGroup G) {
   __shared__ double red[kSolveThreads / 32];
   const int job = find_job(G.oblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  solve_f64_body(J.L, J.poses2, J.gH, J.pred_part, J.st, J.X.sref, J.X.stab2, (int64_t)blockIdx.x - G.oblk[job], red);
+  solve_f64_body<kLanes>(J.L, J.poses2, J.gH, J.pred_part, J.st, J.X.sref, J.X.stab2,
+                         (int64_t)blockIdx.x - G.oblk[job], red);
 }
 
 __global__ void __launch_bounds__(kDecideThreads) decide_kernel(const double* __restrict__ cost_part, int64_t n_cost,
@@ -710,14 +760,15 @@ cudaError_t launch_shard_cost(const double* cost_part, int64_t n_cost, double* o
 
 cudaError_t launch_shard_decide(const DevLayout& L, const double* pred_part, DevState* st, double trial_total,
                                 cudaStream_t stream) {
-  shard_decide_kernel<<<1, kDecideThreads, 0, stream>>>(pred_part, solve_blocks(L.n_scans), st, trial_total);
+  shard_decide_kernel<<<1, kDecideThreads, 0, stream>>>(pred_part, pred_parts(L.n_scans), st, trial_total);
   return cudaGetLastError();
 }
 
 cudaError_t launch_solve_f64(const DevLayout& L, double* poses2, const double* gH, double* pred_part, DevState* st,
                              const double* sref, float* stab2, cudaStream_t stream, bool dependent) {
-  return launch_dependent(solve_f64_kernel, solve_blocks(L.n_scans), kSolveThreads, stream, dependent, L, poses2, gH,
-                          pred_part, st, sref, stab2);
+  const int lanes = solve_lanes(L.n_scans);
+  return launch_dependent(lanes == 8 ? solve_f64_kernel<8> : solve_f64_kernel<1>, solve_blocks(L.n_scans, lanes),
+                          kSolveThreads, stream, dependent, L, poses2, gH, pred_part, st, sref, stab2);
 }
 
 cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double* pred_part, int64_t n_pred,
@@ -727,7 +778,8 @@ cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double*
 }
 
 cudaError_t launch_batch_solve(const JobGroup& T, int64_t n_blocks, cudaStream_t stream) {
-  return launch_dependent(solve_f64_batch_kernel, n_blocks, kSolveThreads, stream, false, T);
+  return launch_dependent(T.solve_lanes == 8 ? solve_f64_batch_kernel<8> : solve_f64_batch_kernel<1>, n_blocks,
+                          kSolveThreads, stream, false, T);
 }
 
 cudaError_t launch_batch_voxel_pass_f64(const JobGroup& T, int64_t n_blocks, int use_trial, cudaStream_t stream) {

@@ -184,7 +184,7 @@ __device__ __forceinline__ void voxel_pass_mixed_body(const DevLayout& L, const 
   // the sum over blocks is FP64
   const float tot = block_sum<kVoxelThreads, float>(lam0, red);
   if (threadIdx.x == 0) cost_part[blk] = (double)tot;
-  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_blocks(L.n_voxels), pred_part, solve_blocks(L.n_scans), st,
+  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_blocks(L.n_voxels), pred_part, pred_parts(L.n_scans), st,
                                    decide_mode, dred, is_last);
 }
 

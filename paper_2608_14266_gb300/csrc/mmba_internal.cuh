@@ -252,6 +252,7 @@ struct JobGroup {
   int32_t sblk[kGroupJobs + 1];  // prefix of scan-pass blocks (one per scan)
   int32_t oblk[kGroupJobs + 1];  // prefix of solve blocks
   int32_t n_jobs;
+  int32_t solve_lanes;  // lanes per scan in the solve (1 or 8, by the group's scans)
 };
 static_assert(sizeof(JobGroup) <= 32000, "a job group must fit the kernel parameter space");
 
@@ -656,36 +657,6 @@ __device__ __forceinline__ double* sq2_of(const double* sref, int64_t n_scans) {
   return const_cast<double*>(sref) + 18 * n_scans;  // 12 doubles + 12 floats per scan before it
 }
 
-// Hamilton product p q of FP64 quaternions (w, x, y, z)
-__device__ __forceinline__ void quat_mul_d(const double* p, const double* q, double* r) {
-  r[0] = p[0] * q[0] - p[1] * q[1] - p[2] * q[2] - p[3] * q[3];
-  r[1] = p[0] * q[1] + p[1] * q[0] + p[2] * q[3] - p[3] * q[2];
-  r[2] = p[0] * q[2] - p[1] * q[3] + p[2] * q[0] + p[3] * q[1];
-  r[3] = p[0] * q[3] + p[1] * q[2] - p[2] * q[1] + p[3] * q[0];
-}
-
-// Unit quaternion of Exp(phi): (cos(th/2), sin(th/2) phi / th), th = |phi|;
-// below th = 0.1 from the Taylor series of both functions (terms to th^8;
-// the first dropped term is below 1e-19).
-__device__ inline void so3_exp_quat(const double* phi, double* q) {
-  const double x = phi[0], y = phi[1], z = phi[2];
-  const double t2 = x * x + y * y + z * z;
-  double c, s;  // cos(th/2), sin(th/2) / th
-  if (t2 < 0.01) {
-    c = 1.0 + t2 * (-1.0 / 8 + t2 * (1.0 / 384 + t2 * (-1.0 / 46080 + t2 * (1.0 / 10321920))));
-    s = 0.5 + t2 * (-1.0 / 48 + t2 * (1.0 / 3840 + t2 * (-1.0 / 645120 + t2 * (1.0 / 185794560))));
-  } else {
-    const double th = sqrt(t2);
-    double sh;
-    sincos(0.5 * th, &sh, &c);
-    s = sh / th;
-  }
-  q[0] = c;
-  q[1] = s * x;
-  q[2] = s * y;
-  q[3] = s * z;
-}
-
 // Hamilton product p q of quaternions held as float4 (w, x, y, z) in the
 // fields (x, y, z, w): rot(p q) = rot(p) rot(q)
 __device__ __forceinline__ float4 quat_mul_f(float4 p, float4 q) {
@@ -732,7 +703,7 @@ __device__ inline bool ldlt6_solve(const double* A, const double* b, double* x) 
 #pragma unroll
       for (int k = 0; k < j; ++k) v = fma(-L[i][k], LD[j][k], v);
       LD[i][j] = v;
-      L[i][j] = v * inv;
+      L[i][j] = __dmul_rn(v, inv);
     }
   }
   double y[6];
@@ -744,12 +715,12 @@ __device__ inline bool ldlt6_solve(const double* A, const double* b, double* x) 
     y[i] = v;
   }
 #pragma unroll
-  for (int i = 0; i < 6; ++i) y[i] *= Di[i];
+  for (int i = 0; i < 6; ++i) y[i] = __dmul_rn(y[i], Di[i]);
 #pragma unroll
   for (int i = 5; i >= 0; --i) {
     double v = y[i];
 #pragma unroll
-    for (int k = i + 1; k < 6; ++k) v -= L[k][i] * x[k];
+    for (int k = 5; k > i; --k) v = fma(-L[k][i], x[k], v);
     x[i] = v;
   }
   bool ok = true;

@@ -32,16 +32,20 @@ __host__ __device__ inline int64_t voxel_pass_f64_blocks(int64_t n_voxels) {
   const int v = voxel_pass_f64_width(n_voxels);
   return (n_voxels + v - 1) / v;
 }
-// Lanes per scan in the solve kernel: 8 while the GPU has few warps to each of
-// its 608 SM sub-partitions, else 1.  Both sides, launch included: 500 scans
-// 18.5 us with one lane and 12.4 with eight, 4000 scans 19.6 and 16.3, 6000
-// scans 20.5 and 18.4, 10,000 scans 21.7 and 31.6.
+// Lanes per scan in the solve kernel, for a launch of n_scans scans in all (a
+// handle's, or a batch group's): 8 while the GPU has few warps to each of its
+// 608 SM sub-partitions, else 1; the results have the same bits.  Both sides,
+// launch included: 500 scans 18.5 us with one lane and 12.4 with eight, 4000
+// scans 19.6 and 16.3, 6000 scans 20.5 and 18.4, 10,000 scans 21.7 and 31.6.
 constexpr int64_t kLaneSolveScans = 6144;
 __host__ __device__ inline int solve_lanes(int64_t n_scans) { return n_scans <= kLaneSolveScans ? 8 : 1; }
-__host__ __device__ inline int64_t solve_blocks(int64_t n_scans) {
-  const int per = kSolveThreads / solve_lanes(n_scans);
+inline int64_t solve_blocks(int64_t n_scans, int lanes) {
+  const int per = kSolveThreads / lanes;
   return (n_scans + per - 1) / per;
 }
+// the solve's partial sums of the predicted reduction: one for every kPredScans scans
+constexpr int kPredScans = 8;
+__host__ __device__ inline int64_t pred_parts(int64_t n_scans) { return (n_scans + kPredScans - 1) / kPredScans; }
 
 // Launch of an iteration kernel; with dependent = true it may start while the
 // kernel before it in the stream drains (see grid_wait in mmba_internal.cuh).

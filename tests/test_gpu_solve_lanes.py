@@ -1,5 +1,5 @@
-"""The solve kernel gives eight lanes to a scan up to 6144 scans and one
-beyond: one LM step on both sides of the line, with ragged last blocks, scans
+"""The solve kernel gives eight lanes to a scan in launches of up to 6144 scans
+and one beyond, with the same bits: one LM step on both sides of the line, with ragged last blocks, scans
 without observations, a fixed scan, steps below and above the small-angle
 series' 0.1 rad, and a factorisation that fails."""
 import numpy as np
@@ -110,3 +110,31 @@ def test_failed_factorisation_keeps_the_pose(mm, n_scans):
         st = ba.iterate(1)
         assert not st["last_accepted"] and st["cost"] == cost
         np.testing.assert_array_equal(ba.poses(), pose)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("tilt", [1e-3, 0.3])
+def test_lanes_give_the_bits_of_one_thread(mm, precision, tilt):
+    """A job alone (500 scans, eight lanes) and in a batch of 7,003 scans (one):
+    poses, cost and damping after three steps have the same bits."""
+    prec = mm.BA_MIXED if precision == "mixed" else mm.BA_FP64
+    kw = dict(precision=prec, hessian_mode=1, mu0=1e-2, fixed_scan=2)
+    jobs = [_problem(n, tilt, n) for n in (500, 6500, 3)]
+    alone = []
+    for ns, off, scan, cen, pose in jobs:
+        with mm.BundleAdjuster(**kw) as ba:
+            ba.load_observations(ns, off, scan, cen, pose)
+            st = ba.iterate(3)
+            alone.append((ba.poses().copy(), st["cost"], st["mu"], st["last_pred"]))
+    bas = [mm.BundleAdjuster(**kw) for _ in jobs]
+    with mm.Batch() as b:
+        for ba, (ns, off, scan, cen, pose) in zip(bas, jobs):
+            ba.load_observations(ns, off, scan, cen, pose)
+            b.add(ba)
+        b.iterate(3)
+        for ba, (poses, cost, mu, pred) in zip(bas, alone):
+            st = ba.stats()
+            np.testing.assert_array_equal(ba.poses(), poses)
+            assert (st["cost"], st["mu"], st["last_pred"]) == (cost, mu, pred)
+    for ba in bas:
+        ba.close()
