@@ -1237,7 +1237,8 @@ ba_status refresh(ba_batch* b) {
   for (size_t k = 0; k < n; ++k) {
     const ba_handle* h = b->jobs[k];
     views[k] = job_view(h);
-    pre[k + 1] = pre[k] + h->n_cost;
+    // (a slice of 32 voxels to a block in the FP64 batch, whatever the width alone)
+    pre[k + 1] = pre[k] + (h->mixed ? h->n_cost : (h->L.n_voxels + 31) / 32);
     pre[(n + 1) + k + 1] = pre[(n + 1) + k] + h->L.n_scans;
     pre[2 * (n + 1) + k + 1] = pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans, solve_lanes(group_scans[k / kGroupJobs]));
   }

@@ -32,15 +32,22 @@ namespace mmba {
 // voxel: 118 -> 32 us at 200 voxels, 258 -> 206 us at 50,000, 2.01 -> 1.97 ms
 // at 500,000 (15M observations).
 // ---------------------------------------------------------------------------
-template <int kV, bool kFull>
+// kTiles > 1: the block takes that many of the tiles of kV voxels one after
+// another, with the same sums, and solves their eigenproblems together (kV
+// kTiles = 32 lanes of the warp at work): what a batch, which fills the GPU,
+// does with the narrow tiles of its small jobs, whose results so have the bits
+// of a job alone (120 FP64 jobs of 1000 to 3000 voxels 1554 us an iteration,
+// with a tile to a block 1905, with a thread per voxel 1652).
+template <int kV, bool kFull, int kTiles>
 __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const double* poses2, double* planes2,
                                                     double* full_out, double* cost_part, const double* pred_part,
                                                     DevState* st, int use_trial, int decide_mode, int64_t blk, double* red,
-                                                    double (*sums)[10][32], int* is_last) {
+                                                    double (*sums)[10][32], double (*anchor)[32], int* is_last) {
   static_assert(kVoxelThreads == 128 && (kV == 8 || kV == 16 || kV == 32), "four warps per block");
-  const int64_t p = blk * kV + (threadIdx.x & (kV - 1));
-  const int len = p < L.n_voxels ? L.vlen[p] : 0;
-  const int64_t base = p < L.n_voxels ? L.slice_off[p >> 5] + (p & 31) : 0;
+  static_assert(kTiles == 1 || kTiles * kV == 32, "a slice");
+  int64_t p = blk * (kV * kTiles) + (threadIdx.x & (kV - 1));
+  int len = p < L.n_voxels ? L.vlen[p] : 0;
+  int64_t base = p < L.n_voxels ? L.slice_off[p >> 5] + (p & 31) : 0;
   grid_wait();
   grid_launch_next();
   st = after_wait(st);
@@ -57,70 +64,91 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
   // the sums n, s, M of this thread's observations
   double acc[10] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   double ax = 0.0, ay = 0.0, az = 0.0;
-  if (p < L.n_voxels) {
-    const int64_t ne = L.n_elems;
-    const int k0 = threadIdx.x / kV;
-    if (k0 < len || w == (int)(blk & 3)) {
-      // the anchor: the first observation's posed mean, formed by every thread
-      const uint32_t sv = (uint32_t)__ldg(L.ve_scan + base);
-      int p0, p1, p2;
-      perm_decode(sv >> kPermShift, p0, p1, p2);
-      const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
-      const double m0 = __ldg(L.ve + 6 * ne + base), m1 = __ldg(L.ve + 7 * ne + base), m2 = __ldg(L.ve + 8 * ne + base);
-      ax = fma(P[p0], m0, fma(P[p1], m1, fma(P[p2], m2, P[9])));
-      ay = fma(P[3 + p0], m0, fma(P[3 + p1], m1, fma(P[3 + p2], m2, P[10])));
-      az = fma(P[6 + p0], m0, fma(P[6 + p1], m1, fma(P[6 + p2], m2, P[11])));
+#pragma unroll 1
+  for (int tile = 0; tile < kTiles; ++tile) {
+    if (kTiles > 1 && tile > 0) {
+      p += kV;
+      len = p < L.n_voxels ? L.vlen[p] : 0;
+      base = p < L.n_voxels ? L.slice_off[p >> 5] + (p & 31) : 0;
+#pragma unroll
+      for (int q = 0; q < 10; ++q) acc[q] = 0.0;
     }
-    for (int k = k0; k < len; k += kRows) {
-      const int64_t e = base + (int64_t)k * kSlice;
-      const uint32_t sv = (uint32_t)__ldg(L.ve_scan + e);
-      int p0, p1, p2;
-      perm_decode(sv >> kPermShift, p0, p1, p2);
-      const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
-      const double l10 = __ldg(L.ve + e), l20 = __ldg(L.ve + ne + e), l21 = __ldg(L.ve + 2 * ne + e);
-      const double D0 = __ldg(L.ve + 3 * ne + e), D1 = __ldg(L.ve + 4 * ne + e), D2 = __ldg(L.ve + 5 * ne + e);
-      const double m0 = __ldg(L.ve + 6 * ne + e), m1 = __ldg(L.ve + 7 * ne + e), m2 = __ldg(L.ve + 8 * ne + e);
-      const double N = __ldg(L.ve + 9 * ne + e);
-      // columns pi0, pi1, pi2 of R
-      const double a0 = P[p0], a1 = P[3 + p0], a2 = P[6 + p0];
-      const double b0 = P[p1], b1 = P[3 + p1], b2 = P[6 + p1];
-      const double c0 = P[p2], c1 = P[3 + p2], c2 = P[6 + p2];
-      const double qx = fma(a0, m0, fma(b0, m1, fma(c0, m2, P[9])));
-      const double qy = fma(a1, m0, fma(b1, m1, fma(c1, m2, P[10])));
-      const double qz = fma(a2, m0, fma(b2, m1, fma(c2, m2, P[11])));
-      const double dx = qx - ax, dy = qy - ay, dz = qz - az;
-      // R S R^T = sum_a D_a W_a W_a^T with W = R P^T L
-      const double w00 = fma(l10, b0, fma(l20, c0, a0)), w01 = fma(l10, b1, fma(l20, c1, a1)),
-                   w02 = fma(l10, b2, fma(l20, c2, a2));
-      const double w10 = fma(l21, c0, b0), w11 = fma(l21, c1, b1), w12 = fma(l21, c2, b2);
-      const double u00 = D0 * w00, u01 = D0 * w01, u02 = D0 * w02;
-      const double u10 = D1 * w10, u11 = D1 * w11, u12 = D1 * w12;
-      const double u20 = D2 * c0, u21 = D2 * c1, u22 = D2 * c2;
-      const double Nx = N * dx, Ny = N * dy, Nz = N * dz;
-      acc[4] = fma(u00, w00, fma(u10, w10, fma(u20, c0, fma(Nx, dx, acc[4]))));
-      acc[5] = fma(u00, w01, fma(u10, w11, fma(u20, c1, fma(Nx, dy, acc[5]))));
-      acc[6] = fma(u00, w02, fma(u10, w12, fma(u20, c2, fma(Nx, dz, acc[6]))));
-      acc[7] = fma(u01, w01, fma(u11, w11, fma(u21, c1, fma(Ny, dy, acc[7]))));
-      acc[8] = fma(u01, w02, fma(u11, w12, fma(u21, c2, fma(Ny, dz, acc[8]))));
-      acc[9] = fma(u02, w02, fma(u12, w12, fma(u22, c2, fma(Nz, dz, acc[9]))));
-      acc[1] += Nx;
-      acc[2] += Ny;
-      acc[3] += Nz;
-      acc[0] += N;
+    if (p < L.n_voxels) {
+      const int64_t ne = L.n_elems;
+      const int k0 = threadIdx.x / kV;
+      if (k0 < len || (kTiles == 1 && w == (int)(blk & 3))) {
+        // the anchor: the first observation's posed mean, formed by every thread
+        const uint32_t sv = (uint32_t)__ldg(L.ve_scan + base);
+        int p0, p1, p2;
+        perm_decode(sv >> kPermShift, p0, p1, p2);
+        const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
+        const double m0 = __ldg(L.ve + 6 * ne + base), m1 = __ldg(L.ve + 7 * ne + base), m2 = __ldg(L.ve + 8 * ne + base);
+        ax = fma(P[p0], m0, fma(P[p1], m1, fma(P[p2], m2, P[9])));
+        ay = fma(P[3 + p0], m0, fma(P[3 + p1], m1, fma(P[3 + p2], m2, P[10])));
+        az = fma(P[6 + p0], m0, fma(P[6 + p1], m1, fma(P[6 + p2], m2, P[11])));
+      }
+      for (int k = k0; k < len; k += kRows) {
+        const int64_t e = base + (int64_t)k * kSlice;
+        const uint32_t sv = (uint32_t)__ldg(L.ve_scan + e);
+        int p0, p1, p2;
+        perm_decode(sv >> kPermShift, p0, p1, p2);
+        const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
+        const double l10 = __ldg(L.ve + e), l20 = __ldg(L.ve + ne + e), l21 = __ldg(L.ve + 2 * ne + e);
+        const double D0 = __ldg(L.ve + 3 * ne + e), D1 = __ldg(L.ve + 4 * ne + e), D2 = __ldg(L.ve + 5 * ne + e);
+        const double m0 = __ldg(L.ve + 6 * ne + e), m1 = __ldg(L.ve + 7 * ne + e), m2 = __ldg(L.ve + 8 * ne + e);
+        const double N = __ldg(L.ve + 9 * ne + e);
+        // columns pi0, pi1, pi2 of R
+        const double a0 = P[p0], a1 = P[3 + p0], a2 = P[6 + p0];
+        const double b0 = P[p1], b1 = P[3 + p1], b2 = P[6 + p1];
+        const double c0 = P[p2], c1 = P[3 + p2], c2 = P[6 + p2];
+        const double qx = fma(a0, m0, fma(b0, m1, fma(c0, m2, P[9])));
+        const double qy = fma(a1, m0, fma(b1, m1, fma(c1, m2, P[10])));
+        const double qz = fma(a2, m0, fma(b2, m1, fma(c2, m2, P[11])));
+        const double dx = qx - ax, dy = qy - ay, dz = qz - az;
+        // R S R^T = sum_a D_a W_a W_a^T with W = R P^T L
+        const double w00 = fma(l10, b0, fma(l20, c0, a0)), w01 = fma(l10, b1, fma(l20, c1, a1)),
+                     w02 = fma(l10, b2, fma(l20, c2, a2));
+        const double w10 = fma(l21, c0, b0), w11 = fma(l21, c1, b1), w12 = fma(l21, c2, b2);
+        const double u00 = D0 * w00, u01 = D0 * w01, u02 = D0 * w02;
+        const double u10 = D1 * w10, u11 = D1 * w11, u12 = D1 * w12;
+        const double u20 = D2 * c0, u21 = D2 * c1, u22 = D2 * c2;
+        const double Nx = N * dx, Ny = N * dy, Nz = N * dz;
+        acc[4] = fma(u00, w00, fma(u10, w10, fma(u20, c0, fma(Nx, dx, acc[4]))));
+        acc[5] = fma(u00, w01, fma(u10, w11, fma(u20, c1, fma(Nx, dy, acc[5]))));
+        acc[6] = fma(u00, w02, fma(u10, w12, fma(u20, c2, fma(Nx, dz, acc[6]))));
+        acc[7] = fma(u01, w01, fma(u11, w11, fma(u21, c1, fma(Ny, dy, acc[7]))));
+        acc[8] = fma(u01, w02, fma(u11, w12, fma(u21, c2, fma(Ny, dz, acc[8]))));
+        acc[9] = fma(u02, w02, fma(u12, w12, fma(u22, c2, fma(Nz, dz, acc[9]))));
+        acc[1] += Nx;
+        acc[2] += Ny;
+        acc[3] += Nz;
+        acc[0] += N;
+      }
+    }
+    // a voxel's threads of one warp (kV < 32), then of the four warps, in a fixed order
+#pragma unroll
+    for (int o = 16; o >= kV; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < 10; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    if (lane < kV)
+#pragma unroll
+      for (int q = 0; q < 10; ++q) sums[w][q][tile * kV + lane] = acc[q];
+    if (kTiles > 1 && threadIdx.x < kV) {  // (the first row's threads: they have the anchor)
+      anchor[0][tile * kV + lane] = ax;
+      anchor[1][tile * kV + lane] = ay;
+      anchor[2][tile * kV + lane] = az;
     }
   }
-  // a voxel's threads of one warp (kV < 32), then of the four warps, in a fixed order
-#pragma unroll
-  for (int o = 16; o >= kV; o >>= 1)
-#pragma unroll
-    for (int q = 0; q < 10; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-  if (lane < kV)
-#pragma unroll
-    for (int q = 0; q < 10; ++q) sums[w][q][lane] = acc[q];
   __syncthreads();
   if (w == (int)(blk & 3)) {
     double lam0 = 0.0;
-    if (lane < kV && p < L.n_voxels) {
+    if (kTiles > 1) {
+      p = blk * (kV * kTiles) + lane;
+      ax = anchor[0][lane];
+      ay = anchor[1][lane];
+      az = anchor[2][lane];
+    }
+    if (lane < kV * kTiles && p < L.n_voxels) {
 #pragma unroll
       for (int q = 0; q < 10; ++q)
         acc[q] = (sums[0][q][lane] + sums[1][q][lane]) + (sums[2][q][lane] + sums[3][q][lane]);
@@ -153,32 +181,41 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
     }
 #pragma unroll
     for (int o = kV / 2; o > 0; o >>= 1) lam0 += __shfl_down_sync(0xffffffffu, lam0, o);
-    if (lane == 0) cost_part[blk] = lam0;
+    // (of each tile, in its first lane)
+#pragma unroll
+    for (int tile = 0; tile < kTiles; ++tile) {
+      const double c = kTiles == 1 ? lam0 : __shfl_sync(0xffffffffu, lam0, tile * kV);
+      const int64_t part = blk * kTiles + tile;
+      if (lane == 0 && (kTiles == 1 || part < voxel_pass_f64_blocks(L.n_voxels))) cost_part[part] = c;
+    }
   }
   voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_f64_blocks(L.n_voxels), pred_part, pred_parts(L.n_scans),
-                                   st, decide_mode, red, is_last, (int)(blk & 3) * 32);
+                                   st, decide_mode, red, is_last, (int)(blk & 3) * 32,
+                                   kTiles == 1 ? voxel_pass_f64_blocks(L.n_voxels) : (L.n_voxels + 31) / 32);
 }
 
-// the body for a problem of this size (voxel_pass_f64_width)
-template <bool kFull>
+// the body for a problem of this size (voxel_pass_f64_width), a tile of its
+// width or (kSlices) a slice of 32 voxels to a block
+template <bool kFull, bool kSlices>
 __device__ __forceinline__ void voxel_pass_f64_sized(const DevLayout& L, const double* poses2, double* planes2,
                                                      double* full_out, double* cost_part, const double* pred_part,
                                                      DevState* st, int use_trial, int decide_mode, int64_t blk) {
   __shared__ double red[kVoxelThreads / 32];
   __shared__ double sums[kVoxelThreads / 32][10][32];
+  __shared__ double anchor[kSlices ? 3 : 1][32];
   __shared__ int is_last;
   switch (voxel_pass_f64_width(L.n_voxels)) {
     case 8:
-      voxel_pass_f64_body<8, kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
-                                    blk, red, sums, &is_last);
+      voxel_pass_f64_body<8, kFull, kSlices ? 4 : 1>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial,
+                                                     decide_mode, blk, red, sums, anchor, &is_last);
       break;
     case 16:
-      voxel_pass_f64_body<16, kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
-                                     blk, red, sums, &is_last);
+      voxel_pass_f64_body<16, kFull, kSlices ? 2 : 1>(L, poses2, planes2, full_out, cost_part, pred_part, st,
+                                                      use_trial, decide_mode, blk, red, sums, anchor, &is_last);
       break;
     default:
-      voxel_pass_f64_body<32, kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
-                                     blk, red, sums, &is_last);
+      voxel_pass_f64_body<32, kFull, 1>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial,
+                                        decide_mode, blk, red, sums, anchor, &is_last);
   }
 }
 
@@ -187,7 +224,7 @@ __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_kernel(DevLayout
                                                                       double* planes2, double* full_out,
                                                                       double* cost_part, const double* pred_part,
                                                                       DevState* st, int use_trial, int decide_mode) {
-  voxel_pass_f64_sized<kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
+  voxel_pass_f64_sized<kFull, false>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
                               blockIdx.x);
 }
 
@@ -195,7 +232,7 @@ __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_batch_kernel(con
                                                                              int use_trial) {
   const int job = find_job(G.vblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  voxel_pass_f64_sized<false>(J.L, J.poses2, J.planes2, nullptr, J.cost_part, J.pred_part, J.st, use_trial,
+  voxel_pass_f64_sized<false, true>(J.L, J.poses2, J.planes2, nullptr, J.cost_part, J.pred_part, J.st, use_trial,
                               use_trial ? 0 : 1, (int64_t)blockIdx.x - G.vblk[job]);
 }
 

@@ -185,7 +185,7 @@ __device__ __forceinline__ void voxel_pass_mixed_body(const DevLayout& L, const 
   const float tot = block_sum<kVoxelThreads, float>(lam0, red);
   if (threadIdx.x == 0) cost_part[blk] = (double)tot;
   voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_blocks(L.n_voxels), pred_part, pred_parts(L.n_scans), st,
-                                   decide_mode, dred, is_last);
+                                   decide_mode, dred, is_last, 0, voxel_pass_blocks(L.n_voxels));
 }
 
 template <bool kFull>

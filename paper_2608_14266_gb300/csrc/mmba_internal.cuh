@@ -954,20 +954,20 @@ __device__ __forceinline__ void decide_apply(DevState* st, double csum, double p
 
 // Epilogue of a voxel pass that decides in its last block: every block adds
 // one to the state's counter after its cost partial is visible device-wide;
-// the block that brings the counter to n_cost sums all partials (in the same
+// the block that brings the counter to n_blocks sums all partials (in the same
 // fixed order as a separate decision launch, so results do not depend on which
 // block finishes last), decides, and re-arms the counter.  mode as for
 // decide_body; with mode < 0 nothing is decided.  leader is the thread that
-// wrote the block's partial.
+// wrote the block's partials.
 template <int kThreads>
 __device__ __forceinline__ void voxel_pass_decide(const double* cost_part, int64_t n_cost, const double* pred_part,
                                                   int64_t n_pred, DevState* st, int mode, double* red,
-                                                  int* is_last, int leader = 0) {
+                                                  int* is_last, int leader, int64_t n_blocks) {
   if (mode < 0) return;
   if (threadIdx.x == leader) {
     __threadfence();
     const unsigned prev = atomicAdd(&st->blocks_done, 1u);
-    *is_last = prev == (unsigned)(n_cost - 1);
+    *is_last = prev == (unsigned)(n_blocks - 1);
   }
   __syncthreads();
   if (!*is_last) return;
