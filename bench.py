@@ -1081,14 +1081,15 @@ def _standalone(fn, args):
 # preprocessing: FP64 peak from the unit counts (152 SMs x 2 FP64 FMA lanes
 # per clock x 2 flops x 2.07 GHz max SM clock)
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# algorithmic work per point of the dominant stages: world point and index
-# (9 FMA + 3 adds = 21 flops); the clusters' shifted sums (3 subtractions,
-# 3 additions, 6 FMA = 18 flops); the level-1 sort of packed 32-bit keys
-# (repack: read 8 B, write 4 B; per 8-bit pass: histogram reads the 4-byte
-# key, scatter reads and writes key and value, 4 + 16 B)
-VOX_KEYS_FLOPS_PER_POINT = 21
-VOX_CLUSTER_FLOPS_PER_POINT = 18
-VOX_SORT_BYTES_PER_POINT = lambda passes: 12 + 20 * passes
+# algorithmic bytes per point of the dominant stages (keys and cluster sums are
+# integer work, with FP64 near voxel faces and per run only): the point read,
+# key and scan written; the point, its index and its key read; the level-1 sort
+# of packed 32-bit keys (repack: read 8 B, write 4 B; the histograms of all
+# digits read the 4-byte key once; per 8-bit pass the scatter reads and writes
+# key and value, 16 B)
+VOX_KEYS_BYTES_PER_POINT = 24 + 8 + 4
+VOX_CLUSTER_BYTES_PER_POINT = 24 + 4 + 4
+VOX_SORT_BYTES_PER_POINT = lambda passes: 12 + 4 + 16 * passes
 
 
 def run_voxelize(args):
@@ -1158,21 +1159,20 @@ def voxelize_result(args, mm, torch, scenegen):
     span = _world_index_range(P_p.numpy(), spo_h, s.pose_init[:n_scans], cfg["voxel_size"])
     passes = -(-int(sum(int(x).bit_length() for x in span)) // 8)
     rl = {
-        "cluster_pass": {"bound": "alu", "achieved": VOX_CLUSTER_FLOPS_PER_POINT * n_pts / (stage_ms["cluster_pass"] / 1e3) / 1e12,
-                         "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s"},
-        "keys": {"bound": "alu", "achieved": VOX_KEYS_FLOPS_PER_POINT * n_pts / (stage_ms["keys"] / 1e3) / 1e12,
-                 "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s"},
+        "cluster_pass": {"bound": "hbm", "achieved": VOX_CLUSTER_BYTES_PER_POINT * n_pts / (stage_ms["cluster_pass"] / 1e3) / 1e9,
+                         "peak": hbm, "unit": "GB/s"},
+        "keys": {"bound": "hbm", "achieved": VOX_KEYS_BYTES_PER_POINT * n_pts / (stage_ms["keys"] / 1e3) / 1e9,
+                 "peak": hbm, "unit": "GB/s"},
         "sort": {"bound": "hbm", "achieved": VOX_SORT_BYTES_PER_POINT(passes) * n_pts / (stage_ms["sort"] / 1e3) / 1e9,
                  "peak": hbm, "unit": "GB/s"},
     }
     for x in rl.values():
         x["frac"] = x["achieved"] / x["peak"]
     top = max(rl, key=lambda k: stage_ms[k])
-    kname = {"cluster_pass": "l1_pieces", "keys": "l1_keys", "sort": "radix sort of the level-1 keys"}[top]
+    kname = {"cluster_pass": "l1_clusters", "keys": "l1_keys", "sort": "radix sort of the level-1 keys"}[top]
     tr = recorded_traffic(f"voxelize_{n_scans}", kname)
     roof = dict(rl[top], traffic=tr, kernel=kname,
-                stage_ms=stage_ms[top], peak_source="FP64: 152 SMs x 2 FMA/clk x 2 flops x 2.07 GHz"
-                if rl[top]["bound"] == "alu" else src)
+                stage_ms=stage_ms[top], peak_source=src)
     # oracle on the first scans' points (bounded sample), scaled by points
     import oracle
     k = 1
