@@ -477,8 +477,9 @@ ba_status ba_aggregate_points(int64_t n_obs, const int64_t* point_offsets, const
  * w = R_j p + t_j (each axis fma(R_a0, p0, fma(R_a1, p1, fma(R_a2, p2,
  * t_a))), the index floor(w / d) per axis, the floor of the correctly
  * rounded quotient; the points of one scan in one voxel form one centred
- * cluster (Eq. 2), summed in point order as shifted sums (deviations from
- * the run's first point) in fixed chunks, so results are deterministic and
+ * cluster (Eq. 2) from the points' deviations from the run's first point, as
+ * exact fixed-point sums (a run outside their range: shifted sums in FP64, in
+ * point order); results are deterministic and
  * agree with the mean-then-scatter definition to rounding.  Bottom-up levels
  * (Eq. 5): the level-k index of a level-(k-1) cluster is floor(index / 2)
  * per axis, and the clusters with the same (level-k index, scan) are merged
