@@ -21,59 +21,103 @@ namespace mmba {
   } while (0)
 
 // ============================================================================
-// Exclusive scan of int64 (three-phase: per-tile scan + tile sums, recursive
-// scan of the tile sums, add back).
+// Exclusive scan of int64: (1) each tile's sum; (2) each tile scanned behind the
+// sum of the tiles before it, which its block adds up itself while there are
+// few (their recursive scan beyond).  Bound by DRAM: two reads and a write (a
+// scan of every tile and a pass that adds the prefixes back wrote twice).  A
+// warp takes 256 consecutive elements, two to a lane, so its accesses are whole
+// lines (120M points: all prefix sums of a call 360 -> 200 us).
 // ============================================================================
 constexpr int kScanBlock = 512;
-constexpr int kScanItems = 8;
-constexpr int64_t kScanTile = (int64_t)kScanBlock * kScanItems;
+constexpr int kScanRounds = 4;  // of 64 elements a warp
+constexpr int64_t kScanTile = (int64_t)kScanBlock * 2 * kScanRounds;
+constexpr int64_t kScanOwnTiles = 4096;  // tiles whose sums a block adds up itself
 
-__global__ void __launch_bounds__(kScanBlock) scan_tiles_kernel(int64_t* data, int64_t n, int64_t* tile_sums) {
+// elements i, i + 1 (0 past the end)
+__device__ __forceinline__ longlong2 scan_load(const int64_t* data, int64_t i, int64_t n, bool pair) {
+  if (pair && i + 1 < n) return *reinterpret_cast<const longlong2*>(data + i);
+  return make_longlong2(i < n ? data[i] : 0, i + 1 < n ? data[i + 1] : 0);
+}
+
+// the block's total of v, in every thread
+__device__ __forceinline__ int64_t scan_block_total(int64_t v, int64_t* warp_tot) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) warp_tot[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int64_t t = 0;
+#pragma unroll
+  for (int k = 0; k < kScanBlock / 32; ++k) t += warp_tot[k];
+  __syncthreads();
+  return t;
+}
+
+__global__ void __launch_bounds__(kScanBlock) scan_sums_kernel(const int64_t* data, int64_t n, int64_t* tile_sums) {
   grid_wait();
   grid_launch_next();
   __shared__ int64_t warp_tot[kScanBlock / 32];
-  const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-  int64_t v[kScanItems];
-  int64_t run = 0;
+  const bool pair = reinterpret_cast<uintptr_t>(data) % 16 == 0;
+  const int64_t i0 = (int64_t)blockIdx.x * kScanTile + 2 * threadIdx.x;
+  longlong2 v[kScanRounds];
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    int64_t x = (base + k < n) ? data[base + k] : 0;
-    v[k] = run;
-    run += x;
-  }
-  // exclusive scan of per-thread totals across the block
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int64_t incl = run;
+  for (int r = 0; r < kScanRounds; ++r) v[r] = scan_load(data, i0 + r * (2 * kScanBlock), n, pair);
+  int64_t t = 0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int64_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) warp_tot[w] = incl;
-  __syncthreads();
-  if (w == 0) {
-    int64_t t = lane < kScanBlock / 32 ? warp_tot[lane] : 0;
-    int64_t ti = t;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int64_t y = __shfl_up_sync(0xffffffffu, ti, o);
-      if (lane >= o) ti += y;
-    }
-    if (lane < kScanBlock / 32) warp_tot[lane] = ti - t;  // exclusive warp prefix
-    if (lane == kScanBlock / 32 - 1 && tile_sums) tile_sums[blockIdx.x] = ti;
-  }
-  __syncthreads();
-  const int64_t pre = warp_tot[w] + incl - run;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k)
-    if (base + k < n) data[base + k] = v[k] + pre;
+  for (int r = 0; r < kScanRounds; ++r) t += v[r].x + v[r].y;
+  t = scan_block_total(t, warp_tot);
+  if (threadIdx.x == 0) tile_sums[blockIdx.x] = t;
 }
 
-__global__ void scan_add_kernel(int64_t* data, int64_t n, const int64_t* tile_pre) {
+// before: the tiles' sums (scanned = false) or their exclusive scan; null with one tile
+__global__ void __launch_bounds__(kScanBlock) scan_tiles_kernel(int64_t* data, int64_t n, const int64_t* before,
+                                                                bool scanned) {
   grid_wait();
   grid_launch_next();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) data[i] += tile_pre[i / kScanTile];
+  __shared__ int64_t warp_tot[kScanBlock / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool pair = reinterpret_cast<uintptr_t>(data) % 16 == 0;
+  const int64_t i0 = (int64_t)blockIdx.x * kScanTile + w * (64 * kScanRounds) + 2 * lane;
+  longlong2 v[kScanRounds];
+#pragma unroll
+  for (int r = 0; r < kScanRounds; ++r) v[r] = scan_load(data, i0 + 64 * r, n, pair);
+  int64_t pre = 0;
+  if (before) {
+    if (scanned) {
+      pre = before[blockIdx.x];
+    } else {
+      for (int64_t k = threadIdx.x; k < blockIdx.x; k += kScanBlock) pre += before[k];
+      pre = scan_block_total(pre, warp_tot);
+    }
+  }
+  // the warp's running sums, round by round
+  int64_t run = 0, start[kScanRounds];
+#pragma unroll
+  for (int r = 0; r < kScanRounds; ++r) {
+    const int64_t x = v[r].x + v[r].y;
+    int64_t incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    start[r] = run + incl - x;
+    run += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (lane == 0) warp_tot[w] = run;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kScanBlock / 32; ++k) pre += k < w ? warp_tot[k] : 0;
+#pragma unroll
+  for (int r = 0; r < kScanRounds; ++r) {
+    const int64_t i = i0 + 64 * r;
+    const int64_t x = pre + start[r], y = x + v[r].x;
+    if (pair && i + 1 < n) {
+      *reinterpret_cast<longlong2*>(data + i) = make_longlong2(x, y);
+    } else {
+      if (i < n) data[i] = x;
+      if (i + 1 < n) data[i + 1] = y;
+    }
+  }
 }
 
 int64_t scan_scratch_count(int64_t n) {
@@ -89,16 +133,17 @@ cudaError_t exclusive_scan_i64(int64_t* data, int64_t n, int64_t* scratch, cudaS
   if (n <= 0) return cudaSuccess;
   const int64_t tiles = (n + kScanTile - 1) / kScanTile;
   if (tiles == 1) {
-    launch_chained(scan_tiles_kernel, 1, kScanBlock, 0, stream, data, n, nullptr);
+    launch_chained(scan_tiles_kernel, 1, kScanBlock, 0, stream, data, n, nullptr, false);
     ++*launches;
     return cudaGetLastError();
   }
   int64_t* sums = scratch;
-  launch_chained(scan_tiles_kernel, (unsigned)tiles, kScanBlock, 0, stream, data, n, sums);
+  launch_chained(scan_sums_kernel, (unsigned)tiles, kScanBlock, 0, stream, data, n, sums);
   ++*launches;
   RETURN_IF(cudaGetLastError());
-  RETURN_IF(exclusive_scan_i64(sums, tiles, scratch + tiles + 1, stream, launches));
-  launch_chained(scan_add_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, data, n, sums);
+  const bool scanned = tiles > kScanOwnTiles;
+  if (scanned) RETURN_IF(exclusive_scan_i64(sums, tiles, scratch + tiles + 1, stream, launches));
+  launch_chained(scan_tiles_kernel, (unsigned)tiles, kScanBlock, 0, stream, data, n, sums, scanned);
   ++*launches;
   return cudaGetLastError();
 }

@@ -69,3 +69,19 @@ def test_loaded_layout_gives_the_oracle_gradient(mm, n_scans, n_voxels):
     # rounding of terms of the Hessian's size)
     np.testing.assert_allclose(g2, g, rtol=0, atol=1e-10 * np.abs(g).max() + 1e-13 * np.abs(H).max())
     np.testing.assert_allclose(H2, H, rtol=0, atol=1e-11 * np.abs(H).max())
+
+
+@pytest.mark.parametrize("n", [4096 * 4096 - 1, 4096 * 4096 + 5])
+def test_prefix_sums_on_both_sides_of_4096_tiles(mm, n):
+    """A point to a voxel, so that the prefix sums run over n + 1 heads: up to
+    4,096 tiles of 4,096 a block adds up the sums of the tiles before its own,
+    beyond they are scanned first.  Every voxel starts where it must."""
+    import torch
+    i = torch.arange(n, dtype=torch.int64, device="cuda")
+    cell = torch.stack([i % 300, (i // 300) % 300, i // 90000], 1)
+    spo = torch.tensor([0, n], dtype=torch.int64, device="cuda")
+    poses = torch.tensor([[1.0, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0]], dtype=torch.float64, device="cuda")
+    got = mm.voxelize(spo, cell.double() + 0.5, poses, 1.0, out="device")
+    assert torch.equal(got["voxel_off"], torch.arange(n + 1, device="cuda"))
+    key = lambda x: (x[:, 0].long() * 300 + x[:, 1].long()) * 300 + x[:, 2].long()
+    assert torch.equal(key(got["index"]), key(cell).sort()[0])
