@@ -400,8 +400,8 @@ int64_t radix_scratch_count(int64_t n) {
 template <typename K>
 static cudaError_t radix_sort_pairs_t(K** keys, uint32_t** vals, K** tmp_keys, uint32_t** tmp_vals, int64_t n, int bits,
                                       bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches) {
-  const int passes = radix_passes(bits);
-  if (n <= 1 || passes == 0) {
+  const int passes = radix_passes(n, bits);
+  if (passes == 0) {
     if (!positions || n <= 0) return cudaSuccess;
     launch_chained(positions_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, n, *vals);
     ++*launches;
@@ -1071,8 +1071,8 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
     RETURN_IF(exclusive_scan_i64(pbase, nv + 1, pscratch, stream, launches));
     out->vstart = defer_scale ? pbase : nullptr;
     // the order, where it is kept, lands in its own buffer: the sort ends in the
-    // buffer it starts from after an even number of digits, else in the other
-    if (order) (radix_passes(scan_bits) % 2 == 0 ? vals : tv) = order;
+    // buffer it starts from after an even number of passes, else in the other
+    if (order) (radix_passes(no, scan_bits) % 2 == 0 ? vals : tv) = order;
     launch_chained(scan_keys_kernel, (unsigned)((no + 255) / 256), 256, 0, stream, in, obs_vox, vrank, pbase, keys, vals, place);
     ++*launches;
     RETURN_IF(cudaGetLastError());
@@ -1100,7 +1100,7 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
   launch_chained(scan_len_keys_kernel, (unsigned)((in.n_scans + 255) / 256), 256, 0, stream, out->scan_off, in.n_scans, no, keys);
   ++*launches;
   RETURN_IF(cudaGetLastError());
-  if (radix_passes(len_digits) % 2 != 0) std::swap(by_len, other);
+  if (radix_passes(in.n_scans, len_digits) % 2 != 0) std::swap(by_len, other);
   RETURN_IF(radix_sort_pairs(&keys, &by_len, &tk, &other, in.n_scans, len_digits, true, scratch, stream, launches));
   return cudaSuccess;
 }

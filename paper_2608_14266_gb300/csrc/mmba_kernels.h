@@ -126,11 +126,12 @@ cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double*
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of the
 // keys (n < 2^32).  Buffers of n entries each and scratch of
 // radix_scratch_count(n) int64 are supplied by the caller; the sorted pairs end
-// in *keys and *vals, which are exchanged with *tmp_keys and *tmp_vals after an
-// odd number of digits (radix_passes(bits)).  With positions = true the values
-// are the positions 0 .. n - 1 and *vals need not be filled.
+// in *keys and *vals, which each pass (radix_passes) exchanges with *tmp_keys
+// and *tmp_vals.  With positions = true the values are the positions 0 .. n - 1
+// and *vals need not be filled.
 int64_t radix_scratch_count(int64_t n);
-inline int radix_passes(int bits) { return bits <= 0 ? 0 : (bits + 7) / 8; }
+// passes of a sort, one a digit: none for one element, which stays where it is
+inline int radix_passes(int64_t n, int bits) { return n <= 1 || bits <= 0 ? 0 : (bits + 7) / 8; }
 cudaError_t radix_sort_pairs(uint32_t** keys, uint32_t** vals, uint32_t** tmp_keys, uint32_t** tmp_vals, int64_t n,
                              int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches);
 // The same for 64-bit keys (bits up to 64).
