@@ -291,29 +291,34 @@ cudaError_t prof_end(ba_handle* h, size_t idx) {
   return cudaEventRecord(h->ev_pool[idx + 1], h->stream);
 }
 
-// The solve may start under the scan pass's tail (launch_dependent) in FP64,
-// and in the mixed path up to this many observations, whose copies L2 holds:
-// a solve block that starts early keeps its SM from changing between the
-// scan pass's split of shared memory and L1 and the voxel pass's, which at
-// larger sizes costs the voxel pass its L1.  Measured, us an iteration without
-// / with: 58.3 / 56.3 at 0.6M observations, 90.7 / 88.6 at 2.4M, 145.4 / 147.9
-// at 4.8M, 307 / 319 at 15M.
+// In the mixed path the solve may start under the scan pass's tail
+// (early_solve) up to this many observations, whose copies L2 holds: a solve
+// block that starts early keeps its SM from changing between the scan pass's
+// split of shared memory and L1 and the voxel pass's, which at larger sizes
+// costs the voxel pass its L1.  Measured, us an iteration without / with: 58.3 /
+// 56.3 at 0.6M observations, 90.7 / 88.6 at 2.4M, 145.4 / 147.9 at 4.8M, 307 /
+// 319 at 15M; of 5,000 scans and 0.17M observations (more than two solve blocks
+// an SM) 41.6 / 45.4.
 constexpr int64_t kDependentSolveObs = 2500000;
 
 ba_status launch_iteration(ba_handle* h) {
-  const bool early_solve = !h->mixed || h->L.n_obs <= kDependentSolveObs;
+  const int64_t nsc = h->L.n_scans;
+  const bool solve_early = early_solve(solve_blocks(nsc, solve_lanes(nsc))) &&
+                           (!h->mixed || h->L.n_obs <= kDependentSolveObs);
+  const bool voxel_early = h->mixed || early_voxel_pass_f64(h->n_cost);
+  const bool scan_early = early_scan_pass_f64(nsc, h->n_cost);
   size_t ev = 0;
   CK(h, prof_begin(h, BA_KERNEL_SOLVE, &ev), "event");
   CK(h, launch_solve_f64(h->L, h->poses2, h->gH, h->pred_part, h->d_state, h->mixed ? h->mb.sref : nullptr,
-                         h->mixed ? h->mb.stab2 : nullptr, h->stream, early_solve),
+                         h->mixed ? h->mb.stab2 : nullptr, h->stream, solve_early),
      "solve");
   CK(h, prof_end(h, ev), "event");
   CK(h, prof_begin(h, BA_KERNEL_VOXEL_PASS, &ev), "event");
   // the trial cost and the LM decision (in the pass's last block)
-  CK(h, voxel_pass(h, nullptr, 1, 0, true), "trial voxel pass");
+  CK(h, voxel_pass(h, nullptr, 1, 0, voxel_early), "trial voxel pass");
   CK(h, prof_end(h, ev), "event");
   CK(h, prof_begin(h, BA_KERNEL_SCAN_PASS, &ev), "event");
-  CK(h, scan_pass(h, 0, true), "scan pass");
+  CK(h, scan_pass(h, 0, scan_early), "scan pass");
   CK(h, prof_end(h, ev), "event");
   h->launches += 3;
   return BA_OK;

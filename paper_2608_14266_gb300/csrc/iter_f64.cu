@@ -820,11 +820,13 @@ cudaError_t launch_batch_solve(const JobGroup& T, int64_t n_blocks, cudaStream_t
 }
 
 cudaError_t launch_batch_voxel_pass_f64(const JobGroup& T, int64_t n_blocks, int use_trial, cudaStream_t stream) {
-  return launch_dependent(voxel_pass_f64_batch_kernel, n_blocks, kVoxelThreads, stream, true, T, use_trial);
+  return launch_dependent(voxel_pass_f64_batch_kernel, n_blocks, kVoxelThreads, stream,
+                          early_voxel_pass_f64(n_blocks) || T.sblk[T.n_jobs] >= 3 * kSMs, T, use_trial);
 }
 
 cudaError_t launch_batch_scan_pass_f64(const JobGroup& T, int64_t n_blocks, cudaStream_t stream) {
-  return launch_dependent(scan_pass_f64_batch_kernel, n_blocks, kScanThreads, stream, true, T);
+  return launch_dependent(scan_pass_f64_batch_kernel, n_blocks, kScanThreads, stream,
+                          early_scan_pass_f64(n_blocks, T.vblk[T.n_jobs]), T);
 }
 
 }  // namespace mmba

@@ -47,6 +47,31 @@ inline int64_t solve_blocks(int64_t n_scans, int lanes) {
 constexpr int kPredScans = 8;
 __host__ __device__ inline int64_t pred_parts(int64_t n_scans) { return (n_scans + kPredScans - 1) / kPredScans; }
 
+// Which FP64 kernels of an iteration may start under the tail of the one before
+// (launch_dependent).  A block that starts early takes the first place that
+// comes free, so a grid that does not fill the chip ends up on the few SMs that
+// drained first and shares their FP64 pipes, with the others idle; started
+// after the drain it is spread over all SMs.  So early only
+//   the solve       of at most two blocks an SM,
+//   the voxel pass  of at most 5/3 blocks an SM (with 282 blocks the scan pass
+//                   behind it loses, with 250 it does not), and in a batch,
+//                   whose groups run beside each other, where the scan pass
+//                   fills the chip,
+//   the scan pass   where it and the voxel pass before it are just under four
+//                   blocks an SM (both then have room on every SM; with 600
+//                   blocks 52 us instead of 55, with 613 95 instead of 85),
+//                   or with a grid that fills the chip (three resident blocks).
+// Measured, us an iteration with none / all / these early: 20 scans and 200
+// voxels 45.8 / 40.5 / 40.2; 20 and 5,500 139 / 204 / 137; 20 and 20,000 382 /
+// 923 / 382; 100 and 20,000 142 / 253 / 138; 1,000 and 50,000 474 / 470 / 470;
+// 10,000 and 300,000 1,155 / 1,158 / 1,151.
+constexpr int64_t kSMs = 152;
+inline bool early_solve(int64_t blocks) { return blocks <= 2 * kSMs; }
+inline bool early_voxel_pass_f64(int64_t blocks) { return 3 * blocks <= 5 * kSMs; }
+inline bool early_scan_pass_f64(int64_t blocks, int64_t voxel_blocks) {
+  return blocks + voxel_blocks <= 4 * kSMs - 8 || blocks >= 3 * kSMs;
+}
+
 // Launch of an iteration kernel; with dependent = true it may start while the
 // kernel before it in the stream drains (see grid_wait in mmba_internal.cuh).
 template <typename... P, typename... A>
