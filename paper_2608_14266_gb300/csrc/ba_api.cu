@@ -257,9 +257,10 @@ cudaError_t voxel_pass(ba_handle* h, double* full, int use_trial, int decide_mod
                                decide_mode, h->stream, dependent);
 }
 
-cudaError_t scan_pass(ba_handle* h, int force, bool dependent = false) {
-  if (h->mixed) return launch_scan_pass_mixed(h->L, h->X, h->poses2, h->gH, h->d_state, force, h->stream);
-  return launch_scan_pass_f64(h->L, h->poses2, h->planes2, h->gH, h->d_state, force, h->stream, dependent);
+// (next_early: the launch after it may start early)
+cudaError_t scan_pass(ba_handle* h, int force, bool dependent = false, bool next_early = false) {
+  if (h->mixed) return launch_scan_pass_mixed(h->L, h->X, h->poses2, h->gH, h->d_state, force, h->stream, next_early);
+  return launch_scan_pass_f64(h->L, h->poses2, h->planes2, h->gH, h->d_state, force, h->stream, dependent, next_early);
 }
 
 ba_status evaluate_current(ba_handle* h) {
@@ -297,14 +298,13 @@ cudaError_t prof_end(ba_handle* h, size_t idx) {
 // split of shared memory and L1 and the voxel pass's, which at larger sizes
 // costs the voxel pass its L1.  Measured, us an iteration without / with: 58.3 /
 // 56.3 at 0.6M observations, 90.7 / 88.6 at 2.4M, 145.4 / 147.9 at 4.8M, 307 /
-// 319 at 15M; of 5,000 scans and 0.17M observations (more than two solve blocks
-// an SM) 41.6 / 45.4.
+// 319 at 15M; of 5,000 scans and 0.17M observations (beyond early_solve) 41.6 /
+// 45.4.
 constexpr int64_t kDependentSolveObs = 2500000;
 
 ba_status launch_iteration(ba_handle* h) {
   const int64_t nsc = h->L.n_scans;
-  const bool solve_early = early_solve(solve_blocks(nsc, solve_lanes(nsc))) &&
-                           (!h->mixed || h->L.n_obs <= kDependentSolveObs);
+  const bool solve_early = early_solve(nsc) && (!h->mixed || h->L.n_obs <= kDependentSolveObs);
   const bool voxel_early = h->mixed || early_voxel_pass_f64(h->n_cost);
   const bool scan_early = early_scan_pass_f64(nsc, h->n_cost);
   size_t ev = 0;
@@ -318,7 +318,7 @@ ba_status launch_iteration(ba_handle* h) {
   CK(h, voxel_pass(h, nullptr, 1, 0, voxel_early), "trial voxel pass");
   CK(h, prof_end(h, ev), "event");
   CK(h, prof_begin(h, BA_KERNEL_SCAN_PASS, &ev), "event");
-  CK(h, scan_pass(h, 0, scan_early), "scan pass");
+  CK(h, scan_pass(h, 0, scan_early, solve_early), "scan pass");
   CK(h, prof_end(h, ev), "event");
   h->launches += 3;
   return BA_OK;

@@ -251,14 +251,21 @@ __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_batch_kernel(con
 // the (w m'^T + m' w^T)/2 - (w^T m') I term.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const double* poses2, const double* planes2,
-                                                   double* gH, const DevState* st, int force, int j,
+                                                   double* gH, const DevState* st, int force, int order, int j,
                                                    double (*red)[32]) {
-  const int64_t lo = L.scan_off[j], hi = L.scan_off[j + 1];
-  grid_wait();
-  grid_launch_next();
+  int64_t lo = 0, hi = 0;
+  if (order & kWaits) {  // (not before the test below in a launch that does not wait)
+    lo = L.scan_off[j];
+    hi = L.scan_off[j + 1];
+  }
+  grid_order(order);
   st = after_wait(st);
   // a rejected step (or an iteration after the solve stopped) leaves g, H unchanged
   if (!force && !st->scan_pending) return;
+  if (!(order & kWaits)) {
+    lo = L.scan_off[j];
+    hi = L.scan_off[j + 1];
+  }
   const int buf = st->cur;
   const double* P = after_wait(poses2) + ((int64_t)buf * L.n_scans + j) * 12;
   const double* planes = after_wait(planes2) + (int64_t)buf * L.n_voxels * kPlaneStride;
@@ -404,16 +411,18 @@ __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const dou
 
 __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_kernel(DevLayout L, const double* poses2,
                                                                     const double* planes2, double* gH,
-                                                                    const DevState* st, int force) {
+                                                                    const DevState* st, int force, int order) {
   __shared__ double red[kScanThreads / 32][32];
-  scan_pass_f64_body(L, poses2, planes2, gH, st, force, MMBA_IDX(scan_of_block(L, blockIdx.x), L.n_scans, st), red);
+  scan_pass_f64_body(L, poses2, planes2, gH, st, force, order,
+                     MMBA_IDX(scan_of_block(L, blockIdx.x), L.n_scans, st), red);
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const __grid_constant__ JobGroup G) {
+__global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const __grid_constant__ JobGroup G,
+                                                                          int order) {
   __shared__ double red[kScanThreads / 32][32];
   const int job = find_job(G.sblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  scan_pass_f64_body(J.L, J.poses2, J.planes2, J.gH, J.st, 0,
+  scan_pass_f64_body(J.L, J.poses2, J.planes2, J.gH, J.st, 0, order,
                      MMBA_IDX(scan_of_block(J.L, (int64_t)blockIdx.x - G.sblk[job]), J.L.n_scans, J.st), red);
 }
 
@@ -784,10 +793,11 @@ cudaError_t launch_voxel_pass_f64(const DevLayout& L, const double* poses2, doub
 }
 
 cudaError_t launch_scan_pass_f64(const DevLayout& L, const double* poses2, const double* planes2, double* gH,
-                                 const DevState* st, int force, cudaStream_t stream, bool dependent) {
+                                 const DevState* st, int force, cudaStream_t stream, bool dependent,
+                                 bool next_early) {
   if (L.n_scans == 0) return cudaSuccess;
   return launch_dependent(scan_pass_f64_kernel, L.n_scans, kScanThreads, stream, dependent, L, poses2, planes2, gH, st,
-                          force);
+                          force, (dependent ? kWaits : 0) | (next_early ? kFreesNext : 0));
 }
 
 cudaError_t launch_shard_cost(const double* cost_part, int64_t n_cost, double* out, cudaStream_t stream) {
@@ -825,8 +835,8 @@ cudaError_t launch_batch_voxel_pass_f64(const JobGroup& T, int64_t n_blocks, int
 }
 
 cudaError_t launch_batch_scan_pass_f64(const JobGroup& T, int64_t n_blocks, cudaStream_t stream) {
-  return launch_dependent(scan_pass_f64_batch_kernel, n_blocks, kScanThreads, stream,
-                          early_scan_pass_f64(n_blocks, T.vblk[T.n_jobs]), T);
+  const bool early = early_scan_pass_f64(n_blocks, T.vblk[T.n_jobs]);
+  return launch_dependent(scan_pass_f64_batch_kernel, n_blocks, kScanThreads, stream, early, T, early ? kWaits : 0);
 }
 
 }  // namespace mmba

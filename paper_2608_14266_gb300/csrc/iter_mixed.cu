@@ -326,14 +326,14 @@ __device__ __forceinline__ void issue_scan_chunk(ScanChunk& S, uint32_t bar, con
 
 __device__ __forceinline__ void scan_pass_mixed_body(const DevLayout& L, const DevMixed& X,
                                                      double* __restrict__ gH, DevState* __restrict__ st, int force,
-                                                     int j, float (*red)[kGH], float* tot, float* dR,
+                                                     int order, int j, float (*red)[kGH], float* tot, float* dR,
                                                      ScanChunk* chunks, uint64_t* bars) {
   // launched after the voxel pass has drained, not dependent on it: its shared
   // memory and the voxel pass's L1 want different splits of the SM's memory,
   // which changes only between blocks (as a dependent launch its first blocks
   // would settle for the voxel pass's split: 61 -> 73 us an iteration at 0.6M
   // observations, 307 -> 316 at 15M)
-  grid_launch_next();
+  grid_order(order);
   if (!force && !st->scan_pending) return;
   const int lane = threadIdx.x & 31;
   const int buf = st->cur;
@@ -475,14 +475,15 @@ __device__ __forceinline__ void scan_pass_mixed_body(const DevLayout& L, const D
 }
 
 __global__ void __launch_bounds__(kScanMixedThreads, 24) scan_pass_mixed_kernel(DevLayout L, DevMixed X,
-                                                                                  double* gH, DevState* st, int force) {
+                                                                                  double* gH, DevState* st, int force,
+                                                                                  int order) {
   __shared__ float red[1][kGH];
   __shared__ float tot[kGH];
   __shared__ float dR[9];
   __shared__ ScanChunk chunks[2];
   __shared__ uint64_t bars[2];
-  scan_pass_mixed_body(L, X, gH, st, force, MMBA_IDX(scan_of_block(L, blockIdx.x), L.n_scans, st), red, tot, dR,
-                       chunks, bars);
+  scan_pass_mixed_body(L, X, gH, st, force, order, MMBA_IDX(scan_of_block(L, blockIdx.x), L.n_scans, st), red, tot,
+                       dR, chunks, bars);
 }
 
 __global__ void __launch_bounds__(kScanMixedThreads, 24)
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(kScanMixedThreads, 24)
   __shared__ uint64_t bars[2];
   const int job = find_job(G.sblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  scan_pass_mixed_body(J.L, J.X, J.gH, J.st, 0,
+  scan_pass_mixed_body(J.L, J.X, J.gH, J.st, 0, 0,
                        MMBA_IDX(scan_of_block(J.L, (int64_t)blockIdx.x - G.sblk[job]), J.L.n_scans, J.st), red, tot,
                        dR, chunks, bars);
 }
@@ -533,10 +534,11 @@ cudaError_t launch_voxel_pass_mixed(const DevLayout& L, const DevMixed& X, doubl
 }
 
 cudaError_t launch_scan_pass_mixed(const DevLayout& L, const DevMixed& X, const double* poses2, double* gH,
-                                   DevState* st, int force, cudaStream_t stream) {
+                                   DevState* st, int force, cudaStream_t stream, bool next_early) {
   if (L.n_scans == 0) return cudaSuccess;
   (void)poses2;
-  return launch_dependent(scan_pass_mixed_kernel, L.n_scans, kScanMixedThreads, stream, false, L, X, gH, st, force);
+  return launch_dependent(scan_pass_mixed_kernel, L.n_scans, kScanMixedThreads, stream, false, L, X, gH, st, force,
+                          next_early ? kFreesNext : 0);
 }
 
 cudaError_t launch_batch_voxel_pass_mixed(const JobGroup& T, int64_t n_blocks, int use_trial, cudaStream_t stream,

@@ -52,7 +52,8 @@ __host__ __device__ inline int64_t pred_parts(int64_t n_scans) { return (n_scans
 // comes free, so a grid that does not fill the chip ends up on the few SMs that
 // drained first and shares their FP64 pipes, with the others idle; started
 // after the drain it is spread over all SMs.  So early only
-//   the solve       of at most two blocks an SM,
+//   the solve       of at most 16 scans an SM, two blocks (and the scan pass
+//                   before it spends 0.5 ns a scan on it, see grid_order),
 //   the voxel pass  of at most 5/3 blocks an SM (with 282 blocks the scan pass
 //                   behind it loses, with 250 it does not), and in a batch,
 //                   whose groups run beside each other, where the scan pass
@@ -60,16 +61,18 @@ __host__ __device__ inline int64_t pred_parts(int64_t n_scans) { return (n_scans
 //   the scan pass   where it and the voxel pass before it are just under four
 //                   blocks an SM (both then have room on every SM; with 600
 //                   blocks 52 us instead of 55, with 613 95 instead of 85),
-//                   or with a grid that fills the chip (three resident blocks).
+//                   or with a grid that fills the chip (three resident blocks)
+//                   and is not so large that the wait itself costs more
+//                   (grid_order: 2 us at 4,000 scans).
 // Measured, us an iteration with none / all / these early: 20 scans and 200
 // voxels 45.8 / 40.5 / 40.2; 20 and 5,500 139 / 204 / 137; 20 and 20,000 382 /
 // 923 / 382; 100 and 20,000 142 / 253 / 138; 1,000 and 50,000 474 / 470 / 470;
 // 10,000 and 300,000 1,155 / 1,158 / 1,151.
 constexpr int64_t kSMs = 152;
-inline bool early_solve(int64_t blocks) { return blocks <= 2 * kSMs; }
+inline bool early_solve(int64_t n_scans) { return n_scans <= 16 * kSMs; }
 inline bool early_voxel_pass_f64(int64_t blocks) { return 3 * blocks <= 5 * kSMs; }
 inline bool early_scan_pass_f64(int64_t blocks, int64_t voxel_blocks) {
-  return blocks + voxel_blocks <= 4 * kSMs - 8 || blocks >= 3 * kSMs;
+  return blocks + voxel_blocks <= 4 * kSMs - 8 || (blocks >= 3 * kSMs && blocks <= 28 * kSMs);
 }
 
 // Launch of an iteration kernel; with dependent = true it may start while the
@@ -127,7 +130,8 @@ cudaError_t launch_batch_scan_pass_mixed(const JobGroup& T, int64_t n_blocks, cu
 
 // ---- iteration (FP64) ----
 // dependent = true: an iteration's launch, which may overlap the tail of the
-// kernel before it (launch_dependent).
+// kernel before it (launch_dependent); next_early = true: the launch after it is
+// one.
 // decide_mode: 0 = LM decision in the launch's last block (an iteration's
 // trial pass), 1 = only install the summed cost (evaluation at the current
 // poses), -1 = no decision (planes for output)
@@ -135,7 +139,8 @@ cudaError_t launch_voxel_pass_f64(const DevLayout& L, const double* poses2, doub
                                   double* cost_part, const double* pred_part, DevState* st, int use_trial,
                                   int decide_mode, cudaStream_t stream, bool dependent = false);
 cudaError_t launch_scan_pass_f64(const DevLayout& L, const double* poses2, const double* planes2, double* gH,
-                                 const DevState* st, int force, cudaStream_t stream, bool dependent = false);
+                                 const DevState* st, int force, cudaStream_t stream, bool dependent = false,
+                                 bool next_early = false);
 // sref/stab2 non-null: also write the trial FP32 scan table (mixed precision)
 // voxel-sharded solve: this handle's summed trial cost into *out (device);
 // the LM decision from the total trial cost over all shards
@@ -291,7 +296,7 @@ cudaError_t launch_voxel_pass_mixed(const DevLayout& L, const DevMixed& X, doubl
                                     const double* pred_part, DevState* st, int use_trial, int decide_mode,
                                     cudaStream_t stream, bool dependent = false);
 cudaError_t launch_scan_pass_mixed(const DevLayout& L, const DevMixed& X, const double* poses2, double* gH,
-                                   DevState* st, int force, cudaStream_t stream);
+                                   DevState* st, int force, cudaStream_t stream, bool next_early = false);
 cudaError_t launch_scan_table(int32_t n_scans, const double* poses2, const double* sref, float* stab2, int buf,
                               cudaStream_t stream);
 // Build (or rebuild) the FP32 copies, frames, anchors and reference poses at
