@@ -305,8 +305,9 @@ constexpr int64_t kDependentSolveObs = 2500000;
 ba_status launch_iteration(ba_handle* h) {
   const int64_t nsc = h->L.n_scans;
   const bool solve_early = early_solve(nsc) && (!h->mixed || h->L.n_obs <= kDependentSolveObs);
-  const bool voxel_early = h->mixed || early_voxel_pass_f64(h->n_cost);
-  const bool scan_early = early_scan_pass_f64(nsc, h->n_cost);
+  const int64_t voxel_blocks = voxel_pass_f64_blocks(h->L.n_voxels, h->L.n_obs);
+  const bool voxel_early = h->mixed || early_voxel_pass_f64(voxel_blocks);
+  const bool scan_early = early_scan_pass_f64(nsc, voxel_blocks);
   size_t ev = 0;
   CK(h, prof_begin(h, BA_KERNEL_SOLVE, &ev), "event");
   CK(h, launch_solve_f64(h->L, h->poses2, h->gH, h->pred_part, h->d_state, h->mixed ? h->mb.sref : nullptr,
@@ -414,7 +415,7 @@ ba_status load_impl(ba_handle* h, int32_t n_scans, int64_t n_voxels, int64_t n_o
   float4* t32;
   uint32_t* box;
   MixedBuffers& mb = h->mb;
-  h->n_cost = h->mixed ? voxel_pass_blocks(n_voxels) : voxel_pass_f64_blocks(n_voxels);
+  h->n_cost = h->mixed ? voxel_pass_blocks(n_voxels) : voxel_pass_f64_parts(n_voxels, n_obs);
   {
     ArrayGroup inputs, keep, temp;
     temp.add(&d_val, 1);
@@ -1237,13 +1238,18 @@ ba_status refresh(ba_batch* b) {
   std::vector<JobView> views(n);
   std::vector<int64_t> pre(3 * (n + 1), 0);
   const size_t ng = (n + kGroupJobs - 1) / kGroupJobs;
-  std::vector<int64_t> group_scans(ng, 0);
-  for (size_t k = 0; k < n; ++k) group_scans[k / kGroupJobs] += b->jobs[k]->L.n_scans;
+  std::vector<int64_t> group_scans(ng, 0), group_voxels(ng, 0);
+  for (size_t k = 0; k < n; ++k) {
+    group_scans[k / kGroupJobs] += b->jobs[k]->L.n_scans;
+    group_voxels[k / kGroupJobs] += b->jobs[k]->L.n_voxels;
+  }
   for (size_t k = 0; k < n; ++k) {
     const ba_handle* h = b->jobs[k];
     views[k] = job_view(h);
-    // (a slice of 32 voxels to a block in the FP64 batch, whatever the width alone)
-    pre[k + 1] = pre[k] + (h->mixed ? h->n_cost : (h->L.n_voxels + 31) / 32);
+    // (FP64: a voxel to a thread, or a slice of 32 voxels to a block whatever the width alone)
+    pre[k + 1] = pre[k] + (h->mixed                                               ? h->n_cost
+                           : batch_voxels_whole(group_voxels[k / kGroupJobs]) ? voxel_pass_blocks(h->L.n_voxels)
+                                                                              : (h->L.n_voxels + 31) / 32);
     pre[(n + 1) + k + 1] = pre[(n + 1) + k] + h->L.n_scans;
     pre[2 * (n + 1) + k + 1] = pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans, solve_lanes(group_scans[k / kGroupJobs]));
   }
@@ -1257,6 +1263,7 @@ ba_status refresh(ba_batch* b) {
     const size_t k0 = g * kGroupJobs, k1 = std::min(n, k0 + kGroupJobs);
     G.n_jobs = (int32_t)(k1 - k0);
     G.solve_lanes = solve_lanes(group_scans[g]);
+    G.whole_voxels = batch_voxels_whole(group_voxels[g]);
     int64_t v = 0, sc = 0, o = 0;
     for (size_t k = k0; k < k1; ++k) {
       const int i = (int)(k - k0);

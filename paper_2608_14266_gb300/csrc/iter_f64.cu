@@ -1,6 +1,8 @@
 // FP64 iteration kernels: voxel pass (CalRes), scan pass (CalJH), per-scan
 // damped solve + retraction (Solver) and the device-side LM decision
 // (Algorithm 2 and Sec. IV-C of the paper).
+#include <type_traits>
+
 #include "checked.cuh"
 #include "mmba_internal.cuh"
 #include "mmba_kernels.h"
@@ -32,17 +34,113 @@ namespace mmba {
 // voxel: 118 -> 32 us at 200 voxels, 258 -> 206 us at 50,000, 2.01 -> 1.97 ms
 // at 500,000 (15M observations).
 // ---------------------------------------------------------------------------
-// kTiles > 1: the block takes that many of the tiles of kV voxels one after
-// another, with the same sums, and solves their eigenproblems together (kV
-// kTiles = 32 lanes of the warp at work): what a batch, which fills the GPU,
-// does with the narrow tiles of its small jobs, whose results so have the bits
-// of a job alone (120 FP64 jobs of 1000 to 3000 voxels 1554 us an iteration,
-// with a tile to a block 1905, with a thread per voxel 1652).
+// Two forms with the same sums in the same order, so the same bits.  The split
+// form (voxel_pass_f64_split) is the above.  The whole form
+// (voxel_pass_f64_whole) gives a voxel to one thread, which forms the partial sums
+// of as many threads as the problem's size asks for (voxel_pass_f64_rows) one
+// after another and adds them up in the order of the split form's shuffles.  It
+// does less work a voxel (an anchor instead of four, no idle rows, the
+// eigenproblems of 128 voxels in four full warps) and has fewer warps, so it
+// serves problems of many short voxels and the batches that fill the GPU.
+
+// Posed mean of the voxel's observation at slot e (x by P's first row and so on)
+__device__ __forceinline__ void voxel_anchor(const DevLayout& L, const double* poses, int64_t e, DevState* st,
+                                             double (&a)[3]) {
+  const int64_t ne = L.n_elems;
+  const uint32_t sv = (uint32_t)__ldg(L.ve_scan + e);
+  int p0, p1, p2;
+  perm_decode(sv >> kPermShift, p0, p1, p2);
+  const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
+  const double m0 = __ldg(L.ve + 6 * ne + e), m1 = __ldg(L.ve + 7 * ne + e), m2 = __ldg(L.ve + 8 * ne + e);
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+    a[r] = fma(P[3 * r + p0], m0, fma(P[3 * r + p1], m1, fma(P[3 * r + p2], m2, P[9 + r])));
+}
+
+// The observation at slot e added to the sums n, s, M about the anchor a
+__device__ __forceinline__ void voxel_add(const DevLayout& L, const double* poses, int64_t e, DevState* st,
+                                          const double (&a)[3], double (&acc)[10]) {
+  const int64_t ne = L.n_elems;
+  const uint32_t sv = (uint32_t)__ldg(L.ve_scan + e);
+  int p0, p1, p2;
+  perm_decode(sv >> kPermShift, p0, p1, p2);
+  const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
+  const double l10 = __ldg(L.ve + e), l20 = __ldg(L.ve + ne + e), l21 = __ldg(L.ve + 2 * ne + e);
+  const double D0 = __ldg(L.ve + 3 * ne + e), D1 = __ldg(L.ve + 4 * ne + e), D2 = __ldg(L.ve + 5 * ne + e);
+  const double m0 = __ldg(L.ve + 6 * ne + e), m1 = __ldg(L.ve + 7 * ne + e), m2 = __ldg(L.ve + 8 * ne + e);
+  const double N = __ldg(L.ve + 9 * ne + e);
+  // columns pi0, pi1, pi2 of R
+  const double a0 = P[p0], a1 = P[3 + p0], a2 = P[6 + p0];
+  const double b0 = P[p1], b1 = P[3 + p1], b2 = P[6 + p1];
+  const double c0 = P[p2], c1 = P[3 + p2], c2 = P[6 + p2];
+  const double qx = fma(a0, m0, fma(b0, m1, fma(c0, m2, P[9])));
+  const double qy = fma(a1, m0, fma(b1, m1, fma(c1, m2, P[10])));
+  const double qz = fma(a2, m0, fma(b2, m1, fma(c2, m2, P[11])));
+  const double dx = qx - a[0], dy = qy - a[1], dz = qz - a[2];
+  // R S R^T = sum_a D_a W_a W_a^T with W = R P^T L
+  const double w00 = fma(l10, b0, fma(l20, c0, a0)), w01 = fma(l10, b1, fma(l20, c1, a1)),
+               w02 = fma(l10, b2, fma(l20, c2, a2));
+  const double w10 = fma(l21, c0, b0), w11 = fma(l21, c1, b1), w12 = fma(l21, c2, b2);
+  const double u00 = D0 * w00, u01 = D0 * w01, u02 = D0 * w02;
+  const double u10 = D1 * w10, u11 = D1 * w11, u12 = D1 * w12;
+  const double u20 = D2 * c0, u21 = D2 * c1, u22 = D2 * c2;
+  const double Nx = __dmul_rn(N, dx), Ny = __dmul_rn(N, dy), Nz = __dmul_rn(N, dz);
+  acc[4] = fma(u00, w00, fma(u10, w10, fma(u20, c0, fma(Nx, dx, acc[4]))));
+  acc[5] = fma(u00, w01, fma(u10, w11, fma(u20, c1, fma(Nx, dy, acc[5]))));
+  acc[6] = fma(u00, w02, fma(u10, w12, fma(u20, c2, fma(Nx, dz, acc[6]))));
+  acc[7] = fma(u01, w01, fma(u11, w11, fma(u21, c1, fma(Ny, dy, acc[7]))));
+  acc[8] = fma(u01, w02, fma(u11, w12, fma(u21, c2, fma(Ny, dz, acc[8]))));
+  acc[9] = fma(u02, w02, fma(u12, w12, fma(u22, c2, fma(Nz, dz, acc[9]))));
+  acc[1] = __dadd_rn(acc[1], Nx);
+  acc[2] = __dadd_rn(acc[2], Ny);
+  acc[3] = __dadd_rn(acc[3], Nz);
+  acc[0] = __dadd_rn(acc[0], N);
+}
+
+// The plane of the voxel at sorted position p from its sums and anchor, written
+// out; returns lambda_min.
+template <bool kFull>
+__device__ __forceinline__ double voxel_plane(const DevLayout& L, double* planes, double* full_out, int64_t p,
+                                              const double (&a)[3], const double (&acc)[10]) {
+  const double inv = 1.0 / acc[0];
+  const double cx = __dmul_rn(acc[1], inv), cy = __dmul_rn(acc[2], inv), cz = __dmul_rn(acc[3], inv);  // - anchor
+  double A[6] = {fma(-cx, cx, __dmul_rn(acc[4], inv)), fma(-cx, cy, __dmul_rn(acc[5], inv)),
+                 fma(-cx, cz, __dmul_rn(acc[6], inv)), fma(-cy, cy, __dmul_rn(acc[7], inv)),
+                 fma(-cy, cz, __dmul_rn(acc[8], inv)), fma(-cz, cz, __dmul_rn(acc[9], inv))};
+  double lam[3], V[9];
+  eig3_sym(A, lam, V);
+  const double ux = V[0], uy = V[1], uz = V[2];
+  const double Cx = __dadd_rn(a[0], cx), Cy = __dadd_rn(a[1], cy), Cz = __dadd_rn(a[2], cz);
+  double* pl = planes + p * kPlaneStride;
+  pl[0] = ux;
+  pl[1] = uy;
+  pl[2] = uz;
+  pl[3] = fma(ux, Cx, fma(uy, Cy, __dmul_rn(uz, Cz)));
+  if (kFull) {
+    double* f = full_out + 9 * (int64_t)L.vperm[p];
+    f[0] = lam[0];
+    f[1] = lam[1];
+    f[2] = lam[2];
+    f[3] = ux;
+    f[4] = uy;
+    f[5] = uz;
+    f[6] = Cx;
+    f[7] = Cy;
+    f[8] = Cz;
+  }
+  return lam[0];
+}
+
+// The split form.  kTiles > 1: the block takes that many of the tiles of kV
+// voxels one after another, with the same sums, and solves their eigenproblems
+// together (kV kTiles = 32 lanes of the warp at work): what a batch too small
+// for the whole form does with the narrow tiles of its jobs.
 template <int kV, bool kFull, int kTiles>
-__device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const double* poses2, double* planes2,
-                                                    double* full_out, double* cost_part, const double* pred_part,
-                                                    DevState* st, int use_trial, int decide_mode, int64_t blk, double* red,
-                                                    double (*sums)[10][32], double (*anchor)[32], int* is_last) {
+__device__ __forceinline__ void voxel_pass_f64_split(const DevLayout& L, const double* poses2, double* planes2,
+                                                     double* full_out, double* cost_part, const double* pred_part,
+                                                     DevState* st, int use_trial, int decide_mode, int64_t blk,
+                                                     double* red, double (*sums)[10][32], double (*anchor)[32],
+                                                     int* is_last) {
   static_assert(kVoxelThreads == 128 && (kV == 8 || kV == 16 || kV == 32), "four warps per block");
   static_assert(kTiles == 1 || kTiles * kV == 32, "a slice");
   int64_t p = blk * (kV * kTiles) + (threadIdx.x & (kV - 1));
@@ -63,7 +161,7 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the sums n, s, M of this thread's observations
   double acc[10] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  double ax = 0.0, ay = 0.0, az = 0.0;
+  double a[3] = {0.0, 0.0, 0.0};
 #pragma unroll 1
   for (int tile = 0; tile < kTiles; ++tile) {
     if (kTiles > 1 && tile > 0) {
@@ -74,56 +172,10 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
       for (int q = 0; q < 10; ++q) acc[q] = 0.0;
     }
     if (p < L.n_voxels) {
-      const int64_t ne = L.n_elems;
       const int k0 = threadIdx.x / kV;
-      if (k0 < len || (kTiles == 1 && w == (int)(blk & 3))) {
-        // the anchor: the first observation's posed mean, formed by every thread
-        const uint32_t sv = (uint32_t)__ldg(L.ve_scan + base);
-        int p0, p1, p2;
-        perm_decode(sv >> kPermShift, p0, p1, p2);
-        const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
-        const double m0 = __ldg(L.ve + 6 * ne + base), m1 = __ldg(L.ve + 7 * ne + base), m2 = __ldg(L.ve + 8 * ne + base);
-        ax = fma(P[p0], m0, fma(P[p1], m1, fma(P[p2], m2, P[9])));
-        ay = fma(P[3 + p0], m0, fma(P[3 + p1], m1, fma(P[3 + p2], m2, P[10])));
-        az = fma(P[6 + p0], m0, fma(P[6 + p1], m1, fma(P[6 + p2], m2, P[11])));
-      }
-      for (int k = k0; k < len; k += kRows) {
-        const int64_t e = base + (int64_t)k * kSlice;
-        const uint32_t sv = (uint32_t)__ldg(L.ve_scan + e);
-        int p0, p1, p2;
-        perm_decode(sv >> kPermShift, p0, p1, p2);
-        const double* P = poses + 12 * (int64_t)MMBA_IDX((int32_t)(sv & kScanMask), L.n_scans, st);
-        const double l10 = __ldg(L.ve + e), l20 = __ldg(L.ve + ne + e), l21 = __ldg(L.ve + 2 * ne + e);
-        const double D0 = __ldg(L.ve + 3 * ne + e), D1 = __ldg(L.ve + 4 * ne + e), D2 = __ldg(L.ve + 5 * ne + e);
-        const double m0 = __ldg(L.ve + 6 * ne + e), m1 = __ldg(L.ve + 7 * ne + e), m2 = __ldg(L.ve + 8 * ne + e);
-        const double N = __ldg(L.ve + 9 * ne + e);
-        // columns pi0, pi1, pi2 of R
-        const double a0 = P[p0], a1 = P[3 + p0], a2 = P[6 + p0];
-        const double b0 = P[p1], b1 = P[3 + p1], b2 = P[6 + p1];
-        const double c0 = P[p2], c1 = P[3 + p2], c2 = P[6 + p2];
-        const double qx = fma(a0, m0, fma(b0, m1, fma(c0, m2, P[9])));
-        const double qy = fma(a1, m0, fma(b1, m1, fma(c1, m2, P[10])));
-        const double qz = fma(a2, m0, fma(b2, m1, fma(c2, m2, P[11])));
-        const double dx = qx - ax, dy = qy - ay, dz = qz - az;
-        // R S R^T = sum_a D_a W_a W_a^T with W = R P^T L
-        const double w00 = fma(l10, b0, fma(l20, c0, a0)), w01 = fma(l10, b1, fma(l20, c1, a1)),
-                     w02 = fma(l10, b2, fma(l20, c2, a2));
-        const double w10 = fma(l21, c0, b0), w11 = fma(l21, c1, b1), w12 = fma(l21, c2, b2);
-        const double u00 = D0 * w00, u01 = D0 * w01, u02 = D0 * w02;
-        const double u10 = D1 * w10, u11 = D1 * w11, u12 = D1 * w12;
-        const double u20 = D2 * c0, u21 = D2 * c1, u22 = D2 * c2;
-        const double Nx = N * dx, Ny = N * dy, Nz = N * dz;
-        acc[4] = fma(u00, w00, fma(u10, w10, fma(u20, c0, fma(Nx, dx, acc[4]))));
-        acc[5] = fma(u00, w01, fma(u10, w11, fma(u20, c1, fma(Nx, dy, acc[5]))));
-        acc[6] = fma(u00, w02, fma(u10, w12, fma(u20, c2, fma(Nx, dz, acc[6]))));
-        acc[7] = fma(u01, w01, fma(u11, w11, fma(u21, c1, fma(Ny, dy, acc[7]))));
-        acc[8] = fma(u01, w02, fma(u11, w12, fma(u21, c2, fma(Ny, dz, acc[8]))));
-        acc[9] = fma(u02, w02, fma(u12, w12, fma(u22, c2, fma(Nz, dz, acc[9]))));
-        acc[1] += Nx;
-        acc[2] += Ny;
-        acc[3] += Nz;
-        acc[0] += N;
-      }
+      // the anchor: the first observation's posed mean, formed by every thread
+      if (k0 < len || (kTiles == 1 && w == (int)(blk & 3))) voxel_anchor(L, poses, base, st, a);
+      for (int k = k0; k < len; k += kRows) voxel_add(L, poses, base + (int64_t)k * kSlice, st, a, acc);
     }
     // a voxel's threads of one warp (kV < 32), then of the four warps, in a fixed order
 #pragma unroll
@@ -133,51 +185,23 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
     if (lane < kV)
 #pragma unroll
       for (int q = 0; q < 10; ++q) sums[w][q][tile * kV + lane] = acc[q];
-    if (kTiles > 1 && threadIdx.x < kV) {  // (the first row's threads: they have the anchor)
-      anchor[0][tile * kV + lane] = ax;
-      anchor[1][tile * kV + lane] = ay;
-      anchor[2][tile * kV + lane] = az;
-    }
+    if (kTiles > 1 && threadIdx.x < kV)  // (the first row's threads: they have the anchor)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) anchor[r][tile * kV + lane] = a[r];
   }
   __syncthreads();
   if (w == (int)(blk & 3)) {
     double lam0 = 0.0;
     if (kTiles > 1) {
       p = blk * (kV * kTiles) + lane;
-      ax = anchor[0][lane];
-      ay = anchor[1][lane];
-      az = anchor[2][lane];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) a[r] = anchor[r][lane];
     }
     if (lane < kV * kTiles && p < L.n_voxels) {
 #pragma unroll
       for (int q = 0; q < 10; ++q)
         acc[q] = (sums[0][q][lane] + sums[1][q][lane]) + (sums[2][q][lane] + sums[3][q][lane]);
-      const double inv = 1.0 / acc[0];
-      const double cx = acc[1] * inv, cy = acc[2] * inv, cz = acc[3] * inv;  // centroid - anchor
-      double A[6] = {fma(-cx, cx, acc[4] * inv), fma(-cx, cy, acc[5] * inv), fma(-cx, cz, acc[6] * inv),
-                     fma(-cy, cy, acc[7] * inv), fma(-cy, cz, acc[8] * inv), fma(-cz, cz, acc[9] * inv)};
-      double lam[3], V[9];
-      eig3_sym(A, lam, V);
-      const double ux = V[0], uy = V[1], uz = V[2];
-      const double Cx = ax + cx, Cy = ay + cy, Cz = az + cz;
-      double* pl = planes + p * kPlaneStride;
-      pl[0] = ux;
-      pl[1] = uy;
-      pl[2] = uz;
-      pl[3] = fma(ux, Cx, fma(uy, Cy, uz * Cz));
-      if (kFull) {
-        double* f = full_out + 9 * (int64_t)L.vperm[p];
-        f[0] = lam[0];
-        f[1] = lam[1];
-        f[2] = lam[2];
-        f[3] = ux;
-        f[4] = uy;
-        f[5] = uz;
-        f[6] = Cx;
-        f[7] = Cy;
-        f[8] = Cz;
-      }
-      lam0 = lam[0];
+      lam0 = voxel_plane<kFull>(L, planes, full_out, p, a, acc);
     }
 #pragma unroll
     for (int o = kV / 2; o > 0; o >>= 1) lam0 += __shfl_down_sync(0xffffffffu, lam0, o);
@@ -186,15 +210,86 @@ __device__ __forceinline__ void voxel_pass_f64_body(const DevLayout& L, const do
     for (int tile = 0; tile < kTiles; ++tile) {
       const double c = kTiles == 1 ? lam0 : __shfl_sync(0xffffffffu, lam0, tile * kV);
       const int64_t part = blk * kTiles + tile;
-      if (lane == 0 && (kTiles == 1 || part < voxel_pass_f64_blocks(L.n_voxels))) cost_part[part] = c;
+      if (lane == 0 && (kTiles == 1 || part < voxel_pass_f64_parts(L.n_voxels, L.n_obs))) cost_part[part] = c;
     }
   }
-  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_f64_blocks(L.n_voxels), pred_part, pred_parts(L.n_scans),
-                                   st, decide_mode, red, is_last, (int)(blk & 3) * 32,
-                                   kTiles == 1 ? voxel_pass_f64_blocks(L.n_voxels) : (L.n_voxels + 31) / 32);
+  const int64_t parts = voxel_pass_f64_parts(L.n_voxels, L.n_obs);
+  voxel_pass_decide<kVoxelThreads>(cost_part, parts, pred_part, pred_parts(L.n_scans), st, decide_mode, red, is_last,
+                                   (int)(blk & 3) * 32, kTiles == 1 ? parts : (L.n_voxels + 31) / 32);
 }
 
-// the body for a problem of this size (voxel_pass_f64_width), a tile of its
+// The whole form: the sums of kRows rows (observations row, row + kRows, ..) are
+// formed one after another and added up pairwise, in the order in which the
+// split form's shuffles pair the rows of a warp (0 with 2 and 1 with 3 of four)
+// and then its warps.  The sums that wait for their partner are kept in shared
+// memory, one place for each level of the tree; a row past the warp's longest
+// voxel is empty, and nothing is added for it.
+template <int kRows, int kLevels, bool kFull>
+__device__ __forceinline__ void voxel_pass_f64_whole(const DevLayout& L, const double* poses2, double* planes2,
+                                                     double* full_out, double* cost_part, const double* pred_part,
+                                                     DevState* st, int use_trial, int decide_mode, int64_t blk,
+                                                     double* red, double (*wait)[10][kVoxelThreads], int* is_last) {
+  static_assert(kRows <= 1 << kLevels, "a place for each level");
+  constexpr int kV = kRows == 1 ? 32 : kVoxelThreads / kRows;  // voxels to a partial sum of the cost
+  const int64_t p = blk * kVoxelThreads + threadIdx.x;
+  const int len = p < L.n_voxels ? L.vlen[p] : 0;
+  const int64_t base = p < L.n_voxels ? L.slice_off[p >> 5] + (p & 31) : 0;
+  const int longest = __reduce_max_sync(0xffffffffu, len);
+  grid_wait();
+  grid_launch_next();
+  st = after_wait(st);
+  if (st->honor_stop && st->stop) {
+    if (decide_mode == 0 && blk == 0 && threadIdx.x == 0) st->scan_pending = 0;
+    return;
+  }
+  const int buf = use_trial ? 1 - st->cur : st->cur;
+  const double* poses = after_wait(poses2) + (int64_t)buf * L.n_scans * 12;
+  double* planes = planes2 + (int64_t)buf * L.n_voxels * kPlaneStride;
+  const int lane = threadIdx.x & 31;
+  double acc[10] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  double a[3] = {0.0, 0.0, 0.0};
+  if (len > 0) voxel_anchor(L, poses, base, st, a);
+  unsigned waiting = 0;  // levels whose place holds a sum
+#pragma unroll 1
+  for (int i = 0; i < kRows; ++i) {
+    const int row = kRows == 16 ? (i & 12) | ((i & 1) << 1) | ((i >> 1) & 1) : i;  // of four: 0, 2, 1, 3
+    bool any = row < longest;
+    if (any) {
+#pragma unroll
+      for (int q = 0; q < 10; ++q) acc[q] = 0.0;
+      for (int k = row; k < len; k += kRows) voxel_add(L, poses, base + (int64_t)k * kSlice, st, a, acc);
+    }
+    int level = 0;
+    for (; (i >> level) & 1; ++level) {
+      if (!((waiting >> level) & 1u)) continue;
+#pragma unroll
+      for (int q = 0; q < 10; ++q) {
+        const double other = wait[level][q][threadIdx.x];
+        acc[q] = any ? other + acc[q] : other;
+      }
+      any = true;
+      waiting &= ~(1u << level);
+    }
+    if (any && i < kRows - 1) {
+      waiting |= 1u << level;
+#pragma unroll
+      for (int q = 0; q < 10; ++q) wait[level][q][threadIdx.x] = acc[q];
+    }
+  }
+  double lam0 = p < L.n_voxels ? voxel_plane<kFull>(L, planes, full_out, p, a, acc) : 0.0;
+#pragma unroll
+  for (int o = kV / 2; o > 0; o >>= 1) lam0 += __shfl_down_sync(0xffffffffu, lam0, o);
+  if (lane % kV == 0 && p < L.n_voxels) {
+    cost_part[p / kV] = lam0;
+    __threadfence();
+  }
+  __syncthreads();
+  voxel_pass_decide<kVoxelThreads>(cost_part, voxel_pass_f64_parts(L.n_voxels, L.n_obs), pred_part,
+                                   pred_parts(L.n_scans), st, decide_mode, red, is_last, 0,
+                                   voxel_pass_blocks(L.n_voxels));
+}
+
+// the split form for a problem of this size (voxel_pass_f64_rows), a tile of its
 // width or (kSlices) a slice of 32 voxels to a block
 template <bool kFull, bool kSlices>
 __device__ __forceinline__ void voxel_pass_f64_sized(const DevLayout& L, const double* poses2, double* planes2,
@@ -204,36 +299,68 @@ __device__ __forceinline__ void voxel_pass_f64_sized(const DevLayout& L, const d
   __shared__ double sums[kVoxelThreads / 32][10][32];
   __shared__ double anchor[kSlices ? 3 : 1][32];
   __shared__ int is_last;
-  switch (voxel_pass_f64_width(L.n_voxels)) {
-    case 8:
-      voxel_pass_f64_body<8, kFull, kSlices ? 4 : 1>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial,
-                                                     decide_mode, blk, red, sums, anchor, &is_last);
-      break;
+  switch (voxel_pass_f64_rows(L.n_voxels, L.n_obs)) {
     case 16:
-      voxel_pass_f64_body<16, kFull, kSlices ? 2 : 1>(L, poses2, planes2, full_out, cost_part, pred_part, st,
+      voxel_pass_f64_split<8, kFull, kSlices ? 4 : 1>(L, poses2, planes2, full_out, cost_part, pred_part, st,
                                                       use_trial, decide_mode, blk, red, sums, anchor, &is_last);
       break;
+    case 8:
+      voxel_pass_f64_split<16, kFull, kSlices ? 2 : 1>(L, poses2, planes2, full_out, cost_part, pred_part, st,
+                                                       use_trial, decide_mode, blk, red, sums, anchor, &is_last);
+      break;
     default:
-      voxel_pass_f64_body<32, kFull, 1>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial,
-                                        decide_mode, blk, red, sums, anchor, &is_last);
+      voxel_pass_f64_split<32, kFull, 1>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial,
+                                         decide_mode, blk, red, sums, anchor, &is_last);
   }
 }
 
-template <bool kFull>
+template <bool kFull, bool kWhole>
 __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_kernel(DevLayout L, const double* poses2,
                                                                       double* planes2, double* full_out,
                                                                       double* cost_part, const double* pred_part,
                                                                       DevState* st, int use_trial, int decide_mode) {
-  voxel_pass_f64_sized<kFull, false>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
-                              blockIdx.x);
+  if (kWhole) {  // one row
+    __shared__ double red[kVoxelThreads / 32];
+    __shared__ int is_last;
+    voxel_pass_f64_whole<1, 0, kFull>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
+                                      blockIdx.x, red, nullptr, &is_last);
+  } else {
+    voxel_pass_f64_sized<kFull, false>(L, poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode,
+                                       blockIdx.x);
+  }
 }
 
+template <bool kWhole>
 __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_batch_kernel(const __grid_constant__ JobGroup G,
                                                                              int use_trial) {
   const int job = find_job(G.vblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  voxel_pass_f64_sized<false, true>(J.L, J.poses2, J.planes2, nullptr, J.cost_part, J.pred_part, J.st, use_trial,
-                              use_trial ? 0 : 1, (int64_t)blockIdx.x - G.vblk[job]);
+  const int64_t blk = (int64_t)blockIdx.x - G.vblk[job];
+  if (!kWhole) {
+    voxel_pass_f64_sized<false, true>(J.L, J.poses2, J.planes2, nullptr, J.cost_part, J.pred_part, J.st, use_trial,
+                                      use_trial ? 0 : 1, blk);
+    return;
+  }
+  __shared__ double red[kVoxelThreads / 32];
+  __shared__ double wait[4][10][kVoxelThreads];
+  __shared__ int is_last;
+  auto whole = [&](auto rows) {
+    voxel_pass_f64_whole<decltype(rows)::value, 4, false>(J.L, J.poses2, J.planes2, nullptr, J.cost_part, J.pred_part,
+                                                          J.st, use_trial, use_trial ? 0 : 1, blk, red, wait, &is_last);
+  };
+  switch (voxel_pass_f64_rows(J.L.n_voxels, J.L.n_obs)) {
+    case 16:
+      whole(std::integral_constant<int, 16>());
+      break;
+    case 8:
+      whole(std::integral_constant<int, 8>());
+      break;
+    case 4:
+      whole(std::integral_constant<int, 4>());
+      break;
+    default:
+      whole(std::integral_constant<int, 1>());
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -787,9 +914,11 @@ __global__ void __launch_bounds__(kDecideThreads) shard_decide_kernel(const doub
 cudaError_t launch_voxel_pass_f64(const DevLayout& L, const double* poses2, double* planes2, double* full_out,
                                   double* cost_part, const double* pred_part, DevState* st, int use_trial,
                                   int decide_mode, cudaStream_t stream, bool dependent) {
-  return launch_dependent(full_out ? voxel_pass_f64_kernel<true> : voxel_pass_f64_kernel<false>,
-                          voxel_pass_f64_blocks(L.n_voxels), kVoxelThreads, stream, dependent, L, poses2, planes2,
-                          full_out, cost_part, pred_part, st, use_trial, decide_mode);
+  const bool whole = voxel_pass_f64_rows(L.n_voxels, L.n_obs) == 1;
+  const auto kernel = full_out ? (whole ? voxel_pass_f64_kernel<true, true> : voxel_pass_f64_kernel<true, false>)
+                               : (whole ? voxel_pass_f64_kernel<false, true> : voxel_pass_f64_kernel<false, false>);
+  return launch_dependent(kernel, voxel_pass_f64_blocks(L.n_voxels, L.n_obs), kVoxelThreads, stream, dependent, L,
+                          poses2, planes2, full_out, cost_part, pred_part, st, use_trial, decide_mode);
 }
 
 cudaError_t launch_scan_pass_f64(const DevLayout& L, const double* poses2, const double* planes2, double* gH,
@@ -830,7 +959,8 @@ cudaError_t launch_batch_solve(const JobGroup& T, int64_t n_blocks, cudaStream_t
 }
 
 cudaError_t launch_batch_voxel_pass_f64(const JobGroup& T, int64_t n_blocks, int use_trial, cudaStream_t stream) {
-  return launch_dependent(voxel_pass_f64_batch_kernel, n_blocks, kVoxelThreads, stream,
+  return launch_dependent(T.whole_voxels ? voxel_pass_f64_batch_kernel<true> : voxel_pass_f64_batch_kernel<false>,
+                          n_blocks, kVoxelThreads, stream,
                           early_voxel_pass_f64(n_blocks) || T.sblk[T.n_jobs] >= 3 * kSMs, T, use_trial);
 }
 

@@ -16,22 +16,42 @@ constexpr int kDecideThreads = 256;  // one block; FP64 sums are 1/64 rate, so f
 constexpr int kSolveThreads = 64;  // small blocks spread the scans over every SM
 
 __host__ __device__ inline int64_t voxel_pass_blocks(int64_t n_voxels) { return (n_voxels + kVoxelThreads - 1) / kVoxelThreads; }
-// FP64 voxel pass: voxels per block of kVoxelThreads (a part of a 32-voxel
-// slice; the rest of the block's threads share the voxels' observations).
-// Fewer voxels per block spread a small problem over more of the FP64 pipes;
-// the price is the eigenproblem's warp, which then holds fewer voxels.
-// Measured (us per pass, 8-40 observations per voxel, event-timed; 8 / 16 / 32
-// voxels per block, and one thread per voxel before):
+// FP64 voxel pass: the threads that share a voxel's observations, whose partial
+// sums are added up in a fixed order.  More of them (fewer voxels per block of
+// kVoxelThreads) spread a small problem over more of the FP64 pipes; the price
+// is the eigenproblem's warp, which then holds fewer voxels.  Measured (us per
+// pass, 8-40 observations per voxel, event-timed; 16 / 8 / 4 threads, and one
+// before):
 //     200 voxels   32 /  37 /  47   (118)      9,728   85 /  66 /  64   (121)
 //   2,432          37 /  38 /  49   (121)     19,456  149 / 116 /  97   (129)
 //   4,864          47 /  43 /  49   (120)     50,000  344 / 245 / 206   (258)
-__host__ __device__ inline int voxel_pass_f64_width(int64_t n_voxels) {
-  return n_voxels <= 2432 ? 8 : n_voxels <= 6144 ? 16 : 32;
+// One thread where voxels are many and short, so that most of four would be idle
+// (us, four and one): 300,000 voxels of 1-2 observations 328 / 248, of 3-4 402 /
+// 315, 200,000 of 5-8 328 / 293, 50,000 of 3-4 89 / 70, of 6-8 105 / 94; 100,000 of
+// 10-12 225 / 221.
+constexpr int64_t kShortVoxels = 50000, kShortObs = 10;
+__host__ __device__ inline int voxel_pass_f64_rows(int64_t n_voxels, int64_t n_obs) {
+  if (n_voxels <= 6144) return n_voxels <= 2432 ? 16 : 8;
+  return n_voxels >= kShortVoxels && n_obs <= kShortObs * n_voxels ? 1 : 4;
 }
-__host__ __device__ inline int64_t voxel_pass_f64_blocks(int64_t n_voxels) {
-  const int v = voxel_pass_f64_width(n_voxels);
+// partial sums of the cost: one for every so many voxels
+__host__ __device__ inline int voxel_pass_f64_width(int rows) { return rows == 1 ? 32 : kVoxelThreads / rows; }
+__host__ __device__ inline int64_t voxel_pass_f64_parts(int64_t n_voxels, int64_t n_obs) {
+  const int v = voxel_pass_f64_width(voxel_pass_f64_rows(n_voxels, n_obs));
   return (n_voxels + v - 1) / v;
 }
+// Blocks of a problem's own launch: a part to a block, or, with one thread to a
+// voxel, kVoxelThreads voxels.
+inline int64_t voxel_pass_f64_blocks(int64_t n_voxels, int64_t n_obs) {
+  return voxel_pass_f64_rows(n_voxels, n_obs) == 1 ? voxel_pass_blocks(n_voxels)
+                                                   : voxel_pass_f64_parts(n_voxels, n_obs);
+}
+// Whether a batch's launch over a group of n_voxels in all gives a voxel to one
+// thread (which then forms the partial sums of 4, 8 or 16 in turn): where the
+// group fills the GPU.  Us a pass, a slice of 32 voxels to a block / so: 60 jobs of
+// 2,000 voxels of 2-3 observations 290 / 154, of 20-30 570 / 514; 128 jobs of 500
+// voxels 215 / 178; but 16 jobs of 100 43 / 64.
+inline bool batch_voxels_whole(int64_t n_voxels) { return n_voxels >= 60000; }
 // Lanes per scan in the solve kernel, for a launch of n_scans scans in all (a
 // handle's, or a batch group's): 8 while the GPU has few warps to each of its
 // 608 SM sub-partitions, else 1; the results have the same bits.  Both sides,
