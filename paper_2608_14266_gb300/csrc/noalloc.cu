@@ -25,56 +25,59 @@
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kLanes = 4;                      // threads per voxel
-constexpr int kVoxels = kThreads / kLanes;     // voxels per block
-constexpr int64_t kMaxPairs = BA_NOALLOC_MAX_VOXELS / (2 * kVoxels);  // two blocks add into one partial
-static_assert(BA_NOALLOC_MAX_VOXELS % (2 * kVoxels) == 0, "capacity must be a whole number of partials");
+template <int kLanes>
+constexpr int kThreadsOf = kLanes == 1 ? 128 : 256;  // per block
+constexpr int64_t kMaxPartials = BA_NOALLOC_MAX_VOXELS / 128;  // the cost's partial sums: of 128 voxels or more
+static_assert(BA_NOALLOC_MAX_VOXELS % 128 == 0, "capacity must be a whole number of partials");
 
 // scratch shared by every call on a device: partials, then the error word
-static __device__ __align__(256) double g_noalloc_scratch[kMaxPairs + 32];
+static __device__ __align__(256) double g_noalloc_scratch[kMaxPartials + 32];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 bool g_ready[kMaxDevices];
 double* g_ptr[kMaxDevices];
 
-// Four lanes per voxel over the caller's voxel-major CSR, each every fourth
+// kLanes lanes per voxel over the caller's voxel-major CSR, each every kLanes-th
 // observation: posed cluster means q = R m + t, anchored sums about the
 // voxel's first q, covariance, smallest eigenvalue (the voxel's cost, Eq. 1).
 // Invalid offsets or scan indices set the error word and leave the voxel out.
 //
 // Bound: the FP64 pipe (~70 operations an observation, a warp instruction 64
-// cycles of its scheduler whatever its active lanes).  A block takes its 64
-// voxels in order of their lengths, so that the eight of a warp are about as
-// long, and solves their eigenproblems in two full warps.  40,003 voxels of
-// 2-40 observations: 352 us with one thread per voxel (warps as long as their
-// longest voxel, each scheduler with one warp), now 206 us with the FP64 pipe
-// 85% active.
-__global__ void __launch_bounds__(kThreads) noalloc_cost_kernel(int64_t n_voxels, int64_t n_obs,
+// cycles of its scheduler whatever its active lanes).  A block takes its
+// voxels in order of their lengths, so that those of a warp are about as
+// long, and solves their eigenproblems in full warps.  Four lanes to a voxel:
+// 40,003 voxels of 2-40 observations in 206 us with the FP64 pipe 85% active
+// (352 us with one thread per voxel in input order: warps as long as their
+// longest voxel, each scheduler with one warp).  One lane where voxels are many
+// and short (noalloc_lanes).
+template <int kLanes>
+__global__ void __launch_bounds__(kThreadsOf<kLanes>) noalloc_cost_kernel(int64_t n_voxels, int64_t n_obs,
                                                                 const int64_t* __restrict__ off,
                                                                 const int32_t* __restrict__ obs_scan,
                                                                 const double* __restrict__ agg,
                                                                 const double* __restrict__ poses, int32_t n_scans,
                                                                 double* __restrict__ lam0_out, double* scratch) {
+  constexpr int kThreads = kThreadsOf<kLanes>, kVoxels = kThreads / kLanes;
   __shared__ double sums[10][kVoxels];
   __shared__ int valid[kVoxels];
   __shared__ double red[kVoxels / 32];
   __shared__ int s_cnt[32], s_order[mmba::kOrderBlock];
-  static_assert(mmba::kOrderBlock == kThreads, "the ordering takes one item per thread");
-  unsigned long long* err = reinterpret_cast<unsigned long long*>(scratch + kMaxPairs);
+  static_assert(kThreads <= mmba::kOrderBlock, "the ordering takes one item per thread");
+  unsigned long long* err = reinterpret_cast<unsigned long long*>(scratch + kMaxPartials);
   const int64_t v0 = (int64_t)blockIdx.x * kVoxels;
   {
     // the block's voxels by length; the threads past them come last
     const int64_t i = v0 + threadIdx.x;
     int64_t len = threadIdx.x < kVoxels && i < n_voxels ? off[i + 1] - off[i] : 0;
     len = len < 0 ? 0 : len;
-    mmba::block_order_by_key(threadIdx.x >= kVoxels ? 31 : len < 60 ? (int)(len >> 1) : 30, s_cnt, s_order);
+    const int key = kLanes == 1 ? (int)(len < 31 ? len : 31) : len < 60 ? (int)(len >> 1) : 30;
+    mmba::block_order_by_key(threadIdx.x >= kVoxels ? 31 : key, s_cnt, s_order);
   }
   const int w = threadIdx.x >> 5;
   {
     // ranks dealt to the warps so that each scheduler's two take short and long ones
-    const int wr = w < 4 ? w : 11 - w;
+    const int wr = kLanes == 1 || w < 4 ? w : 11 - w;
     const int vl = s_order[wr * (32 / kLanes) + (threadIdx.x & 31) / kLanes];
     const int sub = threadIdx.x & (kLanes - 1);
     const int64_t i = v0 + vl;
@@ -86,7 +89,7 @@ __global__ void __launch_bounds__(kThreads) noalloc_cost_kernel(int64_t n_voxels
     if (ok) {
       const int32_t j = obs_scan[a];
       ok = j >= 0 && j < n_scans;
-      if (ok) {  // the anchor, formed by every lane
+      if (ok && kLanes > 1) {  // the anchor, formed by every lane
         const double* P = poses + 12 * (int64_t)j;
         const double* c = agg + 10 * a;
         ax = fma(P[0], c[6], fma(P[1], c[7], fma(P[2], c[8], P[9])));
@@ -102,10 +105,15 @@ __global__ void __launch_bounds__(kThreads) noalloc_cost_kernel(int64_t n_voxels
       }
       const double* P = poses + 12 * (int64_t)j;
       const double* c = agg + 10 * o;
-      const double dx = fma(P[0], c[6], fma(P[1], c[7], fma(P[2], c[8], P[9]))) - ax;
-      const double dy = fma(P[3], c[6], fma(P[4], c[7], fma(P[5], c[8], P[10]))) - ay;
-      const double dz = fma(P[6], c[6], fma(P[7], c[7], fma(P[8], c[8], P[11]))) - az;
-      const double N = c[9];
+      const double qx = fma(P[0], c[6], fma(P[1], c[7], fma(P[2], c[8], P[9])));
+      const double qy = fma(P[3], c[6], fma(P[4], c[7], fma(P[5], c[8], P[10])));
+      const double qz = fma(P[6], c[6], fma(P[7], c[7], fma(P[8], c[8], P[11])));
+      if (kLanes == 1 && o == a) {
+        ax = qx;
+        ay = qy;
+        az = qz;
+      }
+      const double dx = qx - ax, dy = qy - ay, dz = qz - az, N = c[9];
       // R S R^T from the packed scatter (xx, xy, xz, yy, yz, zz)
       double RS[3][3];
       const double S[3][3] = {{c[0], c[1], c[2]}, {c[1], c[3], c[4]}, {c[2], c[4], c[5]}};
@@ -135,30 +143,30 @@ __global__ void __launch_bounds__(kThreads) noalloc_cost_kernel(int64_t n_voxels
 #pragma unroll
       for (int q = 0; q < 10; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
     if (sub == 0) {
-      const double inv = 1.0 / acc[0];
-      const double cx = acc[1] * inv, cy = acc[2] * inv, cz = acc[3] * inv;
-      sums[0][vl] = acc[0];
-      sums[1][vl] = fma(-cx, cx, acc[4] * inv);
-      sums[2][vl] = fma(-cx, cy, acc[5] * inv);
-      sums[3][vl] = fma(-cx, cz, acc[6] * inv);
-      sums[4][vl] = fma(-cy, cy, acc[7] * inv);
-      sums[5][vl] = fma(-cy, cz, acc[8] * inv);
-      sums[6][vl] = fma(-cz, cz, acc[9] * inv);
+#pragma unroll
+      for (int q = 0; q < 10; ++q) sums[q][vl] = acc[q];
       const unsigned group = ((1u << kLanes) - 1u) << (threadIdx.x & 31 & ~(kLanes - 1));
       valid[vl] = (bad & group) == 0u;
     }
   }
   __syncthreads();
-  // the eigenproblems: two warps, on other schedulers from block to block
-  const int first = (int)(blockIdx.x & 3) * 2;
-  if (w - first != 0 && w - first != 1) return;
+  // the eigenproblems, a voxel to a thread of kVoxels / 32 warps: with four lanes
+  // two, on other schedulers from block to block
+  constexpr int kEigWarps = kVoxels / 32;
+  const int first = kLanes == 1 ? 0 : (int)(blockIdx.x & 3) * kEigWarps;
+  if (w < first || w >= first + kEigWarps) return;
   const int vl = threadIdx.x - 32 * first;
   const int64_t i = v0 + vl;
   double lam0 = 0.0;
   if (i < n_voxels) {
     const bool ok = valid[vl] != 0;
-    if (ok && sums[0][vl] > 0.0) {
-      const double A[6] = {sums[1][vl], sums[2][vl], sums[3][vl], sums[4][vl], sums[5][vl], sums[6][vl]};
+    const double n = sums[0][vl];
+    if (ok && n > 0.0) {
+      const double inv = 1.0 / n;
+      const double cx = sums[1][vl] * inv, cy = sums[2][vl] * inv, cz = sums[3][vl] * inv;
+      const double A[6] = {fma(-cx, cx, sums[4][vl] * inv), fma(-cx, cy, sums[5][vl] * inv),
+                           fma(-cx, cz, sums[6][vl] * inv), fma(-cy, cy, sums[7][vl] * inv),
+                           fma(-cy, cz, sums[8][vl] * inv), fma(-cz, cz, sums[9][vl] * inv)};
       double lam[3], V[9];
       mmba::eig3_sym(A, lam, V);
       lam0 = lam[0];
@@ -170,15 +178,27 @@ __global__ void __launch_bounds__(kThreads) noalloc_cost_kernel(int64_t n_voxels
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) lam0 += __shfl_down_sync(0xffffffffu, lam0, o);
   if ((threadIdx.x & 31) == 0) red[w - first] = lam0;
-  asm volatile("bar.sync 1, 64;" ::: "memory");  // the two warps
-  // (0 + x) + y rounds as (0 + y) + x, so the order of the two blocks does not matter
-  if (threadIdx.x == 32 * first) atomicAdd(scratch + (blockIdx.x >> 1), red[0] + red[1]);
+  asm volatile("bar.sync 1, %0;" ::"n"(kVoxels) : "memory");  // these warps
+  if (threadIdx.x == 32 * first) {
+    double tot = red[0];
+#pragma unroll
+    for (int q = 1; q < kEigWarps; ++q) tot += red[q];
+    // two blocks of 64 voxels share a partial: (0 + x) + y rounds as (0 + y) + x, so
+    // their order does not matter
+    atomicAdd(scratch + (kLanes == 1 ? blockIdx.x : blockIdx.x >> 1), tot);
+  }
 }
+
+// Lanes per voxel: one where voxels are many and short, so that most of four
+// would be idle.  Us a call with four / one: 30,000 voxels of 1-2 observations 71
+// / 41, of 4-6 96 / 58; 100,000 of 2-3 140 / 104, of 10-14 279 / 248; 300,000 of
+// 4-6 534 / 356; but 5,000 of 5-12 39 / 57, 40,000 of 2-40 200 / 240.
+int noalloc_lanes(int64_t n_voxels, int64_t n_obs) { return n_voxels >= 25000 && n_obs <= 14 * n_voxels ? 1 : 4; }
 
 __global__ void noalloc_reset_kernel(double* scratch, int64_t n_partials) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n_partials) scratch[k] = 0.0;
-  if (k == 0) *reinterpret_cast<unsigned long long*>(scratch + kMaxPairs) = ~0ull;
+  if (k == 0) *reinterpret_cast<unsigned long long*>(scratch + kMaxPartials) = ~0ull;
 }
 
 // Sums the partials in a fixed order; a recorded error makes the cost NaN.
@@ -188,7 +208,7 @@ __global__ void __launch_bounds__(256) noalloc_sum_kernel(int64_t n_partials, co
   for (int64_t k = threadIdx.x; k < n_partials; k += 256) v += scratch[k];
   const double tot = mmba::block_sum<256>(v, red);
   if (threadIdx.x == 0) {
-    const unsigned long long e = *reinterpret_cast<const unsigned long long*>(scratch + kMaxPairs);
+    const unsigned long long e = *reinterpret_cast<const unsigned long long*>(scratch + kMaxPartials);
     *cost_out = e == ~0ull ? tot : __longlong_as_double(0x7ff8000000000000ll);
   }
 }
@@ -219,15 +239,18 @@ extern "C" ba_status ba_eval_cost_noalloc(int32_t n_scans, int64_t n_voxels, int
     scratch = g_ptr[dev];
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int64_t blocks = (n_voxels + kVoxels - 1) / kVoxels;
+  const int lanes = noalloc_lanes(n_voxels, n_obs);
+  const int threads = lanes == 1 ? kThreadsOf<1> : kThreadsOf<4>;
+  const int64_t per = threads / lanes, blocks = (n_voxels + per - 1) / per;
   // an error left pending by earlier, unrelated work on this thread is not
   // this call's to report: clear it, then check each launch on its own
   (void)cudaGetLastError();
-  const int64_t partials = (blocks + 1) / 2;
+  const int64_t partials = lanes == 1 ? blocks : (blocks + 1) / 2;
   noalloc_reset_kernel<<<(unsigned)((partials + 255) / 256), 256, 0, s>>>(scratch, partials);
   if (cudaGetLastError() != cudaSuccess) return BA_ERR_CUDA;
-  noalloc_cost_kernel<<<(unsigned)blocks, kThreads, 0, s>>>(n_voxels, n_obs, voxel_offsets, obs_scan, agg_centred,
-                                                            poses, n_scans, lambda0_out, scratch);
+  const auto kernel = lanes == 1 ? noalloc_cost_kernel<1> : noalloc_cost_kernel<4>;
+  kernel<<<(unsigned)blocks, threads, 0, s>>>(n_voxels, n_obs, voxel_offsets, obs_scan, agg_centred, poses, n_scans,
+                                              lambda0_out, scratch);
   if (cudaGetLastError() != cudaSuccess) return BA_ERR_CUDA;
   noalloc_sum_kernel<<<1, 256, 0, s>>>(partials, scratch, cost_out);
   return cudaGetLastError() == cudaSuccess ? BA_OK : BA_ERR_CUDA;
