@@ -7,10 +7,9 @@
 // level, then by integer index (x, y, z); the observations of a voxel by scan.
 // Indices are exactly floor(RN(w / d)) with w formed by explicit fma, so the
 // integer structure does not depend on the compiler's choices.  GB300 runs
-// FP64 on a narrow pipe: divisions are replaced by a multiply and an exact
-// check, cluster sums are one pass over fixed chunks of sorted points with
-// no divergence between threads, and the planarity test runs in FP32 unless
-// it is too close to call.
+// FP64 on a narrow pipe: indices are formed in fixed point, with FP64 near voxel
+// faces only, the sums of a cluster's points are exact integer sums, and the
+// planarity test runs in FP32 unless it is too close to call.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -378,12 +377,14 @@ __global__ void head_mask_kernel(int64_t n, const K* keys, const uint32_t* vals,
 }
 
 // group starts from the mask and the words' exclusive head counts, and the
-// end sentinel
+// end sentinel; n_zero words (at most the grid's threads) set to zero for a
+// kernel to come
 __global__ void mask_starts_kernel(int64_t n_words, const uint32_t* mask, const int64_t* base, int64_t n,
-                                   int64_t* start, int64_t n_groups) {
+                                   int64_t* start, int64_t n_groups, uint32_t* zero, int64_t n_zero) {
   grid_wait();
   grid_launch_next();
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (w < n_zero) zero[w] = 0;
   if (w >= n_words) return;
   uint32_t m = mask[w];
   int64_t b = base[w];
@@ -403,7 +404,6 @@ struct Piece {
   double n, s[3], a[3], b[6];
 };
 
-// centred cluster record (S xx..zz, m, N)
 // A cluster's row (80 bytes, 16-byte aligned in every buffer of the library) as
 // five 128-bit accesses: where each thread has a row of its own, half the
 // requests to L1 that single values make.
@@ -422,6 +422,7 @@ __device__ __forceinline__ void store_row(const double* r, double* c) {
   for (int q = 0; q < 5; ++q) p[q] = make_double2(r[2 * q], r[2 * q + 1]);
 }
 
+// centred cluster record (S xx..zz, m, N)
 __device__ __forceinline__ void piece_finish(const Piece& P, double* c) {
   const double r = __drcp_rn(P.n);
   const double u[3] = {P.a[0] * r, P.a[1] * r, P.a[2] * r};
@@ -447,34 +448,56 @@ __device__ __forceinline__ void piece_finish(const Piece& P, double* c) {
 //
 // One thread per run of fewer than kLongRun points, a block's runs in order of
 // their lengths so that a warp's lanes are about as long, each lane with its
-// next point on the way; longer runs by a whole warp each.  The block's two
-// warps take the groups of 32 runs longest first, as they get free (one warp
-// per group leaves the warps of short runs idle until the longest is done).
+// next point on the way.  The block's two warps take the groups of 32 runs
+// longest first, as they get free (one warp per group leaves the warps of short
+// runs idle until the longest is done).  Longer runs go to a list, in pieces of
+// kPiecePoints, which a second kernel hands to warps over the whole chip.
 //
 // Bound: latency of the gathers (a run's points lie together, its neighbours'
-// elsewhere) against four warps a scheduler, instruction issue 45% active.
-// Measured on 120M points in 12.3M runs, before (FP64 sums over fixed chunks
-// of 32 sorted points, pieces of 104 bytes written and merged per run; the
-// FP64 pipe 69% active): 3.12 + 0.91 ms, now 2.88 ms.  Runs ordered in pools of
-// 256, 512 and 1,024 cost their neighbours' lines in L1 and L2: 2.97, 3.6, 3.7
-// ms.  65,000 points in 7,400 runs: 54 -> 30 us.
+// elsewhere) against four warps a scheduler.  120M points in 12.3M runs: FP64 sums
+// over fixed chunks of 32 sorted points, merged per run, 3.12 + 0.91 ms; so 2.88
+// ms.  (Runs ordered in pools of 256, 512 and 1,024 cost their neighbours' lines in
+// L1 and L2: 2.97, 3.6, 3.7 ms.)  65,000 points in 7,400 runs: 54 -> 30 us.  Few long
+// runs: 30 of 33,000 points 1.97 ms in chunks (3.77 with whole runs to the warps of
+// the block that met them), so 0.04.
 constexpr int kLongRun = 192;  // below kHalfPoints
 static_assert(kLongRun <= kHalfPoints, "a thread's sums must fit");
+constexpr int kPiecePoints = 1024;  // of a long run, to a warp
+static_assert(kPiecePoints <= 32 * kHalfPoints, "a warp's sums must fit");
+
+// A piece of a long run; the sums of one of several go to place slot + piece.
+struct __align__(16) WarpItem {
+  uint32_t run, piece, n_pieces, slot;
+};
+// What is left to l1_rest_kernel of a call over n points: the list of pieces, the
+// places for their sums (10 each), and the counters (pieces listed, places taken,
+// then the finished pieces of each slot).
+struct RestRuns {
+  WarpItem* list;
+  double* sums;
+  uint32_t* counters;
+};
+int64_t rest_items(int64_t n) { return n / kPiecePoints + n / kLongRun; }
+int64_t rest_places(int64_t n) { return 2 * (n / kPiecePoints); }  // of runs of two pieces and more
+int64_t rest_counters(int64_t n) { return 2 + rest_places(n); }
 
 // bin of a run's length for the block's ordering; 31 = long
 __device__ __forceinline__ int run_bin(int64_t len) {
-  return len <= 8 ? (int)len : len <= 24 ? 4 + (int)(len >> 1) : len < 96 ? 13 + (int)(len >> 3) : len < kLongRun ? 25 + (int)((len - 96) >> 5) : 31;
+  if (len <= 24) return len <= 8 ? (int)len : 4 + (int)(len >> 1);
+  return len < 96 ? 13 + (int)(len >> 3) : len < kLongRun ? 25 + (int)((len - 96) >> 5) : 31;
 }
 
 // Fixed-point frame of a run: per axis the scale (steps of 2^-F) and the first
 // point in steps.  A step is half the last bit of the first point's coordinate,
 // so that a run's coordinates are whole steps, but no finer than 2^-f_cap, about
-// 2^-53 of the voxel's diagonal: where the coordinate itself is smaller than the
-// voxel, rounding to it is what FP64 loses of an offset of the voxel's size.
+// 2^-53 of the voxel's diagonal (capped): where the coordinate itself is smaller
+// than the voxel, rounding to it is what FP64 loses of an offset of the voxel's
+// size.
 struct RunFrame {
   int F[3];
   long long X[3];
   bool fits;
+  bool capped[3];
 };
 __device__ __forceinline__ RunFrame run_frame(double x, double y, double z, int f_cap) {
   const double p[3] = {x, y, z};
@@ -482,7 +505,9 @@ __device__ __forceinline__ RunFrame run_frame(double x, double y, double z, int 
   f.fits = true;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    f.F[a] = min(1076 - ((__double2hiint(p[a]) >> 20) & 0x7ff), f_cap);
+    const int F = 1076 - ((__double2hiint(p[a]) >> 20) & 0x7ff);
+    f.capped[a] = F > f_cap;
+    f.F[a] = min(F, f_cap);
     f.fits = f.fits && f.F[a] >= -400 && f.F[a] <= 400;
     f.X[a] = fix_round(p[a], f.F[a], f.fits);
   }
@@ -506,22 +531,35 @@ __device__ __forceinline__ void run_record(const RunFrame& f, const __int128* t,
   c[9] = n;
 }
 
-// the sums of every stride-th point from sorted position e on, in FP64 (a = sum d, b = sum d d^T)
+// the sums of every stride-th point from sorted position e on, in FP64 (a = sum d,
+// b = sum d d^T), four points on their way at a time
 __device__ __noinline__ void run_sums_f64(int64_t e, int64_t end, int stride, const uint32_t* vals, const double* pts,
                                           double p0x, double p0y, double p0z, double* t) {
+  constexpr int kAhead = 4;
   for (int q = 0; q < 9; ++q) t[q] = 0.0;
-  for (; e < end; e += stride) {
-    const double* p = pts + 3 * (int64_t)vals[e];
-    const double x = p[0] - p0x, y = p[1] - p0y, z = p[2] - p0z;
-    t[0] = fma(x, x, t[0]);
-    t[1] = fma(x, y, t[1]);
-    t[2] = fma(x, z, t[2]);
-    t[3] = fma(y, y, t[3]);
-    t[4] = fma(y, z, t[4]);
-    t[5] = fma(z, z, t[5]);
-    t[6] += x;
-    t[7] += y;
-    t[8] += z;
+  for (; e < end; e += (int64_t)kAhead * stride) {
+    double p[kAhead][3];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      const int64_t at = e + (int64_t)k * stride;
+      const double* v = pts + 3 * (int64_t)vals[at < end ? at : e];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) p[k][q] = v[q];
+    }
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      if (e + (int64_t)k * stride >= end) break;
+      const double x = p[k][0] - p0x, y = p[k][1] - p0y, z = p[k][2] - p0z;
+      t[0] = fma(x, x, t[0]);
+      t[1] = fma(x, y, t[1]);
+      t[2] = fma(x, z, t[2]);
+      t[3] = fma(y, y, t[3]);
+      t[4] = fma(y, z, t[4]);
+      t[5] = fma(z, z, t[5]);
+      t[6] += x;
+      t[7] += y;
+      t[8] += z;
+    }
   }
 }
 
@@ -571,43 +609,143 @@ __device__ __forceinline__ void run_totals(const HalfSums& h, __int128* t) {
     t[k] = join_halves(h.v[3 * k], h.v[3 * k + 1], k == 0 || k == 3 || k == 5 ? 28 : 27, h.v[3 * k + 2]);
 }
 
-// a run of kLongRun points and more, by a warp
-__device__ __noinline__ void cluster_long(int64_t g, int lane, const int64_t* start, const uint32_t* vals,
-                                          const double* pts, double* c, int f_cap) {
-  const int64_t a = start[g], b = start[g + 1];
-  const uint32_t v0 = vals[a];
-  const double p0x = pts[3 * (int64_t)v0], p0y = pts[3 * (int64_t)v0 + 1], p0z = pts[3 * (int64_t)v0 + 2];
+// Sorted positions [a, b) of a run that starts at a0, by a warp, in FP64: the run's
+// record (kWhole: they are all of it), or n, sum d and sum d d^T of the offsets
+// from the run's first point, in every lane.
+template <bool kWhole>
+__device__ __noinline__ void cluster_f64(int64_t a0, int64_t a, int64_t b, int lane, const uint32_t* vals,
+                                         const double* pts, double* out) {
+  const double* p0 = pts + 3 * (int64_t)vals[a0];
+  const double x = p0[0], y = p0[1], z = p0[2], n = (double)(b - a);
+  double v[9];
+  run_sums_f64(a + lane, b, 32, vals, pts, x, y, z, v);
+#pragma unroll
+  for (int q = 0; q < 9; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+  if (kWhole) {
+    run_record_f64(v, n, x, y, z, out);
+    return;
+  }
+  out[0] = n;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) out[1 + q] = v[6 + q];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) out[4 + q] = v[q];
+}
+
+// At most kPiecePoints of them in exact integer sums, or FP64 where they do not
+// fit: the run's record (kWhole: they are all of it), or n, sum d and sum d d^T
+// of the offsets from the run's first point, in every lane.
+template <bool kWhole>
+__device__ __forceinline__ void cluster_piece(int64_t a0, int64_t a, int64_t b, int lane,
+                                              const uint32_t* __restrict__ vals, const double* __restrict__ pts,
+                                              int f_cap, double* out) {
+  const double* p0 = pts + 3 * (int64_t)vals[a0];
+  const double p0x = p0[0], p0y = p0[1], p0z = p0[2];
   const RunFrame f = run_frame(p0x, p0y, p0z, f_cap);
-  bool ok = f.fits;
-  __int128 t[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (int64_t e = a; ok && e < b; e += 32 * kHalfPoints) {
-    const int64_t left = (b - e - lane + 31) / 32;  // points of this lane from here on: every 32nd
-    const int cnt = left <= 0 ? 0 : (int)(left < kHalfPoints ? left : kHalfPoints);
+  const int n = (int)(b - a);
+  const int cnt = n > lane ? (n - lane + 31) / 32 : 0;  // points of this lane: every 32nd
+  __int128 t[9];
+  bool ok;
+  {
     HalfSums h;
     h.clear();
-    const bool mine = run_sums(h, f, e + lane, cnt, 32, vals, pts);
-    ok = __all_sync(0xffffffffu, mine);
-    __int128 u[6];
-    run_totals(h, u);
+    const bool mine = run_sums(h, f, a + lane, cnt, 32, vals, pts);
+    ok = __all_sync(0xffffffffu, f.fits && mine);
+    run_totals(h, t);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) t[q] += u[q];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) t[6 + q] += h.v[18 + q];
+    for (int q = 0; q < 3; ++q) t[6 + q] = h.v[18 + q];
   }
-  const double n = (double)(b - a);
-  if (ok) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q)
+  for (int q = 0; q < 9; ++q)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t[q] += shfl_xor_i128(0xffffffffu, t[q], o);
-    const double s[3] = {i128_scaled(t[6], -f.F[0]), i128_scaled(t[7], -f.F[1]), i128_scaled(t[8], -f.F[2])};
-    if (lane == 0) run_record(f, t, s, n, 1.0 / n, c + 10 * g);
+    for (int o = 16; o > 0; o >>= 1) t[q] += shfl_xor_i128(0xffffffffu, t[q], o);
+  const double nd = (double)n;
+  double v[9];  // sum d d^T, sum d
+  if (ok) {  // the same in every lane
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[6 + q] = i128_scaled(t[6 + q], -f.F[q]);
+    if (kWhole) {
+      const double sd[3] = {v[6], v[7], v[8]};
+      run_record(f, t, sd, nd, 1.0 / nd, out);
+      return;
+    }
+    int k = 0;
+#pragma unroll
+    for (int x = 0; x < 3; ++x)
+#pragma unroll
+      for (int y = x; y < 3; ++y, ++k) v[k] = i128_scaled(t[k], -(f.F[x] + f.F[y]));
+    if (f.capped[0] || f.capped[1] || f.capped[2]) {
+      // from the first point in whole steps to the point itself, e apart
+      const double e[3] = {i64_scaled(f.X[0], -f.F[0]) - p0x, i64_scaled(f.X[1], -f.F[1]) - p0y,
+                           i64_scaled(f.X[2], -f.F[2]) - p0z};
+      k = 0;
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int y = x; y < 3; ++y, ++k) v[k] += fma(e[x], fma(nd, e[y], v[6 + y]), e[y] * v[6 + x]);
+#pragma unroll
+      for (int x = 0; x < 3; ++x) v[6 + x] = fma(nd, e[x], v[6 + x]);
+    }
   } else {
-    double t64[9];
-    run_sums_f64(a + lane, b, 32, vals, pts, p0x, p0y, p0z, t64);
-    for (int q = 0; q < 9; ++q)
-      for (int o = 16; o > 0; o >>= 1) t64[q] += __shfl_xor_sync(0xffffffffu, t64[q], o);
-    if (lane == 0) run_record_f64(t64, n, p0x, p0y, p0z, c + 10 * g);
+    cluster_f64<kWhole>(a0, a, b, lane, vals, pts, out);
+    return;
+  }
+  out[0] = nd;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) out[1 + q] = v[6 + q];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) out[4 + q] = v[q];
+}
+
+// The listed pieces of the long runs, a warp to a piece; the warp that finishes a
+// run's last piece adds up the pieces' sums, each lane every 32nd of them.
+constexpr int kLongThreads = 128;
+__global__ void __launch_bounds__(kLongThreads, 4) l1_rest_kernel(const int64_t* start, const uint32_t* vals,
+                                                                  const double* pts, RestRuns R, int f_cap, double* c) {
+  grid_wait();
+  grid_launch_next();
+  const int lane = threadIdx.x & 31;
+  const uint32_t n_list = R.counters[0];
+  const uint32_t warp = blockIdx.x * (kLongThreads / 32) + (threadIdx.x >> 5), warps = gridDim.x * (kLongThreads / 32);
+  for (uint32_t i = warp; i < n_list; i += warps) {
+    const WarpItem L = R.list[i];
+    const int64_t a0 = start[L.run], a = a0 + (int64_t)L.piece * kPiecePoints, end = start[L.run + 1];
+    double rec[10];
+    if (L.n_pieces == 1) {
+      cluster_piece<true>(a0, a0, end, lane, vals, pts, f_cap, rec);
+      if (lane == 0) store_row(rec, c + 10 * (int64_t)L.run);
+      continue;
+    }
+    cluster_piece<false>(a0, a, a + kPiecePoints < end ? a + kPiecePoints : end, lane, vals, pts, f_cap, rec);
+    double* sums = R.sums + 10 * (int64_t)L.slot;
+    unsigned done = 0;
+    if (lane == 0) {
+      store_row(rec, sums + 10 * (int64_t)L.piece);
+      __threadfence();
+      done = atomicAdd(&R.counters[2 + L.slot], 1u);
+    }
+    if (__shfl_sync(0xffffffffu, done, 0) != L.n_pieces - 1) continue;
+    __threadfence();
+    double v[10] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (uint32_t k = lane; k < L.n_pieces; k += 32) {
+      const double2* row = reinterpret_cast<const double2*>(sums + 10 * (int64_t)k);
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        const double2 w = __ldcg(row + q);
+        v[2 * q] += w.x;
+        v[2 * q + 1] += w.y;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 10; ++q)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    const double* p0 = pts + 3 * (int64_t)vals[a0];
+    const Piece P{v[0], {p0[0], p0[1], p0[2]}, {v[1], v[2], v[3]}, {v[4], v[5], v[6], v[7], v[8], v[9]}};
+    piece_finish(P, rec);
+    if (lane == 0) store_row(rec, c + 10 * (int64_t)L.run);
   }
 }
 
@@ -621,9 +759,12 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
                                                                      const int32_t* __restrict__ pscan,
                                                                      const double* __restrict__ pts,
                                                                      const uint64_t* __restrict__ raw, int f_cap,
-                                                                     double* c, uint64_t* ckey, int32_t* cscan) {
+                                                                     RestRuns R, double* c, uint64_t* ckey,
+                                                                     int32_t* cscan) {
   grid_launch_next();
   __shared__ int s_cnt[32], s_next;
+  __shared__ uint32_t s_listed, s_placed, s_base[2];  // pieces and places of the block's long runs
+  __shared__ WarpItem s_long[kPool];
   __shared__ uint16_t s_order[kPool];
   __shared__ int64_t s_start[kPool];
   __shared__ int s_len[kPool];
@@ -657,19 +798,41 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
         cscan[r0 + i] = pscan[v0[k]];
       }
     }
-    if (threadIdx.x == 0) s_next = 0;
+    if (threadIdx.x == 0) {
+      s_next = 0;
+      s_listed = s_placed = 0;
+    }
     block_order_items<kPer, kClusterThreads>(bin, s_cnt, s_order);
+    // the long runs' pieces to the list: places in the block, then the block's
+    const int n_long = kPool - s_cnt[31];  // the last ranks
+    if (n_long > 0) {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k)
+        if (bin[k] == 31) {
+          const uint32_t np = (uint32_t)((e[k] - a[k] + kPiecePoints - 1) / kPiecePoints);
+          const uint32_t at = atomicAdd(&s_listed, np);
+          const uint32_t slot = np > 1 ? atomicAdd(&s_placed, np) : 0u;
+          s_long[k * kClusterThreads + threadIdx.x] = WarpItem{(uint32_t)(r0 + k * kClusterThreads + threadIdx.x), at,
+                                                                np, slot};
+        }
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        s_base[0] = atomicAdd(&R.counters[0], s_listed);
+        s_base[1] = s_placed > 0 ? atomicAdd(&R.counters[1], s_placed) : 0u;
+      }
+      __syncthreads();
+      for (int q = 0; q < n_long; ++q) {
+        const WarpItem L = s_long[s_order[kPool - 1 - q]];
+        for (uint32_t k = threadIdx.x; k < L.n_pieces; k += kClusterThreads)
+          R.list[s_base[0] + L.piece + k] = WarpItem{L.run, k, L.n_pieces, s_base[1] + L.slot};
+      }
+    }
   }
-  const int n_long = kPool - s_cnt[31];
   for (;;) {
-    // the next item: the long runs, then the groups of 32, longest first
+    // the groups of 32, longest first
     int item = lane == 0 ? atomicAdd(&s_next, 1) : 0;
     item = __shfl_sync(0xffffffffu, item, 0);
-    if (item < n_long) {
-      cluster_long(r0 + s_order[kPool - 1 - item], lane, start, vals, pts, c, f_cap);
-      continue;
-    }
-    const int group = kPool / 32 - 1 - (item - n_long);
+    const int group = kPool / 32 - 1 - item;
     if (group < 0) break;
     const int i = s_order[group * 32 + lane];
     const int64_t g = r0 + i, a = s_start[i];
@@ -677,10 +840,10 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
     if (len > 0 && len < kLongRun) {
       const uint32_t v0 = s_first[i];
       const double p0x = pts[3 * (int64_t)v0], p0y = pts[3 * (int64_t)v0 + 1], p0z = pts[3 * (int64_t)v0 + 2];
+      double* rec = c + 10 * g;
       const RunFrame f = run_frame(p0x, p0y, p0z, f_cap);
       HalfSums h;
       h.clear();
-      double* rec = c + 10 * g;
       if (f.fits && run_sums(h, f, a + 1, len - 1, 1, vals, pts)) {  // p0's own offset is zero
         __int128 t[6];
         run_totals(h, t);
@@ -1161,10 +1324,12 @@ cudaError_t sort_keys(uint64_t** k, uint32_t** v, uint64_t** tk, uint32_t** tv, 
   return radix_sort_pairs64(k, v, tk, tv, n, bits, positions, scr, st, launches);
 }
 
-// groups of a sorted (key, scan) sequence: start (n_groups + 1 entries)
+// groups of a sorted (key, scan) sequence: start (n_groups + 1 entries); n_zero
+// words (at most n / 512 + 256) are set to zero on the way
 template <typename K>
 ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int32_t* scan, Buf& tmp,
-                       int64_t** start_out, int64_t* n_groups, cudaStream_t st, int64_t* launches) {
+                       int64_t** start_out, int64_t* n_groups, cudaStream_t st, int64_t* launches,
+                       uint32_t* zero = nullptr, int64_t n_zero = 0) {
   const int64_t nw = (n + 31) / 32;
   uint32_t* mask = tmp.get<uint32_t>(nw);
   int64_t* base = tmp.get<int64_t>(nw + 1);
@@ -1180,7 +1345,8 @@ ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int
   VCK(cudaStreamSynchronize(st), "voxelize");
   int64_t* start = tmp.get<int64_t>(ng + 1);
   if (!start) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  launch_chained(mask_starts_kernel, blocks_for(nw), 256, 0, st, nw, mask, base, n, start, ng);
+  launch_chained(mask_starts_kernel, blocks_for(nw), 256, 0, st, nw, mask, base, n, start, ng, zero,
+                 n_zero);
   VCK(cudaGetLastError(), "voxelize");
   *launches += 2;
   *start_out = start;
@@ -1214,7 +1380,8 @@ struct Level {
 // (the clusters go to out, the rest to tmp; raw_keys: clusters keep raw keys)
 template <typename K>
 ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const double* pts, Level& L,
-                 bool raw_keys, int f_cap, Buf& out, Buf& tmp, StageTimer& tm, cudaStream_t st, int64_t* launches) {
+                 bool raw_keys, int f_cap, int n_sm, Buf& out, Buf& tmp, StageTimer& tm, cudaStream_t st,
+                 int64_t* launches) {
   K* keys = tmp.get<K>(n);
   K* tkeys = tmp.get<K>(n);
   uint32_t* vals = tmp.get<uint32_t>(n);
@@ -1231,7 +1398,15 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   int64_t* start = nullptr;
   int64_t n1 = 0;
   tm.begin(BA_VOX_RUNS);
-  ba_status s = group_starts<K>(n, keys, vals, pscan, tmp, &start, &n1, st, launches);
+  RestRuns R{};
+  {
+    char* b = tmp.get<char>(16 * rest_items(n) + 80 * rest_places(n) + 4 * rest_counters(n));
+    if (!b) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
+    R.list = (WarpItem*)b;
+    R.sums = (double*)(R.list + rest_items(n));
+    R.counters = (uint32_t*)(R.sums + 10 * rest_places(n));
+  }
+  ba_status s = group_starts<K>(n, keys, vals, pscan, tmp, &start, &n1, st, launches, R.counters, rest_counters(n));
   tm.end();
   if (s != BA_OK) return s;
   L.nc = n1;
@@ -1242,7 +1417,7 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   tm.begin(BA_VOX_CLUSTER_PASS);
   auto clusters = [&](auto pool) {
     l1_clusters_kernel<K, decltype(pool)::value><<<blocks_for(n1, decltype(pool)::value), kClusterThreads, 0, st>>>(
-        n1, start, keys, vals, pscan, pts, raw_keys ? raw : nullptr, f_cap, L.c, L.key, L.scan);
+        n1, start, keys, vals, pscan, pts, raw_keys ? raw : nullptr, f_cap, R, L.c, L.key, L.scan);
   };
   if (n1 > kPoolRuns)
     clusters(std::integral_constant<int, 128>());
@@ -1251,6 +1426,15 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   tm.end();
   ++*launches;
   VCK(cudaGetLastError(), "voxelize clusters");
+  if (n - (n1 - 1) >= kLongRun) {  // else no run is as long
+    tm.begin(BA_VOX_CLUSTER_FINISH);
+    const int64_t warps = rest_items(n);
+    launch_chained(l1_rest_kernel, (unsigned)std::min<int64_t>(blocks_for(warps, kLongThreads / 32), 4 * n_sm),
+                   kLongThreads, 0, st, start, vals, pts, R, f_cap, L.c);
+    tm.end();
+    ++*launches;
+    VCK(cudaGetLastError(), "voxelize clusters");
+  }
   return BA_OK;
 }
 
@@ -1341,10 +1525,10 @@ ba_status l1_range(const L1Ctx& c, int64_t p0, int64_t m, const double* pts, boo
   // finest fixed-point step of the cluster sums: the diagonal, 2^e (e from ilogb,
   // so diagonal < 2^(e + 1)), in fewer than 2^54 steps
   const int f_cap = 52 - std::ilogb(1.7320508075688772 * c.d);
-  return pack_bits(L.pk) <= 32 ? level1<uint32_t>(m, raw, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
-                                                  c.launches)
-                               : level1<uint64_t>(m, raw, pscan, pts, L, raw_keys, f_cap, out, tmp, *c.tm, c.st,
-                                                  c.launches);
+  return pack_bits(L.pk) <= 32 ? level1<uint32_t>(m, raw, pscan, pts, L, raw_keys, f_cap, c.n_sm, out, tmp, *c.tm,
+                                                  c.st, c.launches)
+                               : level1<uint64_t>(m, raw, pscan, pts, L, raw_keys, f_cap, c.n_sm, out, tmp, *c.tm,
+                                                  c.st, c.launches);
 }
 
 ba_status l1_single(const L1Ctx& c, int64_t n, const double* pts, Level& L, int* bb, Buf& tmp) {
