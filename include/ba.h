@@ -479,9 +479,9 @@ ba_status ba_aggregate_points(int64_t n_obs, const int64_t* point_offsets, const
  * rounded quotient; the points of one scan in one voxel form one centred
  * cluster (Eq. 2) from the points' deviations from the run's first point, as
  * exact fixed-point sums (a run outside their range: shifted sums in FP64; runs
- * of more than 1,024 points: the sums of pieces added in FP64); results are
- * deterministic and agree with the mean-then-scatter definition to rounding.
- * Bottom-up levels
+ * of more than 1,024 points: the sums of pieces added in FP64), which lose no
+ * more than FP64 sums of the deviations do; results are deterministic and agree
+ * with the mean-then-scatter definition to rounding.  Bottom-up levels
  * (Eq. 5): the level-k index of a level-(k-1) cluster is floor(index / 2)
  * per axis, and the clusters with the same (level-k index, scan) are merged
  * in scan-then-child order; level k has voxel size 2^(k-1) d.
@@ -519,8 +519,9 @@ typedef struct {
 /* Stages timed when profile is set (ba_voxels_stage_ms): world points and
  * level-1 keys; the level-1 sort (with the key packing); the (voxel, scan)
  * runs of the sorted points (includes one host synchronisation); the
- * clusters' sums; those of the long runs; all higher levels (includes host
- * synchronisations); the selection's per-observation terms and per-voxel test; the output writes; the ordering of
+ * clusters' sums; those of the long runs and of the runs of close points; all
+ * higher levels (includes host synchronisations); the selection's
+ * per-observation terms and per-voxel test; the output writes; the ordering of
  * the batches' level-1 clusters (batched calls only). */
 enum {
   BA_VOX_KEYS = 0,

@@ -442,44 +442,50 @@ __device__ __forceinline__ void piece_finish(const Piece& P, double* c) {
 // L1 clusters: the points of each (key, scan) run of the sorted order, as sums
 // of their offsets from the run's first point p0, m = p0 + (sum d) / N and
 // S = sum d d^T - (sum d)(sum d)^T / N.  The sums are exact integer sums in
-// fixed point (RunFrame, fixed_sums.cuh); a run whose points do not fit (the
-// poses stretch it over 2^54 steps, or coordinates outside 2^-400 .. 2^400)
-// takes the same sums in FP64.
+// fixed point (RunFrame, fixed_sums.cuh), in finer steps where the points lie so
+// close together that the frame's are not small against them (run_exact,
+// cluster_tight); a run whose points do not fit (the poses stretch it over 2^54
+// steps, or coordinates outside 2^-400 .. 2^400) takes the same sums in FP64.
 //
 // One thread per run of fewer than kLongRun points, a block's runs in order of
 // their lengths so that a warp's lanes are about as long, each lane with its
 // next point on the way.  The block's two warps take the groups of 32 runs
 // longest first, as they get free (one warp per group leaves the warps of short
-// runs idle until the longest is done).  Longer runs go to a list, in pieces of
-// kPiecePoints, which a second kernel hands to warps over the whole chip.
+// runs idle until the longest is done).  Longer runs, in pieces of kPiecePoints,
+// and those of close points go to lists that a second kernel hands to warps over
+// the whole chip.
 //
 // Bound: latency of the gathers (a run's points lie together, its neighbours'
 // elsewhere) against four warps a scheduler.  120M points in 12.3M runs: FP64 sums
-// over fixed chunks of 32 sorted points, merged per run, 3.12 + 0.91 ms; so 2.88
-// ms.  (Runs ordered in pools of 256, 512 and 1,024 cost their neighbours' lines in
-// L1 and L2: 2.97, 3.6, 3.7 ms.)  65,000 points in 7,400 runs: 54 -> 30 us.  Few long
-// runs: 30 of 33,000 points 1.97 ms in chunks (3.77 with whole runs to the warps of
-// the block that met them), so 0.04.
+// over fixed chunks of 32 sorted points, merged per run, 3.12 + 0.91 ms; so 2.91 ms
+// and 0.17 ms for the second kernel.  (Runs ordered in pools of 256, 512 and 1,024
+// cost their neighbours' lines in L1 and L2: 2.97, 3.6, 3.7 ms.)  65,000 points in
+// 7,400 runs: 54 -> 31 + 11 us.  Few long runs: 30 of 33,000 points 1.97 ms in
+// chunks (3.77 with whole runs to the warps of the block that met them), so 0.04.
 constexpr int kLongRun = 192;  // below kHalfPoints
 static_assert(kLongRun <= kHalfPoints, "a thread's sums must fit");
 constexpr int kPiecePoints = 1024;  // of a long run, to a warp
 static_assert(kPiecePoints <= 32 * kHalfPoints, "a warp's sums must fit");
+constexpr int kWarpRun = 64;  // a run of close points takes a warp from so many on
 
-// A piece of a long run; the sums of one of several go to place slot + piece.
+// A warp's share: a piece of a long run (the sums of one of several go to place
+// slot + piece), or, with n_pieces = 0, a run of close points.
 struct __align__(16) WarpItem {
   uint32_t run, piece, n_pieces, slot;
 };
-// What is left to l1_rest_kernel of a call over n points: the list of pieces, the
-// places for their sums (10 each), and the counters (pieces listed, places taken,
-// then the finished pieces of each slot).
+// What is left to l1_rest_kernel of a call over n points: the list of warps'
+// shares, the places for pieces' sums (10 each), the shorter runs of close points,
+// and the counters (shares listed, places taken, those runs, then the finished
+// pieces of each slot).
 struct RestRuns {
   WarpItem* list;
   double* sums;
+  uint32_t* tight;
   uint32_t* counters;
 };
-int64_t rest_items(int64_t n) { return n / kPiecePoints + n / kLongRun; }
+int64_t rest_items(int64_t n) { return n / kPiecePoints + n / kWarpRun; }
 int64_t rest_places(int64_t n) { return 2 * (n / kPiecePoints); }  // of runs of two pieces and more
-int64_t rest_counters(int64_t n) { return 2 + rest_places(n); }
+int64_t rest_counters(int64_t n) { return 3 + rest_places(n); }
 
 // bin of a run's length for the block's ordering; 31 = long
 __device__ __forceinline__ int run_bin(int64_t len) {
@@ -489,10 +495,11 @@ __device__ __forceinline__ int run_bin(int64_t len) {
 
 // Fixed-point frame of a run: per axis the scale (steps of 2^-F) and the first
 // point in steps.  A step is half the last bit of the first point's coordinate,
-// so that a run's coordinates are whole steps, but no finer than 2^-f_cap, about
-// 2^-53 of the voxel's diagonal (capped): where the coordinate itself is smaller
-// than the voxel, rounding to it is what FP64 loses of an offset of the voxel's
-// size.
+// which loses no more of an offset than FP64 does (a smaller coordinate is off
+// by a quarter of that bit at most, and FP64's difference, at least half the
+// first coordinate, by half).  It is no finer than 2^-f_cap, about 2^-53 of the
+// voxel's diagonal, so that the offsets have room; an axis cut off so (capped)
+// rounds its points by up to half a step, which run_exact weighs.
 struct RunFrame {
   int F[3];
   long long X[3];
@@ -512,6 +519,21 @@ __device__ __forceinline__ RunFrame run_frame(double x, double y, double z, int 
     f.X[a] = fix_round(p[a], f.F[a], f.fits);
   }
   return f;
+}
+
+// Whether the rounding of n points to the steps of a capped axis stays within
+// what FP64 sums of the offsets over chunks of 32 points can lose.  With k =
+// min(n, 32) + n / 32 additions on the way of a term and u = 2^-53, those lose up
+// to (3 k + 5) u sum d^2 of an entry (k + 2 in sum d^2, 2 k in (sum d)^2 / n, and
+// the last operations); half a step a point, in both sums, loses up to 2 sum |d|
+// steps.  As (sum |d|)^2 <= n sum d^2, that is less where sum d^2 >= 4 n 2^106 /
+// (3 k + 5)^2 (in steps): points a few percent of the voxel apart, or more.
+// xx, yy, zz: sum d^2.
+__device__ __forceinline__ bool run_exact(const RunFrame& f, __int128 xx, __int128 yy, __int128 zz, int n) {
+  const float k = (float)(3 * (n < 32 ? n : 32 + n / 32) + 5);
+  const float least = 0x1p48f * ((float)n / (k * k));  // in units of 2^60
+  auto enough = [&](bool capped, __int128 v) { return !capped || (float)(long long)(v >> 60) >= least; };
+  return enough(f.capped[0], xx) && enough(f.capped[1], yy) && enough(f.capped[2], zz);
 }
 
 // record from the exact sums: t = sum d d^T, s = sum d as FP64, n points, rn = 1 / n
@@ -663,7 +685,7 @@ __device__ __forceinline__ void cluster_piece(int64_t a0, int64_t a, int64_t b, 
     for (int o = 16; o > 0; o >>= 1) t[q] += shfl_xor_i128(0xffffffffu, t[q], o);
   const double nd = (double)n;
   double v[9];  // sum d d^T, sum d
-  if (ok) {  // the same in every lane
+  if (ok && run_exact(f, t[0], t[3], t[5], n)) {  // the same in every lane
 #pragma unroll
     for (int q = 0; q < 3; ++q) v[6 + q] = i128_scaled(t[6 + q], -f.F[q]);
     if (kWhole) {
@@ -699,20 +721,116 @@ __device__ __forceinline__ void cluster_piece(int64_t a0, int64_t a, int64_t b, 
   for (int q = 0; q < 6; ++q) out[4 + q] = v[q];
 }
 
-// The listed pieces of the long runs, a warp to a piece; the warp that finishes a
-// run's last piece adds up the pieces' sums, each lane every 32nd of them.
+// A run [a, b) of fewer than kLongRun points that lie too close together for the
+// steps of its frame (or that do not fit it), by kLanes lanes (sub: this one's
+// number), in two passes: the largest offset of each capped axis, then exact
+// integer sums in steps of 2^-53 of that offset or finer, which lose nothing that
+// FP64 keeps (run_exact: sum d^2 is then 2^104 and more).  FP64 sums where the
+// points do not fit.  The record in every lane; every lane of the warp calls it.
+template <int kLanes>
+__device__ __forceinline__ void cluster_tight(int64_t a, int64_t b, int sub, const uint32_t* __restrict__ vals,
+                                              const double* __restrict__ pts, int f_cap, double* rec) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const double* first = pts + 3 * (int64_t)vals[a];
+  const double p0[3] = {first[0], first[1], first[2]};
+  RunFrame f = run_frame(p0[0], p0[1], p0[2], f_cap);
+  unsigned long long reach[3] = {0, 0, 0};
+  int emax = -2048;
+  unsigned wide = 0;
+  for (int64_t e = a + 1 + sub; e < b; e += kLanes) {
+    const double* p = pts + 3 * (int64_t)vals[e];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const long long d = fix_offset(p[q], 1075 - f.F[q], f.X[q], emax, wide);
+      reach[q] |= (unsigned long long)(d < 0 ? -d : d);
+    }
+  }
+  __syncwarp();
+  bool ok = f.fits && emax <= 9 && (wide >> 22) == 0u;
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) reach[q] |= __shfl_xor_sync(kAll, reach[q], o);
+    ok = __shfl_xor_sync(kAll, (int)ok, o) != 0 && ok;
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const int finer = f.capped[q] ? 53 - (64 - __clzll((long long)reach[q])) : 0;
+    f.F[q] = min(1076 - ((__double2hiint(p0[q]) >> 20) & 0x7ff), f.F[q] + max(finer, 0));
+    if (!f.capped[q]) f.F[q] = min(f.F[q], f_cap);
+    ok = ok && f.F[q] <= 400;
+    f.X[q] = fix_round(p0[q], f.F[q], ok);
+  }
+  HalfSums h;
+  h.clear();
+  const int n = (int)(b - a), cnt = n - 1 > sub ? (n - 1 - sub + kLanes - 1) / kLanes : 0;
+  ok = run_sums(h, f, a + 1 + sub, cnt, kLanes, vals, pts) && ok;
+  __syncwarp();
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+#pragma unroll
+    for (int q = 0; q < 21; ++q) h.v[q] += __shfl_xor_sync(kAll, h.v[q], o);
+    ok = __shfl_xor_sync(kAll, (int)ok, o) != 0 && ok;
+  }
+  if (ok) {
+    __int128 t[6];
+    run_totals(h, t);
+    const double sd[3] = {i64_scaled(h.v[18], -f.F[0]), i64_scaled(h.v[19], -f.F[1]), i64_scaled(h.v[20], -f.F[2])};
+    const float nf = (float)n;
+    const double nd = f32_to_f64(nf);
+    run_record(f, t, sd, nd, recip_count(nd, nf), rec);
+  }
+  if (__all_sync(kAll, ok)) return;
+  // (a warp's lanes share the points; fewer lanes, whose number the call decides,
+  // sum them all, so that it changes no result)
+  double t[9];
+  constexpr int kShare = kLanes == 32 ? 32 : 1;
+  run_sums_f64(a + 1 + (kShare == 32 ? sub : 0), b, kShare, vals, pts, p0[0], p0[1], p0[2], t);
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 9; ++q)
+#pragma unroll
+    for (int o = 1; o < kShare; o <<= 1) t[q] += __shfl_xor_sync(kAll, t[q], o);
+  if (!ok) run_record_f64(t, (double)n, p0[0], p0[1], p0[2], rec);
+}
+
+// The runs that l1_clusters_kernel leaves: the pieces of the long ones, a warp to
+// a piece (the warp that finishes a run's last piece adds up the pieces' sums,
+// each lane every 32nd of them), and the runs of close points (done there, with
+// FP64 sums, a few lanes held up their warps: 120M points 12.02 ms a call, so
+// 11.69): a lane to each where they fill the grid, else four, which gets the few
+// of a small call done sooner (8 scans of 8,192 points 11 us instead of 19).
 constexpr int kLongThreads = 128;
 __global__ void __launch_bounds__(kLongThreads, 4) l1_rest_kernel(const int64_t* start, const uint32_t* vals,
                                                                   const double* pts, RestRuns R, int f_cap, double* c) {
   grid_wait();
   grid_launch_next();
   const int lane = threadIdx.x & 31;
-  const uint32_t n_list = R.counters[0];
+  const uint32_t n_list = R.counters[0], n_tight = R.counters[2];
   const uint32_t warp = blockIdx.x * (kLongThreads / 32) + (threadIdx.x >> 5), warps = gridDim.x * (kLongThreads / 32);
+  auto tight = [&](auto run_lanes) {
+    constexpr int kLanes = decltype(run_lanes)::value, kRuns = 32 / kLanes;  // of a warp
+    for (int64_t i0 = (int64_t)warp * kRuns; i0 < n_tight; i0 += (int64_t)warps * kRuns) {
+      const int64_t i = i0 + lane / kLanes;
+      const int64_t g = R.tight[i < n_tight ? i : i0];
+      double rec[10];
+      cluster_tight<kLanes>(start[g], start[g + 1], lane % kLanes, vals, pts, f_cap, rec);
+      if (i < n_tight && lane % kLanes == 0) store_row(rec, c + 10 * g);
+    }
+  };
+  if (n_tight >= 32 * warps)
+    tight(std::integral_constant<int, 1>());
+  else
+    tight(std::integral_constant<int, 4>());
   for (uint32_t i = warp; i < n_list; i += warps) {
     const WarpItem L = R.list[i];
     const int64_t a0 = start[L.run], a = a0 + (int64_t)L.piece * kPiecePoints, end = start[L.run + 1];
     double rec[10];
+    if (L.n_pieces == 0) {
+      cluster_tight<32>(a0, end, lane, vals, pts, f_cap, rec);
+      if (lane == 0) store_row(rec, c + 10 * (int64_t)L.run);
+      continue;
+    }
     if (L.n_pieces == 1) {
       cluster_piece<true>(a0, a0, end, lane, vals, pts, f_cap, rec);
       if (lane == 0) store_row(rec, c + 10 * (int64_t)L.run);
@@ -724,7 +842,7 @@ __global__ void __launch_bounds__(kLongThreads, 4) l1_rest_kernel(const int64_t*
     if (lane == 0) {
       store_row(rec, sums + 10 * (int64_t)L.piece);
       __threadfence();
-      done = atomicAdd(&R.counters[2 + L.slot], 1u);
+      done = atomicAdd(&R.counters[3 + L.slot], 1u);
     }
     if (__shfl_sync(0xffffffffu, done, 0) != L.n_pieces - 1) continue;
     __threadfence();
@@ -762,7 +880,8 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
                                                                      RestRuns R, double* c, uint64_t* ckey,
                                                                      int32_t* cscan) {
   grid_launch_next();
-  __shared__ int s_cnt[32], s_next;
+  __shared__ int s_cnt[32], s_next, s_n_tight, s_n_warp;
+  __shared__ uint16_t s_tight[kPool];  // runs of close points: the short ones from the front
   __shared__ uint32_t s_listed, s_placed, s_base[2];  // pieces and places of the block's long runs
   __shared__ WarpItem s_long[kPool];
   __shared__ uint16_t s_order[kPool];
@@ -799,7 +918,7 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
       }
     }
     if (threadIdx.x == 0) {
-      s_next = 0;
+      s_next = s_n_tight = s_n_warp = 0;
       s_listed = s_placed = 0;
     }
     block_order_items<kPer, kClusterThreads>(bin, s_cnt, s_order);
@@ -841,24 +960,41 @@ __global__ void __launch_bounds__(kClusterThreads, 8) l1_clusters_kernel(int64_t
       const uint32_t v0 = s_first[i];
       const double p0x = pts[3 * (int64_t)v0], p0y = pts[3 * (int64_t)v0 + 1], p0z = pts[3 * (int64_t)v0 + 2];
       double* rec = c + 10 * g;
+      if (len == 1) {
+        const double one[10] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, p0x, p0y, p0z, 1.0};
+        store_row(one, rec);
+        continue;
+      }
       const RunFrame f = run_frame(p0x, p0y, p0z, f_cap);
       HalfSums h;
       h.clear();
-      if (f.fits && run_sums(h, f, a + 1, len - 1, 1, vals, pts)) {  // p0's own offset is zero
-        __int128 t[6];
-        run_totals(h, t);
+      bool ok = f.fits && run_sums(h, f, a + 1, len - 1, 1, vals, pts);  // p0's own offset is zero
+      __int128 t[6];
+      run_totals(h, t);
+      ok = ok && run_exact(f, t[0], t[3], t[5], len);
+      if (ok) {
         const double s[3] = {i64_scaled(h.v[18], -f.F[0]), i64_scaled(h.v[19], -f.F[1]),
                              i64_scaled(h.v[20], -f.F[2])};
         const float nf = (float)len;
         const double n = f32_to_f64(nf);
         run_record(f, t, s, n, recip_count(n, nf), rec);
+      } else if (len < kWarpRun) {
+        s_tight[atomicAdd(&s_n_tight, 1)] = (uint16_t)i;
       } else {
-        double t[9];
-        run_sums_f64(a + 1, a + len, 1, vals, pts, p0x, p0y, p0z, t);
-        run_record_f64(t, (double)len, p0x, p0y, p0z, rec);
+        s_tight[kPool - 1 - atomicAdd(&s_n_warp, 1)] = (uint16_t)i;
       }
     }
   }
+  __syncthreads();
+  if (s_n_tight + s_n_warp == 0) return;
+  if (threadIdx.x == 0) {
+    if (s_n_tight > 0) s_base[0] = atomicAdd(&R.counters[2], (uint32_t)s_n_tight);
+    if (s_n_warp > 0) s_base[1] = atomicAdd(&R.counters[0], (uint32_t)s_n_warp);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < s_n_tight; k += kClusterThreads) R.tight[s_base[0] + k] = (uint32_t)(r0 + s_tight[k]);
+  for (int k = threadIdx.x; k < s_n_warp; k += kClusterThreads)
+    R.list[s_base[1] + k] = WarpItem{(uint32_t)(r0 + s_tight[kPool - 1 - k]), 0, 0, 0};
 }
 
 // Eq. 5: parent key of every cluster (level packing pc -> pp); sort keys
@@ -1413,7 +1549,8 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   L.c = out.get<double>(10 * n1);
   L.key = out.get<uint64_t>(n1);
   L.scan = out.get<int32_t>(n1);
-  if (!L.c || !L.key || !L.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
+  R.tight = tmp.get<uint32_t>(n1);
+  if (!L.c || !L.key || !L.scan || !R.tight) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   tm.begin(BA_VOX_CLUSTER_PASS);
   auto clusters = [&](auto pool) {
     l1_clusters_kernel<K, decltype(pool)::value><<<blocks_for(n1, decltype(pool)::value), kClusterThreads, 0, st>>>(
@@ -1426,9 +1563,9 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   tm.end();
   ++*launches;
   VCK(cudaGetLastError(), "voxelize clusters");
-  if (n - (n1 - 1) >= kLongRun) {  // else no run is as long
+  if (n1 < n) {  // else every point is a run of its own
     tm.begin(BA_VOX_CLUSTER_FINISH);
-    const int64_t warps = rest_items(n);
+    const int64_t warps = std::max<int64_t>(rest_items(n), n1 / 8);
     launch_chained(l1_rest_kernel, (unsigned)std::min<int64_t>(blocks_for(warps, kLongThreads / 32), 4 * n_sm),
                    kLongThreads, 0, st, start, vals, pts, R, f_cap, L.c);
     tm.end();
