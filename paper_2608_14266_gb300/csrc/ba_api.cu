@@ -1238,18 +1238,20 @@ ba_status refresh(ba_batch* b) {
   std::vector<JobView> views(n);
   std::vector<int64_t> pre(3 * (n + 1), 0);
   const size_t ng = (n + kGroupJobs - 1) / kGroupJobs;
-  std::vector<int64_t> group_scans(ng, 0), group_voxels(ng, 0);
+  std::vector<int64_t> group_scans(ng, 0);
+  int64_t all_voxels = 0;
   for (size_t k = 0; k < n; ++k) {
     group_scans[k / kGroupJobs] += b->jobs[k]->L.n_scans;
-    group_voxels[k / kGroupJobs] += b->jobs[k]->L.n_voxels;
+    all_voxels += b->jobs[k]->L.n_voxels;
   }
+  const bool whole = batch_voxels_whole(all_voxels);
   for (size_t k = 0; k < n; ++k) {
     const ba_handle* h = b->jobs[k];
     views[k] = job_view(h);
     // (FP64: a voxel to a thread, or a slice of 32 voxels to a block whatever the width alone)
-    pre[k + 1] = pre[k] + (h->mixed                                               ? h->n_cost
-                           : batch_voxels_whole(group_voxels[k / kGroupJobs]) ? voxel_pass_blocks(h->L.n_voxels)
-                                                                              : (h->L.n_voxels + 31) / 32);
+    pre[k + 1] = pre[k] + (h->mixed ? h->n_cost
+                           : whole  ? voxel_pass_blocks(h->L.n_voxels)
+                                    : (h->L.n_voxels + 31) / 32);
     pre[(n + 1) + k + 1] = pre[(n + 1) + k] + h->L.n_scans;
     pre[2 * (n + 1) + k + 1] = pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans, solve_lanes(group_scans[k / kGroupJobs]));
   }
@@ -1263,7 +1265,7 @@ ba_status refresh(ba_batch* b) {
     const size_t k0 = g * kGroupJobs, k1 = std::min(n, k0 + kGroupJobs);
     G.n_jobs = (int32_t)(k1 - k0);
     G.solve_lanes = solve_lanes(group_scans[g]);
-    G.whole_voxels = batch_voxels_whole(group_voxels[g]);
+    G.whole_voxels = whole;
     int64_t v = 0, sc = 0, o = 0;
     for (size_t k = k0; k < k1; ++k) {
       const int i = (int)(k - k0);

@@ -378,21 +378,22 @@ __global__ void __launch_bounds__(kVoxelThreads) voxel_pass_f64_batch_kernel(con
 // the (w m'^T + m' w^T)/2 - (w^T m') I term.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void scan_pass_f64_body(const DevLayout& L, const double* poses2, const double* planes2,
-                                                   double* gH, const DevState* st, int force, int order, int j,
+                                                   double* gH, const DevState* st, int force, int order, int64_t blk,
                                                    double (*red)[32]) {
+  int j = 0;
   int64_t lo = 0, hi = 0;
-  if (order & kWaits) {  // (not before the test below in a launch that does not wait)
+  auto range = [&] {
+    j = MMBA_IDX(scan_of_block(L, blk), L.n_scans, st);
     lo = L.scan_off[j];
     hi = L.scan_off[j + 1];
-  }
+  };
+  // (before the test below only in a launch that waits: 40,000 rejected scans 42.6 us, after it 28.6)
+  if (order & kWaits) range();
   grid_order(order);
   st = after_wait(st);
   // a rejected step (or an iteration after the solve stopped) leaves g, H unchanged
   if (!force && !st->scan_pending) return;
-  if (!(order & kWaits)) {
-    lo = L.scan_off[j];
-    hi = L.scan_off[j + 1];
-  }
+  if (!(order & kWaits)) range();
   const int buf = st->cur;
   const double* P = after_wait(poses2) + ((int64_t)buf * L.n_scans + j) * 12;
   const double* planes = after_wait(planes2) + (int64_t)buf * L.n_voxels * kPlaneStride;
@@ -540,8 +541,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_kernel(DevLayout L
                                                                     const double* planes2, double* gH,
                                                                     const DevState* st, int force, int order) {
   __shared__ double red[kScanThreads / 32][32];
-  scan_pass_f64_body(L, poses2, planes2, gH, st, force, order,
-                     MMBA_IDX(scan_of_block(L, blockIdx.x), L.n_scans, st), red);
+  scan_pass_f64_body(L, poses2, planes2, gH, st, force, order, blockIdx.x, red);
 }
 
 __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const __grid_constant__ JobGroup G,
@@ -549,8 +549,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_pass_f64_batch_kernel(const
   __shared__ double red[kScanThreads / 32][32];
   const int job = find_job(G.sblk, G.n_jobs, blockIdx.x);
   const JobView& J = G.jobs[job];
-  scan_pass_f64_body(J.L, J.poses2, J.planes2, J.gH, J.st, 0, order,
-                     MMBA_IDX(scan_of_block(J.L, (int64_t)blockIdx.x - G.sblk[job]), J.L.n_scans, J.st), red);
+  scan_pass_f64_body(J.L, J.poses2, J.planes2, J.gH, J.st, 0, order, (int64_t)blockIdx.x - G.sblk[job], red);
 }
 
 // ---------------------------------------------------------------------------

@@ -253,7 +253,7 @@ struct JobGroup {
   int32_t oblk[kGroupJobs + 1];  // prefix of solve blocks
   int32_t n_jobs;
   int32_t solve_lanes;  // lanes per scan in the solve (1 or 8, by the group's scans)
-  int32_t whole_voxels;  // FP64 voxel pass: a voxel to a thread (by the group's voxels)
+  int32_t whole_voxels;  // FP64 voxel pass: a voxel to a thread (by the batch's voxels)
 };
 static_assert(sizeof(JobGroup) <= 32000, "a job group must fit the kernel parameter space");
 

@@ -46,9 +46,9 @@ inline int64_t voxel_pass_f64_blocks(int64_t n_voxels, int64_t n_obs) {
   return voxel_pass_f64_rows(n_voxels, n_obs) == 1 ? voxel_pass_blocks(n_voxels)
                                                    : voxel_pass_f64_parts(n_voxels, n_obs);
 }
-// Whether a batch's launch over a group of n_voxels in all gives a voxel to one
-// thread (which then forms the partial sums of 4, 8 or 16 in turn): where the
-// group fills the GPU.  Us a pass, a slice of 32 voxels to a block / so: 60 jobs of
+// Whether a batch of n_voxels in all (its groups run beside each other) gives a
+// voxel to one thread, which then forms the partial sums of 4, 8 or 16 in turn:
+// where it fills the GPU.  Us a pass, a slice of 32 voxels to a block / so: 60 jobs of
 // 2,000 voxels of 2-3 observations 290 / 154, of 20-30 570 / 514; 128 jobs of 500
 // voxels 215 / 178; but 16 jobs of 100 43 / 64.
 inline bool batch_voxels_whole(int64_t n_voxels) { return n_voxels >= 60000; }
