@@ -580,6 +580,22 @@ ba_status ba_check_bounded_wait(int32_t device, int32_t polls);
  * BA_ERR_CUDA. */
 ba_status ba_check_conversions(int32_t device, int64_t n, uint64_t seed, uint64_t* mismatches);
 
+/* Checks of two reciprocals that stand in for divisions (the paper has no
+ * counterpart): n pseudo-random values (seeded) on `device`; worst[0] receives
+ * the largest |1 - d y| of the solve's reciprocals y of pivots d, worst[1] that
+ * of the point clusters' of whole numbers up to 2^24, in units of 2^-53, which a
+ * correctly rounded quotient stays within.  Errors: BA_ERR_INVALID_ARG,
+ * BA_ERR_CUDA. */
+ba_status ba_check_reciprocals(int32_t device, int64_t n, uint64_t seed, double* worst);
+
+/* Check of the library's radix sort: n pseudo-random keys (seeded) of `bits`
+ * bits, half of them on a few values, sorted on `device` with their positions.
+ * With wait = 0 its tiles do not wait for the counts of the tiles before them but
+ * count those keys themselves, as they do when the bounded wait runs out.
+ * mismatches receives the number of pairs that a stable sort would not have left
+ * so (0 expected).  Errors: BA_ERR_INVALID_ARG, BA_ERR_CUDA. */
+ba_status ba_check_sort(int32_t device, int64_t n, int32_t bits, int32_t wait, uint64_t seed, uint64_t* mismatches);
+
 /* Allocation-free cost evaluation.  The paper has no counterpart: this entry
  * point exists for callers that cannot allocate device memory when they need
  * a cost -- a mapping loop on a vehicle under a fixed memory budget, where

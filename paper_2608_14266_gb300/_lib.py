@@ -115,6 +115,8 @@ _SIGNATURES = {
     "ba_check_bounded_wait": (_I32, [_I32, _I32]),
     "ba_release_cached_memory": (_I32, [_I32]),
     "ba_check_conversions": (_I32, [_I32, _I64, ctypes.c_uint64, _P]),
+    "ba_check_reciprocals": (_I32, [_I32, _I64, ctypes.c_uint64, _P]),
+    "ba_check_sort": (_I32, [_I32, _I64, _I32, _I32, ctypes.c_uint64, _P]),
     "ba_batch_autotune": (_I32, [_P, _I32, _I32, _P]),
     "ba_batch_set_launch": (_I32, [_P, _I32, _I32]),
     "ba_voxelize_config_default": (None, [_P]),

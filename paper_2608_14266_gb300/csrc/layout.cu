@@ -167,7 +167,8 @@ cudaError_t exclusive_scan_i64(int64_t* data, int64_t n, int64_t* scratch, cudaS
 // NVIDIA technical report NVR-2016-002).  Tiles are numbered in the order the
 // blocks start, so a tile waits only for tiles whose blocks are running and
 // publish before they wait; a wait that lasts kLookLimit polls all the same
-// ends with the tile counting the keys before it itself.
+// ends with the tile counting the keys before it itself (ba_check_sort has it do
+// so at once).
 //
 // Bound at large sizes: instruction issue (57% active) and the look-back's
 // waits.  Against a histogram kernel and a prefix sum of one to three kernels
@@ -183,7 +184,7 @@ constexpr int kRadixWarps = kRadixBlock / 32;
 constexpr int kRadixPasses = 8;      // digits of a 64-bit key
 constexpr int kLookLimit = 1 << 20;  // polls of one word
 constexpr int kLookAhead = 4;        // words of a look-back in flight
-constexpr int kCountBlocks = 4 * 152;
+constexpr int64_t kCountBlocks = 4 * kSMs;
 
 // a tile's word for one digit: the pass it belongs to, whether it is the
 // running total (tiles up to this one) or the tile's own count, and the value
@@ -257,7 +258,7 @@ struct RadixShared {
   uint32_t wsum[2][kRadixWarps];
 };
 
-template <typename K, bool kFull>
+template <typename K, bool kFull, bool kWait>
 __device__ __forceinline__ void radix_tile(const K* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
                                            K* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int64_t n,
                                            int64_t tile, int pass, uint32_t total, uint64_t* look, K* skey,
@@ -327,7 +328,7 @@ __device__ __forceinline__ void radix_tile(const K* __restrict__ keys_in, const 
 #pragma unroll
     for (int k = 0; k < kLookAhead; ++k) {
       if (done || gave_up || t - k < 0) continue;
-      for (int it = 0; (uint32_t)(v[k] >> 32) < (uint32_t)(2 * pass + 2) && it < kLookLimit; ++it)
+      for (int it = 0; (uint32_t)(v[k] >> 32) < (uint32_t)(2 * pass + 2) && it < (kWait ? kLookLimit : 0); ++it)
         v[k] = look_load(look + 256 * (t - k) + tid);
       const uint32_t tag = (uint32_t)(v[k] >> 32);
       gave_up = tag < (uint32_t)(2 * pass + 2);
@@ -359,7 +360,7 @@ __device__ __forceinline__ void radix_tile(const K* __restrict__ keys_in, const 
 }
 
 // kBlocks: resident blocks per SM that the registers are held to
-template <typename K, int kBlocks>
+template <typename K, int kBlocks, bool kWait>
 __global__ void __launch_bounds__(kRadixBlock, kBlocks)
     radix_scatter_kernel(const K* keys_in, const uint32_t* vals_in,
                          K* keys_out, uint32_t* vals_out, int64_t n, int pass,
@@ -379,9 +380,9 @@ __global__ void __launch_bounds__(kRadixBlock, kBlocks)
   __syncthreads();
   const int64_t tile = s_tile;
   if ((tile + 1) * kRadixTile <= n)
-    radix_tile<K, true>(keys_in, vals_in, keys_out, vals_out, n, tile, pass, total, look, skey, sval, sh);
+    radix_tile<K, true, kWait>(keys_in, vals_in, keys_out, vals_out, n, tile, pass, total, look, skey, sval, sh);
   else
-    radix_tile<K, false>(keys_in, vals_in, keys_out, vals_out, n, tile, pass, total, look, skey, sval, sh);
+    radix_tile<K, false, kWait>(keys_in, vals_in, keys_out, vals_out, n, tile, pass, total, look, skey, sval, sh);
 }
 
 __global__ void positions_kernel(int64_t n, uint32_t* v) {
@@ -399,7 +400,8 @@ int64_t radix_scratch_count(int64_t n) {
 
 template <typename K>
 static cudaError_t radix_sort_pairs_t(K** keys, uint32_t** vals, K** tmp_keys, uint32_t** tmp_vals, int64_t n, int bits,
-                                      bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches) {
+                                      bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches,
+                                      bool wait) {
   const int passes = radix_passes(n, bits);
   if (passes == 0) {
     if (!positions || n <= 0) return cudaSuccess;
@@ -413,14 +415,18 @@ static cudaError_t radix_sort_pairs_t(K** keys, uint32_t** vals, K** tmp_keys, u
   uint32_t* ticket = hist + kRadixPasses * 256;
   // two resident blocks (no spilled registers) while that is one wave, else more
   // in flight: 65,000 points 758 -> 732 us a call with two, 120M 2.59 -> 2.83 ms
-  const auto scatter = tiles <= 2 * 152 ? radix_scatter_kernel<K, 2> : radix_scatter_kernel<K, sizeof(K) == 4 ? 4 : 3>;
+  const auto scatter = !wait                ? radix_scatter_kernel<K, 2, false>
+                       : tiles <= 2 * kSMs ? radix_scatter_kernel<K, 2, true>
+                                           : radix_scatter_kernel<K, sizeof(K) == 4 ? 4 : 3, true>;
   RETURN_IF(cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)radix_scatter_smem<K>()));
   RETURN_IF(cudaMemsetAsync(scratch, 0, sizeof(int64_t) * (size_t)radix_scratch_count(n), stream));
-  launch_chained(radix_count_kernel<K>, (unsigned)(tiles < kCountBlocks ? tiles : kCountBlocks), kRadixBlock, 0, stream, *keys, n, passes, hist);
+  launch_chained(radix_count_kernel<K>, (unsigned)(tiles < kCountBlocks ? tiles : kCountBlocks), kRadixBlock, 0, stream,
+                 *keys, n, passes, hist);
   ++*launches;
   RETURN_IF(cudaGetLastError());
   for (int p = 0; p < passes; ++p) {
-    launch_chained(scatter, (unsigned)tiles, kRadixBlock, radix_scatter_smem<K>(), stream, *keys, p == 0 && positions ? nullptr : *vals, *tmp_keys, *tmp_vals, n, p, hist, ticket, look);
+    launch_chained(scatter, (unsigned)tiles, kRadixBlock, radix_scatter_smem<K>(), stream, *keys,
+                   p == 0 && positions ? nullptr : *vals, *tmp_keys, *tmp_vals, n, p, hist, ticket, look);
     ++*launches;
     RETURN_IF(cudaGetLastError());
     std::swap(*keys, *tmp_keys);
@@ -430,13 +436,17 @@ static cudaError_t radix_sort_pairs_t(K** keys, uint32_t** vals, K** tmp_keys, u
 }
 
 cudaError_t radix_sort_pairs(uint32_t** keys, uint32_t** vals, uint32_t** tmp_keys, uint32_t** tmp_vals, int64_t n,
-                             int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches) {
-  return radix_sort_pairs_t<uint32_t>(keys, vals, tmp_keys, tmp_vals, n, bits, positions, scratch, stream, launches);
+                             int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches,
+                             bool wait) {
+  return radix_sort_pairs_t<uint32_t>(keys, vals, tmp_keys, tmp_vals, n, bits, positions, scratch, stream, launches,
+                                      wait);
 }
 
 cudaError_t radix_sort_pairs64(uint64_t** keys, uint32_t** vals, uint64_t** tmp_keys, uint32_t** tmp_vals, int64_t n,
-                               int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches) {
-  return radix_sort_pairs_t<uint64_t>(keys, vals, tmp_keys, tmp_vals, n, bits, positions, scratch, stream, launches);
+                               int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches,
+                               bool wait) {
+  return radix_sort_pairs_t<uint64_t>(keys, vals, tmp_keys, tmp_vals, n, bits, positions, scratch, stream, launches,
+                                      wait);
 }
 
 // ============================================================================

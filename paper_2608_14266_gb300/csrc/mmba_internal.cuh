@@ -668,8 +668,9 @@ __device__ __forceinline__ float4 quat_mul_f(float4 p, float4 q) {
 }
 
 // 1 / d for a pivot d: the mantissa's binary32 reciprocal r (|1 - m r| < 2^-22)
-// and one step r + r (e + e^2), e = 1 - m r, of the cubic iteration, which
-// leaves e^3 < 2^-66; the exponent is put back in the bits.  Pivots so small or
+// and one step r + r (e + e^2), e = 1 - m r, of Chebyshev's iteration (the third
+// order one for 1 / m - x = 0), which leaves e^3 < 2^-66 and then rounds once
+// (ba_check_reciprocals); the exponent is put back in the bits.  Pivots so small or
 // large that the result is near the ends of the range, and those that are not
 // positive and finite (whose result is not used), divide.
 __device__ __forceinline__ double recip_pivot(double d) {

@@ -182,11 +182,15 @@ cudaError_t launch_decide(const double* cost_part, int64_t n_cost, const double*
 int64_t radix_scratch_count(int64_t n);
 // passes of a sort, one a digit: none for one element, which stays where it is
 inline int radix_passes(int64_t n, int bits) { return n <= 1 || bits <= 0 ? 0 : (bits + 7) / 8; }
+// wait = false: a tile does not wait for the counts of the tiles before it but
+// counts their keys itself, as it does when a wait runs out (a check's sort).
 cudaError_t radix_sort_pairs(uint32_t** keys, uint32_t** vals, uint32_t** tmp_keys, uint32_t** tmp_vals, int64_t n,
-                             int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches);
+                             int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches,
+                             bool wait = true);
 // The same for 64-bit keys (bits up to 64).
 cudaError_t radix_sort_pairs64(uint64_t** keys, uint32_t** vals, uint64_t** tmp_keys, uint32_t** tmp_vals, int64_t n,
-                               int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches);
+                               int bits, bool positions, int64_t* scratch, cudaStream_t stream, int64_t* launches,
+                               bool wait = true);
 // The library's stream-ordered memory pool of a device (freed memory stays
 // mapped for reuse); NULL if it cannot be created.
 cudaMemPool_t library_pool(int device);
