@@ -1253,7 +1253,8 @@ ba_status refresh(ba_batch* b) {
                            : whole  ? voxel_pass_blocks(h->L.n_voxels)
                                     : (h->L.n_voxels + 31) / 32);
     pre[(n + 1) + k + 1] = pre[(n + 1) + k] + h->L.n_scans;
-    pre[2 * (n + 1) + k + 1] = pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans, solve_lanes(group_scans[k / kGroupJobs]));
+    pre[2 * (n + 1) + k + 1] =
+        pre[2 * (n + 1) + k] + solve_blocks(h->L.n_scans, solve_lanes(group_scans[k / kGroupJobs]));
   }
   b->n_vblk = pre[n];
   b->n_sblk = pre[(n + 1) + n];

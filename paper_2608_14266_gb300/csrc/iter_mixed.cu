@@ -560,8 +560,8 @@ cudaError_t launch_wait_probe(int limit, int32_t* out, cudaStream_t stream) {
 
 cudaError_t launch_scan_table(int32_t n_scans, const double* poses2, const double* sref, float* stab2, int buf,
                               cudaStream_t stream) {
-  return launch_chained(scan_table_kernel, (unsigned)((n_scans + 127) / 128), 128, 0, stream, n_scans, poses2, sref, stab2,
-                        buf);
+  return launch_chained(scan_table_kernel, (unsigned)((n_scans + 127) / 128), 128, 0, stream, n_scans, poses2, sref,
+                        stab2, buf);
 }
 
 }  // namespace mmba

@@ -906,7 +906,8 @@ static int bit_width(uint64_t x) {
 static cudaError_t launch_obs_voxel(const LoadInput& in, int64_t v0, int64_t v1, int32_t* obs_vox, double* vscale,
                                     cudaStream_t stream, int64_t* launches) {
   if (v1 <= v0) return cudaSuccess;
-  launch_chained(obs_voxel_kernel, (unsigned)(((v1 - v0) * kVoxelLanes + 255) / 256), 256, 0, stream, in, v0, v1, obs_vox, vscale);
+  launch_chained(obs_voxel_kernel, (unsigned)(((v1 - v0) * kVoxelLanes + 255) / 256), 256, 0, stream, in, v0, v1,
+                 obs_vox, vscale);
   ++*launches;
   return cudaGetLastError();
 }
@@ -1083,17 +1084,19 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
     // the order, where it is kept, lands in its own buffer: the sort ends in the
     // buffer it starts from after an even number of passes, else in the other
     if (order) (radix_passes(no, scan_bits) % 2 == 0 ? vals : tv) = order;
-    launch_chained(scan_keys_kernel, (unsigned)((no + 255) / 256), 256, 0, stream, in, obs_vox, vrank, pbase, keys, vals, place);
+    launch_chained(scan_keys_kernel, (unsigned)((no + 255) / 256), 256, 0, stream, in, obs_vox, vrank, pbase, keys,
+                   vals, place);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
   RETURN_IF(radix_sort_pairs(&keys, &vals, &tk, &tv, no, scan_bits, false, scratch, stream, launches));
-  launch_chained(scan_off_kernel, (unsigned)((no + 1 + 255) / 256), 256, 0, stream, keys, no, in.n_scans, out->scan_off);
+  launch_chained(scan_off_kernel, (unsigned)((no + 1 + 255) / 256), 256, 0, stream, keys, no, in.n_scans,
+                 out->scan_off);
   ++*launches;
   RETURN_IF(cudaGetLastError());
   if (fill_f64) {  // the mixed path fills its own copy, se_vox included
-    launch_chained(fill_scan_major_kernel, (unsigned)((no + 255) / 256), 256, 0, stream, in, vals, obs_vox, vscale, vrank, out->se,
-                                                                             out->se_vox);
+    launch_chained(fill_scan_major_kernel, (unsigned)((no + 255) / 256), 256, 0, stream, in, vals, obs_vox, vscale,
+                   vrank, out->se, out->se_vox);
     ++*launches;
     RETURN_IF(cudaGetLastError());
   }
@@ -1107,7 +1110,8 @@ cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, 
   const int len_digits = bit_width((uint64_t)no);
   uint32_t* by_len = (uint32_t*)out->scans_by_len;
   uint32_t* other = tv;  // free: the scan-major order is in vals
-  launch_chained(scan_len_keys_kernel, (unsigned)((in.n_scans + 255) / 256), 256, 0, stream, out->scan_off, in.n_scans, no, keys);
+  launch_chained(scan_len_keys_kernel, (unsigned)((in.n_scans + 255) / 256), 256, 0, stream, out->scan_off, in.n_scans,
+                 no, keys);
   ++*launches;
   RETURN_IF(cudaGetLastError());
   if (radix_passes(in.n_scans, len_digits) % 2 != 0) std::swap(by_len, other);
@@ -1352,9 +1356,9 @@ __device__ __forceinline__ void aggregate_one(int64_t a, int64_t b, int sub, uns
 // kRounds: times a block's pairs of lanes take an observation each (of 128
 // kRounds observations in order of length).
 template <int kRounds>
-__global__ void __launch_bounds__(kOrderBlock, 2) aggregate_points_kernel(int64_t n_obs, const int64_t* __restrict__ off,
-                                                                       const double* __restrict__ pts,
-                                                                       double* __restrict__ out) {
+__global__ void __launch_bounds__(kOrderBlock, 2)
+    aggregate_points_kernel(int64_t n_obs, const int64_t* __restrict__ off, const double* __restrict__ pts,
+                            double* __restrict__ out) {
   constexpr int kGroups = kOrderBlock / kAggLanes, kItems = kGroups * kRounds;
   static_assert(kItems <= kOrderBlock, "the ordering takes one observation per thread");
   __shared__ int s_cnt[32], s_order[kOrderBlock];

@@ -493,10 +493,10 @@ __device__ __forceinline__ void fill_scan_one(int64_t q, int64_t o, int64_t n_ob
 // [i0, i1); order[q] = its observation (a pipelined load fills each chunk's
 // entries as the chunk is set up)
 constexpr int kFillScanThreads = 256;
-__global__ void __launch_bounds__(kFillScanThreads) fill_scan_mixed_kernel(int64_t n_obs, const uint32_t* qlist, int64_t i0, int64_t i1,
-                                       const uint32_t* order, const int2* place, const float4* vanchor,
-                                       const int64_t* slice_off, const float4* ve32, const int64_t* vstart, const float4* staging,
-                                       float* se32, int32_t* se_vox) {
+__global__ void __launch_bounds__(kFillScanThreads)
+    fill_scan_mixed_kernel(int64_t n_obs, const uint32_t* qlist, int64_t i0, int64_t i1, const uint32_t* order,
+                           const int2* place, const float4* vanchor, const int64_t* slice_off, const float4* ve32,
+                           const int64_t* vstart, const float4* staging, float* se32, int32_t* se_vox) {
   grid_wait();
   grid_launch_next();
   __shared__ float4 slots[kFillScanThreads / 32][96];
@@ -553,8 +553,9 @@ cudaError_t build_mixed_scan_major(const LoadInput& in, const LayoutBuffers& lb,
                                    const float4* staging, const uint32_t* qlist, int64_t i0, int64_t i1,
                                    cudaStream_t stream, int64_t* launches) {
   if (i1 <= i0) return cudaSuccess;
-  launch_chained(fill_scan_mixed_kernel, (unsigned)((i1 - i0 + kFillScanThreads - 1) / kFillScanThreads), kFillScanThreads, 0, stream, in.n_obs, qlist, i0, i1, lb.scan_order, lb.place, mb.vanchor, lb.slice_off, mb.ve32, lb.vstart, staging, mb.se32,
-      mb.se_vox);
+  launch_chained(fill_scan_mixed_kernel, (unsigned)((i1 - i0 + kFillScanThreads - 1) / kFillScanThreads),
+                 kFillScanThreads, 0, stream, in.n_obs, qlist, i0, i1, lb.scan_order, lb.place, mb.vanchor,
+                 lb.slice_off, mb.ve32, lb.vstart, staging, mb.se32, mb.se_vox);
   ++*launches;
   return cudaGetLastError();
 }
@@ -577,8 +578,8 @@ cudaError_t build_mixed(const LoadInput& in, const LayoutBuffers& lb, const doub
   cur.poses = poses2;  // buffer 0
   const int64_t nv = in.n_voxels;
   if (nv > 0) {
-    launch_chained(voxel_frames_kernel, frame_blocks(nv), 128, 0, stream, cur, 0, nv, mb.sref, lb.vrank, lb.vscale, mb.vstate,
-                                                               mb.vanchor, mb.planes32_2);
+    launch_chained(voxel_frames_kernel, frame_blocks(nv), 128, 0, stream, cur, 0, nv, mb.sref, lb.vrank, lb.vscale,
+                   mb.vstate, mb.vanchor, mb.planes32_2);
     ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // every slot, padding included, by sorted position (coalesced writes)
@@ -586,7 +587,8 @@ cudaError_t build_mixed(const LoadInput& in, const LayoutBuffers& lb, const doub
     const int per = fill_rows(in.n_obs);
     const unsigned row_blocks =
         (unsigned)std::min<int64_t>(std::max<int64_t>((lb.max_len + per - 1) / per, 1), 65535);
-    launch_chained(fill_sell_mixed_kernel, dim3((unsigned)((p1 + 127) / 128), row_blocks), 128, 0, stream, cur, lb.vperm, lb.vlen, lb.slice_off, nv, 0, p1, mb.sref, mb.vanchor, mb.ve32, per);
+    launch_chained(fill_sell_mixed_kernel, dim3((unsigned)((p1 + 127) / 128), row_blocks), 128, 0, stream, cur,
+                   lb.vperm, lb.vlen, lb.slice_off, nv, 0, p1, mb.sref, mb.vanchor, mb.ve32, per);
     ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

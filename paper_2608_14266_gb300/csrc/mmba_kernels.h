@@ -299,7 +299,8 @@ struct LayoutBuffers {
 // With defer_scale the clusters are not read (vscale is left for
 // launch_vscale, voxel range by voxel range, as the clusters arrive).
 cudaError_t build_layout(const LoadInput& in, const float4* t32, uint32_t* box, int max_len, bool fill_f64,
-                         bool defer_scale, Allocator keep, Allocator temp, LayoutBuffers* out, cudaStream_t stream, int64_t* launches);
+                         bool defer_scale, Allocator keep, Allocator temp, LayoutBuffers* out, cudaStream_t stream,
+                         int64_t* launches);
 cudaError_t launch_vscale(const LoadInput& in, int64_t v0, int64_t v1, double* vscale, cudaStream_t stream,
                           int64_t* launches);
 // A load that copies its clusters in chunks of observations [o[k], o[k + 1])

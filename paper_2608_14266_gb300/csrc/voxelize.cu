@@ -194,7 +194,7 @@ constexpr int kKeyRounds = 4;  // at most so many times kKeyThreads kKeyPoints c
 // starting at global point p0 (pts, keys and pscan are indexed within the
 // batch); a thread keeps its scan until a point passes the scan's end.
 //
-// Bound: HBM, 24 bytes read and 12 written a point.  120M points: 0.93 ms (5.2
+// Bound: HBM, 24 bytes read and 12 written a point.  120M points: 0.85 ms (5.1
 // TB/s); 2.63 ms with the index in FP64 (9 multiply-adds and 3 additions a
 // point, 88% of the FP64 pipe).
 __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, const int64_t* __restrict__ spo,
@@ -202,7 +202,8 @@ __global__ void __launch_bounds__(kKeyThreads) l1_keys_kernel(int32_t n_scans, c
                                                               const double* __restrict__ poses,
                                                               const double* __restrict__ sposes,
                                                               const ScanFix* __restrict__ fix, int kp, double d,
-                                                              int rounds, int64_t p0, int64_t n, uint64_t* __restrict__ keys,
+                                                              int rounds, int64_t p0, int64_t n,
+                                                              uint64_t* __restrict__ keys,
                                                               int32_t* __restrict__ pscan, long long* bad, int* bbox) {
   grid_launch_next();
   int mn[3] = {INT_MAX, INT_MAX, INT_MAX}, mx[3] = {INT_MIN, INT_MIN, INT_MIN};
@@ -1034,7 +1035,8 @@ __global__ void __launch_bounds__(kOrderBlock) merge_kernel(int64_t np, const in
   __shared__ int s_cnt[32], s_order[kOrderBlock];
   const int64_t g0 = (int64_t)blockIdx.x * kOrderBlock + threadIdx.x;
   const int64_t len0 = g0 < np ? start[g0 + 1] - start[g0] : 0;
-  const int64_t g = (int64_t)blockIdx.x * kOrderBlock + block_order_by_key((int)(len0 < 31 ? len0 : 31), s_cnt, s_order);
+  const int64_t g =
+      (int64_t)blockIdx.x * kOrderBlock + block_order_by_key((int)(len0 < 31 ? len0 : 31), s_cnt, s_order);
   if (g >= np) return;
   const int64_t a = start[g], b = start[g + 1];
   Piece acc;
@@ -1471,8 +1473,8 @@ ba_status group_starts(int64_t n, const K* keys, const uint32_t* vals, const int
   int64_t* base = tmp.get<int64_t>(nw + 1);
   int64_t* scr = tmp.get<int64_t>(scan_scratch_count(nw + 1));
   if (!mask || !base || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  launch_chained(head_mask_kernel<K>, blocks_for((nw + kHeadWords - 1) / kHeadWords, 8), 256, 0, st, n, keys, vals, scan, mask,
-                                                                                         base);
+  launch_chained(head_mask_kernel<K>, blocks_for((nw + kHeadWords - 1) / kHeadWords, 8), 256, 0, st, n, keys, vals,
+                 scan, mask, base);
   VCK(cudaGetLastError(), "voxelize");
   VCK(cudaMemsetAsync(base + nw, 0, sizeof(int64_t), st), "voxelize");
   VCK(exclusive_scan_i64(base, nw + 1, scr, st, launches), "voxelize");
@@ -1525,7 +1527,8 @@ ba_status level1(int64_t n, const uint64_t* raw, const int32_t* pscan, const dou
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(n));
   if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
   tm.begin(BA_VOX_SORT);
-  launch_chained(repack_kernel<K>, blocks_for(n, kRepackThreads * kRepackItems), kRepackThreads, 0, st, n, raw, L.pk, keys);
+  launch_chained(repack_kernel<K>, blocks_for(n, kRepackThreads * kRepackItems), kRepackThreads, 0, st, n, raw, L.pk,
+                 keys);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize keys");
   // stable by key over points in scan order: groups ordered by (key, scan, point)
@@ -1607,8 +1610,8 @@ ba_status level_up(const Level& ch, Level& P, int32_t n_scans, Buf& tmp, cudaStr
   P.key = tmp.get<uint64_t>(np);
   P.scan = tmp.get<int32_t>(np);
   if (!P.c || !P.key || !P.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  launch_chained(merge_kernel<K>, blocks_for(np, kOrderBlock), kOrderBlock, 0, st, np, pst, cv, ch.c, k2, ch.scan, P.c, P.key,
-                                                                       P.scan);
+  launch_chained(merge_kernel<K>, blocks_for(np, kOrderBlock), kOrderBlock, 0, st, np, pst, cv, ch.c, k2, ch.scan, P.c,
+                 P.key, P.scan);
   ++*launches;
   VCK(cudaGetLastError(), "voxelize merge");
   return BA_OK;
@@ -1644,7 +1647,8 @@ ba_status l1_range(const L1Ctx& c, int64_t p0, int64_t m, const double* pts, boo
   VCK(cudaMemcpyAsync(c.bbox, bb_init, sizeof bb_init, cudaMemcpyHostToDevice, c.st), "voxelize");
   VCK(cudaMemcpyAsync(c.bad + 2, &none, sizeof none, cudaMemcpyHostToDevice, c.st), "voxelize");
   const int64_t key_blocks = std::min<int64_t>(blocks_for(m, kKeyThreads * kKeyPoints), (int64_t)c.n_sm * 8);
-  const int rounds = (int)std::min<int64_t>(std::max<int64_t>(m / (key_blocks * kKeyThreads * kKeyPoints), 1), kKeyRounds);
+  const int rounds =
+      (int)std::min<int64_t>(std::max<int64_t>(m / (key_blocks * kKeyThreads * kKeyPoints), 1), kKeyRounds);
   c.tm->begin(BA_VOX_KEYS);
   l1_keys_kernel<<<(unsigned)key_blocks, kKeyThreads, 0, c.st>>>(c.n_scans, c.spo, pts, c.T, c.sposes, c.fix, c.kp,
                                                                  c.d, rounds, p0, m, raw, pscan, c.bad + 2, c.bbox);
@@ -1725,7 +1729,8 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
   uint32_t* tvals = tmp.get<uint32_t>(m);
   int64_t* scr = tmp.get<int64_t>(radix_scratch_count(m));
   if (!keys || !tkeys || !vals || !tvals || !scr) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  launch_chained(repack_kernel<K>, blocks_for(m, kRepackThreads * kRepackItems), kRepackThreads, 0, c.st, m, raw_all, L.pk, keys);
+  launch_chained(repack_kernel<K>, blocks_for(m, kRepackThreads * kRepackItems), kRepackThreads, 0, c.st, m, raw_all,
+                 L.pk, keys);
   ++*c.launches;
   VCK(cudaGetLastError(), "voxelize merge");
   VCK(sort_keys(&keys, &vals, &tkeys, &tvals, m, pack_bits(L.pk), true, scr, c.st, c.launches), "voxelize sort");
@@ -1735,7 +1740,8 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
     L.key = out.get<uint64_t>(m);
     L.scan = out.get<int32_t>(m);
     if (!L.c || !L.key || !L.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-    launch_chained(gather_clusters_kernel<K>, blocks_for(m), 256, 0, c.st, m, vals, keys, c_all, scan_all, L.c, L.key, L.scan);
+    launch_chained(gather_clusters_kernel<K>, blocks_for(m), 256, 0, c.st, m, vals, keys, c_all, scan_all, L.c, L.key,
+                   L.scan);
     ++*c.launches;
     VCK(cudaGetLastError(), "voxelize merge");
     return BA_OK;
@@ -1749,8 +1755,8 @@ ba_status assemble_batches(const L1Ctx& c, int64_t m, const double* c_all, const
   L.key = out.get<uint64_t>(ng);
   L.scan = out.get<int32_t>(ng);
   if (!L.c || !L.key || !L.scan) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
-  launch_chained(merge_kernel<K>, blocks_for(ng, kOrderBlock), kOrderBlock, 0, c.st, ng, start, vals, c_all, keys, scan_all,
-                                                                          L.c, L.key, L.scan);
+  launch_chained(merge_kernel<K>, blocks_for(ng, kOrderBlock), kOrderBlock, 0, c.st, ng, start, vals, c_all, keys,
+                 scan_all, L.c, L.key, L.scan);
   ++*c.launches;
   VCK(cudaGetLastError(), "voxelize merge");
   return BA_OK;
@@ -2007,8 +2013,8 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
     // fixed point of the indices: 1 / d < 2^e
     // (far out of that range no pose fits and every point takes the FP64 path)
     const int e = std::min(std::max(std::ilogb(1.0 / cfg->voxel_size), -200), 200) + 1, kS = 30 - e, kp = 18 + e;
-    launch_chained(scaled_poses_kernel, blocks_for(n_scans, 128), 128, 0, st, n_scans, T, 1.0 / cfg->voxel_size, kS, kp, sposes,
-                                                                  fix);
+    launch_chained(scaled_poses_kernel, blocks_for(n_scans, 128), 128, 0, st, n_scans, T, 1.0 / cfg->voxel_size, kS, kp,
+                   sposes, fix);
     ++launches;
     int n_sm = 0;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
@@ -2101,12 +2107,13 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
       n_close = tmp.get<unsigned long long>(1);
       if (!rel || !rsr || !close || !n_close) return vfail(BA_ERR_OOM, "voxelize: out of device memory");
       VCK(cudaMemsetAsync(n_close, 0, sizeof(unsigned long long), st), "voxelize");
-      launch_chained(world_terms_kernel, blocks_for(L.nc, kTermThreads), kTermThreads, 0, st, L.nc, L.c, L.scan, T, pos, L.vstart, rel, rsr);
+      launch_chained(world_terms_kernel, blocks_for(L.nc, kTermThreads), kTermThreads, 0, st, L.nc, L.c, L.scan, T, pos,
+                     L.vstart, rel, rsr);
       ++launches;
     }
     // tau rounded to FP32 moves the test by 2^-24 tau lambda1, inside the error band
-    launch_chained(select_kernel, blocks_for(L.nv), 256, 0, st, L.nv, L.vstart, rel, rsr, cfg->tau > 0.0 ? (float)cfg->tau : 0.0f,
-                                                   cfg->min_obs, keep_obs[k], keep_vox[k], close, n_close);
+    launch_chained(select_kernel, blocks_for(L.nv), 256, 0, st, L.nv, L.vstart, rel, rsr,
+                   cfg->tau > 0.0 ? (float)cfg->tau : 0.0f, cfg->min_obs, keep_obs[k], keep_vox[k], close, n_close);
     ++launches;
     if (cfg->tau > 0.0) {
       int n_sm = 0;
@@ -2154,9 +2161,8 @@ ba_status ba_voxelize(const ba_voxelize_config* cfg, int32_t n_scans, const int6
     const Level& L = lv[k];
     if (L.nv == 0) continue;
     tm.begin(BA_VOX_EMIT);
-    launch_chained(emit_kernel, blocks_for(L.nv), 256, 0, st, L.nv, L.vstart, L.key, L.pk, L.scan, L.c, obs_pos[k], vox_pos[k],
-                                                 keep_vox[k], k + 1, vb, ob, v->voxel_off, v->obs_scan, v->agg,
-                                                 v->level, v->index);
+    launch_chained(emit_kernel, blocks_for(L.nv), 256, 0, st, L.nv, L.vstart, L.key, L.pk, L.scan, L.c, obs_pos[k],
+                   vox_pos[k], keep_vox[k], k + 1, vb, ob, v->voxel_off, v->obs_scan, v->agg, v->level, v->index);
     tm.end();
     ++launches;
     VCK(cudaGetLastError(), "voxelize emit");
