@@ -50,8 +50,9 @@ inline int64_t voxel_pass_f64_blocks(int64_t n_voxels, int64_t n_obs) {
 // voxel to one thread, which then forms the partial sums of 4, 8 or 16 in turn:
 // where it fills the GPU.  Us a pass, a slice of 32 voxels to a block / so: 60 jobs of
 // 2,000 voxels of 2-3 observations 290 / 154, of 20-30 570 / 514; 128 jobs of 500
-// voxels 215 / 178; but 16 jobs of 100 43 / 64.
-inline bool batch_voxels_whole(int64_t n_voxels) { return n_voxels >= 60000; }
+// voxels 215 / 178; but 16 jobs of 100 43 / 64.  (From kShortVoxels on, so that a
+// job which alone has one thread to a voxel has it in every batch.)
+inline bool batch_voxels_whole(int64_t n_voxels) { return n_voxels >= kShortVoxels; }
 // Lanes per scan in the solve kernel, for a launch of n_scans scans in all (a
 // handle's, or a batch group's): 8 while the GPU has few warps to each of its
 // 608 SM sub-partitions, else 1; the results have the same bits.  Both sides,

@@ -53,8 +53,9 @@ def test_batches_give_the_bits_of_jobs_alone(mm):
             ba.load_observations(ns, off, scan, agg, pose)
             st = ba.iterate(3)
             alone.append((ba.poses().copy(), st["cost"], st["mu"], ba.planes()))
-    # 24,255 voxels (below a large batch's 60,000), then with those of 50,000 each
-    for pick in (range(len(JOBS)), range(len(jobs))):
+    # 24,255 voxels (below a large batch's 50,000), with those of 50,000 each, and
+    # two of the latter by themselves
+    for pick in (range(len(JOBS)), range(len(jobs)), [len(JOBS)], [len(JOBS) + 1]):
         bas = [mm.BundleAdjuster() for _ in pick]
         with mm.Batch() as b:
             for ba, k in zip(bas, pick):
